@@ -153,24 +153,15 @@ class _State:
     pass
 
 
-def prepare(case, seed):
-    """Tokens, parameters, gradients and the layer's buffers on the GPU, from the seed alone."""
-    c, s = case, _State()
+def _inputs(c, seed):
+    """Tokens, expert embeddings, weights and, for a training step, the output's gradient (else None)."""
     act = torch.float32 if c["dtype"] == "f32" else torch.bfloat16
     wt = torch.float32 if c["master"] else act
     T, d, E, h = c["T"], c["d"], c["E"], c["h"]
     gen = torch.Generator(device="cuda")
     gen.manual_seed(seed)
-    s.step = c["direction"] == "step"
-    s.cfg = etr.make_config(T=T, d=d, D=c["D"], E=E, k=c["k"], h=h, capacity=_capacity(c),
-                            dtype=etr.F32 if c["dtype"] == "f32" else etr.BF16,
-                            weight_dtype=etr.F32 if wt == torch.float32 else etr.BF16,
-                            mode=etr.MODE_ECR if c["mode"] == "ecr" else etr.MODE_TCR,
-                            adaptive=c["delta_max"] > 0.0,
-                            delta_max_override=c["delta_max"] if c["delta_max"] > 0.0 else -1.0,
-                            gate_mode=etr.GATE_SOFTMAX if c["gate"] == "softmax" else etr.GATE_AFFINITY)
-    s.R = _expert_embeddings(E, d // c["D"], seed)
-    s.X = _tokens(c, s.R, gen, act)
+    R = _expert_embeddings(E, d // c["D"], seed)
+    X = _tokens(c, R, gen, act)
 
     def weight(*shape):
         w = torch.empty(*shape, dtype=wt, device="cuda")
@@ -178,11 +169,27 @@ def prepare(case, seed):
             w[i] = torch.randn(*shape[1:], generator=gen, device="cuda") / math.sqrt(d)
         return w
 
-    s.W1g, s.W1u, s.W2 = weight(E, h, d), weight(E, h, d), weight(E, d, h)
+    W1g, W1u, W2 = weight(E, h, d), weight(E, h, d), weight(E, d, h)
+    dY = torch.randn(T, d, generator=gen, device="cuda").to(act) if c["direction"] == "step" else None
+    return X, R, W1g, W1u, W2, dY
+
+
+def prepare(case, seed):
+    """Tokens, parameters, gradients and the layer's buffers on the GPU, from the seed alone."""
+    c, s = case, _State()
+    T, d, E, h = c["T"], c["d"], c["E"], c["h"]
+    s.step = c["direction"] == "step"
+    s.X, s.R, s.W1g, s.W1u, s.W2, s.dY = _inputs(c, seed)
+    s.cfg = etr.make_config(T=T, d=d, D=c["D"], E=E, k=c["k"], h=h, capacity=_capacity(c),
+                            dtype=etr.F32 if c["dtype"] == "f32" else etr.BF16,
+                            weight_dtype=etr.F32 if s.W2.dtype == torch.float32 else etr.BF16,
+                            mode=etr.MODE_ECR if c["mode"] == "ecr" else etr.MODE_TCR,
+                            adaptive=c["delta_max"] > 0.0,
+                            delta_max_override=c["delta_max"] if c["delta_max"] > 0.0 else -1.0,
+                            gate_mode=etr.GATE_SOFTMAX if c["gate"] == "softmax" else etr.GATE_AFFINITY)
     s.buf = etr.LayerBuffers(s.cfg)
     s.Y = torch.empty_like(s.X)
     if s.step:
-        s.dY = torch.randn(T, d, generator=gen, device="cuda").to(act)
         s.dX, s.dR = torch.empty_like(s.X), torch.empty_like(s.R)
         s.dW1g, s.dW1u, s.dW2 = torch.empty_like(s.W1g), torch.empty_like(s.W1u), torch.empty_like(s.W2)
     return s
@@ -195,6 +202,58 @@ def run(s):
         return {"Y": s.Y}
     etr.layer_backward(s.cfg, s.X, s.R, s.W1g, s.W1u, s.W2, s.dY, s.buf, s.dX, s.dR, s.dW1g, s.dW1u, s.dW2)
     return {"Y": s.Y, "dX": s.dX, "dR": s.dR, "dW1g": s.dW1g, "dW1u": s.dW1u, "dW2": s.dW2}
+
+
+def exact(case, seed):
+    """What `run` returns for these inputs, in 64 bits throughout (routing included)."""
+    c = case
+    T, d, D, E, k = c["T"], c["d"], c["D"], c["E"], c["k"]
+    m, C, f64 = d // D, min(_rows_per_expert(c), T), torch.float64
+    X, R, W1g, W1u, W2, dY = _inputs(c, seed)
+    x, R = X.to(f64), R.to(f64)
+    z, a, b = x.view(T, m, D).mean(dim=2), x.norm(dim=1), R.norm(dim=1)
+    delta = math.sqrt(D) * (z @ R.T) / (a[:, None] * b[None, :])
+    score = delta
+    if c["mode"] == "tcr":                     # an expert's candidates: the tokens that have it among their k best
+        best = delta.topk(k, dim=1).indices
+        score = torch.full_like(delta, -math.inf).scatter_(1, best, delta.gather(1, best))
+    gates = torch.softmax(delta, dim=1) if c["gate"] == "softmax" else delta
+    rows = []
+    for i in range(E):
+        val, tok = score[:, i].topk(C)
+        rows.append(tok[val > -math.inf].sort().values)
+
+    silu = torch.nn.functional.silu
+    Y = torch.zeros(T, d, dtype=f64, device="cuda")
+    step = c["direction"] == "step"
+    if step:
+        dY = dY.to(f64)
+        dX, dgate = torch.zeros_like(Y), torch.zeros_like(delta)
+        dW = [torch.zeros(w.shape, dtype=f64, device="cuda") for w in (W1g, W1u, W2)]
+    for i, t in enumerate(rows):
+        wg, wu, w2 = W1g[i].to(f64), W1u[i].to(f64), W2[i].to(f64)
+        xp, gt = x[t], gates[t, i][:, None]
+        g, u = xp @ wg.T, xp @ wu.T
+        hid = silu(g) * u
+        o = hid @ w2.T
+        Y.index_add_(0, t, gt * o)
+        if not step:
+            continue
+        dgate[t, i] = (dY[t] * o).sum(dim=1)
+        do = gt * dY[t]
+        dhid, sg = do @ w2, torch.sigmoid(g)
+        dg, du = dhid * u * sg * (1.0 + g * (1.0 - sg)), dhid * g * sg
+        dX.index_add_(0, t, dg @ wg + du @ wu)
+        dW[0][i], dW[1][i], dW[2][i] = dg.T @ xp, du.T @ xp, do.T @ hid
+    if not step:
+        return {"Y": Y}
+    dd = dgate                                 # gradient of the affinities; the selection itself has none
+    if c["gate"] == "softmax":
+        dd = gates * (dgate - (gates * dgate).sum(dim=1, keepdim=True))
+    w = dd * math.sqrt(D) / (a[:, None] * b[None, :])
+    dX += ((w @ R) / D).repeat_interleave(D, dim=1) - ((dd * delta).sum(dim=1) / a ** 2)[:, None] * x
+    dR = w.T @ z - ((dd * delta).sum(dim=0) / b ** 2)[:, None] * R
+    return {"Y": Y, "dX": dX, "dR": dR, "dW1g": dW[0], "dW1u": dW[1], "dW2": dW[2]}
 
 
 def work(case):
