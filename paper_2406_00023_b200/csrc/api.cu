@@ -46,6 +46,9 @@ static bool use_tc(const etr_config* c) {
   return c->dtype == ETR_BF16 && tc_available();
 }
 
+// fp32 layers: the tensor-core GEMMs on split operands, unless the CUDA-core ones are asked for.
+static bool use_tf32x3(const etr_config* c) { return c->dtype == ETR_F32 && c->gemm_impl == ETR_GEMM_AUTO && tc_available(); }
+
 // Token rearrangement fused into the GEMM operand fetch (layer calls, tensor-core path only).
 static bool fuse_dispatch(const etr_config* c) {
   return use_tc(c) && c->fuse_dispatch == ETR_FUSE_ON;
@@ -298,6 +301,8 @@ etr_status etr_expert_ffn(const etr_config* c, const etr_route* route, const voi
     return tc_ffn_forward(&g, route, Xp, nullptr, w.W1g, w.W1u, w.W2, G, U, H, O, stats, ws, nullptr,
                           (cudaStream_t)stream);
   }
+  if (use_tf32x3(c))
+    return tf32x3_ffn_forward(&g, route, Xp, w.W1g, w.W1u, w.W2, G, U, H, O, stats, (cudaStream_t)stream);
   return simt_ffn_forward(&g, route, Xp, w.W1g, w.W1u, w.W2, G, U, H, O, (cudaStream_t)stream);
 }
 
@@ -335,6 +340,9 @@ static etr_status expert_ffn_bwd(const etr_config* c, const etr_route* route, co
     return tc_ffn_backward(&g, route, dO, Xp, nullptr, G, U, H, w.W1g, w.W1u, w.W2, dG, dU, dXp, dW1g, dW1u, dW2,
                            stats, ws, (cudaStream_t)stream);
   }
+  if (use_tf32x3(c))
+    return tf32x3_ffn_backward(&g, route, dO, Xp, G, U, H, w.W1g, w.W1u, w.W2, dG, dU, dXp, dW1g, dW1u, dW2, stats,
+                               (cudaStream_t)stream);
   return simt_ffn_backward(&g, route, dO, Xp, G, U, H, w.W1g, w.W1u, w.W2, dG, dU, dXp, dW1g, dW1u, dW2,
                            (cudaStream_t)stream);
 }

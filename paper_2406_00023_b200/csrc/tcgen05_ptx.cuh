@@ -44,6 +44,14 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t* r) {
 }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+// One lane of a converged warp, the same every time.  The compiler knows the branch on it for uniform: an MMA or a
+// copy behind it issues every 50 cycles, behind a test of the lane number every 94 (MMAs of 16 and 32 columns).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 // Shared-memory matrix descriptor, 128-byte swizzle, tile base 1024-byte aligned.
 __device__ __forceinline__ uint64_t make_smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
   uint64_t d = (uint64_t)((addr & 0x3FFFFu) >> 4);

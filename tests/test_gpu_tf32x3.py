@@ -1,0 +1,94 @@
+"""The fp32 grouped GEMMs on the tensor cores, stage by stage against 64-bit products of the same inputs: sizes at
+the edges of the 128-row and 128- or 64-column tiles and of the 32-wide K blocks, row counts from none to a full
+buffer, and values at the ends of the number range.
+
+Tolerance (relative 2-norm): a value split into two tf32 parts is off by at most 2^-23, the dropped lo*lo by 2^-22 of
+a product at most, and a chain of eight MMAs drops at most eight last bits of its sum (2^-23 each): 1e-6 holds all
+of it with the growth of the running sum's roundings over the K blocks (2^-24 sqrt(K / 64) at K <= 2000)."""
+import math
+
+import pytest
+import torch
+
+from paper_2406_00023_b200 import etr
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-6
+
+
+def rel(got, ref):
+    n = float(ref.norm())
+    return float((got.double() - ref).norm()) / n if n else float(got.double().norm())
+
+
+def layer(E, d, h, cap, counts, seed=0):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    cfg = etr.make_config(T=max(8, cap), d=d, D=1, E=E, k=1, h=h, capacity=cap, dtype=etr.F32, mode=etr.MODE_TCR)
+    assert etr.validate(cfg) == etr.OK
+    b = etr.LayerBuffers(cfg)
+    b.block.fill_(0xFF)                                      # NaN wherever nothing is written
+    b.stats.zero_()
+    b.counts.copy_(torch.tensor(counts, dtype=torch.int32))
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")  # noqa: E731
+    W = [rnd(E, h, d) / math.sqrt(d), rnd(E, h, d) / math.sqrt(d), rnd(E, d, h) / math.sqrt(d)]
+    Cs = etr.c_stride(cfg)
+    for t in (b.Xp, b.dO):
+        v = t.view(E, Cs, d)
+        for i, n in enumerate(counts):
+            v[i, :n] = rnd(n, d)
+            v[i, n:(n + 127) // 128 * 128] = 0.0
+    return cfg, b, W
+
+
+@pytest.mark.parametrize("E,d,h,cap,counts", [
+    (3, 8, 8, 5, (5, 0, 1)),                                 # one partial K block, one partial tile
+    (4, 40, 72, 129, (129, 128, 127, 0)),                    # K blocks and column tiles end inside
+    (5, 256, 1000, 300, (300, 33, 1, 256, 65)),              # several row tiles, 64- and 128-column tiles
+    (2, 1096, 136, 700, (700, 641)),
+    (24, 512, 768, 257, tuple((37 * i) % 258 for i in range(24))),       # more tiles than SMs
+])
+def test_stages_against_64_bits(E, d, h, cap, counts):
+    cfg, b, W = layer(E, d, h, cap, counts)
+    dW = [torch.full_like(w, float("nan")) for w in W]
+    etr.expert_ffn(cfg, b.route, b.Xp, *W, b.G, b.U, b.H, b.O, b.c.stats, b.c.ws)
+    etr.expert_ffn_bwd(cfg, b.route, b.dO, b.Xp, b.G, b.U, b.H, *W, b.dG, b.dU, b.dXp, *dW, b.c.stats, b.c.ws)
+    assert b.read_stats().error_word == 0
+    Cs = etr.c_stride(cfg)
+    for i, n in enumerate(counts):
+        pad = (n + 127) // 128 * 128
+        x, G, U, H, O, dO, dG, dU, dXp = (t.view(E, Cs, -1)[i].double() for t in
+                                          (b.Xp, b.G, b.U, b.H, b.O, b.dO, b.dG, b.dU, b.dXp))
+        for t in (G, U, H, O, dG, dU, dXp):
+            assert bool((t[n:pad] == 0).all()) and bool(t[pad:].isnan().all())
+        x, G, U, H, O, dO, dG, dU, dXp = (t[:n] for t in (x, G, U, H, O, dO, dG, dU, dXp))
+        wg, wu, w2 = (w[i].double() for w in W)
+        s, dh = torch.sigmoid(G), dO @ w2
+        for name, got, ref in (("G", G, x @ wg.T), ("U", U, x @ wu.T), ("H", H, G * s * U), ("O", O, H @ w2.T),
+                               ("dG", dG, dh * U * s * (1 + G * (1 - s))), ("dU", dU, dh * G * s),
+                               ("dXp", dXp, dG @ wg + dU @ wu), ("dW1g", dW[0][i], dG.T @ x),
+                               ("dW1u", dW[1][i], dU.T @ x), ("dW2", dW[2][i], dO.T @ H)):
+            assert rel(got, ref) <= TOL, (name, i, rel(got, ref))
+
+
+def test_ends_of_the_number_range():
+    """An infinity gives the infinities that fp32 products give, a NaN its row, the largest and the smallest finite
+    values their products; the other rows of the tile are as if these were not there."""
+    cfg, b, W = layer(1, 64, 64, 128, (128,))
+    x = b.Xp.view(128, 64)
+    x[3, 7], x[4, 9], x[5, 63] = math.inf, -math.inf, math.nan
+    x[6] = 0.0
+    x[6, 1] = torch.finfo(torch.float32).max
+    x[7] = 0.0
+    x[7, 2] = 1e-30
+    etr.expert_ffn(cfg, b.route, b.Xp, *W, b.G, b.U, b.H, b.O, b.c.stats, b.c.ws)
+    assert b.read_stats().error_word == 0
+    ref = x.double() @ W[0][0].double().T
+    G = b.G.view(128, 64).double()
+    for r in (3, 4):
+        assert bool((G[r] == ref[r]).all())                  # +-inf by the weight's sign
+    assert bool(G[5].isnan().all())
+    for r in (6, 7):
+        ok = ref[r].abs() < 3e38
+        assert bool((G[r][ok] - ref[r][ok]).abs().le(1e-6 * ref[r][ok].abs()).all())
+    rest = [r for r in range(128) if r not in (3, 4, 5, 6, 7)]
+    assert rel(G[rest], ref[rest]) <= TOL
