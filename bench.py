@@ -83,7 +83,6 @@ def algorithmic_work(w, rows, kernel, unrouted=0):
         "select_token_side_kernel": (2 * T * E * 4, "bytes"),
         "select_expert_side_kernel": (T * E * 4 + rows * 8, "bytes"),
         "csr_count_kernel": (T * E * 4, "bytes"),
-        "csr_scan_kernel": (T * 8, "bytes"),
         "csr_fill_kernel": (T * E * 4 + rows * 4, "bytes"),
         "dispatch_kernel": (2 * rows * d * b, "bytes"),
         "combine_kernel": (rows * d * b + T * d * b, "bytes"),

@@ -140,8 +140,11 @@ __device__ inline void pool_token(const T* __restrict__ x, float* __restrict__ z
 // adjacent pieces whose partial sums meet through xor-shuffles.  Pure HBM streaming.
 template <class T, int PPG>
 __global__ void __launch_bounds__(256)
-grap_pool_kernel(const T* __restrict__ X, float* __restrict__ Z, float* __restrict__ xnorm, int Ttok,
-                 int d, int D, int m) {
+grap_pool_kernel(const T* __restrict__ X, float* __restrict__ Z, float* __restrict__ xnorm,
+                 etr_stats* zero_stats, int Ttok, int d, int D, int m) {
+  grid_sync();
+  if (zero_stats != nullptr && blockIdx.x == 0 && threadIdx.x < sizeof(etr_stats) / 4)
+    reinterpret_cast<uint32_t*>(zero_stats)[threadIdx.x] = 0;
   constexpr int PE = Raw16<T>::ELEMS;
   constexpr int BATCH = 8;
   const int lane = threadIdx.x & 31;
@@ -190,6 +193,7 @@ affinity_score_kernel(const float* __restrict__ Z, const float* __restrict__ xno
                       const float* __restrict__ R, float* __restrict__ delta,
                       float* __restrict__ rnorm, etr_stats* stats, int Ttok, int D, int E, int m,
                       int ldm) {
+  grid_sync();
   extern __shared__ __align__(16) float smem[];
   constexpr int EROWS = 32 * EPL;
   const int nw = blockDim.x >> 5;
@@ -311,6 +315,7 @@ affinity_score_tile_kernel(const float* __restrict__ Z, const float* __restrict_
                            const float* __restrict__ R, float* __restrict__ delta,
                            float* __restrict__ rnorm, etr_stats* stats, int Ttok, int D, int E, int m,
                            int ldm) {
+  grid_sync();
   extern __shared__ __align__(16) float smem[];
   constexpr int EROWS = 8 * EPT;
   float* Rs = smem;                               // [EROWS][ldm]
@@ -431,6 +436,7 @@ affinity_fwd_warp_kernel(const T* __restrict__ X, const float* __restrict__ R,
                          float* __restrict__ delta, float* __restrict__ Z, float* __restrict__ xnorm,
                          float* __restrict__ rnorm, etr_stats* stats, int Ttok, int d, int D, int E,
                          int m, int ldm) {
+  grid_sync();
   extern __shared__ __align__(16) float smem[];
   constexpr int EROWS = 32 * EPL;
   const int nw = blockDim.x >> 5;
@@ -542,6 +548,7 @@ __global__ void __launch_bounds__(AFF_THREADS)
 affinity_fwd_kernel(const T* __restrict__ X, const float* __restrict__ R, float* __restrict__ delta,
                     float* __restrict__ Z, float* __restrict__ xnorm, float* __restrict__ rnorm,
                     etr_stats* stats, int Ttok, int d, int D, int E, int m, int ldm, int Epad) {
+  grid_sync();
   extern __shared__ __align__(16) float smem[];
   float* Rs = smem;                          // [Epad][ldm]
   float* Zs = Rs + (size_t)Epad * ldm;       // [TB][ldm]
@@ -655,6 +662,7 @@ affinity_bwd_dx_kernel(const T* __restrict__ X, const float* __restrict__ R,
                        const int32_t* __restrict__ tok_row, const float* __restrict__ dgate,
                        const float* __restrict__ ddelta, const T* __restrict__ dXp, T* __restrict__ dX,
                        int Ttok, int d, int D, int E, int m, int C_stride) {
+  grid_sync();
   extern __shared__ __align__(16) float smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* cz = smem + (size_t)warp * m;
@@ -812,6 +820,7 @@ affinity_bwd_dx_chunk_kernel(const T* __restrict__ X, const float* __restrict__ 
                              const int32_t* __restrict__ tok_row, const float* __restrict__ dgate,
                              const T* __restrict__ dXp, T* __restrict__ dX,
                              int Ttok, int d, int D, int E, int m, int C_stride, int tpb, int d_shift) {
+  grid_sync();
   extern __shared__ __align__(16) float cz[];      // [tpb][m]
   __shared__ int s_ptr[DXC_MAX_TOKENS + 1];
   __shared__ int s_row[DXC_ROWS];
@@ -833,7 +842,7 @@ affinity_bwd_dx_chunk_kernel(const T* __restrict__ X, const float* __restrict__ 
   for (int e = tid; e < staged; e += 256) {
     const int r = tok_row[base + e];
     int tl = 0;
-    while (s_ptr[tl + 1] - base <= e) ++tl;        // the entry's token (at most tpb steps)
+    while (tl + 1 < nt && s_ptr[tl + 1] - base <= e) ++tl;        // the entry's token (at most tpb steps)
     const int i = r / C_stride;
     const float a = s_a[tl], b = rnorm[i], dg = dgate[r];
     s_row[e] = r;
@@ -924,6 +933,7 @@ affinity_bwd_dr_partial_kernel(const float* __restrict__ Z, const float* __restr
                                const int32_t* __restrict__ slot_token,
                                const float* __restrict__ dgate, float* __restrict__ part,
                                int E, int m, int C_stride, int nch, float sqD) {
+  grid_sync();
   __shared__ int s_t[DR_CHUNK];
   __shared__ float s_w[DR_CHUNK], s_dd[DR_CHUNK];
   const int i = blockIdx.x, ch = blockIdx.y, tid = threadIdx.x;
@@ -986,6 +996,7 @@ affinity_bwd_dr_dense_partial_kernel(const float* __restrict__ Z, const float* _
                                      const float* __restrict__ xnorm, const float* __restrict__ rnorm,
                                      const float* __restrict__ ddelta, float* __restrict__ part,
                                      int Ttok, int E, int m, int nch, float sqD) {
+  grid_sync();
   __shared__ __align__(16) float s_w[DR_CHUNK][32];
   __shared__ float s_dd[DR_CHUNK][32];
   const int ch = blockIdx.x, tid = threadIdx.x;
@@ -1040,6 +1051,7 @@ affinity_bwd_dr_dense_partial_kernel(const float* __restrict__ Z, const float* _
 __global__ void __launch_bounds__(256)
 affinity_bwd_dr_final_kernel(const float* __restrict__ part, const float* __restrict__ R,
                              const float* __restrict__ rnorm, float* __restrict__ dR, int m, int nch) {
+  grid_sync();
   const int i = blockIdx.x;
   const float b = rnorm[i];
   const float* base = part + (size_t)i * nch * (m + 1);
@@ -1076,7 +1088,7 @@ static etr_status launch_affinity_warp(const etr_config* c, const void* X, const
     const int ngroups = ceil_div(c->T, TPG);
     const int grid = std::min(current_sm_count(), ceil_div(ngroups, nw));
     ETR_TIME_BEGIN("affinity_fwd_warp_kernel");
-    k<<<grid, nw * 32, smem, st>>>((const T*)X, R, delta, Z, xnorm, rnorm, stats, c->T, c->d, c->D,
+    launch_kernel(k, grid, nw * 32, smem, st, 1, (const T*)X, R, delta, Z, xnorm, rnorm, stats, c->T, c->d, c->D,
                                    c->E, m, ldm);
     ETR_LAUNCH_CHECK();
     *done = true;
@@ -1096,14 +1108,15 @@ static etr_status affinity_forward_warp(const etr_config* c, const void* X, cons
 }
 
 template <class T>
-static etr_status launch_pool(const etr_config* c, const void* X, float* Z, float* xnorm, cudaStream_t st) {
+static etr_status launch_pool(const etr_config* c, const void* X, float* Z, float* xnorm, etr_stats* zero_stats,
+                              cudaStream_t st) {
   constexpr int PE = Raw16<T>::ELEMS;
   const int m = c->d / c->D, grid = ceil_div(c->T, 8), D = c->D;
   ETR_TIME_BEGIN("grap_pool_kernel");
-  if (D == PE) grap_pool_kernel<T, 1><<<grid, 256, 0, st>>>((const T*)X, Z, xnorm, c->T, c->d, D, m);
-  else if (D == 2 * PE) grap_pool_kernel<T, 2><<<grid, 256, 0, st>>>((const T*)X, Z, xnorm, c->T, c->d, D, m);
-  else if (D == 4 * PE) grap_pool_kernel<T, 4><<<grid, 256, 0, st>>>((const T*)X, Z, xnorm, c->T, c->d, D, m);
-  else grap_pool_kernel<T, 0><<<grid, 256, 0, st>>>((const T*)X, Z, xnorm, c->T, c->d, D, m);
+  if (D == PE) launch_kernel(grap_pool_kernel<T, 1>, grid, 256, 0, st, 1, (const T*)X, Z, xnorm, zero_stats, c->T, c->d, D, m);
+  else if (D == 2 * PE) launch_kernel(grap_pool_kernel<T, 2>, grid, 256, 0, st, 1, (const T*)X, Z, xnorm, zero_stats, c->T, c->d, D, m);
+  else if (D == 4 * PE) launch_kernel(grap_pool_kernel<T, 4>, grid, 256, 0, st, 1, (const T*)X, Z, xnorm, zero_stats, c->T, c->d, D, m);
+  else launch_kernel(grap_pool_kernel<T, 0>, grid, 256, 0, st, 1, (const T*)X, Z, xnorm, zero_stats, c->T, c->d, D, m);
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }
@@ -1122,7 +1135,7 @@ static etr_status launch_score(const etr_config* c, const float* Z, const float*
     const int ngroups = ceil_div(c->T, TPG);
     const int grid = std::min(current_sm_count(), ceil_div(ngroups, nw));
     ETR_TIME_BEGIN("affinity_score_kernel");
-    k<<<grid, nw * 32, smem, st>>>(Z, xnorm, R, delta, rnorm, stats, c->T, c->D, c->E, m, ldm);
+    launch_kernel(k, grid, nw * 32, smem, st, 1, Z, xnorm, R, delta, rnorm, stats, c->T, c->D, c->E, m, ldm);
     ETR_LAUNCH_CHECK();
     *done = true;
     return ETR_OK;
@@ -1143,7 +1156,7 @@ static etr_status launch_score_tile(const etr_config* c, const float* Z, const f
     return ETR_ERR_CUDA;
   const int grid = std::min(2 * current_sm_count(), ceil_div(c->T, SC_TM));
   ETR_TIME_BEGIN("affinity_score_kernel");
-  k<<<grid, 256, smem, st>>>(Z, xnorm, R, delta, rnorm, stats, c->T, c->D, c->E, m, ldm);
+  launch_kernel(k, grid, 256, smem, st, 1, Z, xnorm, R, delta, rnorm, stats, c->T, c->D, c->E, m, ldm);
   ETR_LAUNCH_CHECK();
   *done = true;
   return ETR_OK;
@@ -1152,14 +1165,14 @@ static etr_status launch_score_tile(const etr_config* c, const float* Z, const f
 // pool + score as two kernels; *done is false if the score kernel's shared memory does not fit
 static etr_status affinity_forward_split(const etr_config* c, const void* X, const float* R, float* delta,
                                          float* Z, float* xnorm, float* rnorm, etr_stats* stats,
-                                         cudaStream_t st, bool* done) {
+                                         bool zero_stats, cudaStream_t st, bool* done) {
   const int m = c->d / c->D, ldm = (m + 3) / 4 * 4 + 4;
   const int EPL = c->E <= 32 ? 1 : c->E <= 64 ? 2 : c->E <= 128 ? 4 : 8;
   const int TPG = EPL <= 2 ? 8 : EPL == 4 ? 4 : 2;
   *done = false;
   if (((size_t)(32 * EPL + 4 * TPG) * ldm + 32 * EPL) * sizeof(float) > 220 * 1024) return ETR_OK;
-  if (c->dtype == ETR_BF16) ETR_TRY(launch_pool<__nv_bfloat16>(c, X, Z, xnorm, st));
-  else ETR_TRY(launch_pool<float>(c, X, Z, xnorm, st));
+  if (c->dtype == ETR_BF16) ETR_TRY(launch_pool<__nv_bfloat16>(c, X, Z, xnorm, zero_stats ? stats : nullptr, st));
+  else ETR_TRY(launch_pool<float>(c, X, Z, xnorm, zero_stats ? stats : nullptr, st));
   // The product on the tensor cores wherever its shape rules hold, whatever the token count: a token's
   // affinities must not depend on how a batch is cut (an expert-parallel rank scores its own tokens).
   if (affinity_score_tc_takes(c, Z, R, delta)) {
@@ -1181,14 +1194,15 @@ static etr_status affinity_forward_split(const etr_config* c, const void* X, con
 }
 
 etr_status affinity_forward(const etr_config* c, const void* X, const float* R, float* delta,
-                            float* Z, float* xnorm, float* rnorm, etr_stats* stats,
+                            float* Z, float* xnorm, float* rnorm, etr_stats* stats, bool zero_stats,
                             cudaStream_t st) {
   const int m = c->d / c->D;
   bool done = false;
   if (Z != nullptr) {
-    ETR_TRY(affinity_forward_split(c, X, R, delta, Z, xnorm, rnorm, stats, st, &done));
+    ETR_TRY(affinity_forward_split(c, X, R, delta, Z, xnorm, rnorm, stats, zero_stats, st, &done));
     if (done) return ETR_OK;
   }
+  if (zero_stats && cudaMemsetAsync(stats, 0, sizeof(etr_stats), st) != cudaSuccess) return ETR_ERR_CUDA;
   if (c->dtype == ETR_BF16)
     ETR_TRY(affinity_forward_warp<__nv_bfloat16>(c, X, R, delta, Z, xnorm, rnorm, stats, st, &done));
   else
@@ -1203,14 +1217,14 @@ etr_status affinity_forward(const etr_config* c, const void* X, const float* R, 
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return ETR_ERR_CUDA;
     ETR_TIME_BEGIN("affinity_fwd_kernel");
-    k<<<grid, AFF_THREADS, smem, st>>>((const __nv_bfloat16*)X, R, delta, Z, xnorm, rnorm, stats,
+    launch_kernel(k, grid, AFF_THREADS, smem, st, 1, (const __nv_bfloat16*)X, R, delta, Z, xnorm, rnorm, stats,
                                        c->T, c->d, c->D, c->E, m, ldm, Epad);
   } else {
     auto k = affinity_fwd_kernel<float>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return ETR_ERR_CUDA;
     ETR_TIME_BEGIN("affinity_fwd_kernel");
-    k<<<grid, AFF_THREADS, smem, st>>>((const float*)X, R, delta, Z, xnorm, rnorm, stats, c->T,
+    launch_kernel(k, grid, AFF_THREADS, smem, st, 1, (const float*)X, R, delta, Z, xnorm, rnorm, stats, c->T,
                                        c->d, c->D, c->E, m, ldm, Epad);
   }
   ETR_LAUNCH_CHECK();
@@ -1235,7 +1249,7 @@ static etr_status launch_bwd_dx(const etr_config* c, const void* X, const float*
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return ETR_ERR_CUDA;
     ETR_TIME_BEGIN(name);
-    k<<<grid, 256, smem, st>>>((const T*)X, R, delta, xnorm, rnorm, rt->tok_ptr, rt->tok_row, dgate, ddelta,
+    launch_kernel(k, grid, 256, smem, st, 1, (const T*)X, R, delta, xnorm, rnorm, rt->tok_ptr, rt->tok_row, dgate, ddelta,
                                (const T*)dXp_fused, (T*)dX, c->T, c->d, c->D, c->E, m, Cs);
     return ETR_OK;
   };
@@ -1249,7 +1263,7 @@ static etr_status launch_bwd_dx(const etr_config* c, const void* X, const float*
     const size_t csm = (size_t)tpb * m * sizeof(float);
     ETR_TIME_BEGIN("affinity_bwd_dx_fused_kernel");
     auto go = [&](auto k) {
-      k<<<ceil_div(c->T, tpb), 256, csm, st>>>((const T*)X, R, delta, xnorm, rnorm, rt->tok_ptr, rt->tok_row, dgate,
+      launch_kernel(k, ceil_div(c->T, tpb), 256, csm, st, 1, (const T*)X, R, delta, xnorm, rnorm, rt->tok_ptr, rt->tok_row, dgate,
                                                (const T*)dXp_fused, (T*)dX, c->T, c->d, c->D, c->E, m, Cs, tpb,
                                                d_shift);
     };
@@ -1290,17 +1304,16 @@ etr_status affinity_backward(const etr_config* c, const void* X, const float* R,
   float* part = (float*)ws;
   if (ddelta) {
     ETR_TIME_BEGIN("affinity_bwd_dr_dense_partial_kernel");
-    affinity_bwd_dr_dense_partial_kernel<<<nch, 256, 0, st>>>(Z, delta, xnorm, rnorm, ddelta, part, c->T, c->E,
+    launch_kernel(affinity_bwd_dr_dense_partial_kernel, nch, 256, 0, st, 1, Z, delta, xnorm, rnorm, ddelta, part, c->T, c->E,
                                                               m, nch, sqrtf((float)c->D));
   } else {
     ETR_TIME_BEGIN("affinity_bwd_dr_partial_kernel");
-    affinity_bwd_dr_partial_kernel<<<dim3(c->E, nch), 256, 0, st>>>(
-        Z, delta, xnorm, rnorm, rt->counts, rt->slot_token, dgate, part, c->E, m, Cs, nch,
+    launch_kernel(affinity_bwd_dr_partial_kernel, dim3(c->E, nch), 256, 0, st, 1, Z, delta, xnorm, rnorm, rt->counts, rt->slot_token, dgate, part, c->E, m, Cs, nch,
         sqrtf((float)c->D));
   }
   ETR_LAUNCH_CHECK();
   ETR_TIME_BEGIN("affinity_bwd_dr_final_kernel");
-  affinity_bwd_dr_final_kernel<<<c->E, 256, 0, st>>>(part, R, rnorm, dR, m, nch);
+  launch_kernel(affinity_bwd_dr_final_kernel, c->E, 256, 0, st, 1, part, R, rnorm, dR, m, nch);
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }

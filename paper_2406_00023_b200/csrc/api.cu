@@ -268,7 +268,7 @@ etr_status etr_affinity(const etr_config* c, const void* X, const float* R, floa
   ETR_TRY(etr_validate(c));
   ETR_TRY(check_ptrs({X, R, delta, xnorm, rnorm, stats}));
   if (Z && !aligned16(Z)) return ETR_ERR_ALIGN;
-  return affinity_forward(c, X, R, delta, Z, xnorm, rnorm, stats, (cudaStream_t)stream);
+  return affinity_forward(c, X, R, delta, Z, xnorm, rnorm, stats, false, (cudaStream_t)stream);
 }
 
 etr_status etr_select(const etr_config* c, const float* delta, etr_stats* stats,
@@ -422,10 +422,9 @@ etr_status etr_layer_forward(const etr_config* c, const void* X, const float* R,
                              void* stream) {
   if (b == nullptr) return ETR_ERR_ARG;
   ETR_TRY(etr_validate(c));
-  ETR_TRY(check_ptrs({b->stats}));
-  if (cudaMemsetAsync(b->stats, 0, sizeof(etr_stats), (cudaStream_t)stream) != cudaSuccess)
-    return ETR_ERR_CUDA;
-  ETR_TRY(etr_affinity(c, X, R, b->delta, b->Z, b->xnorm, b->rnorm, b->stats, stream));
+  ETR_TRY(check_ptrs({b->stats, X, R, b->delta, b->xnorm, b->rnorm}));
+  if (b->Z && !aligned16(b->Z)) return ETR_ERR_ALIGN;
+  ETR_TRY(affinity_forward(c, X, R, b->delta, b->Z, b->xnorm, b->rnorm, b->stats, true, (cudaStream_t)stream));
   ETR_TRY(etr_select(c, b->delta, b->stats, &b->route, b->ws, stream));
   if (c->gate_mode == ETR_GATE_SOFTMAX) ETR_TRY(etr_gate_softmax(c, b->delta, &b->route, b->lse, stream));
   const bool fc = fuse_combine(c);

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <utility>
 
 #include "../../include/etr.h"
 
@@ -28,6 +29,32 @@ void timing_end(cudaStream_t st);
     etr_status s__ = (expr);                                \
     if (s__ != ETR_OK) return s__;                          \
   } while (0)
+
+// Every kernel is launched with programmatic stream serialization: its blocks may become resident while the last
+// blocks of the kernel before it still run, so that the launch latency and the set-up that touches no memory of
+// others (barriers, tensor memory) overlap.  Each kernel calls grid_sync() before its first access to global
+// memory: it waits for the kernel before it to be complete and visible, and only then lets the next kernel in, so
+// that never more than two kernels of a stream are in flight.
+template <class... P, class... A>
+inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, int cluster,
+                                 A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = 1;
+  if (cluster > 1) {
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+  }
+  cfg.attrs = attr;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 inline int c_stride_of(const etr_config* c) { return (c->capacity + 127) / 128 * 128; }
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -142,6 +169,9 @@ __device__ inline float warp_sum(float v) {
 constexpr long long ETR_WAIT_LIMIT_CYCLES = 4000000000ll;   // about two seconds
 
 #ifdef __CUDACC__
+__device__ __forceinline__ void grid_sync() {
+  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
+}
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
@@ -178,9 +208,38 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 }
 #endif
 
+#ifdef __CUDACC__
+// prefix[e] = tiles(counts[0]) + ... + tiles(counts[e - 1]), e <= E <= 256, by one warp.
+template <class F>
+__device__ __forceinline__ void tile_prefix_warp(int* prefix, const int* counts, int E, int lane, F tiles) {
+  int n[8], mine = 0;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int e = 8 * lane + u;
+    n[u] = e < E ? tiles(counts[e]) : 0;
+    mine += n[u];
+  }
+  int inc = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  int acc = inc - mine;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int e = 8 * lane + u;
+    if (e <= E) prefix[e] = acc;
+    acc += n[u];
+  }
+  if (lane == 31 && E == 256) prefix[256] = acc;
+}
+#endif
+
 // ---- stage entry points, one translation unit each ------------------------------------------
 etr_status affinity_forward(const etr_config* c, const void* X, const float* R, float* delta,
-                            float* Z, float* xnorm, float* rnorm, etr_stats* stats, cudaStream_t st);
+                            float* Z, float* xnorm, float* rnorm, etr_stats* stats, bool zero_stats,
+                            cudaStream_t st);      // zero_stats: *stats is cleared first
 size_t affinity_bwd_workspace_bytes(const etr_config* c);
 // score_tcgen05.cu: the score product on the tensor cores (E <= 64, 32 | d/D, 16-byte aligned Z, R, delta)
 bool affinity_score_tc_takes(const etr_config* c, const float* Z, const float* R, const float* delta);

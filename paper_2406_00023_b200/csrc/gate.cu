@@ -14,6 +14,7 @@ __global__ void __launch_bounds__(256)
 gate_softmax_kernel(const float* __restrict__ delta, const int32_t* __restrict__ tok_ptr,
                     const int32_t* __restrict__ tok_row, float* __restrict__ gate,
                     float* __restrict__ lse, int Ttok, int E, int C_stride) {
+  grid_sync();
   const int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (t >= Ttok) return;
   const float* dt = delta + (size_t)t * E;
@@ -40,6 +41,7 @@ gate_softmax_bwd_kernel(const float* __restrict__ delta, const float* __restrict
                         const int32_t* __restrict__ tok_ptr, const int32_t* __restrict__ tok_row,
                         const float* __restrict__ gate, const float* __restrict__ dgate,
                         float* __restrict__ ddelta, int Ttok, int E, int C_stride) {
+  grid_sync();
   const int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (t >= Ttok) return;
   const int beg = tok_ptr[t], end = tok_ptr[t + 1];
@@ -69,6 +71,7 @@ gate_softmax_bwd_kernel(const float* __restrict__ delta, const float* __restrict
 __global__ void __launch_bounds__(256)
 load_stats_kernel(const int32_t* __restrict__ counts, const float* __restrict__ gate,
                   float* __restrict__ load, float* __restrict__ gate_mean, int Ttok, int C_stride) {
+  grid_sync();
   __shared__ float red[8];
   const int i = blockIdx.x, tid = threadIdx.x;
   const int n = counts[i];
@@ -88,7 +91,7 @@ load_stats_kernel(const int32_t* __restrict__ counts, const float* __restrict__ 
 etr_status gate_softmax_forward(const etr_config* c, const float* delta, const etr_route* rt, float* lse,
                                 cudaStream_t st) {
   ETR_TIME_BEGIN("gate_softmax_kernel");
-  gate_softmax_kernel<<<ceil_div(c->T, 8), 256, 0, st>>>(delta, rt->tok_ptr, rt->tok_row, rt->gate, lse,
+  launch_kernel(gate_softmax_kernel, ceil_div(c->T, 8), 256, 0, st, 1, delta, rt->tok_ptr, rt->tok_row, rt->gate, lse,
                                                          c->T, c->E, c_stride_of(c));
   ETR_LAUNCH_CHECK();
   return ETR_OK;
@@ -97,7 +100,7 @@ etr_status gate_softmax_forward(const etr_config* c, const float* delta, const e
 etr_status gate_softmax_backward(const etr_config* c, const float* delta, const float* lse,
                                  const etr_route* rt, const float* dgate, float* ddelta, cudaStream_t st) {
   ETR_TIME_BEGIN("gate_softmax_bwd_kernel");
-  gate_softmax_bwd_kernel<<<ceil_div(c->T, 8), 256, 0, st>>>(delta, lse, rt->tok_ptr, rt->tok_row, rt->gate,
+  launch_kernel(gate_softmax_bwd_kernel, ceil_div(c->T, 8), 256, 0, st, 1, delta, lse, rt->tok_ptr, rt->tok_row, rt->gate,
                                                              dgate, ddelta, c->T, c->E, c_stride_of(c));
   ETR_LAUNCH_CHECK();
   return ETR_OK;
@@ -106,7 +109,7 @@ etr_status gate_softmax_backward(const etr_config* c, const float* delta, const 
 etr_status load_stats_launch(const etr_config* c, const etr_route* rt, float* load, float* gate_mean,
                              cudaStream_t st) {
   ETR_TIME_BEGIN("load_stats_kernel");
-  load_stats_kernel<<<c->E, 256, 0, st>>>(rt->counts, rt->gate, load, gate_mean, c->T, c_stride_of(c));
+  launch_kernel(load_stats_kernel, c->E, 256, 0, st, 1, rt->counts, rt->gate, load, gate_mean, c->T, c_stride_of(c));
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }

@@ -33,6 +33,7 @@ __device__ inline float sigmoid_f(float v) { return 1.0f / (1.0f + expf(-v)); }
 
 template <class T, int EPI>
 __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g) {
+  grid_sync();
   constexpr int BM = 64, BN = 64, BK = 16;
   constexpr bool SEP = (EPI == EPI_SWIGLU);
   __shared__ __align__(16) float As[BK][BM + 4];
@@ -117,7 +118,7 @@ template <class T, int EPI>
 static etr_status launch(const GemmArgs& g, int E, cudaStream_t st) {
   dim3 grid(ceil_div(g.N, 64), ceil_div(g.dyn == DYN_M ? g.m_cap : g.M, 64), E);
   ETR_TIME_BEGIN("gemm_simt_kernel");
-  gemm_simt_kernel<T, EPI><<<grid, 256, 0, st>>>(g);
+  launch_kernel(gemm_simt_kernel<T, EPI>, grid, 256, 0, st, 1, g);
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }

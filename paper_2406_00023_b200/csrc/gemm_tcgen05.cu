@@ -342,26 +342,24 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_c
   const uint32_t tempty_bar = smem_u32(&bars[2 * TC_STAGES + 2]); // [2]
 
   // ---- set-up ---------------------------------------------------------------------------------
-  for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
-  __syncthreads();
   if (tid == 0) {
     abort_flag_s = 0;
     for (int s = 0; s < TC_STAGES; ++s) { mbar_init(full_bar + 8 * s, 1); mbar_init(empty_bar + 8 * s, 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar + 8 * a, 1); mbar_init(tempty_bar + 8 * a, 8); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    const int nt = (p.N + N_TILE_COLS - 1) / N_TILE_COLS;
-    int acc = 0;
-    for (int e = 0; e < p.E; ++e) {
-      tile_prefix[e] = acc;
-      const int n_e = s_counts[e];
-      const int mt = p.dyn == TC_DYN_M ? (min(n_e, p.M) + TC_BM - 1) / TC_BM : (p.M + TC_BM - 1) / TC_BM;
-      acc += mt * nt;
-    }
-    tile_prefix[p.E] = acc;
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  grid_sync();
+  for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
+  __syncthreads();
+  if (warp == 2) {
+    const int nt = (p.N + N_TILE_COLS - 1) / N_TILE_COLS;
+    tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) {
+      return nt * (p.dyn == TC_DYN_M ? (min(n_e, p.M) + TC_BM - 1) / TC_BM : (p.M + TC_BM - 1) / TC_BM);
+    });
   }
   tc_fence_before();
   __syncthreads();
@@ -659,26 +657,24 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
   const uint32_t tfull_bar = smem_u32(&bars[2 * TC2_STAGES]);      // [2]           in each CTA
   const uint32_t tempty_bar = smem_u32(&bars[2 * TC2_STAGES + 2]); // [2]           used in the leader
 
-  for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
-  __syncthreads();
   if (tid == 0) {
     abort_flag_s = 0;
     for (int s = 0; s < TC2_STAGES; ++s) { mbar_init(full_bar + 8 * s, 1); mbar_init(empty_bar + 8 * s, 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar + 8 * a, 1); mbar_init(tempty_bar + 8 * a, 16); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    const int nt = (p.N + N_TILE_COLS - 1) / N_TILE_COLS;
-    int acc = 0;
-    for (int e = 0; e < p.E; ++e) {
-      tile_prefix[e] = acc;
-      const int n_e = s_counts[e];
-      const int mt = p.dyn == TC_DYN_M ? (min(n_e, p.M) + 255) / 256 : (p.M + 255) / 256;
-      acc += mt * nt;
-    }
-    tile_prefix[p.E] = acc;
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  grid_sync();
+  for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
+  __syncthreads();
+  if (warp == 2) {
+    const int nt = (p.N + N_TILE_COLS - 1) / N_TILE_COLS;
+    tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) {
+      return nt * (p.dyn == TC_DYN_M ? (min(n_e, p.M) + 255) / 256 : (p.M + 255) / 256);
+    });
   }
   tc_fence_before();
   __syncthreads();
@@ -856,6 +852,7 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
   }
+  cluster_sync_all();                 // the next kernel's blocks may start on an SM as soon as its CTA is gone
 }
 
 // ---- CTA-pair kernel, two output tiles per pass ------------------------------------------------------
@@ -924,27 +921,25 @@ tc_grouped_gemm_pair_wide_kernel(const __grid_constant__ CUtensorMap mapA0, cons
   const uint32_t tfull_bar = smem_u32(&bars[2 * TCW_STAGES]);      // [1]           in each CTA
   const uint32_t tempty_bar = smem_u32(&bars[2 * TCW_STAGES + 1]); // [2]           used in the leader
 
-  for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
-  __syncthreads();
   if (tid == 0) {
     abort_flag_s = 0;
     for (int s = 0; s < TCW_STAGES; ++s) { mbar_init(full_bar + 8 * s, 1); mbar_init(empty_bar + 8 * s, 1); }
     mbar_init(tfull_bar, 1);
     for (int a = 0; a < 2; ++a) mbar_init(tempty_bar + 8 * a, 16);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    const int nt = (p.N + 2 * N_TILE_COLS - 1) / (2 * N_TILE_COLS);
-    int acc = 0;
-    for (int e = 0; e < p.E; ++e) {
-      tile_prefix[e] = acc;
-      const int n_e = s_counts[e];
-      const int mt = p.dyn == TC_DYN_M ? (min(n_e, p.M) + 255) / 256 : (p.M + 255) / 256;
-      acc += mt * nt;
-    }
-    tile_prefix[p.E] = acc;
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  grid_sync();
+  for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
+  __syncthreads();
+  if (warp == 2) {
+    const int nt = (p.N + 2 * N_TILE_COLS - 1) / (2 * N_TILE_COLS);
+    tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) {
+      return nt * (p.dyn == TC_DYN_M ? (min(n_e, p.M) + 255) / 256 : (p.M + 255) / 256);
+    });
   }
   tc_fence_before();
   __syncthreads();
@@ -1206,6 +1201,7 @@ tc_grouped_gemm_pair_wide_kernel(const __grid_constant__ CUtensorMap mapA0, cons
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
   }
+  cluster_sync_all();                 // the next kernel's blocks may start on an SM as soon as its CTA is gone
 }
 
 // ---- host side --------------------------------------------------------------------------------------
@@ -1263,7 +1259,7 @@ static etr_status tc_launch(const char* name, const CUtensorMap& a0, const CUten
   p.idesc = make_idesc(p.a_mn, p.b_mn, BN);
   const int grid = max_tiles < sm_count() ? (max_tiles < 1 ? 1 : max_tiles) : sm_count();
   ETR_TIME_BEGIN(name);
-  k<<<grid, TC_THREADS, smem, st>>>(a0, a1, b0, b1, p);
+  launch_kernel(k, grid, TC_THREADS, smem, st, 1, a0, a1, b0, b1, p);
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }
@@ -1279,18 +1275,8 @@ static etr_status tc_launch_pair_cfg(const char* name, const CUtensorMap& a0, co
   p.idesc = make_idesc(p.a_mn, p.b_mn, 256, 256);
   const int pairs_max = sm_count() / 2;
   const int pairs = max_tiles < pairs_max ? (max_tiles < 1 ? 1 : max_tiles) : pairs_max;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * pairs);
-  cfg.blockDim = dim3(TC_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   ETR_TIME_BEGIN(name);
-  if (cudaLaunchKernelEx(&cfg, k, a0, a1, b0, b1, p) != cudaSuccess) { timing_end(st); return ETR_ERR_CUDA; }
+  launch_kernel(k, 2 * pairs, TC_THREADS, smem, st, 2, a0, a1, b0, b1, p);
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }
@@ -1306,18 +1292,8 @@ static etr_status tc_launch_pair_wide_cfg(const char* name, const CUtensorMap& a
   p.idesc = make_idesc(p.a_mn, p.b_mn, 256, 256);
   const int pairs_max = sm_count() / 2;
   const int pairs = max_tiles < pairs_max ? (max_tiles < 1 ? 1 : max_tiles) : pairs_max;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * pairs);
-  cfg.blockDim = dim3(TC_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   ETR_TIME_BEGIN(name);
-  if (cudaLaunchKernelEx(&cfg, k, a0, a1, b0, b1, p) != cudaSuccess) { timing_end(st); return ETR_ERR_CUDA; }
+  launch_kernel(k, 2 * pairs, TC_THREADS, smem, st, 2, a0, a1, b0, b1, p);
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }

@@ -215,8 +215,6 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
   const uint32_t tfull_bar = smem_u32(&bars[3 * F3_STAGES]);         // [2] a chunk's accumulators are complete
   const uint32_t tempty_bar = smem_u32(&bars[3 * F3_STAGES + 2]);    // [2] they have been read
 
-  for (int e = tid; e < p.E; e += F3_THREADS) s_counts[e] = p.counts[e];
-  __syncthreads();
   if (tid == 0) {
     abort_flag_s = 0;
     for (int s = 0; s < F3_STAGES; ++s) {
@@ -224,14 +222,17 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
     }
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar + 8 * a, 1); mbar_init(tempty_bar + 8 * a, 8); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    const int nt = (p.N + COLS - 1) / COLS;
-    int acc = 0;
-    for (int e = 0; e < p.E; ++e) { tile_prefix[e] = acc; acc += f3_mtiles(p, s_counts[e]) * nt; }
-    tile_prefix[p.E] = acc;
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  grid_sync();
+  for (int e = tid; e < p.E; e += F3_THREADS) s_counts[e] = p.counts[e];
+  __syncthreads();
+  if (warp == 2) {
+    const int nt = (p.N + COLS - 1) / COLS;
+    tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) { return f3_mtiles(p, n_e) * nt; });
   }
   tc_fence_before();
   __syncthreads();
@@ -475,7 +476,7 @@ static etr_status f3_launch_bn(const char* name, const F3Operand* A, const F3Ope
     ETR_TRY(f3_map(&b[i], ob.ptr, ob.cols, ob.rows, p.E, B_MN ? F3_BK : (EPI == F3_SWIGLU ? BN / 2 : BN)));
   }
   ETR_TIME_BEGIN(name);
-  k<<<std::max(1, std::min(max_tiles, current_sm_count())), F3_THREADS, smem, st>>>(a[0], a[1], b[0], b[1], p, idesc);
+  launch_kernel(k, std::max(1, std::min(max_tiles, current_sm_count())), F3_THREADS, smem, st, 1, a[0], a[1], b[0], b[1], p, idesc);
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }

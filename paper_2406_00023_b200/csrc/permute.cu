@@ -11,6 +11,7 @@ __global__ void __launch_bounds__(256)
 dispatch_kernel(const T* __restrict__ X, const int32_t* __restrict__ counts,
                 const int32_t* __restrict__ slot_token, T* __restrict__ Xp, int d, int C_stride,
                 int n_rows) {
+  grid_sync();
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= n_rows) return;
   const int i = r / C_stride, p = r - i * C_stride;
@@ -42,6 +43,7 @@ __global__ void __launch_bounds__(256)
 combine_kernel(const T* __restrict__ O, const float* __restrict__ gate,
                const int32_t* __restrict__ tok_ptr, const int32_t* __restrict__ tok_row,
                T* __restrict__ Y, int Ttok, int d) {
+  grid_sync();
   __shared__ int s_ptr[COMBINE_TOKENS + 1];
   __shared__ int s_row[COMBINE_ROWS];
   __shared__ float s_gate[COMBINE_ROWS];
@@ -112,6 +114,7 @@ combine_bwd_kernel(const T* __restrict__ dY, const T* __restrict__ O,
                    const int32_t* __restrict__ counts, const int32_t* __restrict__ slot_token,
                    const float* __restrict__ gate, T* __restrict__ dO, float* __restrict__ dgate,
                    int d, int C_stride, int n_rows) {
+  grid_sync();
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= n_rows) return;
   const int i = r / C_stride, p = r - i * C_stride;
@@ -145,6 +148,7 @@ combine_bwd_kernel(const T* __restrict__ dY, const T* __restrict__ O,
 // down GEMM leaves over).  One warp per token.
 __global__ void __launch_bounds__(256)
 zero_unrouted_kernel(const int32_t* __restrict__ tok_ptr, uint4* __restrict__ Y, int Ttok, int row_vec) {
+  grid_sync();
   const int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (t >= Ttok || tok_ptr[t] != tok_ptr[t + 1]) return;
   uint4* dst = Y + (size_t)t * row_vec;
@@ -153,7 +157,7 @@ zero_unrouted_kernel(const int32_t* __restrict__ tok_ptr, uint4* __restrict__ Y,
 
 etr_status zero_unrouted_rows(const etr_config* c, const etr_route* rt, void* Y, cudaStream_t st) {
   ETR_TIME_BEGIN("zero_unrouted_kernel");
-  zero_unrouted_kernel<<<ceil_div(c->T, 8), 256, 0, st>>>(rt->tok_ptr, (uint4*)Y, c->T,
+  launch_kernel(zero_unrouted_kernel, ceil_div(c->T, 8), 256, 0, st, 1, rt->tok_ptr, (uint4*)Y, c->T,
                                                           (int)((size_t)c->d * elem_bytes(c->dtype) / 16));
   ETR_LAUNCH_CHECK();
   return ETR_OK;
@@ -166,7 +170,7 @@ static etr_status permute_launch(int which, const etr_config* c, const etr_route
   switch (which) {
     case 0:
       ETR_TIME_BEGIN("dispatch_kernel");
-      dispatch_kernel<T><<<ceil_div(n_rows, 8), 256, 0, st>>>((const T*)a, rt->counts, rt->slot_token,
+      launch_kernel(dispatch_kernel<T>, ceil_div(n_rows, 8), 256, 0, st, 1, (const T*)a, rt->counts, rt->slot_token,
                                                              (T*)out, c->d, Cs, n_rows);
       break;
     case 1:
@@ -175,15 +179,14 @@ static etr_status permute_launch(int which, const etr_config* c, const etr_route
       ETR_TIME_BEGIN("combine_kernel");
       const unsigned grid = (unsigned)ceil_div(c->T, COMBINE_TOKENS);
       if (c->d % 16 == 0)
-        combine_kernel<T, 2><<<grid, 256, 0, st>>>((const T*)a, g, rt->tok_ptr, rt->tok_row, (T*)out, c->T, c->d);
+        launch_kernel(combine_kernel<T, 2>, grid, 256, 0, st, 1, (const T*)a, g, rt->tok_ptr, rt->tok_row, (T*)out, c->T, c->d);
       else
-        combine_kernel<T, 1><<<grid, 256, 0, st>>>((const T*)a, g, rt->tok_ptr, rt->tok_row, (T*)out, c->T, c->d);
+        launch_kernel(combine_kernel<T, 1>, grid, 256, 0, st, 1, (const T*)a, g, rt->tok_ptr, rt->tok_row, (T*)out, c->T, c->d);
       break;
     }
     case 2:
       ETR_TIME_BEGIN("combine_bwd_kernel");
-      combine_bwd_kernel<T><<<ceil_div(n_rows, 8), 256, 0, st>>>(
-          (const T*)a, (const T*)b, rt->counts, rt->slot_token, rt->gate, (T*)out, dgate, c->d, Cs, n_rows);
+      launch_kernel(combine_bwd_kernel<T>, ceil_div(n_rows, 8), 256, 0, st, 1, (const T*)a, (const T*)b, rt->counts, rt->slot_token, rt->gate, (T*)out, dgate, c->d, Cs, n_rows);
       break;
   }
   ETR_LAUNCH_CHECK();
@@ -215,6 +218,7 @@ etr_status dispatch_backward(const etr_config* c, const etr_route* rt, const voi
 // fp32 master weights, rounded once per pass for the GEMMs.
 __global__ void __launch_bounds__(256) cast_f32_to_bf16_kernel(const float4* __restrict__ src, uint4* __restrict__ dst,
                                                                size_t n8) {
+  grid_sync();
   for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n8; i += (size_t)gridDim.x * 256) {
     const float4 a = src[2 * i], b = src[2 * i + 1];
     const __nv_bfloat162 p0 = __floats2bfloat162_rn(a.x, a.y), p1 = __floats2bfloat162_rn(a.z, a.w);
@@ -231,7 +235,7 @@ etr_status cast_f32_to_bf16(const void* src, void* dst, size_t n, cudaStream_t s
   const size_t n8 = n / 8;
   const size_t want = (n8 + 255) / 256, cap = (size_t)current_sm_count() * 16;
   ETR_TIME_BEGIN("cast_weights_kernel");
-  cast_f32_to_bf16_kernel<<<(unsigned)(want < cap ? (want ? want : 1) : cap), 256, 0, st>>>((const float4*)src,
+  launch_kernel(cast_f32_to_bf16_kernel, (unsigned)(want < cap ? (want ? want : 1) : cap), 256, 0, st, 1, (const float4*)src,
                                                                                             (uint4*)dst, n8);
   ETR_LAUNCH_CHECK();
   return ETR_OK;

@@ -101,6 +101,7 @@ affinity_score_tc_kernel(const __grid_constant__ CUtensorMap mapZ, const __grid_
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(SCT_TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  grid_sync();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -325,8 +326,7 @@ etr_status affinity_score_tc(const etr_config* c, const float* Z, const float* x
   const int ntiles = ceil_div(c->T, SCT_BM);
   const long long limit = c->wait_limit_cycles > 0 ? (long long)c->wait_limit_cycles : ETR_WAIT_LIMIT_CYCLES;
   ETR_TIME_BEGIN("affinity_score_tc_kernel");
-  affinity_score_tc_kernel<<<std::min(ntiles, current_sm_count()), SCT_THREADS, smem, st>>>(
-      mapZ, mapR, R, xnorm, delta, rnorm, stats, c->T, c->E, m, sqrtf((float)c->D), idesc, limit);
+  launch_kernel(affinity_score_tc_kernel, std::min(ntiles, current_sm_count()), SCT_THREADS, smem, st, 1, mapZ, mapR, R, xnorm, delta, rnorm, stats, c->T, c->E, m, sqrtf((float)c->D), idesc, limit);
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }

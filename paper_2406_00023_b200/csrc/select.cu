@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(256)
 select_token_side_kernel(const float* __restrict__ delta, int32_t* __restrict__ topk_idx,
                          uint32_t* __restrict__ keyT, etr_stats* stats, int32_t* __restrict__ skipped,
                          SelectParams p) {
+  grid_sync();
   __shared__ uint32_t tile[256 * (SEL_TB + 1)];      // [E][33]
   __shared__ int s_skipped;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -188,6 +189,7 @@ __device__ __forceinline__ void pick_bin(const uint32_t* hist, uint32_t rem, int
 __global__ void __launch_bounds__(1024)
 select_threshold_limit_kernel(const uint32_t* __restrict__ keyT, int32_t* __restrict__ limit, int T,
                               long long tq) {
+  grid_sync();
   __shared__ uint32_t hist_cnt[256];
   __shared__ unsigned long long hist_sum[256];
   __shared__ uint32_t s_prefix, s_before;
@@ -272,6 +274,7 @@ __global__ void __launch_bounds__(1024)
 select_expert_side_kernel(uint32_t* __restrict__ keyT, const etr_stats* __restrict__ stats,
                           const int32_t* __restrict__ limit, int32_t* __restrict__ counts,
                           int32_t* __restrict__ slot_token, float* __restrict__ gate, int T, int C_stride) {
+  grid_sync();
   __shared__ uint32_t hist[256];
   __shared__ uint32_t s_prefix, s_remaining, s_ncand;
   __shared__ uint32_t warp_tot[32], warp_pre[32];
@@ -424,6 +427,7 @@ select_expert_side_cluster_kernel(uint32_t* __restrict__ keyT, const etr_stats* 
                                   const int32_t* __restrict__ limit, int32_t* __restrict__ counts,
                                   int32_t* __restrict__ slot_token, float* __restrict__ gate, int T,
                                   int C_stride) {
+  grid_sync();
   __shared__ uint32_t hist[256], tot[256];
   __shared__ uint32_t s_prefix, s_remaining, s_ncand_local, s_ncand;
   __shared__ uint32_t s_cnt_gt, s_cnt_eq;
@@ -593,17 +597,20 @@ select_expert_side_cluster_kernel(uint32_t* __restrict__ keyT, const etr_stats* 
   }
   for (int p = (int)n_keep + (int)rank * 1024 + tid; p < C_stride; p += CL * 1024) { my_slot[p] = -1; my_gate[p] = 0.f; }
   if (tid == 0 && rank == 0) counts[i] = (int)n_keep;
+  __syncthreads();                                // the cluster barrier wants converged warps
   sel_cluster_sync();                             // no CTA leaves while a peer may still read its counters
 }
 
-// Token-major CSR in three small kernels without a long serial scan:
+// Token-major CSR in two small kernels without a long serial scan:
 //   count  per-token row counts, exclusive scan inside each 256-token block (left in
 //          tok_ptr[t+1]), block totals to scratch
-//   scan   exclusive scan of the block totals (one CTA; T/256 values)
-//   fill   tok_row from the position matrix, final tok_ptr
+//   fill   a block's offset as the sum of the totals before it (every block for itself: one value per thread
+//          and 65536 tokens, cheaper than a launch for a scan of them), tok_row from the position matrix, final
+//          tok_ptr; the last block leaves the sums in stats
 __global__ void __launch_bounds__(256)
 csr_count_kernel(const int32_t* __restrict__ posT, int32_t* __restrict__ tok_ptr,
                  int32_t* __restrict__ block_total, etr_stats* stats, int T, int E) {
+  grid_sync();
   __shared__ int wsum[8];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int t = blockIdx.x * 256 + tid;
@@ -627,63 +634,45 @@ csr_count_kernel(const int32_t* __restrict__ posT, int32_t* __restrict__ tok_ptr
   if (tid == 0) block_total[blockIdx.x] = tot;
 }
 
-__global__ void __launch_bounds__(1024)
-csr_scan_kernel(int32_t* __restrict__ block_total, int32_t* __restrict__ tok_ptr, etr_stats* stats,
-                int nblocks, int n_cand, const int32_t* __restrict__ skipped, int n_skipped_blocks) {
-  __shared__ int wsum[32], wpre[32];
-  __shared__ int carry, given_up;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) { carry = 0; given_up = 0; tok_ptr[0] = 0; }
+__device__ __forceinline__ int block_sum_256(int v, int* wsum) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   __syncthreads();
-  if (skipped) {              // candidates the tokens gave up themselves (token-side threshold): integer sum
-    int s = 0;
-    for (int b = tid; b < n_skipped_blocks; b += 1024) s += skipped[b];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0 && s) atomicAdd(&given_up, s);
-    __syncthreads();
-  }
-  for (int c0 = 0; c0 < nblocks; c0 += 1024) {
-    const int b = c0 + tid;
-    const int v = b < nblocks ? block_total[b] : 0;
-    int inc = v;
+  if (lane == 0) wsum[warp] = v;
+  __syncthreads();
+  int tot = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += y;
-    }
-    if (lane == 31) wsum[warp] = inc;
-    __syncthreads();
-    if (warp == 0) {
-      const int wt = wsum[lane];
-      int winc = wt;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, winc, o);
-        if (lane >= o) winc += y;
-      }
-      wpre[lane] = winc - wt;
-      if (lane == 31) wsum[0] = winc;
-    }
-    __syncthreads();
-    if (b < nblocks) block_total[b] = carry + wpre[warp] + inc - v;     // exclusive block offset
-    const int total = wsum[0];
-    __syncthreads();
-    if (tid == 0) carry += total;
-    __syncthreads();
-  }
-  if (tid == 0) {
-    stats->rows_total = carry;
-    stats->dropped = n_cand - given_up - carry;
-  }
+  for (int w = 0; w < 8; ++w) tot += wsum[w];
+  return tot;
 }
 
 __global__ void __launch_bounds__(256)
-csr_fill_kernel(const int32_t* __restrict__ posT, const int32_t* __restrict__ block_offset,
-                int32_t* __restrict__ tok_ptr, int32_t* __restrict__ tok_row, int T, int E,
-                int C_stride) {
-  const int t = blockIdx.x * 256 + threadIdx.x;
+csr_fill_kernel(const int32_t* __restrict__ posT, const int32_t* __restrict__ block_total,
+                int32_t* __restrict__ tok_ptr, int32_t* __restrict__ tok_row, etr_stats* stats, int T, int E,
+                int C_stride, int n_cand, const int32_t* __restrict__ skipped, int n_skipped_blocks) {
+  grid_sync();
+  __shared__ int wsum[8];
+  const int tid = threadIdx.x, b = blockIdx.x;
+  int before = 0;
+  for (int i = tid; i < b; i += 256) before += block_total[i];
+  const int offset = block_sum_256(before, wsum);
+  if (b == (int)gridDim.x - 1) {
+    int given_up = 0;         // candidates the tokens gave up themselves (token-side threshold)
+    if (skipped) {
+      for (int i = tid; i < n_skipped_blocks; i += 256) given_up += skipped[i];
+      given_up = block_sum_256(given_up, wsum);
+    }
+    if (tid == 0) {
+      const int rows = offset + block_total[b];
+      stats->rows_total = rows;
+      stats->dropped = n_cand - given_up - rows;
+    }
+  }
+  if (b == 0 && tid == 0) tok_ptr[0] = 0;
+  const int t = b * 256 + tid;
   if (t >= T) return;
-  int q = block_offset[blockIdx.x] + tok_ptr[t + 1];
+  int q = offset + tok_ptr[t + 1];
   for (int i = 0; i < E; ++i) {
     const int pos = posT[(size_t)i * T + t];
     if (pos >= 0) tok_row[q++] = i * C_stride + pos;
@@ -719,11 +708,11 @@ etr_status select_forward(const etr_config* c, const float* delta, etr_stats* st
   int32_t* limit = (c->threshold_mode & ETR_THRESHOLD_EXPERT) ? reinterpret_cast<int32_t*>(ws_tail) : nullptr;
   int32_t* skipped = p.cut_token ? reinterpret_cast<int32_t*>(ws_tail + select_limit_bytes(c)) : nullptr;
   ETR_TIME_BEGIN("select_token_side_kernel");
-  select_token_side_kernel<<<ceil_div(c->T, SEL_TB), 256, 0, st>>>(delta, rt->topk_idx, keyT, stats, skipped, p);
+  launch_kernel(select_token_side_kernel, ceil_div(c->T, SEL_TB), 256, 0, st, 1, delta, rt->topk_idx, keyT, stats, skipped, p);
   ETR_LAUNCH_CHECK();
   if (limit) {
     ETR_TIME_BEGIN("select_threshold_limit_kernel");
-    select_threshold_limit_kernel<<<c->E, 1024, 0, st>>>(keyT, limit, c->T, quantise_threshold(c->threshold_tau));
+    launch_kernel(select_threshold_limit_kernel, c->E, 1024, 0, st, 1, keyT, limit, c->T, quantise_threshold(c->threshold_tau));
     ETR_LAUNCH_CHECK();
   }
   ETR_TIME_BEGIN("select_expert_side_kernel");
@@ -732,40 +721,22 @@ etr_status select_forward(const etr_config* c, const float* delta, etr_stats* st
     const size_t key_bytes = (size_t)((ceil_div(c->T, CL) + SEL_KPT - 1) / SEL_KPT * SEL_KPT) * sizeof(uint32_t);
     static std::atomic<unsigned long long> attr_done{0};      // one bit per device
     if (!ensure_dyn_smem(select_expert_side_cluster_kernel<CL>, 196608, attr_done)) return ETR_ERR_CUDA;
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(c->E * CL);
-    lc.blockDim = dim3(1024);
-    lc.dynamicSmemBytes = key_bytes;
-    lc.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CL; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    lc.attrs = attr;
-    lc.numAttrs = 1;
-    if (cudaLaunchKernelEx(&lc, select_expert_side_cluster_kernel<CL>, keyT, (const etr_stats*)stats,
-                           (const int32_t*)limit, rt->counts, rt->slot_token, rt->gate, c->T,
-                           p.C_stride) != cudaSuccess) {
-      timing_end(st);
-      return ETR_ERR_CUDA;
-    }
+    launch_kernel(select_expert_side_cluster_kernel<CL>, c->E * CL, 1024, key_bytes, st, CL, keyT, (const etr_stats*)stats,
+                  (const int32_t*)limit, rt->counts, rt->slot_token, rt->gate, c->T, p.C_stride);
   } else {
-    select_expert_side_kernel<<<c->E, 1024, 0, st>>>(keyT, stats, limit, rt->counts, rt->slot_token, rt->gate,
+    launch_kernel(select_expert_side_kernel, c->E, 1024, 0, st, 1, keyT, stats, limit, rt->counts, rt->slot_token, rt->gate,
                                                      c->T, p.C_stride);
   }
   ETR_LAUNCH_CHECK();
   ETR_TIME_BEGIN("csr_count_kernel");
   int32_t* block_total = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(ws) + select_keys_bytes(c));
   const int nblocks = ceil_div(c->T, 256);
-  csr_count_kernel<<<nblocks, 256, 0, st>>>((const int32_t*)keyT, rt->tok_ptr, block_total, stats, c->T, c->E);
+  launch_kernel(csr_count_kernel, nblocks, 256, 0, st, 1, (const int32_t*)keyT, rt->tok_ptr, block_total, stats, c->T, c->E);
   ETR_LAUNCH_CHECK();
   const int n_cand = p.mode == ETR_MODE_TCR ? c->T * c->k : c->T * c->E;
-  ETR_TIME_BEGIN("csr_scan_kernel");
-  csr_scan_kernel<<<1, 1024, 0, st>>>(block_total, rt->tok_ptr, stats, nblocks, n_cand, skipped,
-                                      ceil_div(c->T, SEL_TB));
-  ETR_LAUNCH_CHECK();
   ETR_TIME_BEGIN("csr_fill_kernel");
-  csr_fill_kernel<<<nblocks, 256, 0, st>>>((const int32_t*)keyT, block_total, rt->tok_ptr, rt->tok_row,
-                                           c->T, c->E, p.C_stride);
+  launch_kernel(csr_fill_kernel, nblocks, 256, 0, st, 1, (const int32_t*)keyT, (const int32_t*)block_total, rt->tok_ptr,
+                rt->tok_row, stats, c->T, c->E, p.C_stride, n_cand, (const int32_t*)skipped, ceil_div(c->T, SEL_TB));
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }
