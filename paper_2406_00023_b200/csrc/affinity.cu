@@ -1253,13 +1253,15 @@ static etr_status launch_bwd_dx(const etr_config* c, const void* X, const float*
                                (const T*)dXp_fused, (T*)dX, c->T, c->d, c->D, c->E, m, Cs);
     return ETR_OK;
   };
-  // chunked form of the fused kernel: as many tokens per block as keep cz within 48 KiB (at most 16)
+  // chunked form of the fused kernel: as many tokens per block as keep cz, beside the 10.2 KiB of its row lists,
+  // within the 48 KiB a launch gets without opting in (at most 16)
+  constexpr size_t cz_max = 37 * 1024;
   int tpb = DXC_MAX_TOKENS;
-  while (tpb > 2 && (size_t)tpb * m * sizeof(float) > 48 * 1024) tpb /= 2;
+  while (tpb > 2 && (size_t)tpb * m * sizeof(float) > cz_max) tpb /= 2;
   int d_shift = 0;
   while ((1 << d_shift) < c->D) ++d_shift;
   const bool group8 = c->D >= 8 && (1 << d_shift) == c->D;
-  if (dXp_fused && !ddelta && (size_t)tpb * m * sizeof(float) <= 48 * 1024) {
+  if (dXp_fused && !ddelta && (size_t)tpb * m * sizeof(float) <= cz_max) {
     const size_t csm = (size_t)tpb * m * sizeof(float);
     ETR_TIME_BEGIN("affinity_bwd_dx_fused_kernel");
     auto go = [&](auto k) {

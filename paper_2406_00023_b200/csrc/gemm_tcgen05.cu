@@ -24,6 +24,8 @@
 // device, and tiles are dealt round-robin to the CTAs of a persistent grid.  All waits on
 // mbarriers are bounded; on expiry the kernel records a code in etr_stats.error_word,
 // stops issuing work, releases its tensor memory and returns.
+#include <algorithm>
+
 #include "common.cuh"
 #include "tcgen05_ptx.cuh"
 
@@ -1204,14 +1206,384 @@ tc_grouped_gemm_pair_wide_kernel(const __grid_constant__ CUtensorMap mapA0, cons
   cluster_sync_all();                 // the next kernel's blocks may start on an SM as soon as its CTA is gone
 }
 
+// ---- CTA-pair kernel, operands exchanged ---------------------------------------------------------------
+// The contractions whose rows are the expert's tokens, with the weights as the M operand (256 rows of them per
+// pair, always full) and the tokens as N: N may be any multiple of 16 up to 256, so an expert's n rows are cut
+// into ceil(n / 256) tiles of equal size and only the last 16-row step is padded, where the forms above compute
+// whole tiles of 256 (or 128) token rows.  With few rows per expert (decoding) an MMA costs next to nothing and
+// the kernel is a stream of the weights.
+//
+//   out[t][n] = sum_k tokens[t][k] * weights[n][k]:  accumulator lane = n, column = token
+//
+// The epilogue turns the 32 x 32 blocks (lane = output column) through the warp's scratch with 16-bit stores.
+// SwiGLU: the 128 rows of a CTA are 64 rows of W1g and the same 64 of W1u; the warps that hold U hand it, in
+// fp32, to the warps that hold G through shared memory.  Ring, roles, waits and teardown are those of the pair form.
+constexpr uint32_t TCS_XBUF_BYTES = 16 * 32 * 4;      // per pair of epilogue warps: U of 16 tokens x 32 columns
+
+struct SwapParams {
+  int two_k;             // the first half of the K blocks from (A0, B0), the rest from (A1, B1)
+  int M, N, K, E;        // M: C_stride (bound of an expert's rows), N: output columns, K: of one range
+  int tok_box;           // rows of a token box (8, 16, 32 or 64)
+  const int32_t* counts;
+  __nv_bfloat16* out0; __nv_bfloat16* out1; __nv_bfloat16* out2;
+  const __nv_bfloat16* in0; const __nv_bfloat16* in1;
+  etr_stats* stats;
+  const int32_t* sc_tok; const float* sc_gate; __nv_bfloat16* sc_out; int sc_ld;      // as in TcParams
+  long long wait_limit;
+};
+struct SwapTile { int e, n0, t0, nt, rows, kblocks; };      // nt: tokens of the tile (a multiple of 16)
+
+__device__ __forceinline__ int swap_tile_rows(int n) {      // tokens per tile of an expert with n > 0 rows
+  const int parts = (n + 255) / 256;
+  return ((n + parts - 1) / parts + 15) & ~15;
+}
+__device__ __forceinline__ int swap_tiles(int n) { return n > 0 ? (n - 1) / swap_tile_rows(n) + 1 : 0; }
+__device__ __forceinline__ bool swap_tile(const SwapParams& p, const int* tile_prefix, const int* counts_s, int tile,
+                                          int& e_cur, int cols, SwapTile& t) {
+  if (tile >= tile_prefix[p.E]) return false;
+  while (tile >= tile_prefix[e_cur + 1]) ++e_cur;
+  const int local = tile - tile_prefix[e_cur], n = min(counts_s[e_cur], p.M);
+  const int size = swap_tile_rows(n), parts = (n - 1) / size + 1;
+  t.e = e_cur;
+  t.rows = n;
+  t.t0 = (local % parts) * size;
+  t.nt = min(size, (n - t.t0 + 15) & ~15);
+  t.n0 = (local / parts) * cols;
+  t.kblocks = (p.K + TC_BK - 1) / TC_BK * (p.two_k ? 2 : 1);
+  return true;
+}
+
+// 32 values of this lane (output column nb + lane; rows of the block in order) to rows 0 .. nrows - 1 of dst.
+__device__ __forceinline__ void store_turned(uint8_t* scratch, int lane, int nrows, __nv_bfloat16* dst, int ld,
+                                             const float* v) {
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    *reinterpret_cast<__nv_bfloat16*>(scratch + j * TC_SCRATCH_ROW_BYTES + 2 * lane) = __float2bfloat16_rn(v[j]);
+  __syncwarp();
+  const int sub = lane & 3;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int row = (lane >> 2) + 8 * i;
+    const uint4 w = *reinterpret_cast<const uint4*>(scratch + row * TC_SCRATCH_ROW_BYTES + sub * 16);
+    if (row < nrows) *reinterpret_cast<uint4*>(dst + (long long)row * ld + sub * 8) = w;
+  }
+  __syncwarp();
+}
+// The block just stored once more, scaled, to the rows of its tokens (Top-1 combine, see scatter32_warp); the
+// scratch still holds it.
+__device__ __forceinline__ void scatter_turned(const uint8_t* scratch, int lane, int nrows, const int32_t* tok,
+                                               const float* gate, __nv_bfloat16* out, int ld) {
+  const int sub = lane & 3;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int row = (lane >> 2) + 8 * i;
+    if (row >= nrows) continue;
+    const int t = tok[row];
+    if (t < 0) continue;
+    const float g = gate[row];
+    const uint4 w = *reinterpret_cast<const uint4*>(scratch + row * TC_SCRATCH_ROW_BYTES + sub * 16);
+    const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+    uint32_t y[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) y[k] = pack_bf16(g * __uint_as_float(u[k] << 16), g * __uint_as_float(u[k] & 0xffff0000u));
+    *reinterpret_cast<uint4*>(out + (long long)t * ld + sub * 8) = make_uint4(y[0], y[1], y[2], y[3]);
+  }
+  __syncwarp();
+}
+// A 32-row x 32-column block of a row-major tensor to this lane's column: v[j] = src[j][lane] (rows past nrows: 0).
+__device__ __forceinline__ void load_turned(uint8_t* scratch, int lane, const uint4 (&t)[4], float* v) {
+  const int sub = lane & 3;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    *reinterpret_cast<uint4*>(scratch + ((lane >> 2) + 8 * i) * TC_SCRATCH_ROW_BYTES + sub * 16) = t[i];
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    v[j] = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(scratch + j * TC_SCRATCH_ROW_BYTES + 2 * lane));
+  __syncwarp();
+}
+// Zeros to rows r0 .. r1 - 1 of a 32-column block (the pad rows behind an expert's last tile), 8 rows at a time.
+__device__ __forceinline__ void zero_rows32(__nv_bfloat16* dst, int ld, int r0, int r1, int lane) {
+  for (int r = r0 + (lane >> 2); r < r1; r += 8)
+    *reinterpret_cast<uint4*>(dst + (long long)r * ld + (lane & 3) * 8) = make_uint4(0, 0, 0, 0);
+}
+
+template <int EPI, bool A_MN>
+__global__ void __launch_bounds__(TC_THREADS, 1)
+tc_grouped_gemm_swap_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
+                            const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
+                            const SwapParams p, uint32_t idesc) {
+  constexpr bool DUAL = EPI == TC_EPI_SWIGLU;
+  constexpr int COLS = DUAL ? 128 : 256;           // output columns of a pair tile
+  constexpr uint32_t TMEM_COLS = 512;              // two accumulator stages of 256 tokens
+
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t bars[2 * TC2_STAGES + 4 + 8];
+  __shared__ uint32_t tmem_base_slot;
+  __shared__ int abort_flag_s;
+  __shared__ int tile_prefix[257];
+  __shared__ int s_counts[256];
+
+  volatile int* abort_flag = &abort_flag_s;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t rank = cluster_ctarank();
+  const int pair = (int)cluster_id_x(), npairs = (int)cluster_count_x();
+  const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const uint32_t full_bar = smem_u32(&bars[0]);                    // [TC2_STAGES]  used in the leader
+  const uint32_t empty_bar = smem_u32(&bars[TC2_STAGES]);          // [TC2_STAGES]  in each CTA
+  const uint32_t tfull_bar = smem_u32(&bars[2 * TC2_STAGES]);      // [2]           in each CTA
+  const uint32_t tempty_bar = smem_u32(&bars[2 * TC2_STAGES + 2]); // [2]           used in the leader
+  const uint32_t xfull_bar = smem_u32(&bars[2 * TC2_STAGES + 4]);  // [4]  SwiGLU: U is in the exchange buffer
+  const uint32_t xempty_bar = smem_u32(&bars[2 * TC2_STAGES + 8]); // [4]  ... and has been read
+
+  if (tid == 0) {
+    abort_flag_s = 0;
+    for (int s = 0; s < TC2_STAGES; ++s) { mbar_init(full_bar + 8 * s, 1); mbar_init(empty_bar + 8 * s, 1); }
+    for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar + 8 * a, 1); mbar_init(tempty_bar + 8 * a, 16); }
+    for (int x = 0; x < 4; ++x) { mbar_init(xfull_bar + 8 * x, 1); mbar_init(xempty_bar + 8 * x, 1); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(TMEM_COLS) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  grid_sync();
+  for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
+  __syncthreads();
+  if (warp == 2) {
+    const int nc = (p.N + COLS - 1) / COLS;
+    tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) { return nc * swap_tiles(min(n_e, p.M)); });
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();                 // both CTAs' barriers exist before any remote arrive
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_base_slot;
+  const uint32_t leader_full = map_to_cta(full_bar, 0);
+  const uint32_t leader_tempty = map_to_cta(tempty_bar, 0);
+
+  if (warp == 0) {
+    // ---- TMA producer (both CTAs) ---------------------------------------------------------------
+    int e_cur = 0, stage = 0;
+    uint32_t phase = 0;
+    SwapTile t;
+    bool ok = true;
+    for (int tile = pair; ok && swap_tile(p, tile_prefix, s_counts, tile, e_cur, COLS, t); tile += npairs) {
+      const int kb1 = p.two_k ? t.kblocks / 2 : t.kblocks;
+      const int tr0 = t.t0 + (int)rank * (t.nt / 2), boxes = (t.nt / 2 + p.tok_box - 1) / p.tok_box;
+      const uint32_t box_bytes = (uint32_t)p.tok_box * 128u;
+      for (int kb = 0; kb < t.kblocks; ++kb) {
+        ok = __all_sync(0xffffffffu, mbar_wait_cluster(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.wait_limit));
+        if (!ok) break;
+        if (elect_one()) {
+          if (rank == 0) mbar_expect_tx(full_bar + 8 * stage, 2 * (2 * TC_BOX_BYTES + boxes * box_bytes));
+          const uint32_t fb = leader_full + 8 * stage;
+          const bool second = kb >= kb1;
+          const int k0 = (second ? kb - kb1 : kb) * TC_BK;
+          const uint32_t sa = tiles_base + stage * TC2_STAGE_BYTES, sb = sa + 2 * TC_BOX_BYTES;
+          const CUtensorMap* ma = second ? &mapA1 : &mapA0;
+          const CUtensorMap* mb = second ? &mapB1 : &mapB0;
+          if (DUAL) {
+            tma_load_3d_pair(sa, &mapA0, fb, k0, t.n0 + 64 * (int)rank, t.e);
+            tma_load_3d_pair(sa + TC_BOX_BYTES, &mapA1, fb, k0, t.n0 + 64 * (int)rank, t.e);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+              const int n = t.n0 + 128 * (int)rank + 64 * j;
+              if (A_MN) tma_load_3d_pair(sa + j * TC_BOX_BYTES, ma, fb, n, k0, t.e);
+              else      tma_load_3d_pair(sa + j * TC_BOX_BYTES, ma, fb, k0, n, t.e);
+            }
+          }
+          for (int i = 0; i < boxes; ++i) tma_load_3d_pair(sb + i * box_bytes, mb, fb, k0, tr0 + i * p.tok_box, t.e);
+        }
+        __syncwarp();
+        if (++stage == TC2_STAGES) { stage = 0; phase ^= 1u; }
+      }
+    }
+  } else if (warp == 1) {
+    // ---- MMA issuer (leader CTA only) --------------------------------------------------------------
+    if (rank == 0) {
+      int e_cur = 0, stage = 0, acc_stage = 0;
+      uint32_t phase = 0, acc_phase = 0;
+      SwapTile t;
+      bool ok = true;
+      constexpr uint32_t a_lbo = A_MN ? TC_BOX_BYTES : 16u, a_kstep = A_MN ? 2048u : 32u;
+      for (int tile = pair; ok && swap_tile(p, tile_prefix, s_counts, tile, e_cur, COLS, t); tile += npairs) {
+        ok = __all_sync(0xffffffffu, mbar_wait_cluster(tempty_bar + 8 * acc_stage, acc_phase ^ 1u, abort_flag, p.wait_limit));
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t d_tmem = tmem_base + (uint32_t)(acc_stage * 256);
+        const uint32_t id = idesc | ((uint32_t)(t.nt >> 3) << 17);
+        for (int kb = 0; kb < t.kblocks; ++kb) {
+          ok = __all_sync(0xffffffffu, mbar_wait_cluster(full_bar + 8 * stage, phase, abort_flag, p.wait_limit));
+          if (!ok) break;
+          tc_fence_after();
+          if (elect_one()) {
+            const uint32_t sa = tiles_base + stage * TC2_STAGE_BYTES, sb = sa + 2 * TC_BOX_BYTES;
+#pragma unroll
+            for (int kk = 0; kk < TC_BK / 16; ++kk)
+              tc_mma_pair(d_tmem, make_smem_desc(sa + kk * a_kstep, a_lbo, 1024u), make_smem_desc(sb + kk * 32u, 16u, 1024u),
+                          id, (kb > 0 || kk > 0) ? 1u : 0u);
+            tc_commit_pair(empty_bar + 8 * stage);                       // frees the stage in both CTAs
+            if (kb + 1 == t.kblocks) tc_commit_pair(tfull_bar + 8 * acc_stage);      // accumulators complete in both CTAs
+          }
+          __syncwarp();
+          if (++stage == TC2_STAGES) { stage = 0; phase ^= 1u; }
+        }
+        if (++acc_stage == 2) { acc_stage = 0; acc_phase ^= 1u; }
+      }
+    }
+  } else {
+    // ---- epilogue warps (both CTAs, own 128 lanes) -----------------------------------------------------
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    uint8_t* scratch = smem_raw + (tiles_base - smem_u32(smem_raw)) + TC2_STAGES * TC2_STAGE_BYTES + (warp - 2) * TC_SCRATCH_BYTES;
+    const int x = 2 * half + (q & 1);               // SwiGLU: the exchange this warp takes part in
+    const bool is_u = DUAL && q >= 2;
+    float* xbuf = reinterpret_cast<float*>(smem_raw + (tiles_base - smem_u32(smem_raw)) + TC2_STAGES * TC2_STAGE_BYTES +
+                                           8 * TC_SCRATCH_BYTES + x * TCS_XBUF_BYTES);
+    uint32_t x_phase = 0;
+    int e_cur = 0, acc_stage = 0;
+    uint32_t acc_phase = 0;
+    SwapTile t;
+    bool ok = true;
+    for (int tile = pair; ok && swap_tile(p, tile_prefix, s_counts, tile, e_cur, COLS, t); tile += npairs) {
+      const int nb = DUAL ? t.n0 + 64 * (int)rank + 32 * (q & 1) : t.n0 + 128 * (int)rank + 32 * q;      // first column
+      const bool live = nb < p.N;
+      const long long row0 = (long long)t.e * p.M + t.t0;
+      const int chunks = (t.nt + 31) / 32;
+      const long long ob = row0 * p.N + nb;
+      uint4 pg[4], pu[4];
+      if (EPI == TC_EPI_DSWIGLU && live && half < chunks) {      // the saved G and U of the first chunk
+        const int nv = min(32, t.nt - 32 * half);
+        load32_warp_issue(p.in0 + ob + (long long)(32 * half) * p.N, p.N, lane, nv, pg);
+        load32_warp_issue(p.in1 + ob + (long long)(32 * half) * p.N, p.N, lane, nv, pu);
+      }
+      ok = __all_sync(0xffffffffu, mbar_wait_cluster(tfull_bar + 8 * acc_stage, acc_phase, abort_flag, p.wait_limit));
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t taddr = tmem_base + (uint32_t)(acc_stage * 256) + ((uint32_t)(32 * q) << 16);
+      for (int c = half; c < chunks; c += 2) {
+        const int nv = min(32, t.nt - 32 * c);                   // rows of this chunk (columns past nt hold nothing of use)
+        const long long cb = ob + (long long)(32 * c) * p.N;
+        __syncwarp();
+        uint32_t r[32];
+        tc_ld32(taddr + 32 * c, r);
+        tc_wait_ld();
+        float v[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+        if (EPI == TC_EPI_SWIGLU) {
+          if (is_u) {
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+              ok = __all_sync(0xffffffffu, mbar_wait(xempty_bar + 8 * x, x_phase ^ 1u, abort_flag, p.wait_limit));
+              if (!ok) break;
+#pragma unroll
+              for (int j = 0; j < 16; ++j) xbuf[32 * j + lane] = v[16 * s + j];
+              __syncwarp();
+              if (lane == 0) mbar_arrive(xfull_bar + 8 * x);
+              x_phase ^= 1u;
+            }
+            if (!ok) break;
+            if (live) store_turned(scratch, lane, nv, p.out1 + cb, p.N, v);
+          } else {
+            float hv[32];
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+              ok = __all_sync(0xffffffffu, mbar_wait(xfull_bar + 8 * x, x_phase, abort_flag, p.wait_limit));
+              if (!ok) break;
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const float g = v[16 * s + j];
+                hv[16 * s + j] = __fdividef(g, 1.0f + __expf(-g)) * xbuf[32 * j + lane];
+              }
+              __syncwarp();
+              if (lane == 0) mbar_arrive(xempty_bar + 8 * x);
+              x_phase ^= 1u;
+            }
+            if (!ok) break;
+            if (live) {
+              store_turned(scratch, lane, nv, p.out0 + cb, p.N, v);
+              store_turned(scratch, lane, nv, p.out2 + cb, p.N, hv);
+            }
+          }
+        } else if (EPI == TC_EPI_DSWIGLU) {
+          if (live) {
+            float g[32], u[32];
+            load_turned(scratch, lane, pg, g);
+            load_turned(scratch, lane, pu, u);
+            if (c + 2 < chunks) {
+              const int nx = min(32, t.nt - 32 * (c + 2));
+              load32_warp_issue(p.in0 + cb + 64ll * p.N, p.N, lane, nx, pg);
+              load32_warp_issue(p.in1 + cb + 64ll * p.N, p.N, lane, nx, pu);
+            }
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              const float dh = v[j], sgm = __fdividef(1.0f, 1.0f + __expf(-g[j]));
+              const float dgj = dh * u[j] * sgm * (1.0f + g[j] * (1.0f - sgm));
+              v[j] = dh * g[j] * sgm;
+              g[j] = dgj;
+            }
+            store_turned(scratch, lane, nv, p.out0 + cb, p.N, g);
+            store_turned(scratch, lane, nv, p.out1 + cb, p.N, v);
+          }
+        } else if (live) {
+          store_turned(scratch, lane, nv, p.out0 + cb, p.N, v);
+          if (p.sc_out != nullptr)
+            scatter_turned(scratch, lane, nv, p.sc_tok + row0 + 32 * c, p.sc_gate + row0 + 32 * c, p.sc_out + nb, p.sc_ld);
+        }
+      }
+      if (!ok) break;
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(leader_tempty + 8 * acc_stage);
+      if (++acc_stage == 2) { acc_stage = 0; acc_phase ^= 1u; }
+      if (live && t.t0 + t.nt >= t.rows) {           // the expert's last tile: its pad rows, half of them per warp
+        const int z0 = t.t0 + t.nt, z1 = min((t.rows + TC_BM - 1) / TC_BM * TC_BM, p.M);
+        if (z0 < z1) {
+          const int zm = z0 + (z1 - z0) / 2, a = half ? zm : z0, b = half ? z1 : zm;
+          const long long eb = (long long)t.e * p.M * p.N + nb;
+          if (EPI == TC_EPI_SWIGLU) {
+            if (is_u) {
+              zero_rows32(p.out1 + eb, p.N, a, b, lane);
+            } else {
+              zero_rows32(p.out0 + eb, p.N, a, b, lane);
+              zero_rows32(p.out2 + eb, p.N, a, b, lane);
+            }
+          } else {
+            zero_rows32(p.out0 + eb, p.N, a, b, lane);
+            if (EPI == TC_EPI_DSWIGLU) zero_rows32(p.out1 + eb, p.N, a, b, lane);
+          }
+        }
+      }
+    }
+  }
+
+  // ---- teardown: neither CTA leaves while the other may still touch its barriers or memory -------
+  __syncwarp();
+  if (*abort_flag) {
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2000000ll) { }
+    if (tid == 0) atomicExch(&p.stats->error_word, 0x7c0b);
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+  }
+  cluster_sync_all();                 // the next kernel's blocks may start on an SM as soon as its CTA is gone
+}
+
 // ---- host side --------------------------------------------------------------------------------------
-// Row-major bf16 tensor [E, rows, cols] as a 3-D map (cols, rows, E), 64x64 boxes, 128-byte swizzle.
-static etr_status make_map(CUtensorMap* m, const void* base, int cols, int rows, int E) {
+// Row-major bf16 tensor [E, rows, cols] as a 3-D map (cols, rows, E), boxes of 64 columns x box_rows, 128-byte swizzle.
+static etr_status make_map(CUtensorMap* m, const void* base, int cols, int rows, int E, int box_rows = 64) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return ETR_ERR_CUDA;
   const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)E};
   const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * 2 * (cuuint64_t)rows};
-  const cuuint32_t box[3] = {64, 64, 1};
+  const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
   const cuuint32_t estr[3] = {1, 1, 1};
   const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
                         estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -1379,6 +1751,34 @@ static etr_status tc_run(TcForm form, const char* name, const CUtensorMap& a0, c
   return tc_launch<256, EPI>(name, a0, a1, b0, b1, p, max_tiles, st);
 }
 
+// ---- exchanged operands: host side ----------------------------------------------------------------------
+// Rows of a token box: half of a tile's tokens at most, so that a layer with few rows per expert fetches few.
+static int swap_tok_box(const etr_config* c) {
+  const int half = std::min(64, ceil_div(std::min(c->capacity, 256), 16) * 8);
+  return half <= 8 ? 8 : half <= 16 ? 16 : half <= 32 ? 32 : 64;
+}
+static bool use_swap(const etr_config* c) { return c->gemm_impl == ETR_GEMM_AUTO; }
+static SwapParams swap_params(const etr_config* c, const etr_route* rt, etr_stats* stats) {
+  SwapParams p = {};
+  p.M = c_stride_of(c); p.E = c->E; p.tok_box = swap_tok_box(c); p.counts = rt->counts; p.stats = stats;
+  p.wait_limit = c->wait_limit_cycles > 0 ? (long long)c->wait_limit_cycles : TC_WAIT_LIMIT_CYCLES;
+  return p;
+}
+template <int EPI, bool A_MN>
+static etr_status swap_launch(const char* name, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0,
+                              const CUtensorMap& b1, const SwapParams& p, cudaStream_t st) {
+  constexpr size_t smem = (size_t)TC2_STAGES * TC2_STAGE_BYTES + 1024 + 8 * TC_SCRATCH_BYTES + 4 * TCS_XBUF_BYTES;
+  auto k = tc_grouped_gemm_swap_kernel<EPI, A_MN>;
+  static std::atomic<unsigned long long> attr_done{0};      // one bit per device
+  if (!ensure_dyn_smem(k, smem, attr_done)) return ETR_ERR_CUDA;
+  const int tiles = p.E * ceil_div(p.M, 256) * ceil_div(p.N, EPI == TC_EPI_SWIGLU ? 128 : 256);
+  const int pairs = std::max(1, std::min(tiles, sm_count() / 2));
+  ETR_TIME_BEGIN(name);
+  launch_kernel(k, 2 * pairs, TC_THREADS, smem, st, 2, a0, a1, b0, b1, p, make_idesc(A_MN, 0, 0, 256));
+  ETR_LAUNCH_CHECK();
+  return ETR_OK;
+}
+
 static TcParams tc_params(const etr_config* c) {
   TcParams p = {};
   p.wait_limit = c->wait_limit_cycles > 0 ? (long long)c->wait_limit_cycles : TC_WAIT_LIMIT_CYCLES;
@@ -1393,6 +1793,21 @@ etr_status tc_ffn_forward(const etr_config* c, const etr_route* rt, const void* 
                           etr_stats* stats, void*, void* Y_top1, cudaStream_t st) {
   const int d = c->d, h = c->h, Cs = c_stride_of(c), E = c->E;
   CUtensorMap mXp, mW1g, mW1u, mW2, mH;
+  if (use_swap(c) && !Xtok) {
+    SwapParams p = swap_params(c, rt, stats);
+    ETR_TRY(make_map(&mXp, Xp, d, Cs, E, p.tok_box));
+    ETR_TRY(make_map(&mH, H, h, Cs, E, p.tok_box));
+    ETR_TRY(make_map(&mW1g, W1g, d, h, E));
+    ETR_TRY(make_map(&mW1u, W1u, d, h, E));
+    ETR_TRY(make_map(&mW2, W2, h, d, E));
+    p.N = h; p.K = d;
+    p.out0 = (__nv_bfloat16*)G; p.out1 = (__nv_bfloat16*)U; p.out2 = (__nv_bfloat16*)H;
+    ETR_TRY((swap_launch<TC_EPI_SWIGLU, false>("tc_gemm_swiglu", mW1g, mW1u, mXp, mXp, p, st)));
+    p.N = d; p.K = h;
+    p.out0 = (__nv_bfloat16*)O; p.out1 = p.out2 = nullptr;
+    if (Y_top1) { p.sc_tok = rt->slot_token; p.sc_gate = rt->gate; p.sc_out = (__nv_bfloat16*)Y_top1; p.sc_ld = d; }
+    return swap_launch<TC_EPI_STORE, false>("tc_gemm_down", mW2, mW2, mH, mH, p, st);
+  }
   if (Xtok) ETR_TRY(make_gather_map(&mXp, Xtok, d, c->T));
   else ETR_TRY(make_map(&mXp, Xp, d, Cs, E));
   ETR_TRY(make_map(&mW1g, W1g, d, h, E));
@@ -1437,22 +1852,37 @@ etr_status tc_ffn_backward(const etr_config* c, const etr_route* rt, const void*
   ETR_TRY(make_map(&mW1u, W1u, d, h, E));
   ETR_TRY(make_map(&mW2, W2, h, d, E));
   const int mt = Cs / TC_BM;
-  {  // dH = dO W2 (W2 read with its output index contiguous), then dG, dU
-    TcParams p = tc_params(c);
-    p.b_mn = 1; p.M = Cs; p.N = h; p.K = d; p.dyn = TC_DYN_M; p.E = E; p.counts = rt->counts;
+  if (use_swap(c) && !Xtok) {      // (with the dispatch fused the forms below serve every contraction)
+    SwapParams p = swap_params(c, rt, stats);
+    CUtensorMap tdO, tdG, tdU;
+    ETR_TRY(make_map(&tdO, dO, d, Cs, E, p.tok_box));
+    ETR_TRY(make_map(&tdG, dG, h, Cs, E, p.tok_box));
+    ETR_TRY(make_map(&tdU, dU, h, Cs, E, p.tok_box));
+    p.N = h; p.K = d;
     p.out0 = (__nv_bfloat16*)dG; p.out1 = (__nv_bfloat16*)dU;
     p.in0 = (const __nv_bfloat16*)G; p.in1 = (const __nv_bfloat16*)U;
-    p.out_bs = (long long)Cs * h; p.ld_out = h; p.stats = stats;
-    ETR_TRY((tc_run<TC_EPI_DSWIGLU>(tc_form_of(c, TC_EPI_DSWIGLU, p), "tc_gemm_dswiglu", mdO, mdO, mW2, mW2, p,
-                                            E * mt * ceil_div(h, 256), st)));
-  }
-  {  // dXp = dG W1g + dU W1u: one contraction over 2h
-    TcParams p = tc_params(c);
-    p.b_mn = 1; p.k1_blocks = ceil_div(h, TC_BK); p.M = Cs; p.N = d; p.K = 2 * h; p.dyn = TC_DYN_M;
-    p.E = E; p.counts = rt->counts;
-    p.out0 = (__nv_bfloat16*)dXp; p.out_bs = (long long)Cs * d; p.ld_out = d; p.stats = stats;
-    ETR_TRY((tc_run<TC_EPI_STORE>(tc_form_of(c, TC_EPI_STORE, p), "tc_gemm_dxp", mdG, mdU, mW1g, mW1u, p,
-                                          E * mt * ceil_div(d, 256), st)));
+    ETR_TRY((swap_launch<TC_EPI_DSWIGLU, true>("tc_gemm_dswiglu", mW2, mW2, tdO, tdO, p, st)));
+    p.N = d; p.K = h; p.two_k = 1;
+    p.out0 = (__nv_bfloat16*)dXp; p.out1 = nullptr; p.in0 = p.in1 = nullptr;
+    ETR_TRY((swap_launch<TC_EPI_STORE, true>("tc_gemm_dxp", mW1g, mW1u, tdG, tdU, p, st)));
+  } else {
+    {  // dH = dO W2 (W2 read with its output index contiguous), then dG, dU
+      TcParams p = tc_params(c);
+      p.b_mn = 1; p.M = Cs; p.N = h; p.K = d; p.dyn = TC_DYN_M; p.E = E; p.counts = rt->counts;
+      p.out0 = (__nv_bfloat16*)dG; p.out1 = (__nv_bfloat16*)dU;
+      p.in0 = (const __nv_bfloat16*)G; p.in1 = (const __nv_bfloat16*)U;
+      p.out_bs = (long long)Cs * h; p.ld_out = h; p.stats = stats;
+      ETR_TRY((tc_run<TC_EPI_DSWIGLU>(tc_form_of(c, TC_EPI_DSWIGLU, p), "tc_gemm_dswiglu", mdO, mdO, mW2, mW2, p,
+                                              E * mt * ceil_div(h, 256), st)));
+    }
+    {  // dXp = dG W1g + dU W1u: one contraction over 2h
+      TcParams p = tc_params(c);
+      p.b_mn = 1; p.k1_blocks = ceil_div(h, TC_BK); p.M = Cs; p.N = d; p.K = 2 * h; p.dyn = TC_DYN_M;
+      p.E = E; p.counts = rt->counts;
+      p.out0 = (__nv_bfloat16*)dXp; p.out_bs = (long long)Cs * d; p.ld_out = d; p.stats = stats;
+      ETR_TRY((tc_run<TC_EPI_STORE>(tc_form_of(c, TC_EPI_STORE, p), "tc_gemm_dxp", mdG, mdU, mW1g, mW1u, p,
+                                            E * mt * ceil_div(d, 256), st)));
+    }
   }
   {  // dW2 = dO^T H: contraction over the expert's rows, both operands MN-major
     TcParams p = tc_params(c);

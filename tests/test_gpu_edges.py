@@ -205,3 +205,11 @@ def test_sweep_modes_follow_the_step():
         assert st.C == ob.capacity_bound(w.d, w.E, w.capacity, 1, True, st.delta_max)
         if want == etr.MODE_ECR:
             assert np.all(hz.to_np(buf.counts) == min(st.C, w.T))
+
+
+@pytest.mark.parametrize("d,D", [(2560, 4), (2432, 4), (3072, 4), (2368, 4), (4096, 4), (1216, 1)])
+def test_pooled_widths_at_the_shared_memory_limit_of_the_fused_dx_kernel(d, D):
+    """608 to 768 (and 1216 to 1536) pooled columns: cz of 16 (8) tokens together with the row lists is more shared
+    memory than a launch gets without opting in."""
+    w = gw.scaled(W["small"], T=70, d=d, D=D, E=4, h=64)
+    layer_vs_oracle(w, gw.make_inputs(w), ob.MODE_TCR)
