@@ -1215,7 +1215,8 @@ tc_grouped_gemm_pair_wide_kernel(const __grid_constant__ CUtensorMap mapA0, cons
 //
 //   out[t][n] = sum_k tokens[t][k] * weights[n][k]:  accumulator lane = n, column = token
 //
-// The epilogue turns the 32 x 32 blocks (lane = output column) through the warp's scratch with 16-bit stores.
+// The epilogue turns the 32 x 32 blocks (lane = output column) through the warp's scratch with transposing stmatrix
+// (16-bit stores instead made the fused epilogues the bound of contractions over 1024 or less).
 // SwiGLU: the 128 rows of a CTA are 64 rows of W1g and the same 64 of W1u; the warps that hold U hand it, in
 // fp32, to the warps that hold G through shared memory.  Ring, roles, waits and teardown are those of the pair form.
 constexpr uint32_t TCS_XBUF_BYTES = 16 * 32 * 4;      // per pair of epilogue warps: U of 16 tokens x 32 columns
@@ -1237,7 +1238,6 @@ __device__ __forceinline__ int swap_tile_rows(int n) {      // tokens per tile o
   const int parts = (n + 255) / 256;
   return ((n + parts - 1) / parts + 15) & ~15;
 }
-__device__ __forceinline__ int swap_tiles(int n) { return n > 0 ? (n - 1) / swap_tile_rows(n) + 1 : 0; }
 __device__ __forceinline__ bool swap_tile(const SwapParams& p, const int* tile_prefix, const int* counts_s, int tile,
                                           int& e_cur, int cols, SwapTile& t) {
   if (tile >= tile_prefix[p.E]) return false;
@@ -1253,12 +1253,35 @@ __device__ __forceinline__ bool swap_tile(const SwapParams& p, const int* tile_p
   return true;
 }
 
-// 32 values of this lane (output column nb + lane; rows of the block in order) to rows 0 .. nrows - 1 of dst.
+// A 32 x 32 block of accumulators (lanes = output columns, columns = tokens) as matrix fragments: two loads of
+// 16 lanes, each thread lane t / 4 (and + 8) at the token pair 2 (t % 4) of every eight tokens.  Value index
+// 16 * (lane half) + 4 * (eight tokens) + 2 * (+ 8 lanes) + (token of the pair): the fragment of stmatrix and
+// ldmatrix, whose transposing forms turn the block to and from row-major bf16.
+__device__ __forceinline__ void tc_ld_block(uint32_t taddr, uint32_t* r) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t* p = r + 16 * h;
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(p[0]), "=r"(p[1]), "=r"(p[2]), "=r"(p[3]), "=r"(p[4]), "=r"(p[5]), "=r"(p[6]), "=r"(p[7]),
+          "=r"(p[8]), "=r"(p[9]), "=r"(p[10]), "=r"(p[11]), "=r"(p[12]), "=r"(p[13]), "=r"(p[14]), "=r"(p[15])
+        : "r"(taddr + ((uint32_t)(16 * h) << 16)));
+  }
+}
+// Address of this lane's row of the 8 x 8 matrices of eight tokens (i): token row, 16 bytes per 8 output columns.
+__device__ __forceinline__ uint32_t turn_addr(const uint8_t* scratch, int lane, int i) {
+  return smem_u32(scratch) + (8 * i + (lane & 7)) * TC_SCRATCH_ROW_BYTES + (lane >> 3) * 16;
+}
+// Such a block, rounded to bf16, to rows 0 .. nrows - 1 of dst (first row, first of the 32 columns).
 __device__ __forceinline__ void store_turned(uint8_t* scratch, int lane, int nrows, __nv_bfloat16* dst, int ld,
                                              const float* v) {
 #pragma unroll
-  for (int j = 0; j < 32; ++j)
-    *reinterpret_cast<__nv_bfloat16*>(scratch + j * TC_SCRATCH_ROW_BYTES + 2 * lane) = __float2bfloat16_rn(v[j]);
+  for (int i = 0; i < 4; ++i)
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};"
+                 ::"r"(turn_addr(scratch, lane, i)), "r"(pack_bf16(v[4 * i], v[4 * i + 1])),
+                 "r"(pack_bf16(v[4 * i + 2], v[4 * i + 3])), "r"(pack_bf16(v[16 + 4 * i], v[16 + 4 * i + 1])),
+                 "r"(pack_bf16(v[16 + 4 * i + 2], v[16 + 4 * i + 3])) : "memory");
   __syncwarp();
   const int sub = lane & 3;
 #pragma unroll
@@ -1290,16 +1313,19 @@ __device__ __forceinline__ void scatter_turned(const uint8_t* scratch, int lane,
   }
   __syncwarp();
 }
-// A 32-row x 32-column block of a row-major tensor to this lane's column: v[j] = src[j][lane] (rows past nrows: 0).
-__device__ __forceinline__ void load_turned(uint8_t* scratch, int lane, const uint4 (&t)[4], float* v) {
+// The reverse: a 32-row x 32-column block fetched by load32_warp_issue, as fragments of bf16 pairs (word
+// 4 * (eight tokens) + matrix, the pairs that store_turned packs).
+__device__ __forceinline__ void load_turned(uint8_t* scratch, int lane, const uint4 (&t)[4], uint32_t* w) {
   const int sub = lane & 3;
 #pragma unroll
   for (int i = 0; i < 4; ++i)
     *reinterpret_cast<uint4*>(scratch + ((lane >> 2) + 8 * i) * TC_SCRATCH_ROW_BYTES + sub * 16) = t[i];
   __syncwarp();
 #pragma unroll
-  for (int j = 0; j < 32; ++j)
-    v[j] = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(scratch + j * TC_SCRATCH_ROW_BYTES + 2 * lane));
+  for (int i = 0; i < 4; ++i)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(w[4 * i]), "=r"(w[4 * i + 1]), "=r"(w[4 * i + 2]), "=r"(w[4 * i + 3])
+                 : "r"(turn_addr(scratch, lane, i)) : "memory");
   __syncwarp();
 }
 // Zeros to rows r0 .. r1 - 1 of a 32-column block (the pad rows behind an expert's last tile), 8 rows at a time.
@@ -1352,7 +1378,10 @@ tc_grouped_gemm_swap_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
   __syncthreads();
   if (warp == 2) {
     const int nc = (p.N + COLS - 1) / COLS;
-    tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) { return nc * swap_tiles(min(n_e, p.M)); });
+    tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) {
+      const int n = min(n_e, p.M);
+      return n > 0 ? nc * ((n - 1) / swap_tile_rows(n) + 1) : 0;
+    });
   }
   tc_fence_before();
   __syncthreads();
@@ -1453,6 +1482,18 @@ tc_grouped_gemm_swap_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
       const int chunks = (t.nt + 31) / 32;
       const long long ob = row0 * p.N + nb;
       uint4 pg[4], pu[4];
+      if (EPI == TC_EPI_DSWIGLU) {                   // G and U of the warp's part of the NEXT tile, towards L2
+        SwapTile tn;
+        int e_next = e_cur;
+        if (swap_tile(p, tile_prefix, s_counts, tile + npairs, e_next, COLS, tn)) {
+          const int nn = tn.n0 + 128 * (int)rank + 32 * q;
+          for (int r = 32 * half + lane; nn < p.N && r < tn.nt; r += 64) {
+            const long long o = ((long long)tn.e * p.M + tn.t0 + r) * p.N + nn;
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.in0 + o));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.in1 + o));
+          }
+        }
+      }
       if (EPI == TC_EPI_DSWIGLU && live && half < chunks) {      // the saved G and U of the first chunk
         const int nv = min(32, t.nt - 32 * half);
         load32_warp_issue(p.in0 + ob + (long long)(32 * half) * p.N, p.N, lane, nv, pg);
@@ -1467,7 +1508,7 @@ tc_grouped_gemm_swap_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
         const long long cb = ob + (long long)(32 * c) * p.N;
         __syncwarp();
         uint32_t r[32];
-        tc_ld32(taddr + 32 * c, r);
+        tc_ld_block(taddr + 32 * c, r);
         tc_wait_ld();
         float v[32];
 #pragma unroll
@@ -1509,9 +1550,10 @@ tc_grouped_gemm_swap_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
           }
         } else if (EPI == TC_EPI_DSWIGLU) {
           if (live) {
-            float g[32], u[32];
-            load_turned(scratch, lane, pg, g);
-            load_turned(scratch, lane, pu, u);
+            uint32_t gw[16], uw[16];
+            float g[32];
+            load_turned(scratch, lane, pg, gw);
+            load_turned(scratch, lane, pu, uw);
             if (c + 2 < chunks) {
               const int nx = min(32, t.nt - 32 * (c + 2));
               load32_warp_issue(p.in0 + cb + 64ll * p.N, p.N, lane, nx, pg);
@@ -1519,10 +1561,12 @@ tc_grouped_gemm_swap_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
             }
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
-              const float dh = v[j], sgm = __fdividef(1.0f, 1.0f + __expf(-g[j]));
-              const float dgj = dh * u[j] * sgm * (1.0f + g[j] * (1.0f - sgm));
-              v[j] = dh * g[j] * sgm;
-              g[j] = dgj;
+              const int k = 4 * ((j & 15) >> 2) + 2 * (j >> 4) + ((j >> 1) & 1);      // value j is half (j & 1) of word k
+              const float gj = __uint_as_float((j & 1) ? gw[k] & 0xffff0000u : gw[k] << 16);
+              const float uj = __uint_as_float((j & 1) ? uw[k] & 0xffff0000u : uw[k] << 16);
+              const float dh = v[j], sgm = __fdividef(1.0f, 1.0f + __expf(-gj));
+              g[j] = dh * uj * sgm * (1.0f + gj * (1.0f - sgm));
+              v[j] = dh * gj * sgm;
             }
             store_turned(scratch, lane, nv, p.out0 + cb, p.N, g);
             store_turned(scratch, lane, nv, p.out1 + cb, p.N, v);
@@ -1757,7 +1801,24 @@ static int swap_tok_box(const etr_config* c) {
   const int half = std::min(64, ceil_div(std::min(c->capacity, 256), 16) * 8);
   return half <= 8 ? 8 : half <= 16 ? 16 : half <= 32 ? 32 : 64;
 }
-static bool use_swap(const etr_config* c) { return c->gemm_impl == ETR_GEMM_AUTO; }
+// Where the exchanged form runs (gemm_impl AUTO; the other forms otherwise).  Measured against the form that
+// tc_form_of takes, same box, in us:
+//   capacity <= 192: a 256-row tile would be padding by a quarter or more.  8 rows per expert (E 13, d 1216,
+//     h 6144): SwiGLU 92 -> 86, down 56 -> 48, derivative 80 -> 52, dXp 95 -> 75.
+//   plain stores with at least three rounds of tiles: down 153 -> 139 and dXp 258 -> 244 at 1024 rows (E 32, d 2048,
+//     h 1408), 147 -> 127 and 248 -> 223 at 769 rows of 1280, 656 -> 582 and 1183 -> 1117 at 717 rows (E 64, d 4096,
+//     h 2048).  With fewer rounds the last one weighs more than the padding saved: 54 -> 59 and 91 -> 99 at 512
+//     rows (E 16, d 1024, h 2816; 2.2 rounds).  (Tiles of 128 tokens there: 64 and 109.)
+//   the fused epilogues are longer here (an exchange, a transposed read), so they need a longer contraction:
+//     SwiGLU from K = 2048 (365 -> 348 at E 128, d 2048, h 768; 97 -> 105 at d 1024), its derivative from
+//     K = 4096 (702 -> 668 at d 4096; 183 -> 219 at d 2048).
+static bool use_swap(const etr_config* c, int epi) {
+  if (c->gemm_impl != ETR_GEMM_AUTO) return false;
+  if (c->capacity <= 192) return true;
+  if (epi == TC_EPI_SWIGLU) return c->d >= 2048;
+  if (epi == TC_EPI_DSWIGLU) return c->d >= 4096;
+  return (long long)c->E * ceil_div(c->capacity, 256) * ceil_div(c->d, 256) >= 3 * (sm_count() / 2);
+}
 static SwapParams swap_params(const etr_config* c, const etr_route* rt, etr_stats* stats) {
   SwapParams p = {};
   p.M = c_stride_of(c); p.E = c->E; p.tok_box = swap_tok_box(c); p.counts = rt->counts; p.stats = stats;
@@ -1771,8 +1832,8 @@ static etr_status swap_launch(const char* name, const CUtensorMap& a0, const CUt
   auto k = tc_grouped_gemm_swap_kernel<EPI, A_MN>;
   static std::atomic<unsigned long long> attr_done{0};      // one bit per device
   if (!ensure_dyn_smem(k, smem, attr_done)) return ETR_ERR_CUDA;
-  const int tiles = p.E * ceil_div(p.M, 256) * ceil_div(p.N, EPI == TC_EPI_SWIGLU ? 128 : 256);
-  const int pairs = std::max(1, std::min(tiles, sm_count() / 2));
+  const long long tiles = (long long)p.E * ceil_div(p.M, 256) * ceil_div(p.N, EPI == TC_EPI_SWIGLU ? 128 : 256);
+  const int pairs = (int)std::max(1ll, std::min(tiles, (long long)(sm_count() / 2)));
   ETR_TIME_BEGIN(name);
   launch_kernel(k, 2 * pairs, TC_THREADS, smem, st, 2, a0, a1, b0, b1, p, make_idesc(A_MN, 0, 0, 256));
   ETR_LAUNCH_CHECK();
@@ -1793,21 +1854,6 @@ etr_status tc_ffn_forward(const etr_config* c, const etr_route* rt, const void* 
                           etr_stats* stats, void*, void* Y_top1, cudaStream_t st) {
   const int d = c->d, h = c->h, Cs = c_stride_of(c), E = c->E;
   CUtensorMap mXp, mW1g, mW1u, mW2, mH;
-  if (use_swap(c) && !Xtok) {
-    SwapParams p = swap_params(c, rt, stats);
-    ETR_TRY(make_map(&mXp, Xp, d, Cs, E, p.tok_box));
-    ETR_TRY(make_map(&mH, H, h, Cs, E, p.tok_box));
-    ETR_TRY(make_map(&mW1g, W1g, d, h, E));
-    ETR_TRY(make_map(&mW1u, W1u, d, h, E));
-    ETR_TRY(make_map(&mW2, W2, h, d, E));
-    p.N = h; p.K = d;
-    p.out0 = (__nv_bfloat16*)G; p.out1 = (__nv_bfloat16*)U; p.out2 = (__nv_bfloat16*)H;
-    ETR_TRY((swap_launch<TC_EPI_SWIGLU, false>("tc_gemm_swiglu", mW1g, mW1u, mXp, mXp, p, st)));
-    p.N = d; p.K = h;
-    p.out0 = (__nv_bfloat16*)O; p.out1 = p.out2 = nullptr;
-    if (Y_top1) { p.sc_tok = rt->slot_token; p.sc_gate = rt->gate; p.sc_out = (__nv_bfloat16*)Y_top1; p.sc_ld = d; }
-    return swap_launch<TC_EPI_STORE, false>("tc_gemm_down", mW2, mW2, mH, mH, p, st);
-  }
   if (Xtok) ETR_TRY(make_gather_map(&mXp, Xtok, d, c->T));
   else ETR_TRY(make_map(&mXp, Xp, d, Cs, E));
   ETR_TRY(make_map(&mW1g, W1g, d, h, E));
@@ -1815,7 +1861,14 @@ etr_status tc_ffn_forward(const etr_config* c, const etr_route* rt, const void* 
   ETR_TRY(make_map(&mW2, W2, h, d, E));
   ETR_TRY(make_map(&mH, H, h, Cs, E));
   const int mt = Cs / TC_BM;
-  {  // G, U, H = SwiGLU(Xp W1g^T, Xp W1u^T)
+  // G, U, H = SwiGLU(Xp W1g^T, Xp W1u^T)
+  if (!Xtok && use_swap(c, TC_EPI_SWIGLU)) {
+    SwapParams p = swap_params(c, rt, stats);
+    ETR_TRY(make_map(&mXp, Xp, d, Cs, E, p.tok_box));
+    p.N = h; p.K = d;
+    p.out0 = (__nv_bfloat16*)G; p.out1 = (__nv_bfloat16*)U; p.out2 = (__nv_bfloat16*)H;
+    ETR_TRY((swap_launch<TC_EPI_SWIGLU, false>("tc_gemm_swiglu", mW1g, mW1u, mXp, mXp, p, st)));
+  } else {
     TcParams p = tc_params(c);
     if (Xtok) { p.gather = 1; p.gather_ld = Cs; p.gather_oob = c->T; p.gather_idx = rt->slot_token; }
     p.dual_b = 1; p.M = Cs; p.N = h; p.K = d; p.dyn = TC_DYN_M; p.E = E; p.counts = rt->counts;
@@ -1824,11 +1877,18 @@ etr_status tc_ffn_forward(const etr_config* c, const etr_route* rt, const void* 
     ETR_TRY((tc_run<TC_EPI_SWIGLU>(tc_form_of(c, TC_EPI_SWIGLU, p), "tc_gemm_swiglu", mXp, mXp, mW1g, mW1u, p,
                                            E * mt * ceil_div(h, 128), st)));
   }
-  {  // O = H W2^T
+  // O = H W2^T.  Y_top1 (Top-1): the combine in this epilogue (the caller has zeroed the rows of unrouted tokens)
+  if (use_swap(c, TC_EPI_STORE)) {
+    SwapParams p = swap_params(c, rt, stats);
+    ETR_TRY(make_map(&mH, H, h, Cs, E, p.tok_box));
+    p.N = d; p.K = h; p.out0 = (__nv_bfloat16*)O;
+    if (Y_top1) { p.sc_tok = rt->slot_token; p.sc_gate = rt->gate; p.sc_out = (__nv_bfloat16*)Y_top1; p.sc_ld = d; }
+    ETR_TRY((swap_launch<TC_EPI_STORE, false>("tc_gemm_down", mW2, mW2, mH, mH, p, st)));
+  } else {
     TcParams p = tc_params(c);
     p.M = Cs; p.N = d; p.K = h; p.dyn = TC_DYN_M; p.E = E; p.counts = rt->counts;
     p.out0 = (__nv_bfloat16*)O; p.out_bs = (long long)Cs * d; p.ld_out = d; p.stats = stats;
-    if (Y_top1) {      // Top-1: the combine in this epilogue (the caller has zeroed the rows of unrouted tokens)
+    if (Y_top1) {
       p.sc_tok = rt->slot_token; p.sc_gate = rt->gate; p.sc_out = (__nv_bfloat16*)Y_top1; p.sc_ld = d;
     }
     ETR_TRY((tc_run<TC_EPI_STORE>(tc_form_of(c, TC_EPI_STORE, p), "tc_gemm_down", mH, mH, mW2, mW2, p, E * mt * ceil_div(d, 256), st)));
@@ -1852,37 +1912,39 @@ etr_status tc_ffn_backward(const etr_config* c, const etr_route* rt, const void*
   ETR_TRY(make_map(&mW1u, W1u, d, h, E));
   ETR_TRY(make_map(&mW2, W2, h, d, E));
   const int mt = Cs / TC_BM;
-  if (use_swap(c) && !Xtok) {      // (with the dispatch fused the forms below serve every contraction)
+  // dH = dO W2 (W2 read with its output index contiguous), then dG, dU
+  if (use_swap(c, TC_EPI_DSWIGLU)) {
     SwapParams p = swap_params(c, rt, stats);
-    CUtensorMap tdO, tdG, tdU;
-    ETR_TRY(make_map(&tdO, dO, d, Cs, E, p.tok_box));
-    ETR_TRY(make_map(&tdG, dG, h, Cs, E, p.tok_box));
-    ETR_TRY(make_map(&tdU, dU, h, Cs, E, p.tok_box));
+    CUtensorMap t;
+    ETR_TRY(make_map(&t, dO, d, Cs, E, p.tok_box));
     p.N = h; p.K = d;
     p.out0 = (__nv_bfloat16*)dG; p.out1 = (__nv_bfloat16*)dU;
     p.in0 = (const __nv_bfloat16*)G; p.in1 = (const __nv_bfloat16*)U;
-    ETR_TRY((swap_launch<TC_EPI_DSWIGLU, true>("tc_gemm_dswiglu", mW2, mW2, tdO, tdO, p, st)));
-    p.N = d; p.K = h; p.two_k = 1;
-    p.out0 = (__nv_bfloat16*)dXp; p.out1 = nullptr; p.in0 = p.in1 = nullptr;
-    ETR_TRY((swap_launch<TC_EPI_STORE, true>("tc_gemm_dxp", mW1g, mW1u, tdG, tdU, p, st)));
+    ETR_TRY((swap_launch<TC_EPI_DSWIGLU, true>("tc_gemm_dswiglu", mW2, mW2, t, t, p, st)));
   } else {
-    {  // dH = dO W2 (W2 read with its output index contiguous), then dG, dU
-      TcParams p = tc_params(c);
-      p.b_mn = 1; p.M = Cs; p.N = h; p.K = d; p.dyn = TC_DYN_M; p.E = E; p.counts = rt->counts;
-      p.out0 = (__nv_bfloat16*)dG; p.out1 = (__nv_bfloat16*)dU;
-      p.in0 = (const __nv_bfloat16*)G; p.in1 = (const __nv_bfloat16*)U;
-      p.out_bs = (long long)Cs * h; p.ld_out = h; p.stats = stats;
-      ETR_TRY((tc_run<TC_EPI_DSWIGLU>(tc_form_of(c, TC_EPI_DSWIGLU, p), "tc_gemm_dswiglu", mdO, mdO, mW2, mW2, p,
-                                              E * mt * ceil_div(h, 256), st)));
-    }
-    {  // dXp = dG W1g + dU W1u: one contraction over 2h
-      TcParams p = tc_params(c);
-      p.b_mn = 1; p.k1_blocks = ceil_div(h, TC_BK); p.M = Cs; p.N = d; p.K = 2 * h; p.dyn = TC_DYN_M;
-      p.E = E; p.counts = rt->counts;
-      p.out0 = (__nv_bfloat16*)dXp; p.out_bs = (long long)Cs * d; p.ld_out = d; p.stats = stats;
-      ETR_TRY((tc_run<TC_EPI_STORE>(tc_form_of(c, TC_EPI_STORE, p), "tc_gemm_dxp", mdG, mdU, mW1g, mW1u, p,
-                                            E * mt * ceil_div(d, 256), st)));
-    }
+    TcParams p = tc_params(c);
+    p.b_mn = 1; p.M = Cs; p.N = h; p.K = d; p.dyn = TC_DYN_M; p.E = E; p.counts = rt->counts;
+    p.out0 = (__nv_bfloat16*)dG; p.out1 = (__nv_bfloat16*)dU;
+    p.in0 = (const __nv_bfloat16*)G; p.in1 = (const __nv_bfloat16*)U;
+    p.out_bs = (long long)Cs * h; p.ld_out = h; p.stats = stats;
+    ETR_TRY((tc_run<TC_EPI_DSWIGLU>(tc_form_of(c, TC_EPI_DSWIGLU, p), "tc_gemm_dswiglu", mdO, mdO, mW2, mW2, p,
+                                            E * mt * ceil_div(h, 256), st)));
+  }
+  // dXp = dG W1g + dU W1u: one contraction over 2h
+  if (use_swap(c, TC_EPI_STORE)) {
+    SwapParams p = swap_params(c, rt, stats);
+    CUtensorMap tg, tu;
+    ETR_TRY(make_map(&tg, dG, h, Cs, E, p.tok_box));
+    ETR_TRY(make_map(&tu, dU, h, Cs, E, p.tok_box));
+    p.N = d; p.K = h; p.two_k = 1; p.out0 = (__nv_bfloat16*)dXp;
+    ETR_TRY((swap_launch<TC_EPI_STORE, true>("tc_gemm_dxp", mW1g, mW1u, tg, tu, p, st)));
+  } else {
+    TcParams p = tc_params(c);
+    p.b_mn = 1; p.k1_blocks = ceil_div(h, TC_BK); p.M = Cs; p.N = d; p.K = 2 * h; p.dyn = TC_DYN_M;
+    p.E = E; p.counts = rt->counts;
+    p.out0 = (__nv_bfloat16*)dXp; p.out_bs = (long long)Cs * d; p.ld_out = d; p.stats = stats;
+    ETR_TRY((tc_run<TC_EPI_STORE>(tc_form_of(c, TC_EPI_STORE, p), "tc_gemm_dxp", mdG, mdU, mW1g, mW1u, p,
+                                          E * mt * ceil_div(d, 256), st)));
   }
   {  // dW2 = dO^T H: contraction over the expert's rows, both operands MN-major
     TcParams p = tc_params(c);
