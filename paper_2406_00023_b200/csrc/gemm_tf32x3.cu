@@ -5,9 +5,10 @@
 //
 // The tensor core's fp32 accumulator drops the bits that do not fit instead of rounding them, an error that
 // always points towards zero and would add up over a long contraction.  So a chain of MMAs is never longer
-// than two K blocks (64 values: eight MMAs): hi*hi and the cross terms of such a chunk go to accumulators of
+// than one K block (32 values: four MMAs): hi*hi and the cross terms of such a chunk go to accumulators of
 // their own in tensor memory, and the epilogue warps add each chunk to running sums in registers with rounded
-// fp32 additions while the next one is multiplied.
+// fp32 additions while the next one is multiplied.  (Chunks of two K blocks: contractions off by 2.0e-7 instead of
+// 1.4e-7, an fp32 step of width 256 by 1.0e-6 where fp32 FMAs are off by 8.3e-7.)
 //
 // One persistent kernel serves the six contractions.  Roles in a CTA of 640 threads:
 //   warp 0       TMA: a K block arrives as plain fp32 in the place of its hi tiles
@@ -36,7 +37,7 @@ constexpr int F3_THREADS = 640;
 // registers per thread by role; 640 threads are launched with 96 each (61440), the split takes 60416
 constexpr int F3_REGS_LAUNCH = 96, F3_REGS_IO = 40, F3_REGS_CONV = 88, F3_REGS_EPI = 128;
 static_assert(128 * F3_REGS_IO + 256 * F3_REGS_CONV + 256 * F3_REGS_EPI <= F3_THREADS * F3_REGS_LAUNCH, "register split");
-constexpr int F3_CHUNK = 2;                      // K blocks that one chain of MMAs adds up
+constexpr int F3_CHUNK = 1;                      // K blocks that one chain of MMAs adds up
 constexpr int F3_SCRATCH = 32 * 80;              // per epilogue warp: 32 rows of 64 bytes, 16 bytes of pad each
 
 enum { F3_STORE = 0, F3_SWIGLU = 1, F3_DSWIGLU = 2 };
