@@ -681,13 +681,37 @@ affinity_bwd_dx_kernel(const T* __restrict__ X, const float* __restrict__ R,
   float beta = 0.f;
   const float sqD = sqrtf((float)D);
   if (DENSE && a != 0.f) {
-    // dense d delta (softmax gate): every expert contributes, in ascending expert order
-    for (int i = 0; i < E; ++i) {
-      const float b = rnorm[i], dg = ddelta[(size_t)t * E + i];
-      if (b == 0.f || dg == 0.f) continue;
-      const float w = dg * sqD / (a * b) / (float)D;
-      beta += dg * delta[(size_t)t * E + i];
-      for (int j = lane; j < m; j += 32) cz[j] = fmaf(w, R[(size_t)i * m + j], cz[j]);
+    // dense d delta (softmax gate): every expert contributes, in ascending expert order.  Lane i holds the
+    // scalars of expert e0 + i; a pooled column then takes eight experts' R values at a time.
+    for (int e0 = 0; e0 < E; e0 += 32) {
+      const int i = e0 + lane, ne = min(32, E - e0);
+      float w = 0.f, bd = 0.f;
+      bool use = false;
+      if (i < E) {
+        const float b = rnorm[i], dg = ddelta[(size_t)t * E + i];
+        use = b != 0.f && dg != 0.f;
+        if (use) { w = dg * sqD / (a * b) / (float)D; bd = dg * delta[(size_t)t * E + i]; }
+      }
+      const uint32_t live = __ballot_sync(0xffffffffu, use);
+      for (int u = 0; u < ne; ++u) {
+        const float x = __shfl_sync(0xffffffffu, bd, u);
+        if (live >> u & 1u) beta += x;
+      }
+      for (int j0 = 0; j0 < m; j0 += 32) {
+        const int j = j0 + lane;
+        float acc = j < m ? cz[j] : 0.f;
+        for (int u0 = 0; u0 < ne; u0 += 8) {
+          float r[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) r[u] = j < m && u0 + u < ne ? R[(size_t)(e0 + u0 + u) * m + j] : 0.f;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const float wu = __shfl_sync(0xffffffffu, w, (u0 + u) & 31);
+            if (live >> (u0 + u) & 1u) acc = fmaf(wu, r[u], acc);
+          }
+        }
+        if (j < m) cz[j] = acc;
+      }
     }
     beta /= (a * a);
   } else if (!DENSE && a != 0.f) {
@@ -924,8 +948,16 @@ affinity_bwd_dx_chunk_kernel(const T* __restrict__ X, const float* __restrict__ 
 // Partial dR over chunks of 128 slots of one expert (fixed order inside a chunk):
 //   part[i][ch][j] = sum_p w_p Z[t_p][j], w_p = dgate_p sqrt(D)/(a_t b_i);
 //   part[i][ch][m] = sum_p dgate_p delta_ti
+// The gathered rows of Z are short (m floats), so what counts is how many rounds of dependent loads a chunk takes:
+// V = 4 columns per thread (4 | m), the threads left over by a row take slots of their own (256 / (m / 4) groups of
+// consecutive slots, added in group order), eight slots requested together.  One column per thread and no groups
+// took 27 us at 512 rows per expert (E 16, m 128), this 11 us.
 constexpr int DR_CHUNK = 128;
 constexpr int DR_MAXJ = 16;     // m <= 256 * DR_MAXJ
+template <int V> struct DrVec;
+template <> struct DrVec<1> { typedef float type; };
+template <> struct DrVec<4> { typedef float4 type; };
+template <int V>
 __global__ void __launch_bounds__(256)
 affinity_bwd_dr_partial_kernel(const float* __restrict__ Z, const float* __restrict__ delta,
                                const float* __restrict__ xnorm, const float* __restrict__ rnorm,
@@ -934,8 +966,10 @@ affinity_bwd_dr_partial_kernel(const float* __restrict__ Z, const float* __restr
                                const float* __restrict__ dgate, float* __restrict__ part,
                                int E, int m, int C_stride, int nch, float sqD) {
   grid_sync();
+  typedef typename DrVec<V>::type vec;
   __shared__ int s_t[DR_CHUNK];
   __shared__ float s_w[DR_CHUNK], s_dd[DR_CHUNK];
+  __shared__ __align__(16) float s_red[256 * V];
   const int i = blockIdx.x, ch = blockIdx.y, tid = threadIdx.x;
   const int n = counts[i];
   const int p0 = ch * DR_CHUNK;
@@ -946,123 +980,162 @@ affinity_bwd_dr_partial_kernel(const float* __restrict__ Z, const float* __restr
     return;
   }
   const float b = rnorm[i];
-  if (tid < np) {
-    const size_t r = (size_t)i * C_stride + p0 + tid;
-    const int t = slot_token[r];
-    const float a = xnorm[t], dg = dgate[r];
-    const bool dead = (a == 0.f || b == 0.f);
-    s_t[tid] = t;
-    s_w[tid] = dead ? 0.f : dg * sqD / (a * b);
-    s_dd[tid] = dead ? 0.f : dg * delta[(size_t)t * E + i];
+  if (tid < DR_CHUNK) {
+    int t = 0;
+    float w = 0.f, dd = 0.f;
+    if (tid < np) {
+      const size_t r = (size_t)i * C_stride + p0 + tid;
+      t = slot_token[r];
+      const float a = xnorm[t], dg = dgate[r];
+      if (a != 0.f && b != 0.f) { w = dg * sqD / (a * b); dd = dg * delta[(size_t)t * E + i]; }
+    }
+    s_t[tid] = t; s_w[tid] = w; s_dd[tid] = dd;
   }
   __syncthreads();
-  float acc[DR_MAXJ];
+  const int cols = m / V;                                     // vectors of a row
+  const int groups = max(1, min(256 / cols, DR_CHUNK / 8)), per = (np + groups - 1) / groups;
+  const int g = groups > 1 ? tid / cols : 0;
+  const int beg = min(np, g * per), end = g < groups ? min(np, beg + per) : beg;
+  for (int j0 = 0; j0 < cols; j0 += 256) {
+    const int j = groups > 1 ? tid - g * cols : j0 + tid;
+    float acc[V];
 #pragma unroll
-  for (int u = 0; u < DR_MAXJ; ++u) acc[u] = 0.f;
-  float sdd = 0.f;
-  // slots in batches of 8: the gathered Z values of a batch are all requested before the first
-  // is used; the accumulation order (ascending slot) is unchanged
-  for (int p0 = 0; p0 < np; p0 += 8) {
+    for (int v = 0; v < V; ++v) acc[v] = 0.f;
+    if (j < cols) {
+      for (int p = beg; p < end; p += 8) {
+        vec z[8];
 #pragma unroll
-    for (int u = 0; u < DR_MAXJ; ++u) {
-      const int j = tid + u * 256;
-      if (j >= m) break;
-      float zv[8];
+        for (int u = 0; u < 8; ++u) z[u] = *(reinterpret_cast<const vec*>(Z + (size_t)s_t[min(p + u, np - 1)] * m) + j);
 #pragma unroll
-      for (int b = 0; b < 8; ++b) zv[b] = p0 + b < np ? Z[(size_t)s_t[p0 + b] * m + j] : 0.f;
+        for (int u = 0; u < 8; ++u) {
+          const float* zu = reinterpret_cast<const float*>(&z[u]);
+          if (p + u < end) {
+            const float w = s_w[p + u];
 #pragma unroll
-      for (int b = 0; b < 8; ++b)
-        if (p0 + b < np) acc[u] = fmaf(s_w[p0 + b], zv[b], acc[u]);
+            for (int v = 0; v < V; ++v) acc[v] = fmaf(w, zu[v], acc[v]);
+          }
+        }
+      }
     }
+    if (groups > 1) {
 #pragma unroll
-    for (int b = 0; b < 8; ++b)
-      if (p0 + b < np) sdd += s_dd[p0 + b];
-  }
+      for (int v = 0; v < V; ++v) s_red[tid * V + v] = acc[v];
+      __syncthreads();
+      if (g == 0) {
+        for (int k = 1; k < groups; ++k)
 #pragma unroll
-  for (int u = 0; u < DR_MAXJ; ++u) {
-    const int j = tid + u * 256;
-    if (j < m) out[j] = acc[u];
+          for (int v = 0; v < V; ++v) acc[v] += s_red[(k * cols + j) * V + v];
+      }
+    }
+    if (g == 0 && j < cols) {
+#pragma unroll
+      for (int v = 0; v < V; ++v) out[j * V + v] = acc[v];
+    }
   }
-  if (tid == 0) out[m] = sdd;
+  if (tid < 32) {
+    float sdd = 0.f;
+#pragma unroll
+    for (int u = 0; u < DR_CHUNK; u += 32) sdd += s_dd[u + tid];
+    sdd = warp_sum(sdd);
+    if (tid == 0) out[m] = sdd;
+  }
 }
 
-// The same partial sums for a dense d delta [T, E] (softmax gate): chunks of DR_DENSE_TOKENS
-// consecutive tokens, every expert.  A block takes one chunk and 32 experts at a time: thread j keeps
-// column j of the 32 partial rows, so each Z value is loaded once per 32 experts; tokens in ascending
-// order (sub-chunks of 128 staged in shared memory).
+// The same partial sums for a dense d delta [T, E] (softmax gate): a block takes one chunk of consecutive tokens, 32
+// experts (blockIdx.y) and 256 columns (blockIdx.z): thread j keeps column j of the 32 partial rows, so each Z value
+// is loaded once per 32 experts; tokens in ascending order.  `tok` tokens per chunk: 256, or fewer, so that a
+// short batch fills the GPU (3001 tokens, E 12, m 136: 12 chunks of 256 on 12 SMs took 99 us).
 constexpr int DR_DENSE_TOKENS = 256;
+constexpr int DR_DENSE_STEP = 32;
+static int dr_dense_tokens(const etr_config* c) {
+  const long long groups = (long long)ceil_div(c->E, 32) * ceil_div(c->d / c->D, 256);
+  const long long want = ((long long)c->T * groups + 2 * current_sm_count() - 1) / (2 * current_sm_count());
+  return (int)std::min<long long>(DR_DENSE_TOKENS, std::max<long long>(DR_DENSE_STEP, (want + DR_DENSE_STEP - 1) / DR_DENSE_STEP * DR_DENSE_STEP));
+}
 __global__ void __launch_bounds__(256)
 affinity_bwd_dr_dense_partial_kernel(const float* __restrict__ Z, const float* __restrict__ delta,
                                      const float* __restrict__ xnorm, const float* __restrict__ rnorm,
                                      const float* __restrict__ ddelta, float* __restrict__ part,
-                                     int Ttok, int E, int m, int nch, float sqD) {
+                                     int Ttok, int E, int m, int nch, int tok, float sqD) {
   grid_sync();
-  __shared__ __align__(16) float s_w[DR_CHUNK][32];
-  __shared__ float s_dd[DR_CHUNK][32];
-  const int ch = blockIdx.x, tid = threadIdx.x;
-  const int t_beg = ch * DR_DENSE_TOKENS, t_end = min(Ttok, t_beg + DR_DENSE_TOKENS);
-  for (int e0 = 0; e0 < E; e0 += 32) {
-    for (int j0 = 0; j0 < m; j0 += 256) {
-      const int j = j0 + tid;
-      float acc[32];
+  __shared__ __align__(16) float s_w[DR_DENSE_STEP][32];
+  __shared__ float s_dd[DR_DENSE_STEP][32];
+  const int ch = blockIdx.x, e0 = 32 * blockIdx.y, j0 = 256 * blockIdx.z, tid = threadIdx.x;
+  const int t_beg = ch * tok, t_end = min(Ttok, t_beg + tok);
+  const int j = j0 + tid;
+  float acc[32];
 #pragma unroll
-      for (int ii = 0; ii < 32; ++ii) acc[ii] = 0.f;
-      float sdd = 0.f;
-      for (int t0 = t_beg; t0 < t_end; t0 += DR_CHUNK) {
-        const int np = min(DR_CHUNK, t_end - t0);
-        __syncthreads();
-        for (int idx = tid; idx < DR_CHUNK * 32; idx += 256) {
-          const int p = idx >> 5, i = e0 + (idx & 31);
-          float w = 0.f, dd = 0.f;
-          if (p < np && i < E) {
-            const int t = t0 + p;
-            const float a = xnorm[t], b = rnorm[i], dg = ddelta[(size_t)t * E + i];
-            if (a != 0.f && b != 0.f) { w = dg * sqD / (a * b); dd = dg * delta[(size_t)t * E + i]; }
-          }
-          s_w[p][idx & 31] = w;
-          s_dd[p][idx & 31] = dd;
-        }
-        __syncthreads();
-        if (j < m) {
-          for (int p = 0; p < np; ++p) {
-            const float zv = Z[(size_t)(t0 + p) * m + j];
+  for (int ii = 0; ii < 32; ++ii) acc[ii] = 0.f;
+  float sdd = 0.f;
+  for (int t0 = t_beg; t0 < t_end; t0 += DR_DENSE_STEP) {
+    const int np = min(DR_DENSE_STEP, t_end - t0);
+    __syncthreads();
 #pragma unroll
-            for (int q4 = 0; q4 < 8; ++q4) {
-              const float4 w = *reinterpret_cast<const float4*>(&s_w[p][4 * q4]);
-              acc[4 * q4] = fmaf(w.x, zv, acc[4 * q4]);         acc[4 * q4 + 1] = fmaf(w.y, zv, acc[4 * q4 + 1]);
-              acc[4 * q4 + 2] = fmaf(w.z, zv, acc[4 * q4 + 2]); acc[4 * q4 + 3] = fmaf(w.w, zv, acc[4 * q4 + 3]);
-            }
-          }
-        }
-        if (j0 == 0 && tid < 32)
-          for (int p = 0; p < np; ++p) sdd += s_dd[p][tid];
+    for (int u = 0; u < DR_DENSE_STEP * 32 / 256; ++u) {
+      const int idx = tid + 256 * u, p = idx >> 5, i = e0 + (idx & 31);
+      float w = 0.f, dd = 0.f;
+      if (p < np && i < E) {
+        const int t = t0 + p;
+        const float a = xnorm[t], b = rnorm[i], dg = ddelta[(size_t)t * E + i];
+        if (a != 0.f && b != 0.f) { w = dg * sqD / (a * b); dd = dg * delta[(size_t)t * E + i]; }
       }
-      if (j < m) {
-#pragma unroll
-        for (int ii = 0; ii < 32; ++ii)
-          if (e0 + ii < E) part[((size_t)(e0 + ii) * nch + ch) * (m + 1) + j] = acc[ii];
-      }
-      if (j0 == 0 && tid < 32 && e0 + tid < E) part[((size_t)(e0 + tid) * nch + ch) * (m + 1) + m] = sdd;
+      s_w[p][idx & 31] = w;
+      s_dd[p][idx & 31] = dd;
     }
+    __syncthreads();
+    if (j < m) {
+      for (int p0 = 0; p0 < np; p0 += 8) {
+        float z[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) z[u] = Z[(size_t)(t0 + min(p0 + u, np - 1)) * m + j];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          if (p0 + u >= np) break;
+#pragma unroll
+          for (int q4 = 0; q4 < 8; ++q4) {
+            const float4 w = *reinterpret_cast<const float4*>(&s_w[p0 + u][4 * q4]);
+            acc[4 * q4] = fmaf(w.x, z[u], acc[4 * q4]);         acc[4 * q4 + 1] = fmaf(w.y, z[u], acc[4 * q4 + 1]);
+            acc[4 * q4 + 2] = fmaf(w.z, z[u], acc[4 * q4 + 2]); acc[4 * q4 + 3] = fmaf(w.w, z[u], acc[4 * q4 + 3]);
+          }
+        }
+      }
+    }
+    if (j0 == 0 && tid < 32)
+      for (int p = 0; p < np; ++p) sdd += s_dd[p][tid];
   }
+  if (j < m) {
+#pragma unroll
+    for (int ii = 0; ii < 32; ++ii)
+      if (e0 + ii < E) part[((size_t)(e0 + ii) * nch + ch) * (m + 1) + j] = acc[ii];
+  }
+  if (j0 == 0 && tid < 32 && e0 + tid < E) part[((size_t)(e0 + tid) * nch + ch) * (m + 1) + m] = sdd;
 }
 
-// dR[i][j] = sum_ch part[i][ch][j] - (sum_ch part[i][ch][m]) R[i][j] / b_i^2, chunks in order.
+// dR[i][j] = sum_ch part[i][ch][j] - (sum_ch part[i][ch][m]) R[i][j] / b_i^2.  A block takes 32 columns of an
+// expert; its eight warps take every eighth chunk, their sums are added in warp order (fixed whatever runs first).
 __global__ void __launch_bounds__(256)
 affinity_bwd_dr_final_kernel(const float* __restrict__ part, const float* __restrict__ R,
                              const float* __restrict__ rnorm, float* __restrict__ dR, int m, int nch) {
   grid_sync();
-  const int i = blockIdx.x;
-  const float b = rnorm[i];
+  __shared__ float s_acc[8][32], s_sdd[8];
+  const int i = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = 32 * blockIdx.y + lane;
   const float* base = part + (size_t)i * nch * (m + 1);
-  float sdd = 0.f;
+  float acc = 0.f, sdd = 0.f;
+  for (int ch = threadIdx.x; ch < nch; ch += 256) sdd += base[(size_t)ch * (m + 1) + m];
+  if (j < m) {
 #pragma unroll 8
-  for (int ch = 0; ch < nch; ++ch) sdd += base[(size_t)ch * (m + 1) + m];
-  for (int j = threadIdx.x; j < m; j += 256) {
-    float acc = 0.f;
-#pragma unroll 8
-    for (int ch = 0; ch < nch; ++ch) acc += base[(size_t)ch * (m + 1) + j];
-    dR[(size_t)i * m + j] = b == 0.f ? 0.f : acc - sdd * R[(size_t)i * m + j] / (b * b);
+    for (int ch = warp; ch < nch; ch += 8) acc += base[(size_t)ch * (m + 1) + j];
+  }
+  sdd = warp_sum(sdd);
+  s_acc[warp][lane] = acc;
+  if (lane == 0) s_sdd[warp] = sdd;
+  __syncthreads();
+  if (warp == 0 && j < m) {
+    float a = 0.f, d = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) { a += s_acc[w][lane]; d += s_sdd[w]; }
+    const float b = rnorm[i];
+    dR[(size_t)i * m + j] = b == 0.f ? 0.f : a - d * R[(size_t)i * m + j] / (b * b);
   }
 }
 
@@ -1233,7 +1306,7 @@ etr_status affinity_forward(const etr_config* c, const void* X, const float* R, 
 
 size_t affinity_bwd_workspace_bytes(const etr_config* c) {
   const int m = c->d / c->D;
-  const int nch = c->gate_mode == ETR_GATE_SOFTMAX ? std::max(c_stride_of(c) / DR_CHUNK, ceil_div(c->T, DR_DENSE_TOKENS))
+  const int nch = c->gate_mode == ETR_GATE_SOFTMAX ? std::max(c_stride_of(c) / DR_CHUNK, ceil_div(c->T, dr_dense_tokens(c)))
                                                    : c_stride_of(c) / DR_CHUNK;
   return (size_t)c->E * nch * (m + 1) * sizeof(float);
 }
@@ -1258,6 +1331,8 @@ static etr_status launch_bwd_dx(const etr_config* c, const void* X, const float*
   constexpr size_t cz_max = 37 * 1024;
   int tpb = DXC_MAX_TOKENS;
   while (tpb > 2 && (size_t)tpb * m * sizeof(float) > cz_max) tpb /= 2;
+  // a short batch: fewer tokens, so that every SM has two blocks (512 tokens, d 256: 16.8 -> 10.9 us)
+  while (tpb > 2 && ceil_div(c->T, tpb) < 2 * current_sm_count()) tpb /= 2;
   int d_shift = 0;
   while ((1 << d_shift) < c->D) ++d_shift;
   const bool group8 = c->D >= 8 && (1 << d_shift) == c->D;
@@ -1296,7 +1371,7 @@ etr_status affinity_backward(const etr_config* c, const void* X, const float* R,
                              const void* dXp_fused, void* dX, float* dR, void* ws, etr_stats* stats,
                              cudaStream_t st) {
   const int m = c->d / c->D, Cs = c_stride_of(c);
-  const int nch = ddelta ? ceil_div(c->T, DR_DENSE_TOKENS) : Cs / DR_CHUNK;
+  const int nch = ddelta ? ceil_div(c->T, dr_dense_tokens(c)) : Cs / DR_CHUNK;
   if (m > 256 * DR_MAXJ) return ETR_ERR_UNSUPPORTED;
   const size_t smem = (size_t)8 * m * sizeof(float);
   if (smem > 200 * 1024) return ETR_ERR_UNSUPPORTED;
@@ -1306,16 +1381,20 @@ etr_status affinity_backward(const etr_config* c, const void* X, const float* R,
   float* part = (float*)ws;
   if (ddelta) {
     ETR_TIME_BEGIN("affinity_bwd_dr_dense_partial_kernel");
-    launch_kernel(affinity_bwd_dr_dense_partial_kernel, nch, 256, 0, st, 1, Z, delta, xnorm, rnorm, ddelta, part, c->T, c->E,
-                                                              m, nch, sqrtf((float)c->D));
+    launch_kernel(affinity_bwd_dr_dense_partial_kernel, dim3(nch, ceil_div(c->E, 32), ceil_div(m, 256)), 256, 0, st, 1, Z,
+                  delta, xnorm, rnorm, ddelta, part, c->T, c->E, m, nch, dr_dense_tokens(c), sqrtf((float)c->D));
   } else {
     ETR_TIME_BEGIN("affinity_bwd_dr_partial_kernel");
-    launch_kernel(affinity_bwd_dr_partial_kernel, dim3(c->E, nch), 256, 0, st, 1, Z, delta, xnorm, rnorm, rt->counts, rt->slot_token, dgate, part, c->E, m, Cs, nch,
-        sqrtf((float)c->D));
+    auto go = [&](auto k) {
+      launch_kernel(k, dim3(c->E, nch), 256, 0, st, 1, Z, delta, xnorm, rnorm, rt->counts, rt->slot_token, dgate, part,
+                    c->E, m, Cs, nch, sqrtf((float)c->D));
+    };
+    if (m % 4 == 0) go(affinity_bwd_dr_partial_kernel<4>);
+    else go(affinity_bwd_dr_partial_kernel<1>);
   }
   ETR_LAUNCH_CHECK();
   ETR_TIME_BEGIN("affinity_bwd_dr_final_kernel");
-  launch_kernel(affinity_bwd_dr_final_kernel, c->E, 256, 0, st, 1, part, R, rnorm, dR, m, nch);
+  launch_kernel(affinity_bwd_dr_final_kernel, dim3(c->E, ceil_div(m, 32)), 256, 0, st, 1, part, R, rnorm, dR, m, nch);
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }

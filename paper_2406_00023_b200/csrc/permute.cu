@@ -30,26 +30,26 @@ dispatch_kernel(const T* __restrict__ X, const int32_t* __restrict__ counts,
 }
 
 // Y[t,:] = sum_{r in rows(t)} gate[r] O[r,:]   (gate == nullptr: plain sum, used for dX).
-// A block takes COMBINE_TOKENS consecutive tokens.  It first copies their row lists and gates to
+// A block takes tpb <= COMBINE_TOKENS consecutive tokens.  It first copies their row lists and gates to
 // shared memory (two rounds of dependent loads for the whole chunk instead of two per token), then
 // every thread owns NV groups of 8 consecutive elements of a token, 1/NV of a row apart, and walks
 // the token's rows two at a time: 2 NV independent 16-byte loads in flight per thread, none of them
 // waiting for an index.  Rows are added in list order (the result does not depend on the chunking).
-constexpr int COMBINE_TOKENS = 8;
+constexpr int COMBINE_TOKENS = 8;      // at most; fewer where a short batch would leave SMs without a block
 constexpr int COMBINE_ROWS = 512;     // row entries held in shared memory; later ones are read in place
 
 template <class T, int NV>
 __global__ void __launch_bounds__(256)
 combine_kernel(const T* __restrict__ O, const float* __restrict__ gate,
                const int32_t* __restrict__ tok_ptr, const int32_t* __restrict__ tok_row,
-               T* __restrict__ Y, int Ttok, int d) {
+               T* __restrict__ Y, int Ttok, int d, int tpb) {
   grid_sync();
   __shared__ int s_ptr[COMBINE_TOKENS + 1];
   __shared__ int s_row[COMBINE_ROWS];
   __shared__ float s_gate[COMBINE_ROWS];
   const int tid = threadIdx.x;
-  const int t0 = blockIdx.x * COMBINE_TOKENS;
-  const int nt = min(COMBINE_TOKENS, Ttok - t0);
+  const int t0 = blockIdx.x * tpb;
+  const int nt = min(tpb, Ttok - t0);
   if (tid <= nt) s_ptr[tid] = tok_ptr[t0 + tid];
   __syncthreads();
   const int base = s_ptr[0];
@@ -177,11 +177,13 @@ static etr_status permute_launch(int which, const etr_config* c, const etr_route
     case 3: {
       const float* g = which == 1 ? rt->gate : nullptr;
       ETR_TIME_BEGIN("combine_kernel");
-      const unsigned grid = (unsigned)ceil_div(c->T, COMBINE_TOKENS);
+      int tpb = COMBINE_TOKENS;
+      while (tpb > 1 && ceil_div(c->T, tpb) < 2 * current_sm_count()) tpb /= 2;
+      const unsigned grid = (unsigned)ceil_div(c->T, tpb);
       if (c->d % 16 == 0)
-        launch_kernel(combine_kernel<T, 2>, grid, 256, 0, st, 1, (const T*)a, g, rt->tok_ptr, rt->tok_row, (T*)out, c->T, c->d);
+        launch_kernel(combine_kernel<T, 2>, grid, 256, 0, st, 1, (const T*)a, g, rt->tok_ptr, rt->tok_row, (T*)out, c->T, c->d, tpb);
       else
-        launch_kernel(combine_kernel<T, 1>, grid, 256, 0, st, 1, (const T*)a, g, rt->tok_ptr, rt->tok_row, (T*)out, c->T, c->d);
+        launch_kernel(combine_kernel<T, 1>, grid, 256, 0, st, 1, (const T*)a, g, rt->tok_ptr, rt->tok_row, (T*)out, c->T, c->d, tpb);
       break;
     }
     case 2:
