@@ -175,16 +175,23 @@ __device__ __forceinline__ void scatter32_warp(uint8_t* scratch, int lane, int t
   }
   __syncwarp();
 }
-// 32 zeros at element offset `off` of the output (this lane's row of a block with nothing to contract).
-__device__ __forceinline__ void store_zero32(const TcParams& p, long long off) {
-  if (p.out_f32) {
-    float4* q = reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out0) + off);
+// Zeros to a 32-row x 32-column block of the output (nothing to contract): wbase is the element offset of its first
+// row and column.  Like any store, 8 rows of 64 bytes per instruction.
+__device__ __forceinline__ void store_zero_block(const TcParams& p, long long wbase, int lane, int nvalid) {
+  const uint4 z = make_uint4(0, 0, 0, 0);
+  const int sub = lane & 3;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  } else {
-    uint4* q = reinterpret_cast<uint4*>(p.out0 + off);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) q[i] = make_uint4(0, 0, 0, 0);
+  for (int i = 0; i < 4; ++i) {
+    const int row = (lane >> 2) + 8 * i;
+    if (row >= nvalid) continue;
+    const long long o = wbase + (long long)row * p.ld_out;
+    if (p.out_f32) {
+      float* q = reinterpret_cast<float*>(p.out0) + o + sub * 4;
+      *reinterpret_cast<uint4*>(q) = z;
+      *reinterpret_cast<uint4*>(q + 16) = z;
+    } else {
+      *reinterpret_cast<uint4*>(p.out0 + o + sub * 8) = z;
+    }
   }
 }
 
@@ -456,8 +463,9 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_c
       const int c_beg = half * NCH;
       const long long obase = (long long)tc.e * p.out_bs + (long long)grow * p.ld_out + tc.n0;
       if (tc.kblocks == 0) {        // nothing to contract: the block of the output is zero
-        if (row_ok)
-          for (int c = c_beg; c < c_beg + NCH && tc.n0 + 32 * c < p.N; ++c) store_zero32(p, obase + 32 * c);
+        const int nz = min(32, max(0, tc.m_lim - (grow - lane)));
+        for (int c = c_beg; c < c_beg + NCH && tc.n0 + 32 * c < p.N; ++c)
+          store_zero_block(p, obase - (long long)lane * p.ld_out + 32 * c, lane, nz);
         continue;
       }
       // SwiGLU derivative: the saved G and U of the first chunk are fetched before the
@@ -812,8 +820,9 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
       const int c_beg = half * NCH;
       const long long obase = (long long)tc.e * p.out_bs + (long long)grow * p.ld_out + tc.n0;
       if (tc.kblocks == 0) {
-        if (row_ok)
-          for (int c = c_beg; c < c_beg + NCH && tc.n0 + 32 * c < p.N; ++c) store_zero32(p, obase + 32 * c);
+        const int nz = min(32, max(0, tc.m_lim - (grow - lane)));
+        for (int c = c_beg; c < c_beg + NCH && tc.n0 + 32 * c < p.N; ++c)
+          store_zero_block(p, obase - (long long)lane * p.ld_out + 32 * c, lane, nz);
         continue;
       }
       uint4 pg[4], pu[4];
@@ -832,10 +841,36 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
         sc_t = p.sc_tok[(long long)tc.e * p.M + grow];
         sc_g = p.sc_gate[(long long)tc.e * p.M + grow];
       }
-      epilogue_chunks<EPI, BN>(p, tc.n0, taddr, obase, row_ok, c_beg, NCH, pg, pu, scratch, lane, nvalid, sc_t, sc_g);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(leader_tempty + 8 * acc_stage);
+      if (EPI == TC_EPI_STORE && CFG == 3) {
+        // Weight gradients: a tile of a few rows' contraction is all epilogue, so the accumulators are read in one go
+        // (four loads in flight instead of a wait per chunk) and released before the stores.
+        constexpr int NC = EPI == TC_EPI_STORE ? NCH : 1;
+        uint32_t r[NC][32];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) tc_ld32(taddr + 32 * (c_beg + c), r[c]);
+        tc_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(leader_tempty + 8 * acc_stage);
+        const long long wb = obase - (long long)lane * p.ld_out + 32 * c_beg;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          if (tc.n0 + 32 * (c_beg + c) >= p.N) break;
+          if (p.out_f32) {
+            store32_warp_f32(scratch, lane, nvalid, reinterpret_cast<float*>(p.out0) + wb + 32 * c, p.ld_out, r[c]);
+          } else {
+            uint32_t pk[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(__uint_as_float(r[c][2 * i]), __uint_as_float(r[c][2 * i + 1]));
+            store32_warp_packed(scratch, lane, nvalid, p.out0 + wb + 32 * c, p.ld_out, pk);
+          }
+        }
+      } else {
+        epilogue_chunks<EPI, BN>(p, tc.n0, taddr, obase, row_ok, c_beg, NCH, pg, pu, scratch, lane, nvalid, sc_t, sc_g);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(leader_tempty + 8 * acc_stage);
+      }
       if (++acc_stage == 2) { acc_stage = 0; acc_phase ^= 1u; }
     }
   }
@@ -1071,10 +1106,10 @@ tc_grouped_gemm_pair_wide_kernel(const __grid_constant__ CUtensorMap mapA0, cons
       const bool two = tc.n0 + N_TILE_COLS < p.N;
       const long long obase = (long long)tc.e * p.out_bs + (long long)grow * p.ld_out + tc.n0;
       if (tc.kblocks == 0) {
-        if (row_ok)
-          for (int hf = 0; hf < (two ? 2 : 1); ++hf)
-            for (int c = c_beg; c < c_beg + NCH && tc.n0 + hf * N_TILE_COLS + 32 * c < p.N; ++c)
-              store_zero32(p, obase + hf * N_TILE_COLS + 32 * c);
+        const int nz = min(32, max(0, tc.m_lim - (grow - lane)));
+        for (int hf = 0; hf < (two ? 2 : 1); ++hf)
+          for (int c = c_beg; c < c_beg + NCH && tc.n0 + hf * N_TILE_COLS + 32 * c < p.N; ++c)
+            store_zero_block(p, obase - (long long)lane * p.ld_out + hf * N_TILE_COLS + 32 * c, lane, nz);
         continue;
       }
       uint4 pg[4], pu[4];
