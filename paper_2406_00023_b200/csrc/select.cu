@@ -18,7 +18,6 @@
 namespace etr {
 
 constexpr int SEL_TB = 32;         // tokens per CTA on the token side
-constexpr int SEL_MAX_EPL = 8;     // experts per lane: E <= 256
 
 struct SelectParams {
   int T, E, k, d, C_stride, capacity, c_floor, adaptive, mode;
@@ -50,12 +49,16 @@ __device__ inline int capacity_from_delta(const SelectParams& p, float delta_max
   return (int)c;
 }
 
+// EPL: experts per lane (E <= 32 EPL).  A rank's winner is found by two warp reductions of 32 bits, the largest key
+// and the lowest index that has it (64-bit shuffles over eight slots per lane took 24 us at T 8192, E 128, k 8; this
+// 17 us).
+template <int EPL>
 __global__ void __launch_bounds__(256)
 select_token_side_kernel(const float* __restrict__ delta, int32_t* __restrict__ topk_idx,
                          uint32_t* __restrict__ keyT, etr_stats* stats, int32_t* __restrict__ skipped,
                          SelectParams p) {
   grid_sync();
-  __shared__ uint32_t tile[256 * (SEL_TB + 1)];      // [E][33]
+  __shared__ uint32_t tile[32 * EPL * (SEL_TB + 1)];      // [E][33]
   __shared__ int s_skipped;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int t0 = blockIdx.x * SEL_TB;
@@ -73,45 +76,48 @@ select_token_side_kernel(const float* __restrict__ delta, int32_t* __restrict__ 
     stats->dropped = 0;
     stats->rows_total = 0;
   }
+  auto load = [&](int t, uint32_t (&k)[EPL]) {
+#pragma unroll
+    for (int u = 0; u < EPL; ++u) {
+      const int i = lane + 32 * u;
+      k[u] = (t < p.T && i < p.E) ? ordered_key(delta[(size_t)t * p.E + i]) : 0u;
+    }
+  };
+  uint32_t key[EPL], next[EPL];
+  load(t0 + warp, next);
   for (int tt = warp; tt < SEL_TB; tt += 8) {
     const int t = t0 + tt;
-    uint32_t key[SEL_MAX_EPL];
-    bool cand[SEL_MAX_EPL], taken[SEL_MAX_EPL];
+    bool cand[EPL], taken[EPL];
 #pragma unroll
-    for (int u = 0; u < SEL_MAX_EPL; ++u) {
+    for (int u = 0; u < EPL; ++u) key[u] = next[u];
+    if (tt + 8 < SEL_TB) load(t + 8, next);          // under this token's ranks
+#pragma unroll
+    for (int u = 0; u < EPL; ++u) {
       const int i = lane + 32 * u;
-      key[u] = (t < p.T && i < p.E) ? ordered_key(delta[(size_t)t * p.E + i]) : 0u;
       cand[u] = (p.mode == ETR_MODE_ECR);
-      taken[u] = false;
+      taken[u] = i >= p.E;
     }
     if (p.mode == ETR_MODE_TCR && t < p.T) {
       long long sum_before = 0;                      // of the affinities of the ranks before j (threshold walk)
       bool open = true;
       for (int j = 0; j < p.k; ++j) {
         // arg-max over (key, lower index wins) among experts not yet taken
-        unsigned long long best = 0ull;
+        uint32_t best = 0u;
+        int first = 0x7fffffff;
 #pragma unroll
-        for (int u = 0; u < SEL_MAX_EPL; ++u) {
-          const int i = lane + 32 * u;
-          if (i < p.E && !taken[u]) {
-            const unsigned long long v = ((unsigned long long)key[u] << 32) | (uint32_t)(0x7fffffff - i);
-            best = v > best ? v : best;
-          }
+        for (int u = 0; u < EPL; ++u) {
+          if (!taken[u] && (first == 0x7fffffff || key[u] > best)) { best = key[u]; first = lane + 32 * u; }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
-          best = other > best ? other : best;
-        }
-        const int win = 0x7fffffff - (int)(uint32_t)(best & 0xffffffffull);
+        const uint32_t top = __reduce_max_sync(0xffffffffu, best);
+        const int win = __reduce_min_sync(0xffffffffu, best == top ? first : 0x7fffffff);
         if (p.cut_token) {                           // the walk stops at the first rank it does not keep
           open = open && sum_before < p.tq_token;
-          sum_before += quantise_affinity(key_to_float((uint32_t)(best >> 32)));
+          sum_before += quantise_affinity(key_to_float(top));
           n_skipped += !open;
         }
         if (lane == (win & 31)) {
 #pragma unroll
-          for (int u = 0; u < SEL_MAX_EPL; ++u) if (u == (win >> 5)) { taken[u] = true; cand[u] = open; }
+          for (int u = 0; u < EPL; ++u) if (u == (win >> 5)) { taken[u] = true; cand[u] = open; }
         }
         if (lane == 0) topk_idx[(size_t)t * p.k + j] = open ? win : -1;
       }
@@ -119,7 +125,7 @@ select_token_side_kernel(const float* __restrict__ delta, int32_t* __restrict__ 
       for (int j = lane; j < p.k; j += 32) topk_idx[(size_t)t * p.k + j] = -1;
     }
 #pragma unroll
-    for (int u = 0; u < SEL_MAX_EPL; ++u) {
+    for (int u = 0; u < EPL; ++u) {
       const int i = lane + 32 * u;
       if (i < p.E) tile[i * (SEL_TB + 1) + tt] = cand[u] ? key[u] : 0u;
     }
@@ -316,6 +322,7 @@ select_expert_side_kernel(uint32_t* __restrict__ keyT, const etr_stats* __restri
     __syncthreads();
     if (pass == 0) n_keep = min((uint32_t)C, s_ncand);
     if (n_keep == 0) break;                       // uniform across the CTA
+    if (n_keep == s_ncand) break;                 // every candidate is kept: nothing to search, tau = 0
     if (warp == 0) {
       uint32_t b, rem;
       pick_bin(hist, pass == 0 ? n_keep : s_remaining, lane, b, rem);
@@ -326,7 +333,7 @@ select_expert_side_kernel(uint32_t* __restrict__ keyT, const etr_stats* __restri
     }
     __syncthreads();
   }
-  if (n_keep > 0) { tau = s_prefix; quota = s_remaining; }
+  if (n_keep > 0 && n_keep < s_ncand) { tau = s_prefix; quota = s_remaining; }
 
   // slot assignment in ascending token order
   if (tid == 0) { base_sel = 0; base_eq = 0; }
@@ -708,7 +715,13 @@ etr_status select_forward(const etr_config* c, const float* delta, etr_stats* st
   int32_t* limit = (c->threshold_mode & ETR_THRESHOLD_EXPERT) ? reinterpret_cast<int32_t*>(ws_tail) : nullptr;
   int32_t* skipped = p.cut_token ? reinterpret_cast<int32_t*>(ws_tail + select_limit_bytes(c)) : nullptr;
   ETR_TIME_BEGIN("select_token_side_kernel");
-  launch_kernel(select_token_side_kernel, ceil_div(c->T, SEL_TB), 256, 0, st, 1, delta, rt->topk_idx, keyT, stats, skipped, p);
+  auto token_side = [&](auto k) {
+    launch_kernel(k, ceil_div(c->T, SEL_TB), 256, 0, st, 1, delta, rt->topk_idx, keyT, stats, skipped, p);
+  };
+  if (c->E <= 32) token_side(select_token_side_kernel<1>);
+  else if (c->E <= 64) token_side(select_token_side_kernel<2>);
+  else if (c->E <= 128) token_side(select_token_side_kernel<4>);
+  else token_side(select_token_side_kernel<8>);      // E <= 256
   ETR_LAUNCH_CHECK();
   if (limit) {
     ETR_TIME_BEGIN("select_threshold_limit_kernel");
