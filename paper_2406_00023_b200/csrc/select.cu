@@ -11,6 +11,7 @@
 //      scan in token order assigns slots (ascending token id).  The row of keyT is
 //      overwritten with the slot position (or -1).
 //   3. token-major CSR from the position matrix: count, exclusive scan, fill.
+// Short batches take all three steps in one kernel (select_small_kernel), with the same result.
 #include <mutex>
 
 #include "common.cuh"
@@ -687,6 +688,177 @@ csr_fill_kernel(const int32_t* __restrict__ posT, const int32_t* __restrict__ bl
   tok_ptr[t + 1] = q;
 }
 
+// ---- short batches: the whole selection in one kernel ---------------------------------------------------------
+// With a few hundred tokens the four kernels above are launch latency and block start-up; one CTA does the same
+// with the keys in shared memory, in the same order of decisions: a thread per token for the top-k, a warp per expert
+// for the C-th largest key (its row in NK registers per lane, a binary search over the bits that ends as soon as a
+// prefix separates exactly C keys) and the slots in token order, a thread per token for the CSR.
+// NK: keys per lane, T <= 32 NK <= 512.
+template <int NK>
+__global__ void __launch_bounds__(1024)
+select_small_kernel(const float* __restrict__ delta, int32_t* __restrict__ topk_idx, etr_stats* stats,
+                    int32_t* __restrict__ counts, int32_t* __restrict__ slot_token, float* __restrict__ gate,
+                    int32_t* __restrict__ tok_ptr, int32_t* __restrict__ tok_row, SelectParams p, int n_cand) {
+  grid_sync();
+  extern __shared__ uint32_t sk[];                   // [E][T, odd stride]: keys, then slot positions (-1: not kept)
+  __shared__ int s_C, wsum[32], s_un;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int T = p.T, E = p.E, Ts = T | 1;            // odd: lanes along the experts hit different banks
+  if (tid == 0) {
+    const uint32_t mk = stats->delta_max_key;
+    const float dm = mk ? key_to_float(mk) : 0.f;
+    s_C = capacity_from_delta(p, dm);
+    s_un = 0;
+    stats->delta_max = dm;
+    stats->mode = p.mode;
+    stats->C = s_C;
+  }
+  const bool tcr = p.mode == ETR_MODE_TCR;
+  for (int idx = tid; idx < T * E; idx += 1024) {
+    const int t = idx / E, i = idx - t * E;
+    sk[i * Ts + t] = ordered_key(delta[idx]);
+  }
+  __syncthreads();
+  // token side: the k best experts of a token keep their keys, the others are cleared
+  if (tcr) {
+    // a thread per token: rank j is the largest (key, lower index first) behind rank j - 1 (a warp per token, by
+    // reductions as above, took 31 us instead of 8 at 512 tokens, E 8, k 2)
+    for (int t = tid; t < T; t += 1024) {
+      uint32_t last = 0xffffffffu;
+      int last_i = -1;
+      for (int j = 0; j < p.k; ++j) {
+        uint32_t best = 0u;
+        int win = E;
+#pragma unroll 4
+        for (int i = 0; i < E; ++i) {
+          const uint32_t x = sk[i * Ts + t];
+          const bool behind = j == 0 || x < last || (x == last && i > last_i);
+          if (behind && (win == E || x > best)) { best = x; win = i; }
+        }
+        topk_idx[(size_t)t * p.k + j] = win;
+        last = best;
+        last_i = win;
+      }
+      for (int i = 0; i < E; ++i) {
+        const uint32_t x = sk[i * Ts + t];
+        if (x < last || (x == last && i > last_i)) sk[i * Ts + t] = 0u;
+      }
+    }
+  } else {
+    for (int idx = tid; idx < T * p.k; idx += 1024) topk_idx[idx] = -1;
+  }
+  __syncthreads();
+  // expert side
+  const int C = s_C;
+  for (int i = warp; i < E; i += 32) {
+    uint32_t* row = sk + i * Ts;
+    uint32_t key[NK];
+    int nc = 0;
+#pragma unroll
+    for (int u = 0; u < NK; ++u) {
+      const int t = 32 * u + lane;
+      key[u] = t < T ? row[t] : 0u;
+      nc += key[u] != 0u;
+    }
+    nc = __reduce_add_sync(0xffffffffu, nc);
+    const int n_keep = min(C, nc);
+    uint32_t tau = 0u;                               // kept: keys above tau, and the first `quota` keys equal to it
+    int quota = 0;
+    if (n_keep < nc && n_keep > 0) {
+      uint32_t pre = 0u;
+      bool exact = false;
+      for (int bit = 31; bit >= 0 && !exact; --bit) {
+        const uint32_t trial = pre | (1u << bit);
+        int cnt = 0;
+#pragma unroll
+        for (int u = 0; u < NK; ++u) cnt += key[u] >= trial;
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if (cnt >= n_keep) { pre = trial; exact = cnt == n_keep; }
+      }
+      if (exact) {
+        tau = pre - 1;                               // pre > 0: a bit was set
+      } else {
+        tau = pre;
+        int above = 0;
+#pragma unroll
+        for (int u = 0; u < NK; ++u) above += key[u] > tau;
+        quota = n_keep - __reduce_add_sync(0xffffffffu, above);
+      }
+    }
+    int base = 0, eq_seen = 0;
+    int32_t* my_slot = slot_token + (size_t)i * p.C_stride;
+    float* my_gate = gate + (size_t)i * p.C_stride;
+#pragma unroll
+    for (int u = 0; u < NK; ++u) {
+      const int t = 32 * u + lane;
+      const bool live = n_keep > 0 && key[u] != 0u, eq = live && quota > 0 && key[u] == tau;
+      const uint32_t below = (1u << lane) - 1u, eqm = __ballot_sync(0xffffffffu, eq);
+      const bool kept = (live && key[u] > tau) || (eq && eq_seen + __popc(eqm & below) < quota);
+      const uint32_t km = __ballot_sync(0xffffffffu, kept);
+      const int pos = kept ? base + __popc(km & below) : -1;
+      if (kept) { my_slot[pos] = t; my_gate[pos] = key_to_float(key[u]); }
+      if (t < T) row[t] = (uint32_t)pos;
+      base += __popc(km);
+      eq_seen += __popc(eqm);
+    }
+    for (int q = n_keep + lane; q < p.C_stride; q += 32) { my_slot[q] = -1; my_gate[q] = 0.f; }
+    if (lane == 0) counts[i] = n_keep;
+  }
+  __syncthreads();
+  // token-major CSR
+  int n = 0;
+  if (tid < T)
+    for (int i = 0; i < E; ++i) n += (int)sk[i * Ts + tid] >= 0;
+  const uint32_t un = __ballot_sync(0xffffffffu, tid < T && n == 0);
+  if (lane == 0 && un) atomicAdd(&s_un, __popc(un));
+  int inc = n;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) wsum[warp] = inc;
+  __syncthreads();
+  int q = inc - n;
+  int total = 0;
+#pragma unroll
+  for (int w = 0; w < 32; ++w) { const int x = wsum[w]; q += w < warp ? x : 0; total += x; }
+  if (tid < T) {
+    for (int i = 0; i < E; ++i) {
+      const int pos = (int)sk[i * Ts + tid];
+      if (pos >= 0) tok_row[q++] = i * p.C_stride + pos;
+    }
+    tok_ptr[tid + 1] = q;
+  }
+  if (tid == 0) {
+    tok_ptr[0] = 0;
+    stats->unrouted = s_un;
+    stats->rows_total = total;
+    stats->dropped = n_cand - total;
+  }
+}
+// Up to 512 tokens and 16 Ki keys; beyond, the kernels above have more SMs to win than launches to lose (expert choice,
+// this against those, us: 6 / 15 at T 64, E 16; 10 / 13 at T 512, E 8; 17 / 18 at T 512, E 32; 20 / 16 at T 1024, E 16).
+// Token choice also reads E k keys per token in one thread: 8 / 15 at T 64, E 16, k 2; 11 / 16 at T 128, E 32, k 2;
+// 22 / 18 at T 512, E 32, k 4; 30 / 25 at T 64, E 128, k 2.
+constexpr int SEL_SMALL_TOKENS = 512, SEL_SMALL_KEYS = 16384, SEL_SMALL_RANKS = 96;
+constexpr size_t SEL_SMALL_BYTES = (SEL_SMALL_KEYS + 256) * sizeof(uint32_t);
+static etr_status select_small(const etr_config* c, const float* delta, etr_stats* stats, const etr_route* rt,
+                               const SelectParams& p, int n_cand, cudaStream_t st) {
+  auto go = [&](auto k, std::atomic<unsigned long long>& done) -> etr_status {
+    if (!ensure_dyn_smem(k, SEL_SMALL_BYTES, done)) return ETR_ERR_CUDA;
+    ETR_TIME_BEGIN("select_small_kernel");
+    launch_kernel(k, 1, 1024, (size_t)(c->T | 1) * c->E * sizeof(uint32_t), st, 1, delta, rt->topk_idx, stats, rt->counts,
+                  rt->slot_token, rt->gate, rt->tok_ptr, rt->tok_row, p, n_cand);
+    ETR_LAUNCH_CHECK();
+    return ETR_OK;
+  };
+  static std::atomic<unsigned long long> done[3] = {};      // one bit per device
+  if (c->T <= 128) return go(select_small_kernel<4>, done[0]);
+  if (c->T <= 256) return go(select_small_kernel<8>, done[1]);
+  return go(select_small_kernel<16>, done[2]);
+}
+
 // key / position matrix [E][T], then one int per 256-token block
 static size_t select_keys_bytes(const etr_config* c) { return align_up((size_t)c->T * c->E * sizeof(uint32_t), 256); }
 // ... then the per-expert threshold limits and the per-block counts of given-up candidates
@@ -714,6 +886,10 @@ etr_status select_forward(const etr_config* c, const float* delta, etr_stats* st
   char* ws_tail = reinterpret_cast<char*>(ws) + select_keys_bytes(c) + select_scan_bytes(c);
   int32_t* limit = (c->threshold_mode & ETR_THRESHOLD_EXPERT) ? reinterpret_cast<int32_t*>(ws_tail) : nullptr;
   int32_t* skipped = p.cut_token ? reinterpret_cast<int32_t*>(ws_tail + select_limit_bytes(c)) : nullptr;
+  const int n_cand = p.mode == ETR_MODE_TCR ? c->T * c->k : c->T * c->E;
+  if (!limit && !skipped && c->T <= SEL_SMALL_TOKENS && c->T * c->E <= SEL_SMALL_KEYS &&
+      (p.mode == ETR_MODE_ECR || c->E * c->k <= SEL_SMALL_RANKS))
+    return select_small(c, delta, stats, rt, p, n_cand, st);
   ETR_TIME_BEGIN("select_token_side_kernel");
   auto token_side = [&](auto k) {
     launch_kernel(k, ceil_div(c->T, SEL_TB), 256, 0, st, 1, delta, rt->topk_idx, keyT, stats, skipped, p);
@@ -746,7 +922,6 @@ etr_status select_forward(const etr_config* c, const float* delta, etr_stats* st
   const int nblocks = ceil_div(c->T, 256);
   launch_kernel(csr_count_kernel, nblocks, 256, 0, st, 1, (const int32_t*)keyT, rt->tok_ptr, block_total, stats, c->T, c->E);
   ETR_LAUNCH_CHECK();
-  const int n_cand = p.mode == ETR_MODE_TCR ? c->T * c->k : c->T * c->E;
   ETR_TIME_BEGIN("csr_fill_kernel");
   launch_kernel(csr_fill_kernel, nblocks, 256, 0, st, 1, (const int32_t*)keyT, (const int32_t*)block_total, rt->tok_ptr,
                 rt->tok_row, stats, c->T, c->E, p.C_stride, n_cand, (const int32_t*)skipped, ceil_div(c->T, SEL_TB));
