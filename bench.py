@@ -97,7 +97,15 @@ def algorithmic_work(w, rows, kernel, unrouted=0):
         "gate_softmax_kernel": (T * E * 4 + rows * 12 + T * 4, "bytes"),
         "gate_softmax_bwd_kernel": (2 * T * E * 4 + rows * 12, "bytes"),
         "load_stats_kernel": (rows * 4, "bytes"),
+        "select_small_kernel": (T * E * 4 + rows * 12, "bytes"),
         "gemm_simt_kernel": (18 * rows * d * h, "flops"),
+        # fp32 layers: flops of the fp32 product (three tf32 products each)
+        "tf32x3_gemm_swiglu": (4 * rows * d * h, "flops"),
+        "tf32x3_gemm_down": (2 * rows * d * h, "flops"),
+        "tf32x3_gemm_dswiglu": (2 * rows * d * h, "flops"),
+        "tf32x3_gemm_dxp": (4 * rows * d * h, "flops"),
+        "tf32x3_gemm_dw2": (2 * rows * d * h, "flops"),
+        "tf32x3_gemm_dw1": (4 * rows * d * h, "flops"),
         # tcgen05 grouped GEMMs: selected rows only (not the rows padding a 128-row tile)
         "tc_gemm_swiglu": (4 * rows * d * h, "flops"),
         "tc_gemm_down": (2 * rows * d * h, "flops"),

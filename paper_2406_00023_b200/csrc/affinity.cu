@@ -1047,9 +1047,10 @@ affinity_bwd_dr_partial_kernel(const float* __restrict__ Z, const float* __restr
 // short batch fills the GPU (3001 tokens, E 12, m 136: 12 chunks of 256 on 12 SMs took 99 us).
 constexpr int DR_DENSE_TOKENS = 256;
 constexpr int DR_DENSE_STEP = 32;
+constexpr int DR_DENSE_BLOCKS = 296;   // two per SM; a constant, because the workspace size must not depend on the device
 static int dr_dense_tokens(const etr_config* c) {
   const long long groups = (long long)ceil_div(c->E, 32) * ceil_div(c->d / c->D, 256);
-  const long long want = ((long long)c->T * groups + 2 * current_sm_count() - 1) / (2 * current_sm_count());
+  const long long want = ((long long)c->T * groups + DR_DENSE_BLOCKS - 1) / DR_DENSE_BLOCKS;
   return (int)std::min<long long>(DR_DENSE_TOKENS, std::max<long long>(DR_DENSE_STEP, (want + DR_DENSE_STEP - 1) / DR_DENSE_STEP * DR_DENSE_STEP));
 }
 __global__ void __launch_bounds__(256)

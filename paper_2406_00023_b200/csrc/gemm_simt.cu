@@ -1,6 +1,6 @@
-// Grouped GEMMs of the expert FFN on the CUDA cores (fp32 accumulate).  This is the path
-// for fp32 layers and the cross-check for the tensor-core kernels; the bf16 layer runs on
-// gemm_tcgen05.cu.  One generic kernel: 64x64x16 tiles, 4x4 outputs per thread, operands
+// Grouped GEMMs of the expert FFN on the CUDA cores (fp32 accumulate).  The cross-check
+// for the tensor-core kernels (gemm_impl SIMT); bf16 layers run on gemm_tcgen05.cu, fp32 layers on
+// gemm_tf32x3.cu.  One generic kernel: 64x64x16 tiles, 4x4 outputs per thread, operands
 // addressed by (row stride, column stride) so the same code serves K-major and MN-major
 // inputs; blockIdx.z is the expert and the row (or contraction) extent comes from counts.
 #include "common.cuh"

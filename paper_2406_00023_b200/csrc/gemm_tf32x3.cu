@@ -20,7 +20,9 @@
 //   warps 12-19  add the chunks' accumulators, then SwiGLU / its derivative / plain stores
 // Registers are split unevenly (setmaxnreg): the epilogue holds 64 running sums per thread.
 // What bounds it is shared memory: 12 KiB and 8 KiB of operands per pair of MMAs, 32 KiB in by TMA, 32 KiB read and
-// 64 KiB written by the split, about 1600 cycles of its port per K block at BN = 128.
+// 64 KiB written by the split, about 1600 cycles of its port per K block at BN = 128, of about 1850 that a block
+// takes (the MMAs alone: 940).  An fp32 step of T 1531, d 768, h 1000, 12 experts: 2.8 ms with the CUDA-core kernels,
+// 0.65 ms with these.
 // A tile is 128 x BN, BN = 128, or 64 where 128 would leave SMs without a tile.  All waits are bounded; on
 // expiry the kernel leaves 0x7c0a in etr_stats.error_word, frees its tensor memory and returns.
 #include <algorithm>

@@ -213,3 +213,11 @@ def test_pooled_widths_at_the_shared_memory_limit_of_the_fused_dx_kernel(d, D):
     memory than a launch gets without opting in."""
     w = gw.scaled(W["small"], T=70, d=d, D=D, E=4, h=64)
     layer_vs_oracle(w, gw.make_inputs(w), ob.MODE_TCR)
+
+
+@pytest.mark.parametrize("d,D,T", [(264, 8, 300), (24, 1, 150), (1312, 1, 140), (520, 4, 700)])
+def test_router_gradient_sums_at_the_edges_of_their_groups(d, D, T):
+    """33, 24, 1312 and 130 pooled columns: rows of Z that are no multiple of 16 bytes, shorter than a warp, longer than
+    a block, and of a width that leaves threads over; chunks of 128 slots that end inside (fp32, 1e-4)."""
+    w = gw.scaled(W["small"], T=T, d=d, D=D, E=4, h=64, dtype="f32")
+    layer_vs_oracle(w, gw.make_inputs(w), ob.MODE_TCR)
