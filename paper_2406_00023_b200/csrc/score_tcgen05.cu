@@ -140,7 +140,7 @@ affinity_score_tc_kernel(const __grid_constant__ CUtensorMap mapZ, const __grid_
           if (!mbar_wait(conv_bar + 8 * stage, phase, abort_flag, wait_limit)) { ok = false; break; }
           tc_fence_after();
           const uint32_t a_hi = tiles_base + stage * SCT_STAGE_BYTES, a_lo = a_hi + SCT_A_BYTES;
-          const uint32_t b_hi = a_hi + 2 * SCT_A_BYTES, b_lo = b_hi + SCT_B_BYTES;
+          const uint32_t b_hi = a_hi + 2 * SCT_A_BYTES;
           // 8 floats (32 bytes) per MMA, two MMAs per step: the hi and lo tiles of R lie one behind the other in
           // the stage, so A_hi x [R_hi; R_lo]^T is ONE MMA of 128 expert columns (hi*hi in columns 0-63 of the
           // chain, hi*lo in 64-127), and A_lo x R_hi^T adds lo*hi to columns 0-63.  These are small MMAs whose
@@ -192,22 +192,31 @@ affinity_score_tc_kernel(const __grid_constant__ CUtensorMap mapZ, const __grid_
     float* stg = reinterpret_cast<float*>(tiles + (size_t)SCT_STAGES * SCT_STAGE_BYTES) + (warp - 6) * 32 * 33;
     // ||R_i|| while the first tile is on its way: a warp per row, lanes over the columns, the same sums
     // as the other score kernels (eight columns per lane requested together)
-    for (int i = q; i < SCT_N; i += 4) {
-      float acc_q = 0.f;
-      if (i < E) {
-        const float* row = R + (size_t)i * m;
+    // (and four rows of a warp: a row at a time is a round of L2 latency each, sixteen of them at E = 64)
+    for (int i0 = q; i0 < SCT_N; i0 += 16) {
+      float sq[4] = {0.f, 0.f, 0.f, 0.f};
+      if (i0 < E) {
         for (int j0 = lane; j0 < m; j0 += 256) {
-          float v[8];
+          float v[4][8];
 #pragma unroll
-          for (int u = 0; u < 8; ++u) v[u] = j0 + 32 * u < m ? row[j0 + 32 * u] : 0.f;
+          for (int r = 0; r < 4; ++r)
 #pragma unroll
-          for (int u = 0; u < 8; ++u) acc_q += v[u] * v[u];
+            for (int u = 0; u < 8; ++u)
+              v[r][u] = i0 + 4 * r < E && j0 + 32 * u < m ? R[(size_t)(i0 + 4 * r) * m + j0 + 32 * u] : 0.f;
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int u = 0; u < 8; ++u) sq[r] += v[r][u] * v[r][u];
         }
       }
-      acc_q = warp_sum(acc_q);
-      if (lane == 0) {
-        rn[i] = sqrtf(acc_q);
-        if (blockIdx.x == 0 && i < E) rnorm[i] = rn[i];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int i = i0 + 4 * r;
+        const float acc_q = warp_sum(sq[r]);
+        if (lane == 0) {
+          rn[i] = sqrtf(acc_q);
+          if (blockIdx.x == 0 && i < E) rnorm[i] = rn[i];
+        }
       }
     }
     asm volatile("bar.sync 1, 128;" ::: "memory");      // the four epilogue warps: rn is complete
