@@ -557,7 +557,7 @@ def main():
         # The six tcgen05 contractions run on one persistent grouped-GEMM design in two tile forms
         # (--gemm can force one); the roofline entry covers all their launches.
         pair = args.gemm == "auto"          # the ncu traffic ratio was taken with the library's own choice
-        kname = {"auto": "tc_grouped_gemm_pair_kernel + tc_grouped_gemm_pair_wide_kernel (chosen per contraction)",
+        kname = {"auto": "tc_grouped_gemm_pair_kernel + tc_grouped_gemm_swap_kernel (chosen per contraction)",
                  "tcgen05_2cta": "tc_grouped_gemm_pair_kernel", "tcgen05_2cta_wide": "tc_grouped_gemm_pair_wide_kernel",
                  "tcgen05": "tc_grouped_gemm_kernel"}.get(args.gemm, "tc_grouped_gemm")
         roofline = {"kernel": kname, "launches_per_step": g["launches_per_step"], "bound": "tensor",
