@@ -168,7 +168,8 @@ typedef struct etr_buffers {
   void* Xp; void* G; void* U; void* H; void* O;          /* forward activations */
   void* dO; void* dG; void* dU; void* dXp; float* dgate; /* backward activations */
   void* ws;                   /* scratch, ws_bytes long */
-  size_t ws_bytes;
+  size_t ws_bytes;            /* the layer and host-step calls return ETR_ERR_WORKSPACE, before any launch, where this
+                                 is less than they need; 0: not stated, not checked */
   /* staging used only by etr_layer_step_host */
   void* X_dev; void* dY_dev; void* Y_dev; void* dX_dev;
   /* softmax gate only (NULL otherwise): per-token log-sum-exp [T] and the dense d delta [T,E] */
@@ -183,7 +184,8 @@ etr_status etr_validate(const etr_config* cfg);
 /* C_stride for a config (capacity rounded up to 128). */
 int32_t etr_c_stride(const etr_config* cfg);
 
-/* Scratch bytes the calls below need in `ws` (max over all of them). */
+/* Scratch bytes the calls below need in `ws` (max over all of them).  Never less for a larger T, E, d/D, h or
+ * capacity with the other options equal: buffers of the longest batch serve every shorter one. */
 etr_status etr_workspace_bytes(const etr_config* cfg, size_t* bytes);
 
 /* Size of one block holding every etr_buffers member, and the carving of such a block

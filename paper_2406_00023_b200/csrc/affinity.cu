@@ -1047,7 +1047,7 @@ affinity_bwd_dr_partial_kernel(const float* __restrict__ Z, const float* __restr
 // short batch fills the GPU (3001 tokens, E 12, m 136: 12 chunks of 256 on 12 SMs took 99 us).
 constexpr int DR_DENSE_TOKENS = 256;
 constexpr int DR_DENSE_STEP = 32;
-constexpr int DR_DENSE_BLOCKS = 296;   // two per SM; a constant, because the workspace size must not depend on the device
+constexpr int DR_DENSE_BLOCKS = 296;   // two per SM; a constant: the workspace size follows from it and must not depend on the device
 static int dr_dense_tokens(const etr_config* c) {
   const long long groups = (long long)ceil_div(c->E, 32) * ceil_div(c->d / c->D, 256);
   const long long want = ((long long)c->T * groups + DR_DENSE_BLOCKS - 1) / DR_DENSE_BLOCKS;
@@ -1305,11 +1305,19 @@ etr_status affinity_forward(const etr_config* c, const void* X, const float* R, 
   return ETR_OK;
 }
 
+// Partials of dR.  A dense d delta is cut into ceil(T / dr_dense_tokens) chunks, a number that falls wherever the chunk
+// length steps up by 32, while buffers made for one batch have to serve every shorter one (and every smaller E, m and
+// capacity).  So the size is a bound that never falls: chunks have at least 32 tokens; where they have fewer than 256,
+// groups of 32 experts x 256 columns times chunks stay below DR_DENSE_BLOCKS + 1 per group (at most 9.7 MB).
 size_t affinity_bwd_workspace_bytes(const etr_config* c) {
-  const int m = c->d / c->D;
-  const int nch = c->gate_mode == ETR_GATE_SOFTMAX ? std::max(c_stride_of(c) / DR_CHUNK, ceil_div(c->T, dr_dense_tokens(c)))
-                                                   : c_stride_of(c) / DR_CHUNK;
-  return (size_t)c->E * nch * (m + 1) * sizeof(float);
+  const size_t row = (size_t)c->E * (c->d / c->D + 1);
+  size_t floats = row * (c_stride_of(c) / DR_CHUNK);
+  if (c->gate_mode == ETR_GATE_SOFTMAX) {
+    const size_t few = row * ceil_div(c->T, DR_DENSE_STEP), many = row * ceil_div(c->T, DR_DENSE_TOKENS);
+    const size_t spread = (size_t)DR_DENSE_BLOCKS * 32 * 257 + row;
+    floats = std::max(floats, std::min(few, std::max(spread, many)));
+  }
+  return floats * sizeof(float);
 }
 
 template <class T>

@@ -1,4 +1,5 @@
 // C ABI of libetr: argument checks, buffer carving, stage wrappers, whole-layer calls.
+#include <algorithm>
 #include <atomic>
 #include <cstring>
 #include <mutex>
@@ -101,6 +102,16 @@ static etr_status check_ptrs(std::initializer_list<const void*> ps) {
     if (!aligned16(p)) return ETR_ERR_ALIGN;
   }
   return ETR_OK;
+}
+
+// The layer calls know how long their scratch is: one made for another configuration is refused before anything is
+// launched.  ws_bytes = 0: the caller does not say.
+static etr_status check_workspace(const etr_config* c, const etr_buffers* b, bool forward, bool backward) {
+  size_t need = use_tc(c) ? tc_workspace_bytes(c) : 0;
+  if (forward) need = std::max(need, select_workspace_bytes(c));
+  if (backward) need = std::max(need, affinity_bwd_workspace_bytes(c));
+  if (mixed_weights(c)) need = scratch_bytes(c) + 3 * 2 * weight_elems(c);
+  return b->ws_bytes != 0 && b->ws_bytes < need ? ETR_ERR_WORKSPACE : ETR_OK;
 }
 
 static etr_status check_route(const etr_route* r) {
@@ -424,6 +435,7 @@ etr_status etr_layer_forward(const etr_config* c, const void* X, const float* R,
   ETR_TRY(etr_validate(c));
   ETR_TRY(check_ptrs({b->stats, X, R, b->delta, b->xnorm, b->rnorm}));
   if (b->Z && !aligned16(b->Z)) return ETR_ERR_ALIGN;
+  ETR_TRY(check_workspace(c, b, true, false));
   ETR_TRY(affinity_forward(c, X, R, b->delta, b->Z, b->xnorm, b->rnorm, b->stats, true, (cudaStream_t)stream));
   ETR_TRY(etr_select(c, b->delta, b->stats, &b->route, b->ws, stream));
   if (c->gate_mode == ETR_GATE_SOFTMAX) ETR_TRY(etr_gate_softmax(c, b->delta, &b->route, b->lse, stream));
@@ -453,6 +465,8 @@ etr_status etr_layer_backward(const etr_config* c, const void* X, const float* R
                               const void* W1u, const void* W2, const void* dY, const etr_buffers* b,
                               void* dX, float* dR, void* dW1g, void* dW1u, void* dW2, void* stream) {
   if (b == nullptr) return ETR_ERR_ARG;
+  ETR_TRY(etr_validate(c));
+  ETR_TRY(check_workspace(c, b, false, true));
   ETR_TRY(etr_combine_bwd(c, &b->route, dY, b->O, b->dO, b->dgate, stream));
   if (fuse_dispatch(c)) {
     ETR_TRY(etr_validate(c));
@@ -523,6 +537,7 @@ etr_status etr_layer_step_host(const etr_config* c, const void* X_host, const vo
     return ETR_ERR_ARG;
   ETR_TRY(etr_validate(c));
   if (!b->X_dev || !b->dY_dev || !b->Y_dev || !b->dX_dev) return ETR_ERR_WORKSPACE;
+  ETR_TRY(check_workspace(c, b, true, true));
   cudaStream_t st = (cudaStream_t)stream;
   HostStepCtx* hc = nullptr;
   ETR_TRY(host_step_ctx(&hc));
@@ -558,6 +573,7 @@ etr_status etr_layer_step_host_begin(const etr_config* c, const void* X_host, co
     return ETR_ERR_ARG;
   ETR_TRY(etr_validate(c));
   ETR_TRY(check_ptrs({sg->X_dev, sg->dY_dev, sg->Y_dev, sg->dX_dev}));
+  ETR_TRY(check_workspace(c, b, true, true));
   cudaStream_t st = (cudaStream_t)stream;
   HostStepCtx* hc = nullptr;
   ETR_TRY(host_step_ctx(&hc));

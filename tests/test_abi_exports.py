@@ -74,3 +74,46 @@ def test_layout_gives_the_offsets_bind_uses():
             assert b.X_dev == base + lay.X_dev and b.lse == base + lay.lse and lay.ddelta > lay.lse > 0
         else:
             assert lay.X_dev == 0 and lay.lse == 0 and not b.X_dev
+
+
+def test_workspace_never_shrinks_with_the_batch():
+    """Buffers made for one batch serve every shorter one: their size and that of the scratch in them never fall as T,
+    E or the pooled width grows, for both gates."""
+    from paper_2406_00023_b200 import etr
+
+    def sizes(**kw):
+        cfg = etr.make_config(**dict(dict(T=512, d=2048, D=8, E=32, k=2, h=64, capacity=64, dtype=etr.BF16), **kw))
+        n = ctypes.c_size_t(0)
+        assert etr.lib().etr_buffers_bytes(ctypes.byref(cfg), 0, ctypes.byref(n)) == etr.OK
+        return etr.workspace_bytes(cfg), n.value
+
+    for gate in (etr.GATE_AFFINITY, etr.GATE_SOFTMAX):
+        for d, D, E in ((2048, 8, 32), (64, 8, 8), (1088, 8, 12), (4096, 1, 256), (512, 4, 100)):
+            last = (0, 0)
+            for T in sorted({*range(1, 2000), *range(2000, 70001, 31), 9471, 9472, 9473, 18944, 18945, 37888, 37889}):
+                now = sizes(T=T, d=d, D=D, E=E, gate_mode=gate)
+                assert now[0] >= last[0] and now[1] >= last[1], (gate, d, D, E, T)
+                last = now
+        for T in (3001, 9472, 60000):
+            by_E = [sizes(T=T, E=E, gate_mode=gate)[0] for E in range(2, 257)]
+            by_m = [sizes(T=T, d=8 * m, D=8, E=8, dtype=etr.F32, gate_mode=gate)[0] for m in range(8, 700)]
+            assert by_E == sorted(by_E) and by_m == sorted(by_m)
+
+
+def test_layer_calls_refuse_a_small_workspace():
+    """A scratch shorter than the configuration needs is refused before anything is launched (there is no GPU here: a
+    launch would fail with another status)."""
+    from paper_2406_00023_b200 import etr
+    big, small = (etr.make_config(T=T, d=2048, D=8, E=32, k=2, h=64, capacity=64, dtype=etr.BF16,
+                                  gate_mode=etr.GATE_SOFTMAX) for T in (16384, 512))
+    b, n = etr.Buffers(), ctypes.c_size_t(0)
+    assert etr.lib().etr_buffers_bytes(ctypes.byref(small), 1, ctypes.byref(n)) == etr.OK
+    assert etr.lib().etr_buffers_bind(ctypes.byref(small), 1, ctypes.c_void_p(1 << 20), n, ctypes.byref(b)) == etr.OK
+    p, s = ctypes.c_void_p(1 << 20), ctypes.c_void_p(0)
+    L, cfg, bb = etr.lib(), ctypes.byref(big), ctypes.byref(b)
+    slot = etr.HostSlotC(p, p, p, p)
+    assert L.etr_layer_forward(cfg, p, p, p, p, p, bb, p, s) == etr.ERR_WORKSPACE
+    assert L.etr_layer_backward(cfg, p, p, p, p, p, p, bb, p, p, p, p, p, s) == etr.ERR_WORKSPACE
+    assert L.etr_layer_step_host(cfg, p, p, p, p, p, p, bb, p, p, p, p, p, p, s) == etr.ERR_WORKSPACE
+    assert L.etr_layer_step_host_begin(cfg, p, p, p, p, p, p, bb, ctypes.byref(slot), ctypes.c_int32(0), p, p, p, p,
+                                       p, p, s) == etr.ERR_WORKSPACE

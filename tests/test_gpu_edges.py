@@ -221,3 +221,26 @@ def test_router_gradient_sums_at_the_edges_of_their_groups(d, D, T):
     a block, and of a width that leaves threads over; chunks of 128 slots that end inside (fp32, 1e-4)."""
     w = gw.scaled(W["small"], T=T, d=d, D=D, E=4, h=64, dtype="f32")
     layer_vs_oracle(w, gw.make_inputs(w), ob.MODE_TCR)
+
+
+@pytest.mark.parametrize("gate", [etr.GATE_AFFINITY, etr.GATE_SOFTMAX])
+def test_buffers_of_a_longer_batch_serve_a_shorter_one(gate):
+    """A step of 9000 tokens on buffers made for 16384 gives the bits of buffers made for 9000 (the dense router
+    gradient cuts the shorter batch into more chunks than the longer one)."""
+    T, d, D, E, h = 9000, 2048, 8, 32, 64
+    g = torch.Generator(device="cuda").manual_seed(5)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")  # noqa: E731
+    X, dY = rnd(T, d).bfloat16(), rnd(T, d).bfloat16()
+    R = rnd(E, d // D)
+    W1g, W1u, W2 = ((rnd(*s) / d ** 0.5).bfloat16() for s in ((E, h, d), (E, h, d), (E, d, h)))
+    short, longer = (etr.make_config(T=n, d=d, D=D, E=E, k=2, h=h, capacity=700, dtype=etr.BF16, mode=etr.MODE_TCR,
+                                     gate_mode=gate) for n in (T, 16384))
+    outs = []
+    for made_for in (short, longer):
+        buf = etr.LayerBuffers(made_for)
+        out = [torch.empty_like(t) for t in (X, X, R, W1g, W1u, W2)]
+        etr.layer_forward(short, X, R, W1g, W1u, W2, buf, out[0])
+        etr.layer_backward(short, X, R, W1g, W1u, W2, dY, buf, *out[1:])
+        assert buf.read_stats().error_word == 0
+        outs.append(out)
+    assert all(torch.equal(a, b) for a, b in zip(*outs))
