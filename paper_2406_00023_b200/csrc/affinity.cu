@@ -1398,7 +1398,7 @@ etr_status affinity_backward(const etr_config* c, const void* X, const float* R,
       launch_kernel(k, dim3(c->E, nch), 256, 0, st, 1, Z, delta, xnorm, rnorm, rt->counts, rt->slot_token, dgate, part,
                     c->E, m, Cs, nch, sqrtf((float)c->D));
     };
-    if (m % 4 == 0) go(affinity_bwd_dr_partial_kernel<4>);
+    if (m % 4 == 0 && aligned16(Z)) go(affinity_bwd_dr_partial_kernel<4>);      // the layer call takes any float Z
     else go(affinity_bwd_dr_partial_kernel<1>);
   }
   ETR_LAUNCH_CHECK();

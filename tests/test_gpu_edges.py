@@ -244,3 +244,24 @@ def test_buffers_of_a_longer_batch_serve_a_shorter_one(gate):
         assert buf.read_stats().error_word == 0
         outs.append(out)
     assert all(torch.equal(a, b) for a, b in zip(*outs))
+
+
+def test_layer_backward_takes_pooled_tokens_at_any_float_address():
+    """The backward layer call reads Z where the caller has put it, here one float behind a 16-byte boundary: the sums
+    of dR are taken in another order (fp32 sums of at most 160 products: 1e-6), everything else has the same bits."""
+    w = gw.scaled(W["small"], T=512, d=256, D=4, E=8, h=64, dtype="f32")
+    inp = gw.make_inputs(w)
+    cfg, dev = hz.make_cfg(w, mode=ob.MODE_TCR), hz.upload(w, inp)
+    buf = etr.LayerBuffers(cfg)
+    Y = torch.empty_like(dev.X)
+    etr.layer_forward(cfg, dev.X, dev.R, dev.W1g, dev.W1u, dev.W2, buf, Y)
+    outs = []
+    shifted = torch.empty(buf.Z.numel() + 1, device="cuda")
+    shifted[1:].copy_(buf.Z.flatten())
+    for Z in (buf.c.Z, shifted.data_ptr() + 4):
+        buf.c.Z = Z
+        outs.append([torch.empty_like(t) for t in (dev.X, dev.R, dev.W1g, dev.W1u, dev.W2)])
+        etr.layer_backward(cfg, dev.X, dev.R, dev.W1g, dev.W1u, dev.W2, dev.dY, buf, *outs[-1])
+    torch.cuda.synchronize()
+    for i, (a, b) in enumerate(zip(*outs)):
+        assert float((a - b).norm()) <= 1e-6 * float(a.norm()) if i == 1 else torch.equal(a, b)
