@@ -92,3 +92,24 @@ def test_ends_of_the_number_range():
         assert bool((G[r][ok] - ref[r][ok]).abs().le(1e-6 * ref[r][ok].abs()).all())
     rest = [r for r in range(128) if r not in (3, 4, 5, 6, 7)]
     assert rel(G[rest], ref[rest]) <= TOL
+
+
+@pytest.mark.parametrize("bits", [0x7f800001, 0x7f801fff, -0x7fffff, -0x7fe001, 0x7fc00000, -1])
+def test_every_nan_stays_a_nan(bits):
+    """Payloads in the low 13 bits only (0x7f800001, 0x7f801fff and the negative ones), the canonical NaN and all ones,
+    in a token, a weight and a gradient: NaN in exactly the outputs whose products hold it."""
+    cfg, b, W = layer(1, 64, 64, 128, (128,))
+    put = lambda t, *at: t.view(torch.int32).__setitem__(at, bits)  # noqa: E731
+    x, dO = b.Xp.view(128, 64), b.dO.view(128, 64)
+    put(x, 3, 7)
+    put(W[1], 0, 5, 9)
+    put(dO, 11, 2)
+    dW = [torch.empty_like(w) for w in W]
+    etr.expert_ffn(cfg, b.route, b.Xp, *W, b.G, b.U, b.H, b.O, b.c.stats, b.c.ws)
+    etr.expert_ffn_bwd(cfg, b.route, b.dO, b.Xp, b.G, b.U, b.H, *W, b.dG, b.dU, b.dXp, *dW, b.c.stats, b.c.ws)
+    assert b.read_stats().error_word == 0
+    G, U, dG = (t.view(128, 64).isnan() for t in (b.G, b.U, b.dG))
+    row, col = torch.arange(128, device="cuda")[:, None], torch.arange(64, device="cuda")[None, :]
+    assert G.equal((row == 3).expand(128, 64)) and U.equal((row == 3) | (col == 5))
+    assert dG.equal((row == 3) | (row == 11) | (col == 5))
+    assert bool(dW[2].isnan()[0, 2].all())                   # its row of dO, transposed on the way
