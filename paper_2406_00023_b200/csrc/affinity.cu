@@ -33,7 +33,7 @@ template <class T> struct Raw16;
 template <> struct Raw16<__nv_bfloat16> {          // 8 elements
   static constexpr int ELEMS = 8;
   uint4 w;
-  __device__ void load(const __nv_bfloat16* p) { w = __ldg(reinterpret_cast<const uint4*>(p)); }
+  __device__ void load(const __nv_bfloat16* p) { w = *reinterpret_cast<const uint4*>(p); }
   __device__ void reduce(float& s, float& sq) const {
     const uint32_t u[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
@@ -46,7 +46,7 @@ template <> struct Raw16<__nv_bfloat16> {          // 8 elements
 template <> struct Raw16<float> {                  // 4 elements
   static constexpr int ELEMS = 4;
   float4 w;
-  __device__ void load(const float* p) { w = __ldg(reinterpret_cast<const float4*>(p)); }
+  __device__ void load(const float* p) { w = *reinterpret_cast<const float4*>(p); }
   __device__ void reduce(float& s, float& sq) const {
     s += w.x; s += w.y; s += w.z; s += w.w;
     sq = fmaf(w.x, w.x, sq); sq = fmaf(w.y, w.y, sq); sq = fmaf(w.z, w.z, sq); sq = fmaf(w.w, w.w, sq);
@@ -140,7 +140,7 @@ __device__ inline void pool_token(const T* __restrict__ x, float* __restrict__ z
 // adjacent pieces whose partial sums meet through xor-shuffles.  Pure HBM streaming.
 template <class T, int PPG>
 __global__ void __launch_bounds__(256)
-grap_pool_kernel(const T* __restrict__ X, float* __restrict__ Z, float* __restrict__ xnorm,
+grap_pool_kernel(const T* X, float* __restrict__ Z, float* __restrict__ xnorm,
                  etr_stats* zero_stats, int Ttok, int d, int D, int m) {
   grid_sync();
   if (zero_stats != nullptr && blockIdx.x == 0 && threadIdx.x < sizeof(etr_stats) / 4)
@@ -163,6 +163,7 @@ grap_pool_kernel(const T* __restrict__ X, float* __restrict__ Z, float* __restri
         const int p = p0 + 32 * g + lane;
         q[g].load(x + (size_t)(p < npieces ? p : lane) * PE);
       }
+      asm volatile("" ::: "memory");      // no load moves behind the stores below
 #pragma unroll
       for (int g = 0; g < BATCH; ++g) {
         const int p = p0 + 32 * g + lane;
@@ -189,8 +190,8 @@ grap_pool_kernel(const T* __restrict__ X, float* __restrict__ Z, float* __restri
 // FMA rate (2 m E flop per token against 4 m bytes), not by HBM.
 template <int EPL, int TPG>
 __global__ void __launch_bounds__(512, 1)
-affinity_score_kernel(const float* __restrict__ Z, const float* __restrict__ xnorm,
-                      const float* __restrict__ R, float* __restrict__ delta,
+affinity_score_kernel(const float* Z, const float* xnorm,
+                      const float* R, float* __restrict__ delta,
                       float* __restrict__ rnorm, etr_stats* stats, int Ttok, int D, int E, int m,
                       int ldm) {
   grid_sync();
@@ -230,21 +231,19 @@ affinity_score_kernel(const float* __restrict__ Z, const float* __restrict__ xno
     const int t0 = g * TPG;
     float xn[TPG];
 #pragma unroll
-    for (int u = 0; u < TPG; ++u) {
-      const int t = t0 + u;
-      xn[u] = t < Ttok ? xnorm[t] : 0.f;
-      float* zr = zs + (size_t)u * ldm;
-      if (t < Ttok) {
-        const float* src = Z + (size_t)t * m;
-        if (vec_ok) {
-          for (int j = lane; j < m / 4; j += 32)
-            reinterpret_cast<float4*>(zr)[j] = __ldg(reinterpret_cast<const float4*>(src) + j);
-        } else {
-          for (int j = lane; j < m; j += 32) zr[j] = src[j];
-        }
-      } else {
-        for (int j = lane; j < m; j += 32) zr[j] = 0.f;
+    for (int u = 0; u < TPG; ++u) xn[u] = t0 + u < Ttok ? xnorm[t0 + u] : 0.f;
+    if (vec_ok) {
+      for (int j = lane; j < m / 4; j += 32) {          // a vector of every token in flight before the first store
+        float4 q[TPG];
+#pragma unroll
+        for (int u = 0; u < TPG; ++u)
+          q[u] = t0 + u < Ttok ? reinterpret_cast<const float4*>(Z + (size_t)(t0 + u) * m)[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < TPG; ++u) reinterpret_cast<float4*>(zs + (size_t)u * ldm)[j] = q[u];
       }
+    } else {
+      for (int u = 0; u < TPG; ++u)
+        for (int j = lane; j < m; j += 32) zs[(size_t)u * ldm + j] = t0 + u < Ttok ? Z[(size_t)(t0 + u) * m + j] : 0.f;
     }
     __syncwarp();
     float acc[TPG][EPL];
@@ -311,8 +310,8 @@ constexpr int SC_ZLD = SC_KC + 4;     // row stride of a stage buffer, in floats
 
 template <int EPT>
 __global__ void __launch_bounds__(256, 2)
-affinity_score_tile_kernel(const float* __restrict__ Z, const float* __restrict__ xnorm,
-                           const float* __restrict__ R, float* __restrict__ delta,
+affinity_score_tile_kernel(const float* Z, const float* xnorm,
+                           const float* R, float* __restrict__ delta,
                            float* __restrict__ rnorm, etr_stats* stats, int Ttok, int D, int E, int m,
                            int ldm) {
   grid_sync();
@@ -432,7 +431,7 @@ affinity_score_tile_kernel(const float* __restrict__ Z, const float* __restrict_
 // No block-wide barrier after set-up, so the loads of some warps overlap the FMAs of others.
 template <class T, int EPL, int TPG>
 __global__ void __launch_bounds__(512, 1)
-affinity_fwd_warp_kernel(const T* __restrict__ X, const float* __restrict__ R,
+affinity_fwd_warp_kernel(const T* X, const float* R,
                          float* __restrict__ delta, float* __restrict__ Z, float* __restrict__ xnorm,
                          float* __restrict__ rnorm, etr_stats* stats, int Ttok, int d, int D, int E,
                          int m, int ldm) {
@@ -545,7 +544,7 @@ affinity_fwd_warp_kernel(const T* __restrict__ X, const float* __restrict__ R,
 // ---- forward, tiled form (fallback for shapes whose R does not fit next to the warp slices) ----
 template <class T>
 __global__ void __launch_bounds__(AFF_THREADS)
-affinity_fwd_kernel(const T* __restrict__ X, const float* __restrict__ R, float* __restrict__ delta,
+affinity_fwd_kernel(const T* X, const float* R, float* __restrict__ delta,
                     float* __restrict__ Z, float* __restrict__ xnorm, float* __restrict__ rnorm,
                     etr_stats* stats, int Ttok, int d, int D, int E, int m, int ldm, int Epad) {
   grid_sync();
@@ -656,11 +655,11 @@ affinity_fwd_kernel(const T* __restrict__ X, const float* __restrict__ R, float*
 // token rearrangement, dX[t] = sum of the token's rows of dXp), so dX is written exactly once.
 template <class T, bool FUSED, bool DENSE>
 __global__ void __launch_bounds__(256)
-affinity_bwd_dx_kernel(const T* __restrict__ X, const float* __restrict__ R,
-                       const float* __restrict__ delta, const float* __restrict__ xnorm,
-                       const float* __restrict__ rnorm, const int32_t* __restrict__ tok_ptr,
-                       const int32_t* __restrict__ tok_row, const float* __restrict__ dgate,
-                       const float* __restrict__ ddelta, const T* __restrict__ dXp, T* __restrict__ dX,
+affinity_bwd_dx_kernel(const T* X, const float* R,
+                       const float* delta, const float* xnorm,
+                       const float* rnorm, const int32_t* tok_ptr,
+                       const int32_t* tok_row, const float* dgate,
+                       const float* ddelta, const T* dXp, T* __restrict__ dX,
                        int Ttok, int d, int D, int E, int m, int C_stride) {
   grid_sync();
   extern __shared__ __align__(16) float smem[];
@@ -838,11 +837,11 @@ __device__ __forceinline__ void dx_chunk_cz(float* __restrict__ cz, float* __res
 
 template <class T, int NV, bool GROUP8>
 __global__ void __launch_bounds__(256, 4)
-affinity_bwd_dx_chunk_kernel(const T* __restrict__ X, const float* __restrict__ R,
-                             const float* __restrict__ delta, const float* __restrict__ xnorm,
-                             const float* __restrict__ rnorm, const int32_t* __restrict__ tok_ptr,
-                             const int32_t* __restrict__ tok_row, const float* __restrict__ dgate,
-                             const T* __restrict__ dXp, T* __restrict__ dX,
+affinity_bwd_dx_chunk_kernel(const T* X, const float* R,
+                             const float* delta, const float* xnorm,
+                             const float* rnorm, const int32_t* tok_ptr,
+                             const int32_t* tok_row, const float* dgate,
+                             const T* dXp, T* __restrict__ dX,
                              int Ttok, int d, int D, int E, int m, int C_stride, int tpb, int d_shift) {
   grid_sync();
   extern __shared__ __align__(16) float cz[];      // [tpb][m]
@@ -959,11 +958,11 @@ template <> struct DrVec<1> { typedef float type; };
 template <> struct DrVec<4> { typedef float4 type; };
 template <int V>
 __global__ void __launch_bounds__(256)
-affinity_bwd_dr_partial_kernel(const float* __restrict__ Z, const float* __restrict__ delta,
-                               const float* __restrict__ xnorm, const float* __restrict__ rnorm,
-                               const int32_t* __restrict__ counts,
-                               const int32_t* __restrict__ slot_token,
-                               const float* __restrict__ dgate, float* __restrict__ part,
+affinity_bwd_dr_partial_kernel(const float* Z, const float* delta,
+                               const float* xnorm, const float* rnorm,
+                               const int32_t* counts,
+                               const int32_t* slot_token,
+                               const float* dgate, float* __restrict__ part,
                                int E, int m, int C_stride, int nch, float sqD) {
   grid_sync();
   typedef typename DrVec<V>::type vec;
@@ -1054,9 +1053,9 @@ static int dr_dense_tokens(const etr_config* c) {
   return (int)std::min<long long>(DR_DENSE_TOKENS, std::max<long long>(DR_DENSE_STEP, (want + DR_DENSE_STEP - 1) / DR_DENSE_STEP * DR_DENSE_STEP));
 }
 __global__ void __launch_bounds__(256)
-affinity_bwd_dr_dense_partial_kernel(const float* __restrict__ Z, const float* __restrict__ delta,
-                                     const float* __restrict__ xnorm, const float* __restrict__ rnorm,
-                                     const float* __restrict__ ddelta, float* __restrict__ part,
+affinity_bwd_dr_dense_partial_kernel(const float* Z, const float* delta,
+                                     const float* xnorm, const float* rnorm,
+                                     const float* ddelta, float* __restrict__ part,
                                      int Ttok, int E, int m, int nch, int tok, float sqD) {
   grid_sync();
   __shared__ __align__(16) float s_w[DR_DENSE_STEP][32];
@@ -1115,8 +1114,8 @@ affinity_bwd_dr_dense_partial_kernel(const float* __restrict__ Z, const float* _
 // dR[i][j] = sum_ch part[i][ch][j] - (sum_ch part[i][ch][m]) R[i][j] / b_i^2.  A block takes 32 columns of an
 // expert; its eight warps take every eighth chunk, their sums are added in warp order (fixed whatever runs first).
 __global__ void __launch_bounds__(256)
-affinity_bwd_dr_final_kernel(const float* __restrict__ part, const float* __restrict__ R,
-                             const float* __restrict__ rnorm, float* __restrict__ dR, int m, int nch) {
+affinity_bwd_dr_final_kernel(const float* part, const float* R,
+                             const float* rnorm, float* __restrict__ dR, int m, int nch) {
   grid_sync();
   __shared__ float s_acc[8][32], s_sdd[8];
   const int i = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = 32 * blockIdx.y + lane;

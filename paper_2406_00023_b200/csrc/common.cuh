@@ -32,9 +32,20 @@ void timing_end(cudaStream_t st);
 
 // Every kernel is launched with programmatic stream serialization: its blocks may become resident while the last
 // blocks of the kernel before it still run, so that the launch latency and the set-up that touches no memory of
-// others (barriers, tensor memory) overlap.  Each kernel calls grid_sync() before its first access to global
-// memory: it waits for the kernel before it to be complete and visible, and only then lets the next kernel in, so
-// that never more than two kernels of a stream are in flight.
+// others (barriers, tensor memory) overlap.  What makes that safe:
+//   - A kernel waits (grid_wait) before its first access to global memory: the kernel before it is then complete and
+//     its writes are visible.  Only after that wait does it let the next kernel in (grid_release), so never more than two
+//     kernels of a stream are in flight, and a kernel sees the writes of all kernels before it.
+//   - Inputs are plain `const` pointers, not `const __restrict__`, and never read by __ldg: the compiler may send such reads
+//     through the read-only path, which asks for memory that nobody writes during the kernel's lifetime, and that
+//     lifetime begins while the kernel before it still writes.  (Outputs are `__restrict__`: that orders nothing away.)
+//   - A block that allocates tensor memory has done so (a block barrier) before it lets the next kernel in.  A block of
+//     the next kernel that allocates on the same SM then only ever waits for one that already holds its columns and
+//     gives them back without waiting for anybody later; the other way round, the two would wait for each other.
+//   - The two blocks of a pair leave together, after both have given their tensor memory back (a cluster barrier behind
+//     tcgen05.dealloc).  Freeing for a pair involves both SMs; once one of them is free a block of the next kernel may
+//     start there and allocate for its own pair, with the first pair still freeing on the other SM.  Without overlapped
+//     launches nothing started on an SM before the whole kernel had ended.
 template <class... P, class... A>
 inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, int cluster,
                                  A&&... args) {
@@ -169,9 +180,9 @@ __device__ inline float warp_sum(float v) {
 constexpr long long ETR_WAIT_LIMIT_CYCLES = 4000000000ll;   // about two seconds
 
 #ifdef __CUDACC__
-__device__ __forceinline__ void grid_sync() {
-  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
-}
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_sync() { grid_wait(); grid_release(); }
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }

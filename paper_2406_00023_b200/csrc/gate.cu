@@ -11,8 +11,8 @@ namespace etr {
 
 // lse[t] = log sum_j exp(delta_tj); gate[r] = exp(delta_ti - lse[t]) for every row r of token t.
 __global__ void __launch_bounds__(256)
-gate_softmax_kernel(const float* __restrict__ delta, const int32_t* __restrict__ tok_ptr,
-                    const int32_t* __restrict__ tok_row, float* __restrict__ gate,
+gate_softmax_kernel(const float* delta, const int32_t* tok_ptr,
+                    const int32_t* tok_row, float* __restrict__ gate,
                     float* __restrict__ lse, int Ttok, int E, int C_stride) {
   grid_sync();
   const int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -37,9 +37,9 @@ gate_softmax_kernel(const float* __restrict__ delta, const int32_t* __restrict__
 // ddelta[t][j] = p_tj (g_tj - s_t), p_tj = exp(delta_tj - lse[t]), g_tj = dgate of the row of (t, j)
 // if selected, else 0.
 __global__ void __launch_bounds__(256)
-gate_softmax_bwd_kernel(const float* __restrict__ delta, const float* __restrict__ lse,
-                        const int32_t* __restrict__ tok_ptr, const int32_t* __restrict__ tok_row,
-                        const float* __restrict__ gate, const float* __restrict__ dgate,
+gate_softmax_bwd_kernel(const float* delta, const float* lse,
+                        const int32_t* tok_ptr, const int32_t* tok_row,
+                        const float* gate, const float* dgate,
                         float* __restrict__ ddelta, int Ttok, int E, int C_stride) {
   grid_sync();
   const int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -69,7 +69,7 @@ gate_softmax_bwd_kernel(const float* __restrict__ delta, const float* __restrict
 // load[i] = counts[i] / T; gate_mean[i] = (sum of the gates of expert i's rows) / T.  One block
 // per expert; a fixed-shape tree reduction.
 __global__ void __launch_bounds__(256)
-load_stats_kernel(const int32_t* __restrict__ counts, const float* __restrict__ gate,
+load_stats_kernel(const int32_t* counts, const float* gate,
                   float* __restrict__ load, float* __restrict__ gate_mean, int Ttok, int C_stride) {
   grid_sync();
   __shared__ float red[8];

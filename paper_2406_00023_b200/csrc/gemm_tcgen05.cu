@@ -363,9 +363,10 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_c
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  grid_sync();
+  grid_wait();
   for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
   __syncthreads();
+  grid_release();
   if (warp == 2) {
     const int nt = (p.N + N_TILE_COLS - 1) / N_TILE_COLS;
     tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) {
@@ -591,7 +592,7 @@ __device__ __forceinline__ void tma_gather4_pair(uint32_t dst, const CUtensorMap
 }
 // Token ids of four consecutive slots, -1 replaced by the out-of-range row.
 __device__ __forceinline__ int4 gather_rows(const int32_t* idx, int oob) {
-  int4 r = __ldg(reinterpret_cast<const int4*>(idx));
+  int4 r = *reinterpret_cast<const int4*>(idx);
   r.x = r.x < 0 ? oob : r.x; r.y = r.y < 0 ? oob : r.y; r.z = r.z < 0 ? oob : r.z; r.w = r.w < 0 ? oob : r.w;
   return r;
 }
@@ -679,9 +680,10 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
-  grid_sync();
+  grid_wait();
   for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
   __syncthreads();
+  grid_release();
   if (warp == 2) {
     const int nt = (p.N + N_TILE_COLS - 1) / N_TILE_COLS;
     tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) {
@@ -971,9 +973,10 @@ tc_grouped_gemm_pair_wide_kernel(const __grid_constant__ CUtensorMap mapA0, cons
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
-  grid_sync();
+  grid_wait();
   for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
   __syncthreads();
+  grid_release();
   if (warp == 2) {
     const int nt = (p.N + 2 * N_TILE_COLS - 1) / (2 * N_TILE_COLS);
     tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) {
@@ -1410,9 +1413,10 @@ tc_grouped_gemm_swap_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
-  grid_sync();
+  grid_wait();
   for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
   __syncthreads();
+  grid_release();
   if (warp == 2) {
     const int nc = (p.N + COLS - 1) / COLS;
     tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) {

@@ -222,9 +222,10 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  grid_sync();
+  grid_wait();
   for (int e = tid; e < p.E; e += F3_THREADS) s_counts[e] = p.counts[e];
   __syncthreads();
+  grid_release();
   if (warp == 2) {
     const int nt = (p.N + COLS - 1) / COLS;
     tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) { return f3_mtiles(p, n_e) * nt; });

@@ -8,8 +8,8 @@ namespace etr {
 // after counts[i]) are zero-filled; rows beyond are left alone.  One warp per row.
 template <class T>
 __global__ void __launch_bounds__(256)
-dispatch_kernel(const T* __restrict__ X, const int32_t* __restrict__ counts,
-                const int32_t* __restrict__ slot_token, T* __restrict__ Xp, int d, int C_stride,
+dispatch_kernel(const T* X, const int32_t* counts,
+                const int32_t* slot_token, T* __restrict__ Xp, int d, int C_stride,
                 int n_rows) {
   grid_sync();
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -22,8 +22,14 @@ dispatch_kernel(const T* __restrict__ X, const int32_t* __restrict__ counts,
   const int nv = d * (int)sizeof(T) / 16;
   if (t >= 0) {
     const uint4* src = reinterpret_cast<const uint4*>(X + (size_t)t * d);
-#pragma unroll 4
-    for (int v = lane; v < nv; v += 32) dst[v] = __ldg(src + v);
+    for (int v0 = lane; v0 < nv; v0 += 128) {        // four loads in flight before the first store
+      uint4 q[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) q[u] = src[v0 + 32 * u < nv ? v0 + 32 * u : v0];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (v0 + 32 * u < nv) dst[v0 + 32 * u] = q[u];
+    }
   } else {
     for (int v = lane; v < nv; v += 32) dst[v] = make_uint4(0, 0, 0, 0);
   }
@@ -40,8 +46,8 @@ constexpr int COMBINE_ROWS = 512;     // row entries held in shared memory; late
 
 template <class T, int NV>
 __global__ void __launch_bounds__(256)
-combine_kernel(const T* __restrict__ O, const float* __restrict__ gate,
-               const int32_t* __restrict__ tok_ptr, const int32_t* __restrict__ tok_row,
+combine_kernel(const T* O, const float* gate,
+               const int32_t* tok_ptr, const int32_t* tok_row,
                T* __restrict__ Y, int Ttok, int d, int tpb) {
   grid_sync();
   __shared__ int s_ptr[COMBINE_TOKENS + 1];
@@ -110,9 +116,9 @@ combine_kernel(const T* __restrict__ O, const float* __restrict__ gate,
 // dO[r,:] = gate[r] dY[t(r),:], dgate[r] = <dY[t(r),:], O[r,:]>; pad rows zero.  Warp per row.
 template <class T>
 __global__ void __launch_bounds__(256)
-combine_bwd_kernel(const T* __restrict__ dY, const T* __restrict__ O,
-                   const int32_t* __restrict__ counts, const int32_t* __restrict__ slot_token,
-                   const float* __restrict__ gate, T* __restrict__ dO, float* __restrict__ dgate,
+combine_bwd_kernel(const T* dY, const T* O,
+                   const int32_t* counts, const int32_t* slot_token,
+                   const float* gate, T* __restrict__ dO, float* __restrict__ dgate,
                    int d, int C_stride, int n_rows) {
   grid_sync();
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -147,7 +153,7 @@ combine_bwd_kernel(const T* __restrict__ dY, const T* __restrict__ O,
 // Y[t,:] = 0 for tokens without a row (the part of the combine that the fused Top-1 epilogue of the
 // down GEMM leaves over).  One warp per token.
 __global__ void __launch_bounds__(256)
-zero_unrouted_kernel(const int32_t* __restrict__ tok_ptr, uint4* __restrict__ Y, int Ttok, int row_vec) {
+zero_unrouted_kernel(const int32_t* tok_ptr, uint4* __restrict__ Y, int Ttok, int row_vec) {
   grid_sync();
   const int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (t >= Ttok || tok_ptr[t] != tok_ptr[t + 1]) return;
@@ -218,7 +224,7 @@ etr_status dispatch_backward(const etr_config* c, const etr_route* rt, const voi
 
 // fp32 -> bf16 (round to nearest even), eight values per thread: the expert weights of a layer that keeps
 // fp32 master weights, rounded once per pass for the GEMMs.
-__global__ void __launch_bounds__(256) cast_f32_to_bf16_kernel(const float4* __restrict__ src, uint4* __restrict__ dst,
+__global__ void __launch_bounds__(256) cast_f32_to_bf16_kernel(const float4* src, uint4* __restrict__ dst,
                                                                size_t n8) {
   grid_sync();
   for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n8; i += (size_t)gridDim.x * 256) {

@@ -69,7 +69,7 @@ __device__ __forceinline__ void split_chunks(uint8_t* hi_tile, uint8_t* lo_tile,
 
 __global__ void __launch_bounds__(SCT_THREADS, 1)
 affinity_score_tc_kernel(const __grid_constant__ CUtensorMap mapZ, const __grid_constant__ CUtensorMap mapR,
-                         const float* __restrict__ R, const float* __restrict__ xnorm, float* __restrict__ delta,
+                         const float* R, const float* xnorm, float* __restrict__ delta,
                          float* __restrict__ rnorm, etr_stats* stats, int Ttok, int E, int m, float sqD,
                          uint32_t idesc, long long wait_limit) {
   extern __shared__ uint8_t smem_raw[];
@@ -100,9 +100,10 @@ affinity_score_tc_kernel(const __grid_constant__ CUtensorMap mapZ, const __grid_
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(SCT_TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  grid_sync();
+  grid_wait();
   tc_fence_before();
   __syncthreads();
+  grid_release();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_slot;
   const uint32_t idesc_wide = (idesc & ~(0x3fu << 17)) | ((uint32_t)(2 * SCT_N >> 3) << 17);      // N = 128

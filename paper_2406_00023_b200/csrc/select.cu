@@ -55,7 +55,7 @@ __device__ inline int capacity_from_delta(const SelectParams& p, float delta_max
 // 17 us).
 template <int EPL>
 __global__ void __launch_bounds__(256)
-select_token_side_kernel(const float* __restrict__ delta, int32_t* __restrict__ topk_idx,
+select_token_side_kernel(const float* delta, int32_t* __restrict__ topk_idx,
                          uint32_t* __restrict__ keyT, etr_stats* stats, int32_t* __restrict__ skipped,
                          SelectParams p) {
   grid_sync();
@@ -194,7 +194,7 @@ __device__ __forceinline__ void pick_bin(const uint32_t* hist, uint32_t rem, int
 // of sums per pass, walking the bins from the top to the first one whose cumulated sum reaches what
 // is left of tq.  In the last pass a bin is a single key value q > 0, of which ceil(left / q) are needed.
 __global__ void __launch_bounds__(1024)
-select_threshold_limit_kernel(const uint32_t* __restrict__ keyT, int32_t* __restrict__ limit, int T,
+select_threshold_limit_kernel(const uint32_t* keyT, int32_t* __restrict__ limit, int T,
                               long long tq) {
   grid_sync();
   __shared__ uint32_t hist_cnt[256];
@@ -278,8 +278,8 @@ __device__ __forceinline__ void load_keys(const uint32_t* __restrict__ row, int 
 }
 
 __global__ void __launch_bounds__(1024)
-select_expert_side_kernel(uint32_t* __restrict__ keyT, const etr_stats* __restrict__ stats,
-                          const int32_t* __restrict__ limit, int32_t* __restrict__ counts,
+select_expert_side_kernel(uint32_t* __restrict__ keyT, const etr_stats* stats,
+                          const int32_t* limit, int32_t* __restrict__ counts,
                           int32_t* __restrict__ slot_token, float* __restrict__ gate, int T, int C_stride) {
   grid_sync();
   __shared__ uint32_t hist[256];
@@ -431,8 +431,8 @@ __device__ __forceinline__ uint32_t sel_peer_load(const uint32_t* local, uint32_
 
 template <int CL>
 __global__ void __launch_bounds__(1024, 2)
-select_expert_side_cluster_kernel(uint32_t* __restrict__ keyT, const etr_stats* __restrict__ stats,
-                                  const int32_t* __restrict__ limit, int32_t* __restrict__ counts,
+select_expert_side_cluster_kernel(uint32_t* __restrict__ keyT, const etr_stats* stats,
+                                  const int32_t* limit, int32_t* __restrict__ counts,
                                   int32_t* __restrict__ slot_token, float* __restrict__ gate, int T,
                                   int C_stride) {
   grid_sync();
@@ -616,7 +616,7 @@ select_expert_side_cluster_kernel(uint32_t* __restrict__ keyT, const etr_stats* 
 //          and 65536 tokens, cheaper than a launch for a scan of them), tok_row from the position matrix, final
 //          tok_ptr; the last block leaves the sums in stats
 __global__ void __launch_bounds__(256)
-csr_count_kernel(const int32_t* __restrict__ posT, int32_t* __restrict__ tok_ptr,
+csr_count_kernel(const int32_t* posT, int32_t* __restrict__ tok_ptr,
                  int32_t* __restrict__ block_total, etr_stats* stats, int T, int E) {
   grid_sync();
   __shared__ int wsum[8];
@@ -656,9 +656,9 @@ __device__ __forceinline__ int block_sum_256(int v, int* wsum) {
 }
 
 __global__ void __launch_bounds__(256)
-csr_fill_kernel(const int32_t* __restrict__ posT, const int32_t* __restrict__ block_total,
+csr_fill_kernel(const int32_t* posT, const int32_t* block_total,
                 int32_t* __restrict__ tok_ptr, int32_t* __restrict__ tok_row, etr_stats* stats, int T, int E,
-                int C_stride, int n_cand, const int32_t* __restrict__ skipped, int n_skipped_blocks) {
+                int C_stride, int n_cand, const int32_t* skipped, int n_skipped_blocks) {
   grid_sync();
   __shared__ int wsum[8];
   const int tid = threadIdx.x, b = blockIdx.x;
@@ -681,9 +681,13 @@ csr_fill_kernel(const int32_t* __restrict__ posT, const int32_t* __restrict__ bl
   const int t = b * 256 + tid;
   if (t >= T) return;
   int q = offset + tok_ptr[t + 1];
-  for (int i = 0; i < E; ++i) {
-    const int pos = posT[(size_t)i * T + t];
-    if (pos >= 0) tok_row[q++] = i * C_stride + pos;
+  for (int i0 = 0; i0 < E; i0 += 8) {                // eight loads in flight before the first store
+    int pos[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) pos[u] = i0 + u < E ? posT[(size_t)(i0 + u) * T + t] : -1;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (pos[u] >= 0) tok_row[q++] = (i0 + u) * C_stride + pos[u];
   }
   tok_ptr[t + 1] = q;
 }
@@ -696,7 +700,7 @@ csr_fill_kernel(const int32_t* __restrict__ posT, const int32_t* __restrict__ bl
 // NK: keys per lane, T <= 32 NK <= 512.
 template <int NK>
 __global__ void __launch_bounds__(1024)
-select_small_kernel(const float* __restrict__ delta, int32_t* __restrict__ topk_idx, etr_stats* stats,
+select_small_kernel(const float* delta, int32_t* __restrict__ topk_idx, etr_stats* stats,
                     int32_t* __restrict__ counts, int32_t* __restrict__ slot_token, float* __restrict__ gate,
                     int32_t* __restrict__ tok_ptr, int32_t* __restrict__ tok_row, SelectParams p, int n_cand) {
   grid_sync();

@@ -1,0 +1,48 @@
+"""The rules that overlapped launches rest on, checked in the kernels' source (a violation is a race or a mutual wait, which
+no test may provoke on a GPU): every kernel waits for its predecessor, reads its inputs through ordinary loads only, and
+lets its successor in only when its own tensor memory is allocated."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2406_00023_b200", "csrc")
+SOURCES = sorted(f for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh")))
+
+
+def text(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def kernels(src):
+    """(name, parameters, body) of every kernel."""
+    for m in re.finditer(r"__global__\s+void\s+(?:__launch_bounds__\([^)]*\)\s*)?(\w+)\s*\(([^{;]*)\)\s*\{", src):
+        depth, end = 1, m.end()
+        while depth:
+            depth += {"{": 1, "}": -1}.get(src[end], 0)
+            end += 1
+        yield m.group(1), m.group(2), src[m.end():end]
+
+
+@pytest.mark.parametrize("name", SOURCES)
+def test_overlapped_launches(name):
+    src = text(name)
+    assert "__ldg" not in src and "ld.global.nc" not in src
+    for kernel, params, body in kernels(src):
+        assert not re.search(r"const\s+\w+\s*\*\s*(const\s+)?__restrict__", params), kernel
+        if re.search(kernel + r"\s*<<<", src):
+            continue                                         # launched without overlap
+        if "tcgen05.alloc" not in body:
+            first = body.index("grid_sync();")
+            assert not re.search(r"\bp\.\w+\[|stats->|\w+\[", re.sub(r"__shared__[^;]*;", "", body[:first])), kernel
+            continue
+        order = [body.index(s) for s in ("tcgen05.alloc", "grid_wait();", "__syncthreads();", "grid_release();")]
+        assert order == sorted(order) and "grid_sync" not in body, kernel
+        if "tcgen05.dealloc.cta_group::2" in body:           # the pair leaves together
+            assert "cluster_sync_all();" in body[body.index("tcgen05.dealloc.cta_group::2"):], kernel
+
+
+def test_the_kernels_are_found():
+    names = [k for f in SOURCES for k, _, _ in kernels(text(f))]
+    assert len(names) >= 30 and "tc_grouped_gemm_swap_kernel" in names and "combine_kernel" in names
