@@ -74,6 +74,18 @@ __device__ __forceinline__ void f3_ld16(uint32_t taddr, uint32_t* r) {
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
+// v -> (hi, lo), both tf32 values (round to nearest, on the integer image: a cvt per value costs twice the time),
+// hi + lo = v up to 2^-23 |v|; the tensor core does not read the low 13 bits of lo.  Values that rounding would carry past
+// the largest finite one are cut; an infinity or NaN is hi (lo then holds nothing of use).  minus_zero is -0.0 in a register
+// that the compiler knows nothing about: the addition leaves every number as it is and makes any NaN the canonical one
+// (a payload in the bits that are cut would leave an infinity; a test and an OR instead took 5 % of a layer).
+__device__ __forceinline__ void f3_split(float v, float minus_zero, float& hi, float& lo) {
+  v += minus_zero;
+  uint32_t u = __float_as_uint(v);
+  if (fabsf(v) < __uint_as_float(0x7f7ff000u)) u += 0x1000u;
+  hi = __uint_as_float(u & 0xffffe000u);
+  lo = __uint_as_float(__float_as_uint(v - hi) + 0x1000u);
+}
 // sum[i] += hh[i] + xx[i].  Where an operand is infinite the cross terms hold inf * 0 or inf - inf; hi*hi alone
 // then has the value that fp32 products would give.
 __device__ __forceinline__ void f3_add16(float* sum, const uint32_t* hh, const uint32_t* xx) {
@@ -117,7 +129,8 @@ __device__ __forceinline__ bool f3_tile(const F3Params& p, const int* prefix, co
 // klim: rows of K that exist in this block (MN-major; what lies behind them is not an operand value).
 template <bool MN>
 __device__ __forceinline__ void f3_split_box(uint8_t* hi, uint8_t* lo, int klim, int lane) {
-  const float mz = opaque_minus_zero();
+  float mz;
+  asm volatile("mov.b32 %0, 0x80000000;" : "=f"(mz));
   float4 v[8];
   const int q = (lane >> 3) * 2 + ((lane >> 2) & 1), c0 = lane & 3;          // MN: quad of rows, chunk of K of the first block
 #pragma unroll
@@ -145,7 +158,7 @@ __device__ __forceinline__ void f3_split_box(uint8_t* hi, uint8_t* lo, int klim,
       x = make_float4(at(b[0]), at(b[1]), at(b[2]), at(b[3]));
     }
     float4 h, l;
-    tf32_split(x.x, mz, h.x, l.x); tf32_split(x.y, mz, h.y, l.y); tf32_split(x.z, mz, h.z, l.z); tf32_split(x.w, mz, h.w, l.w);
+    f3_split(x.x, mz, h.x, l.x); f3_split(x.y, mz, h.y, l.y); f3_split(x.z, mz, h.z, l.z); f3_split(x.w, mz, h.w, l.w);
     *reinterpret_cast<float4*>(hi + off) = h;
     *reinterpret_cast<float4*>(lo + off) = l;
   }

@@ -2,12 +2,10 @@
 // 128 tokens x up to 64 experts per pass, the product <z_t, R_i> as a tcgen05 MMA of kind tf32.
 //
 // The router decides on these numbers, so they keep fp32 accuracy: every fp32 operand v is split in
-// shared memory into hi = v rounded to tf32 and lo = (v - hi) rounded to tf32, and the product is
-// accumulated as hi*hi + hi*lo + lo*hi in fp32 accumulators in tensor memory.  The products of two tf32
-// values are exact in fp32; what is dropped is lo*lo (at most 2^-22 of a product) and the rounding of lo (2^-23).
-// (With both parts cut instead of rounded every affinity came out short, by 4.4e-7 at m = 32 and 9e-7 at 256;
-// rounded 0.9e-7 and 5.6e-7, which is the accumulators' own cutting; 46 -> 48 us for 65536 tokens, E 64, m 256.)
-// Both operand splits are made by a group
+// shared memory into hi = v with its low 13 mantissa bits cleared (exactly a tf32 value) and
+// lo = (v - hi) cut the same way, and the product is accumulated as hi*hi + hi*lo + lo*hi in fp32
+// accumulators in tensor memory.  The products of two tf32 values are exact in fp32; what is dropped is
+// lo*lo (2^-22 of a product) and the second cut of lo (2^-24).  Both operand splits are made by a group
 // of converter warps between the TMA load and the MMA, in place, so the caller's Z and R stay plain
 // fp32 and no scratch memory is needed.
 //
@@ -48,20 +46,23 @@ __device__ __forceinline__ void tc_mma_tf32(uint32_t d_tmem, uint64_t adesc, uin
       "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
+// v -> (hi, lo), both exactly tf32 values, v = hi + lo up to 2^-24 |v|
+__device__ __forceinline__ void split_tf32(float v, float& hi, float& lo) {
+  hi = __uint_as_float(__float_as_uint(v) & 0xffffe000u);
+  lo = __uint_as_float(__float_as_uint(v - hi) & 0xffffe000u);
+}
 // The N 16-byte chunks per thread of a tile (chunk ct, ct + 128, ...: consecutive threads, consecutive chunks),
 // split in place.  All loads are issued before the first store: the two tiles could alias as far as the
 // compiler knows, and a load behind a store would wait for it.
 template <int N>
 __device__ __forceinline__ void split_chunks(uint8_t* hi_tile, uint8_t* lo_tile, int ct) {
-  const float mz = opaque_minus_zero();
   float4 v[N];
 #pragma unroll
   for (int j = 0; j < N; ++j) v[j] = *reinterpret_cast<const float4*>(hi_tile + 16 * (ct + 128 * j));
 #pragma unroll
   for (int j = 0; j < N; ++j) {
     float4 h, l;
-    tf32_split(v[j].x, mz, h.x, l.x); tf32_split(v[j].y, mz, h.y, l.y);
-    tf32_split(v[j].z, mz, h.z, l.z); tf32_split(v[j].w, mz, h.w, l.w);
+    split_tf32(v[j].x, h.x, l.x); split_tf32(v[j].y, h.y, l.y); split_tf32(v[j].z, h.z, l.z); split_tf32(v[j].w, h.w, l.w);
     *reinterpret_cast<float4*>(hi_tile + 16 * (ct + 128 * j)) = h;
     *reinterpret_cast<float4*>(lo_tile + 16 * (ct + 128 * j)) = l;
   }

@@ -52,25 +52,6 @@ __device__ __forceinline__ bool elect_one() {
   return p != 0;
 }
 
-// -0.0 in a register that the compiler knows nothing about.
-__device__ __forceinline__ float opaque_minus_zero() {
-  float z;
-  asm volatile("mov.b32 %0, 0x80000000;" : "=f"(z));
-  return z;
-}
-// v -> (hi, lo), both tf32 values (round to nearest, on the integer image: a cvt per value costs twice the time),
-// hi + lo = v up to 2^-23 |v|; the tensor core does not read the low 13 bits of lo.  Values that rounding would carry past
-// the largest finite one are cut; an infinity or NaN is hi (lo then holds nothing of use).  Adding minus_zero
-// (opaque_minus_zero) leaves every number as it is and makes any NaN the canonical one: a payload in the bits that are cut
-// would leave an infinity (a test and an OR instead took 5 % of an fp32 layer).
-__device__ __forceinline__ void tf32_split(float v, float minus_zero, float& hi, float& lo) {
-  v += minus_zero;
-  uint32_t u = __float_as_uint(v);
-  if (fabsf(v) < __uint_as_float(0x7f7ff000u)) u += 0x1000u;
-  hi = __uint_as_float(u & 0xffffe000u);
-  lo = __uint_as_float(__float_as_uint(v - hi) + 0x1000u);
-}
-
 // Shared-memory matrix descriptor, 128-byte swizzle, tile base 1024-byte aligned.
 __device__ __forceinline__ uint64_t make_smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
   uint64_t d = (uint64_t)((addr & 0x3FFFFu) >> 4);

@@ -7,14 +7,10 @@ a product at most, and a chain of eight MMAs drops at most eight last bits of it
 of it with the growth of the running sum's roundings over the K blocks (2^-24 sqrt(K / 64) at K <= 2000)."""
 import math
 
-import numpy as np
 import pytest
 import torch
 
-from gen import workloads as gw
-from oracle import binding as ob
 from paper_2406_00023_b200 import etr
-from tests import harness as hz
 
 pytestmark = pytest.mark.gpu
 TOL = 1e-6
@@ -117,40 +113,3 @@ def test_every_nan_stays_a_nan(bits):
     assert G.equal((row == 3).expand(128, 64)) and U.equal((row == 3) | (col == 5))
     assert dG.equal((row == 3) | (row == 11) | (col == 5))
     assert bool(dW[2].isnan()[0, 2].all())                   # its row of dO, transposed on the way
-
-
-@pytest.mark.parametrize("d,D,E", [(128, 4, 4), (256, 4, 8), (1024, 8, 16), (4096, 16, 64)])
-@pytest.mark.parametrize("positive", [False, True])
-def test_affinities_against_64_bits(d, D, E, positive):
-    """The affinities that an fp32 layer's gates are, relative 2-norm: the rounding of lo and the dropped lo*lo, of either sign and
-    2^-24 of a product or less on average (together 1.5e-7 with the quotient's rounding), and m / 16 accumulations in a row that cut
-    2^-24 of the sum on average, all in one direction (positive products make every one of them count)."""
-    T, m = 777, d // D
-    g = torch.Generator(device="cuda").manual_seed(d)
-    X, R = (torch.rand(*s, generator=g, device="cuda") - (0.0 if positive else 0.5) for s in ((T, d), (E, m)))
-    cfg = etr.make_config(T=T, d=d, D=D, E=E, k=2, h=64, capacity=16, dtype=etr.F32, mode=etr.MODE_TCR)
-    b = etr.LayerBuffers(cfg)
-    b.stats.zero_()
-    etr.affinity(cfg, X, R, b.delta, b.Z, b.xnorm, b.rnorm, b.c.stats)
-    x, r = X.double(), R.double()
-    ref = math.sqrt(D) * (x.view(T, m, D).mean(2) @ r.T) / (x.norm(dim=1)[:, None] * r.norm(dim=1)[None, :])
-    assert rel(b.delta, ref) <= 1.5e-7 + m / 16 * 2.0 ** -24
-
-
-def test_layer_of_short_contractions_against_64_bits():
-    """Forward and backward of a layer whose contractions have 128 to 512 values: no output further from the oracle in 64
-    bits than the CUDA-core kernels left it (relative 2-norm 7e-7)."""
-    w = gw.WORKLOADS["tiny"]
-    inp = gw.make_inputs(w)
-    o = ob.Oracle("f64")
-    x = {k: v.astype(np.float64) for k, v in inp.items() if isinstance(v, np.ndarray)}
-    fw = o.forward(x["X"], x["R"], x["W1g"], x["W1u"], x["W2"], D=w.D, k=w.k, capacity=w.capacity, mode=ob.MODE_TCR)
-    bw = o.backward(fw, x["X"], x["R"], x["W1g"], x["W1u"], x["W2"], x["dY"])
-    cfg, dev = hz.make_cfg(w, mode=ob.MODE_TCR), hz.upload(w, inp)
-    buf = etr.LayerBuffers(cfg)
-    out = [torch.empty_like(t) for t in (dev.X, dev.X, dev.R, dev.W1g, dev.W1u, dev.W2)]
-    etr.layer_forward(cfg, dev.X, dev.R, dev.W1g, dev.W1u, dev.W2, buf, out[0])
-    etr.layer_backward(cfg, dev.X, dev.R, dev.W1g, dev.W1u, dev.W2, dev.dY, buf, *out[1:])
-    assert buf.read_stats().error_word == 0
-    for got, ref in zip(out, (fw.Y, bw.dX, bw.dR, bw.dW1g, bw.dW1u, bw.dW2)):
-        assert rel(got, torch.from_numpy(np.asarray(ref)).cuda()) <= 7e-7
