@@ -5,10 +5,14 @@
 //
 // The tensor core's fp32 accumulator drops the bits that do not fit instead of rounding them, an error that
 // always points towards zero and would add up over a long contraction.  So a chain of MMAs is never longer
-// than one K block (32 values: four MMAs): hi*hi and the cross terms of such a chunk go to accumulators of
-// their own in tensor memory, and the epilogue warps add each chunk to running sums in registers with rounded
-// fp32 additions while the next one is multiplied.  (Chunks of two K blocks: contractions off by 2.0e-7 instead of
-// 1.4e-7, an fp32 step of width 256 by 1.0e-6 where fp32 FMAs are off by 8.3e-7.)
+// than one K block (32 values: four MMAs): hi*hi and the cross terms of such a chain go to accumulators of
+// their own in tensor memory, and the epilogue warps add each chain to running sums in registers with rounded
+// fp32 additions while the next one is multiplied.  Even so a contraction of positive products comes out 1.2e-7 short,
+// where fp32 FMAs are off by 1.2e-7 at 64 values and 4.3e-7 at 1024 (products of either sign: 1.4e-7 against 1.4e-7 to
+// 5.7e-7), and in a layer of short contractions these add up with what the scores are short by (weight gradients of
+// T 512, d 256, h 512: 8.0e-7, with the CUDA-core GEMMs 7.0e-7).  Contractions over at most 384 columns or 256 rows
+// therefore end a chain after two MMAs: 0.6e-7 short, that layer 7.1e-7, 158 -> 161 us.  (For all of them that would be
+// 651 -> 739 us at T 1531, d 768, h 1000; four MMAs are already below the FMAs there.  Chains of eight: 2.0e-7.)
 //
 // One persistent kernel serves the six contractions.  Roles in a CTA of 640 threads:
 //   warp 0       TMA: a K block arrives as plain fp32 in the place of its hi tiles
@@ -39,7 +43,8 @@ constexpr int F3_THREADS = 640;
 // registers per thread by role; 640 threads are launched with 96 each (61440), the split takes 60416
 constexpr int F3_REGS_LAUNCH = 96, F3_REGS_IO = 40, F3_REGS_CONV = 88, F3_REGS_EPI = 128;
 static_assert(128 * F3_REGS_IO + 256 * F3_REGS_CONV + 256 * F3_REGS_EPI <= F3_THREADS * F3_REGS_LAUNCH, "register split");
-constexpr int F3_CHUNK = 1;                      // K blocks that one chain of MMAs adds up
+// Contractions of at most so many values end a chain of MMAs after 16 values instead of 32.
+constexpr int F3_SHORT_WIDTH = 384, F3_SHORT_ROWS = 256;
 constexpr int F3_SCRATCH = 32 * 80;              // per epilogue warp: 32 rows of 64 bytes, 16 bytes of pad each
 
 enum { F3_STORE = 0, F3_SWIGLU = 1, F3_DSWIGLU = 2 };
@@ -86,21 +91,48 @@ __device__ __forceinline__ void f3_split(float v, float minus_zero, float& hi, f
   hi = __uint_as_float(u & 0xffffe000u);
   lo = __uint_as_float(__float_as_uint(v - hi) + 0x1000u);
 }
-// sum[i] += hh[i] + xx[i].  Where an operand is infinite the cross terms hold inf * 0 or inf - inf; hi*hi alone
-// then has the value that fp32 products would give.
-__device__ __forceinline__ void f3_add16(float* sum, const uint32_t* hh, const uint32_t* xx) {
-  float odd = 0.f;
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 f3_pair(uint32_t x, uint32_t y) { return (f32x2)y << 32 | x; }
+__device__ __forceinline__ f32x2 f3_add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 f3_zero_times(f32x2 a, f32x2 c) {      // 0 * a + c: c, or NaN where a is infinite or NaN
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(0ull), "l"(c));
+  return d;
+}
+// x, or the largest finite value of its sign where x is infinite or NaN.
+__device__ __forceinline__ uint32_t f3_finite(uint32_t x) {
+  float d;
+  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(d) : "f"(__uint_as_float(x)), "f"(3.402823466e38f));
+  return __float_as_uint(d);
+}
+// sum[i] += hh[i] + xx[i].  Where an operand is infinite the cross terms hold inf * 0 or inf - inf; hi*hi alone then has the
+// value that fp32 products would give, an infinity or NaN, which no finite number added to it changes.  Chains of four MMAs:
+// one test for the sixteen columns.  Of two, where the epilogue is the longest stage: no test, whose latency counts twice
+// as often, but every cross term made finite (fp32 step of T 1531: 880 us with the test, 739 without).
+template <int CHAIN>
+__device__ __forceinline__ void f3_add16(f32x2* sum, const uint32_t* hh, const uint32_t* xx) {
+  bool all_finite = false;
+  if (CHAIN == 4) {
+    f32x2 odd[4];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) odd = fmaf(__uint_as_float(xx[i]), 0.f, odd);
-  if (odd == odd) {
+    for (int i = 0; i < 4; ++i)
+      odd[i] = f3_zero_times(f3_pair(xx[4 * i], xx[4 * i + 1]), f3_zero_times(f3_pair(xx[4 * i + 2], xx[4 * i + 3]), 0ull));
+    const f32x2 o2 = f3_add2(f3_add2(odd[0], odd[1]), f3_add2(odd[2], odd[3]));
+    const float o = __uint_as_float((uint32_t)o2) + __uint_as_float((uint32_t)(o2 >> 32));
+    all_finite = o == o;
+  }
+  if (CHAIN == 4 && all_finite) {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) sum[i] += __uint_as_float(hh[i]) + __uint_as_float(xx[i]);
+    for (int i = 0; i < 8; ++i)
+      sum[i] = f3_add2(sum[i], f3_add2(f3_pair(hh[2 * i], hh[2 * i + 1]), f3_pair(xx[2 * i], xx[2 * i + 1])));
   } else {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const float h = __uint_as_float(hh[i]), x = __uint_as_float(xx[i]);
-      sum[i] += fabsf(x) < INFINITY ? h + x : h;
-    }
+    for (int i = 0; i < 8; ++i)
+      sum[i] = f3_add2(sum[i], f3_add2(f3_pair(hh[2 * i], hh[2 * i + 1]), f3_pair(f3_finite(xx[2 * i]), f3_finite(xx[2 * i + 1]))));
   }
 }
 
@@ -194,7 +226,7 @@ __device__ __forceinline__ void f3_store16(uint8_t* scratch, int lane, int nvali
   __syncwarp();
 }
 
-template <int EPI, bool A_MN, bool B_MN, int BN>
+template <int EPI, bool A_MN, bool B_MN, int BN, int CHAIN>
 __global__ void __launch_bounds__(F3_THREADS, 1)
 tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
                    const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
@@ -203,11 +235,12 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
   constexpr int COLS = EPI == F3_SWIGLU ? BN / 2 : BN;               // output columns of a tile
   constexpr uint32_t A_BYTES = F3_BM * 128, B_BYTES = BN * 128;      // one of hi, lo
   constexpr uint32_t STAGE = 2 * A_BYTES + 2 * B_BYTES;
-  constexpr uint32_t TMEM_COLS = 4 * BN;                             // two accumulator stages of hi*hi and cross terms
+  constexpr int F3_ACC = 256 / BN;                                   // accumulator stages of hi*hi and cross terms
+  constexpr uint32_t TMEM_COLS = F3_ACC * 2 * BN;
   constexpr int GW = BN / 4;                                         // columns of a thread's two groups
 
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t bars[3 * F3_STAGES + 4];
+  __shared__ __align__(8) uint64_t bars[3 * F3_STAGES + 2 * F3_ACC];
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag_s;
   __shared__ int tile_prefix[257];
@@ -220,15 +253,15 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
   const uint32_t full_bar = smem_u32(&bars[0]);                      // [STAGES] the TMA boxes have landed
   const uint32_t conv_bar = smem_u32(&bars[F3_STAGES]);              // [STAGES] both operands are split
   const uint32_t empty_bar = smem_u32(&bars[2 * F3_STAGES]);         // [STAGES] the MMAs have read the stage
-  const uint32_t tfull_bar = smem_u32(&bars[3 * F3_STAGES]);         // [2] a chunk's accumulators are complete
-  const uint32_t tempty_bar = smem_u32(&bars[3 * F3_STAGES + 2]);    // [2] they have been read
+  const uint32_t tfull_bar = smem_u32(&bars[3 * F3_STAGES]);         // [ACC] a chain's accumulators are complete
+  const uint32_t tempty_bar = smem_u32(&bars[3 * F3_STAGES + F3_ACC]);      // [ACC] they have been read
 
   if (tid == 0) {
     abort_flag_s = 0;
     for (int s = 0; s < F3_STAGES; ++s) {
       mbar_init(full_bar + 8 * s, 1); mbar_init(conv_bar + 8 * s, 4); mbar_init(empty_bar + 8 * s, 1);
     }
-    for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar + 8 * a, 1); mbar_init(tempty_bar + 8 * a, 8); }
+    for (int a = 0; a < F3_ACC; ++a) { mbar_init(tfull_bar + 8 * a, 1); mbar_init(tempty_bar + 8 * a, 8); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -284,30 +317,33 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
       bool ok = true;
       for (int tile = blockIdx.x; ok && f3_tile(p, tile_prefix, s_counts, tile, e_cur, COLS, t); tile += gridDim.x) {
         for (int kb = 0; kb < t.kblocks; ++kb) {
-          const bool first = kb % F3_CHUNK == 0, last = kb % F3_CHUNK == F3_CHUNK - 1 || kb + 1 == t.kblocks;
-          ok = !first || __all_sync(0xffffffffu, mbar_wait(tempty_bar + 8 * acc, acc_phase ^ 1u, abort_flag, p.wait_limit));
-          ok = ok && __all_sync(0xffffffffu, mbar_wait(conv_bar + 8 * stage, phase, abort_flag, p.wait_limit));
-          if (!ok) break;
-          tc_fence_after();
-          if (elect_one()) {
-            const uint32_t a_hi = tiles_base + stage * STAGE, a_lo = a_hi + A_BYTES, b_hi = a_hi + 2 * A_BYTES;
-            const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 2 * BN);
-            // hi and lo of B lie one behind the other: A_hi x [B_hi; B_lo]^T is one MMA of 2 BN columns (hi*hi in the
-            // first BN, hi*lo in the others), and A_lo x B_hi^T adds lo*hi to the latter
+          ok = __all_sync(0xffffffffu, mbar_wait(conv_bar + 8 * stage, phase, abort_flag, p.wait_limit));
+          const uint32_t a_hi = tiles_base + stage * STAGE, a_lo = a_hi + A_BYTES, b_hi = a_hi + 2 * A_BYTES;
 #pragma unroll
-            for (int kk = 0; kk < F3_BK / 8; ++kk)
-              f3_mma(d_tmem, make_smem_desc(a_hi + 32 * kk, 16u, 1024u), make_smem_desc(b_hi + 32 * kk, 16u, 1024u),
-                     idesc_wide, !first || kk > 0 ? 1u : 0u);
+          for (int k0 = 0; k0 < F3_BK / 8; k0 += CHAIN) {
+            ok = ok && __all_sync(0xffffffffu, mbar_wait(tempty_bar + 8 * acc, acc_phase ^ 1u, abort_flag, p.wait_limit));
+            if (!ok) break;
+            tc_fence_after();
+            if (elect_one()) {
+              const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 2 * BN);
+              // hi and lo of B lie one behind the other: A_hi x [B_hi; B_lo]^T is one MMA of 2 BN columns (hi*hi in the
+              // first BN, hi*lo in the others), and A_lo x B_hi^T adds lo*hi to the latter
 #pragma unroll
-            for (int kk = 0; kk < F3_BK / 8; ++kk)
-              f3_mma(d_tmem + BN, make_smem_desc(a_lo + 32 * kk, 16u, 1024u), make_smem_desc(b_hi + 32 * kk, 16u, 1024u),
-                     idesc, 1u);
-            tc_commit(empty_bar + 8 * stage);
-            if (last) tc_commit(tfull_bar + 8 * acc);
+              for (int kk = k0; kk < k0 + CHAIN; ++kk)
+                f3_mma(d_tmem, make_smem_desc(a_hi + 32 * kk, 16u, 1024u), make_smem_desc(b_hi + 32 * kk, 16u, 1024u),
+                       idesc_wide, kk > k0 ? 1u : 0u);
+#pragma unroll
+              for (int kk = k0; kk < k0 + CHAIN; ++kk)
+                f3_mma(d_tmem + BN, make_smem_desc(a_lo + 32 * kk, 16u, 1024u), make_smem_desc(b_hi + 32 * kk, 16u, 1024u),
+                       idesc, 1u);
+              if (k0 + CHAIN == F3_BK / 8) tc_commit(empty_bar + 8 * stage);
+              tc_commit(tfull_bar + 8 * acc);
+            }
+            __syncwarp();
+            if (++acc == F3_ACC) { acc = 0; acc_phase ^= 1u; }
           }
-          __syncwarp();
+          if (!ok) break;
           if (++stage == F3_STAGES) { stage = 0; phase ^= 1u; }
-          if (last && ++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
       }
     }
@@ -355,36 +391,38 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
     F3Tile t;
     bool ok = true;
     for (int tile = blockIdx.x; ok && f3_tile(p, tile_prefix, s_counts, tile, e_cur, COLS, t); tile += gridDim.x) {
-      float sum[2][GW];
+      f32x2 run[GW];                                                 // 2 GW running sums
 #pragma unroll
-      for (int g = 0; g < 2; ++g)
-#pragma unroll
-        for (int i = 0; i < GW; ++i) sum[g][i] = 0.f;
-      for (int kb = 0; kb < t.kblocks; kb += F3_CHUNK) {
+      for (int i = 0; i < GW; ++i) run[i] = 0ull;
+      // first column in the tile of the j-th sixteen sums
+      auto col = [&](int j) { return (uint32_t)(16 * j < GW ? g0 + 16 * j : g1 + 16 * j - GW); };
+      for (int chain = 0; chain < t.kblocks * (F3_BK / 8 / CHAIN); ++chain) {
         ok = __all_sync(0xffffffffu, mbar_wait(tfull_bar + 8 * acc, acc_phase, abort_flag, p.wait_limit));
         if (!ok) break;
         tc_fence_after();
         const uint32_t taddr = tmem_base + (uint32_t)(acc * 2 * BN) + ((uint32_t)(32 * q) << 16);
 #pragma unroll
-        for (int g = 0; g < 2; ++g) {
-#pragma unroll
-          for (int c = 0; c < GW; c += 16) {
-            uint32_t hh[16], xx[16];
-            const uint32_t col = (uint32_t)((g ? g1 : g0) + c);
-            f3_ld16(taddr + col, hh);
-            f3_ld16(taddr + BN + col, xx);
-            tc_wait_ld();
-            f3_add16(&sum[g][c], hh, xx);
-          }
+        for (int j = 0; j < GW / 8; ++j) {
+          uint32_t hh[16], xx[16];
+          f3_ld16(taddr + col(j), hh);
+          f3_ld16(taddr + BN + col(j), xx);
+          tc_wait_ld();
+          f3_add16<CHAIN>(run + 8 * j, hh, xx);
         }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(tempty_bar + 8 * acc);
-        if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+        if (++acc == F3_ACC) { acc = 0; acc_phase ^= 1u; }
       }
       if (!ok) break;
       const int row0 = t.m0 + 32 * q, nvalid = min(32, t.m_lim - row0);
       const long long wb = (long long)t.e * p.out_bs + (long long)row0 * p.ld_out;
+      float sum[2][GW];
+#pragma unroll
+      for (int i = 0; i < GW; ++i) {
+        sum[i / (GW / 2)][2 * i % GW] = __uint_as_float((uint32_t)run[i]);
+        sum[i / (GW / 2)][2 * i % GW + 1] = __uint_as_float((uint32_t)(run[i] >> 32));
+      }
       __syncwarp();
       if (EPI == F3_SWIGLU) {
 #pragma unroll
@@ -465,11 +503,11 @@ static etr_status f3_map(CUtensorMap* m, const void* base, int cols, int rows, i
 // A row-major [E, rows, cols] operand.  K-major: the columns are the contraction; MN-major: the rows are.
 struct F3Operand { const void* ptr; int cols, rows; };
 
-template <int EPI, bool A_MN, bool B_MN, int BN>
+template <int EPI, bool A_MN, bool B_MN, int BN, int CHAIN>
 static etr_status f3_launch_bn(const char* name, const F3Operand* A, const F3Operand* B, const F3Params& p,
                                int max_tiles, cudaStream_t st) {
   constexpr size_t smem = (size_t)F3Ring<BN>::STAGES * (2 * F3_BM + 2 * BN) * 128 + 1024 + 8 * F3_SCRATCH;
-  auto k = tf32x3_gemm_kernel<EPI, A_MN, B_MN, BN>;
+  auto k = tf32x3_gemm_kernel<EPI, A_MN, B_MN, BN, CHAIN>;
   static std::atomic<unsigned long long> attr_done{0};      // one bit per device
   if (!ensure_dyn_smem(k, smem, attr_done)) return ETR_ERR_CUDA;
   uint32_t idesc = 0;
@@ -489,14 +527,19 @@ static etr_status f3_launch_bn(const char* name, const F3Operand* A, const F3Ope
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }
+// k_max: the longest contraction that the launch can hold.
 template <int EPI, bool A_MN, bool B_MN>
 static etr_status f3_launch(const char* name, const F3Operand (&A)[2], const F3Operand (&B)[2], const F3Params& p,
-                            int tiles_m, cudaStream_t st) {
+                            int tiles_m, int k_max, cudaStream_t st) {
   // 128-column tiles unless they leave SMs without one
   constexpr int C128 = EPI == F3_SWIGLU ? 64 : 128, C64 = C128 / 2;
-  const int t128 = tiles_m * ceil_div(p.N, C128);
-  if (t128 >= current_sm_count()) return f3_launch_bn<EPI, A_MN, B_MN, 128>(name, A, B, p, t128, st);
-  return f3_launch_bn<EPI, A_MN, B_MN, 64>(name, A, B, p, tiles_m * ceil_div(p.N, C64), st);
+  const int t128 = tiles_m * ceil_div(p.N, C128), t64 = tiles_m * ceil_div(p.N, C64);
+  const bool wide = t128 >= current_sm_count();
+  if (k_max <= (p.dyn_m ? F3_SHORT_WIDTH : F3_SHORT_ROWS))
+    return wide ? f3_launch_bn<EPI, A_MN, B_MN, 128, 2>(name, A, B, p, t128, st)
+                : f3_launch_bn<EPI, A_MN, B_MN, 64, 2>(name, A, B, p, t64, st);
+  return wide ? f3_launch_bn<EPI, A_MN, B_MN, 128, 4>(name, A, B, p, t128, st)
+              : f3_launch_bn<EPI, A_MN, B_MN, 64, 4>(name, A, B, p, t64, st);
 }
 
 static F3Params f3_params(const etr_config* c, const etr_route* rt, etr_stats* stats) {
@@ -516,12 +559,12 @@ etr_status tf32x3_ffn_forward(const etr_config* c, const etr_route* rt, const vo
     const F3Operand A[2] = {{Xp, d, Cs}, {}}, B[2] = {{W1g, d, h}, {W1u, d, h}};
     p.M = Cs; p.N = h; p.K = d; p.dyn_m = 1;
     p.out0 = (float*)G; p.out1 = (float*)U; p.out2 = (float*)H; p.out_bs = lhx; p.ld_out = h;
-    ETR_TRY((f3_launch<F3_SWIGLU, false, false>("tf32x3_gemm_swiglu", A, B, p, mt, st)));
+    ETR_TRY((f3_launch<F3_SWIGLU, false, false>("tf32x3_gemm_swiglu", A, B, p, mt, d, st)));
   }
   F3Params p = f3_params(c, rt, stats);      // O = H W2^T
   const F3Operand A[2] = {{H, h, Cs}, {}}, B[2] = {{W2, h, d}, {}};
   p.M = Cs; p.N = d; p.K = h; p.dyn_m = 1; p.out0 = (float*)O; p.out_bs = ldx; p.ld_out = d;
-  return f3_launch<F3_STORE, false, false>("tf32x3_gemm_down", A, B, p, mt, st);
+  return f3_launch<F3_STORE, false, false>("tf32x3_gemm_down", A, B, p, mt, h, st);
 }
 
 etr_status tf32x3_ffn_backward(const etr_config* c, const etr_route* rt, const void* dO, const void* Xp,
@@ -536,25 +579,25 @@ etr_status tf32x3_ffn_backward(const etr_config* c, const etr_route* rt, const v
     p.M = Cs; p.N = h; p.K = d; p.dyn_m = 1;
     p.out0 = (float*)dG; p.out1 = (float*)dU; p.in0 = (const float*)G; p.in1 = (const float*)U;
     p.out_bs = lhx; p.ld_out = h;
-    ETR_TRY((f3_launch<F3_DSWIGLU, false, true>("tf32x3_gemm_dswiglu", A, B, p, mt, st)));
+    ETR_TRY((f3_launch<F3_DSWIGLU, false, true>("tf32x3_gemm_dswiglu", A, B, p, mt, d, st)));
   }
   {  // dXp = dG W1g + dU W1u
     F3Params p = f3_params(c, rt, stats);
     const F3Operand A[2] = {{dG, h, Cs}, {dU, h, Cs}}, B[2] = {{W1g, d, h}, {W1u, d, h}};
     p.two_k = 1; p.M = Cs; p.N = d; p.K = h; p.dyn_m = 1; p.out0 = (float*)dXp; p.out_bs = ldx; p.ld_out = d;
-    ETR_TRY((f3_launch<F3_STORE, false, true>("tf32x3_gemm_dxp", A, B, p, mt, st)));
+    ETR_TRY((f3_launch<F3_STORE, false, true>("tf32x3_gemm_dxp", A, B, p, mt, 2 * h, st)));
   }
   {  // dW2 = dO^T H over the expert's rows
     F3Params p = f3_params(c, rt, stats);
     const F3Operand A[2] = {{dO, d, Cs}, {}}, B[2] = {{H, h, Cs}, {}};
     p.M = d; p.N = h; p.out0 = (float*)dW2; p.out_bs = w; p.ld_out = h;
-    ETR_TRY((f3_launch<F3_STORE, true, true>("tf32x3_gemm_dw2", A, B, p, E * ceil_div(d, F3_BM), st)));
+    ETR_TRY((f3_launch<F3_STORE, true, true>("tf32x3_gemm_dw2", A, B, p, E * ceil_div(d, F3_BM), c->capacity, st)));
   }
   for (int which = 0; which < 2; ++which) {  // dW1g = dG^T Xp, dW1u = dU^T Xp
     F3Params p = f3_params(c, rt, stats);
     const F3Operand A[2] = {{which ? dU : dG, h, Cs}, {}}, B[2] = {{Xp, d, Cs}, {}};
     p.M = h; p.N = d; p.out0 = (float*)(which ? dW1u : dW1g); p.out_bs = w; p.ld_out = d;
-    ETR_TRY((f3_launch<F3_STORE, true, true>("tf32x3_gemm_dw1", A, B, p, E * ceil_div(h, F3_BM), st)));
+    ETR_TRY((f3_launch<F3_STORE, true, true>("tf32x3_gemm_dw1", A, B, p, E * ceil_div(h, F3_BM), c->capacity, st)));
   }
   return ETR_OK;
 }
