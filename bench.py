@@ -38,11 +38,11 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu captures summarised
 # under profiles/ (absent: not captured for the current version of that kernel).
 NCU_TRAFFIC_BYTES = {}
-# tc_grouped_gemm_pair_kernel and its wide form: measured on the mid workload, all 7 launches of one step
-# (profiles/tc_grouped_gemm_pair_kernels_mid_ncu_full.md): 3674.3 MB of DRAM traffic against 3799.7 MB
-# of algorithmic bytes (part of the output is still in L2 when a kernel ends).  The large workload is
-# too big for a multi-pass capture, so its traffic is this ratio times its own algorithmic bytes.
-TC_GEMM_DRAM_OVER_ALGORITHMIC = 3674.3 / 3799.7
+# The grouped GEMMs as AUTO launches them at the mid workload (d = 2048), all 7 launches of one step
+# (profiles/tc_grouped_gemm_mid_ncu.md): 3636.2 MB of DRAM traffic against 3799.7 MB of algorithmic bytes
+# (part of the output is still in L2 when a kernel ends).  The large workload is too big for a
+# multi-pass capture, so its traffic is this ratio times its own algorithmic bytes.
+TC_GEMM_DRAM_OVER_ALGORITHMIC = 3636.2 / 3799.7
 
 
 def tc_gemm_algorithmic_bytes(w, rows_padded):
@@ -554,10 +554,11 @@ def main():
     g = gemm_summary(w, kernels, rows)
     roofline = None
     if g and g["share_of_step"] >= 0.5:
-        # The six tcgen05 contractions run on one persistent grouped-GEMM design in two tile forms
-        # (--gemm can force one); the roofline entry covers all their launches.
-        pair = args.gemm == "auto"          # the ncu traffic ratio was taken with the library's own choice
-        kname = {"auto": "tc_grouped_gemm_pair_kernel + tc_grouped_gemm_swap_kernel (chosen per contraction)",
+        # The six tcgen05 contractions run on one persistent grouped-GEMM design in several tile forms
+        # (--gemm can force one); the roofline entry covers all their launches.  The ncu traffic ratio was
+        # taken with the library's own choice at d = 2048; narrower layers take other forms.
+        pair = args.gemm == "auto" and w.d >= 2048
+        kname = {"auto": "tc_grouped_gemm_*_kernel (form chosen per contraction)",
                  "tcgen05_2cta": "tc_grouped_gemm_pair_kernel", "tcgen05_2cta_wide": "tc_grouped_gemm_pair_wide_kernel",
                  "tcgen05": "tc_grouped_gemm_kernel"}.get(args.gemm, "tc_grouped_gemm")
         roofline = {"kernel": kname, "launches_per_step": g["launches_per_step"], "bound": "tensor",

@@ -1844,7 +1844,10 @@ static int swap_tok_box(const etr_config* c) {
 //     rows (E 16, d 1024, h 2816; 2.2 rounds).  (Tiles of 128 tokens there: 64 and 109.)
 //   the fused epilogues are longer here (an exchange, a transposed read), so they need a longer contraction:
 //     SwiGLU from K = 2048 (365 -> 348 at E 128, d 2048, h 768; 97 -> 105 at d 1024), its derivative from
-//     K = 4096 (702 -> 668 at d 4096; 183 -> 219 at d 2048).
+//     K = 4096 (702 -> 668 at d 4096; 183 -> 219 at d 2048).  Between the measured lines (E 32, h 1408): SwiGLU at d 1536
+//     222 -> 228 with 1024 rows, 119 -> 121 with 512, 213 -> 203 with 769 of 1280, 113 -> 103 with 300 of 1024;
+//     derivative at d 3072 278 -> 281, 158 -> 162, 269 -> 236, 152 -> 130.  So at the line the two forms are even on full
+//     buffers, and rows in use well below the capacity, which the host does not know, favour the exchanged form.
 static bool use_swap(const etr_config* c, int epi) {
   if (c->gemm_impl != ETR_GEMM_AUTO) return false;
   if (c->capacity <= 192) return true;

@@ -51,7 +51,7 @@ __device__ inline int capacity_from_delta(const SelectParams& p, float delta_max
 }
 
 // EPL: experts per lane (E <= 32 EPL).  A rank's winner is found by two warp reductions of 32 bits, the largest key
-// and the lowest index that has it (64-bit shuffles over eight slots per lane took 24 us at T 8192, E 128, k 8; this
+// and the lowest index that has it (64-bit shuffles over eight slots per lane took 29 us at T 8192, E 128, k 8; this
 // 17 us).
 template <int EPL>
 __global__ void __launch_bounds__(256)
