@@ -108,7 +108,8 @@ typedef struct etr_config {
   int32_t dtype;              /* etr_dtype of activations and expert weights */
   int32_t gemm_impl;          /* etr_gemm_impl; AUTO = CTA-pair tcgen05 for bf16; for fp32, tensor-core products of
                                  operands split into two tf32 parts each, summed in fp32 (relative error of a
-                                 contraction about 1.5e-7; the SIMT kernels: 2e-7 to 1.2e-6, growing with its length).
+                                 contraction 1.1e-7 to 2.5e-7, SIMT kernels 1.4e-7 to 1.2e-6, growing with its length;
+                                 operands below 2^-113 lose low bits).
                                  SIMT: the CUDA-core kernels */
   int32_t fuse_dispatch;      /* etr_fuse: token rearrangement fused into the GEMM operand fetch */
   int32_t gate_mode;          /* etr_gate: what weighs an expert's output in the combine */

@@ -99,6 +99,17 @@ def test_ends_of_the_number_range(d):
     assert rel(G[rest], ref[rest]) <= TOL
 
 
+@pytest.mark.parametrize("exponent", [-100, -112, -116, -120, -124])
+def test_small_values_lose_the_bits_below_the_tf32_range(exponent):
+    """The smallest step of a tf32 value is 2^-136, so that lo is off by up to 2^-137 whatever the size of the value: below
+    the format's own error down to values of 2^-113, and 2^-137 of the value's size beyond."""
+    cfg, b, W = layer(1, 64, 64, 128, (128,))
+    b.Xp.view(128, 64).mul_(2.0 ** exponent)
+    etr.expert_ffn(cfg, b.route, b.Xp, *W, b.G, b.U, b.H, b.O, b.c.stats, b.c.ws)
+    ref = b.Xp.view(128, 64).double() @ W[0][0].double().T
+    assert rel(b.G.view(128, 64), ref) <= 2e-7 + 2.0 ** (-137 - exponent)
+
+
 @pytest.mark.parametrize("d", [64, 512])
 @pytest.mark.parametrize("bits", [0x7f800001, 0x7f801fff, -0x7fffff, -0x7fe001, 0x7fc00000, -1])
 def test_every_nan_stays_a_nan(bits, d):
