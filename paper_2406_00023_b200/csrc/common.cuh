@@ -220,14 +220,21 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 #endif
 
 #ifdef __CUDACC__
-// prefix[e] = tiles(counts[0]) + ... + tiles(counts[e - 1]), e <= E <= 256, by one warp.
+// prefix[e] = tiles(counts[0]) + ... + tiles(counts[e - 1]), e <= E <= 256, by one warp, straight from global memory (one
+// round of latency between the wait for the predecessor and the first tile); counts_s: a copy for the tiles' extents.
 template <class F>
-__device__ __forceinline__ void tile_prefix_warp(int* prefix, const int* counts, int E, int lane, F tiles) {
+__device__ __forceinline__ void tile_prefix_warp(int* prefix, int* counts_s, const int32_t* counts, int E, int lane, F tiles) {
   int n[8], mine = 0;
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     const int e = 8 * lane + u;
-    n[u] = e < E ? tiles(counts[e]) : 0;
+    n[u] = e < E ? counts[e] : 0;
+  }
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int e = 8 * lane + u;
+    if (e < E) counts_s[e] = n[u];
+    n[u] = e < E ? tiles(n[u]) : 0;
     mine += n[u];
   }
   int inc = mine;

@@ -364,17 +364,15 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_c
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   grid_wait();
-  for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
-  __syncthreads();
-  grid_release();
   if (warp == 2) {
     const int nt = (p.N + N_TILE_COLS - 1) / N_TILE_COLS;
-    tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) {
+    tile_prefix_warp(tile_prefix, s_counts, p.counts, p.E, lane, [&](int n_e) {
       return nt * (p.dyn == TC_DYN_M ? (min(n_e, p.M) + TC_BM - 1) / TC_BM : (p.M + TC_BM - 1) / TC_BM);
     });
   }
   tc_fence_before();
   __syncthreads();
+  grid_release();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_slot;
 
@@ -680,19 +678,18 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
+  __syncwarp();
+  cluster_sync_all();                 // both CTAs' barriers exist before any remote arrive
   grid_wait();
-  for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
-  __syncthreads();
-  grid_release();
   if (warp == 2) {
     const int nt = (p.N + N_TILE_COLS - 1) / N_TILE_COLS;
-    tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) {
+    tile_prefix_warp(tile_prefix, s_counts, p.counts, p.E, lane, [&](int n_e) {
       return nt * (p.dyn == TC_DYN_M ? (min(n_e, p.M) + 255) / 256 : (p.M + 255) / 256);
     });
   }
   tc_fence_before();
   __syncthreads();
-  cluster_sync_all();                 // both CTAs' barriers exist before any remote arrive
+  grid_release();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_slot;
   const uint32_t leader_full = map_to_cta(full_bar, 0);
@@ -973,19 +970,18 @@ tc_grouped_gemm_pair_wide_kernel(const __grid_constant__ CUtensorMap mapA0, cons
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
+  __syncwarp();
+  cluster_sync_all();                 // both CTAs' barriers exist before any remote arrive
   grid_wait();
-  for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
-  __syncthreads();
-  grid_release();
   if (warp == 2) {
     const int nt = (p.N + 2 * N_TILE_COLS - 1) / (2 * N_TILE_COLS);
-    tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) {
+    tile_prefix_warp(tile_prefix, s_counts, p.counts, p.E, lane, [&](int n_e) {
       return nt * (p.dyn == TC_DYN_M ? (min(n_e, p.M) + 255) / 256 : (p.M + 255) / 256);
     });
   }
   tc_fence_before();
   __syncthreads();
-  cluster_sync_all();                 // both CTAs' barriers exist before any remote arrive
+  grid_release();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_slot;
   const uint32_t leader_full = map_to_cta(full_bar, 0);
@@ -1413,20 +1409,19 @@ tc_grouped_gemm_swap_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
+  __syncwarp();
+  cluster_sync_all();                 // both CTAs' barriers exist before any remote arrive
   grid_wait();
-  for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
-  __syncthreads();
-  grid_release();
   if (warp == 2) {
     const int nc = (p.N + COLS - 1) / COLS;
-    tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) {
+    tile_prefix_warp(tile_prefix, s_counts, p.counts, p.E, lane, [&](int n_e) {
       const int n = min(n_e, p.M);
       return n > 0 ? nc * ((n - 1) / swap_tile_rows(n) + 1) : 0;
     });
   }
   tc_fence_before();
   __syncthreads();
-  cluster_sync_all();                 // both CTAs' barriers exist before any remote arrive
+  grid_release();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_slot;
   const uint32_t leader_full = map_to_cta(full_bar, 0);

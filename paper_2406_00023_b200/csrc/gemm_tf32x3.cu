@@ -269,15 +269,13 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   grid_wait();
-  for (int e = tid; e < p.E; e += F3_THREADS) s_counts[e] = p.counts[e];
-  __syncthreads();
-  grid_release();
   if (warp == 2) {
     const int nt = (p.N + COLS - 1) / COLS;
-    tile_prefix_warp(tile_prefix, s_counts, p.E, lane, [&](int n_e) { return f3_mtiles(p, n_e) * nt; });
+    tile_prefix_warp(tile_prefix, s_counts, p.counts, p.E, lane, [&](int n_e) { return f3_mtiles(p, n_e) * nt; });
   }
   tc_fence_before();
   __syncthreads();
+  grid_release();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_slot;
 
