@@ -111,6 +111,7 @@ def algorithmic_work(w, rows, kernel, unrouted=0):
         "tc_gemm_down": (2 * rows * d * h, "flops"),
         "tc_gemm_dswiglu": (2 * rows * d * h, "flops"),
         "tc_gemm_dxp": (4 * rows * d * h, "flops"),
+        "tc_gemm_dw": (6 * rows * d * h, "flops"),
         "tc_gemm_dw2": (2 * rows * d * h, "flops"),
         "tc_gemm_dw1": (4 * rows * d * h, "flops"),
     }

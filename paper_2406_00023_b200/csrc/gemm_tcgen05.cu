@@ -1656,6 +1656,256 @@ tc_grouped_gemm_swap_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
   cluster_sync_all();                 // the next kernel's blocks may start on an SM as soon as its CTA is gone
 }
 
+// ---- weight gradients ------------------------------------------------------------------------------------
+// dW2 = dO^T H, dW1g = dG^T Xp and dW1u = dU^T Xp of every expert in ONE launch: contractions over the expert's rows, both
+// operands MN-major, CTA pairs on tiles of 256 x up to 256 (the last column tile has 128 columns where that is all that is
+// left).  What bounds it: with many rows per expert the tensor pipe and the operands' way into the SMs; with few (one to
+// four K blocks a tile) the stream of outputs to HBM.  For the latter the epilogue writes nothing itself: it packs 64
+// columns of its 32 rows into a swizzled box in shared memory and hands that to TMA, two boxes per warp in turn, so that the
+// stores of one tile drain under the next ones.  Before, each warp turned 32 x 32 blocks and stored 64-byte row pieces, 1.5
+// to 3 us a tile, and a launch per gradient left the last round of tiles of each part-filled.
+constexpr int WG_STAGES = 5;
+constexpr uint32_t WG_STAGE_BYTES = 4 * TC_BOX_BYTES;        // per CTA: 128 columns of A, 128 of B, 64 rows each
+constexpr uint32_t WG_BOX_BYTES = 32 * 128;                  // an output box: 32 rows of 128 bytes
+constexpr size_t WG_SMEM = WG_STAGES * WG_STAGE_BYTES + 8 * 2 * WG_BOX_BYTES + 1024;
+
+struct WgradParams {
+  int d, h, E;
+  int nout;              // 3: dW2, dW1g, dW1u; 1: dW2 alone (dW1 gathers its rows elsewhere)
+  int krows;             // rows of a K block: 64, or 16 or 32 where the capacity is no larger
+  int out_f32;
+  const int32_t* counts;
+  etr_stats* stats;
+  long long wait_limit;
+  uint32_t idesc;        // without N
+};
+struct WgradMaps { CUtensorMap dO, H, dG, dU, Xp, W2, W1g, W1u; };
+struct WgradTile { int e, which, m0, n0, nt, M, N, rows; };      // nt: columns of the tile, 128 or 256
+
+__device__ __forceinline__ bool wgrad_tile(const WgradParams& p, const int* counts_s, int tile, WgradTile& t) {
+  const int td = (p.d + 255) >> 8, th = (p.h + 255) >> 8, per = td * th;
+  t.e = tile / (p.nout * per);
+  if (t.e >= p.E) return false;
+  const int in_e = tile - t.e * p.nout * per;
+  t.which = in_e / per;
+  const int local = in_e - t.which * per, tm = t.which ? th : td;
+  t.M = t.which ? p.h : p.d;
+  t.N = t.which ? p.d : p.h;
+  t.m0 = (local % tm) * 256;
+  t.n0 = (local / tm) * 256;
+  t.nt = t.N - t.n0 > 128 ? 256 : 128;
+  t.rows = counts_s[t.e];
+  return true;
+}
+
+__device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar_cluster, int c0, int c1,
+                                                 int c2, int c3) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4, %5, %6}], [%2];"
+      ::"r"(dst), "l"(map), "r"(bar_cluster), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
+}
+// 32 words of this lane's row (128 bytes) into the swizzled box at buf, then the whole box to (col, row, e) of the output.
+__device__ __forceinline__ void wgrad_store_box(uint32_t buf, int lane, const uint32_t* w, const CUtensorMap* map, int col,
+                                                int row, int e) {
+  if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");      // the box before last has been read
+  __syncwarp();
+#pragma unroll
+  for (int c = 0; c < 8; ++c)
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(buf + lane * 128 + ((c ^ (lane & 7)) << 4)), "r"(w[4 * c]),
+                 "r"(w[4 * c + 1]), "r"(w[4 * c + 2]), "r"(w[4 * c + 3]) : "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncwarp();
+  if (lane == 0) {
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4}], [%1];"
+                 ::"l"(map), "r"(buf), "r"(col), "r"(row), "r"(e) : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+  }
+}
+
+__global__ void __launch_bounds__(TC_THREADS, 1)
+tc_wgrad_pair_kernel(const __grid_constant__ WgradMaps maps, const WgradParams p) {
+  constexpr uint32_t TMEM_COLS = 512;              // two accumulator stages
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t bars[2 * WG_STAGES + 4];
+  __shared__ uint32_t tmem_base_slot;
+  __shared__ int abort_flag_s;
+  __shared__ int s_counts[256];
+
+  volatile int* abort_flag = &abort_flag_s;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t rank = cluster_ctarank();
+  const int pair = (int)cluster_id_x(), npairs = (int)cluster_count_x();
+  const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const uint32_t full_bar = smem_u32(&bars[0]);                    // [WG_STAGES]  used in the leader
+  const uint32_t empty_bar = smem_u32(&bars[WG_STAGES]);           // [WG_STAGES]  in each CTA
+  const uint32_t tfull_bar = smem_u32(&bars[2 * WG_STAGES]);       // [2]          in each CTA
+  const uint32_t tempty_bar = smem_u32(&bars[2 * WG_STAGES + 2]);  // [2]          used in the leader
+
+  if (tid == 0) {
+    abort_flag_s = 0;
+    for (int s = 0; s < WG_STAGES; ++s) { mbar_init(full_bar + 8 * s, 1); mbar_init(empty_bar + 8 * s, 1); }
+    for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar + 8 * a, 1); mbar_init(tempty_bar + 8 * a, 16); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(TMEM_COLS) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  __syncwarp();
+  cluster_sync_all();                 // both CTAs' barriers exist before any remote arrive
+  grid_wait();
+  for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
+  tc_fence_before();
+  __syncthreads();
+  grid_release();
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_base_slot;
+  const uint32_t leader_full = map_to_cta(full_bar, 0);
+  const uint32_t leader_tempty = map_to_cta(tempty_bar, 0);
+  const uint32_t blk = (uint32_t)p.krows * 128u;   // bytes of 64 columns of a K block
+
+  if (warp == 0) {
+    // ---- TMA producer (both CTAs) ---------------------------------------------------------------
+    int stage = 0;
+    uint32_t phase = 0;
+    WgradTile t;
+    bool ok = true;
+    for (int tile = pair; ok && wgrad_tile(p, s_counts, tile, t); tile += npairs) {
+      const CUtensorMap* ma = t.which == 0 ? &maps.dO : t.which == 1 ? &maps.dG : &maps.dU;
+      const CUtensorMap* mb = t.which == 0 ? &maps.H : &maps.Xp;
+      const int ca = (t.m0 + 128 * (int)rank) >> 6, cb = (t.n0 + (t.nt >> 1) * (int)rank) >> 6;      // in blocks of 64 columns
+      for (int k0 = 0; k0 < t.rows; k0 += p.krows) {
+        ok = __all_sync(0xffffffffu, mbar_wait_cluster(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.wait_limit));
+        if (!ok) break;
+        if (elect_one()) {
+          if (rank == 0) mbar_expect_tx(full_bar + 8 * stage, 8 * blk);
+          const uint32_t fb = leader_full + 8 * stage, sa = tiles_base + stage * WG_STAGE_BYTES;
+          tma_load_4d_pair(sa, ma, fb, 0, k0, ca, t.e);
+          tma_load_4d_pair(sa + 2 * TC_BOX_BYTES, mb, fb, 0, k0, cb, t.e);      // of a tile of 128 columns, half is not used
+        }
+        __syncwarp();
+        if (++stage == WG_STAGES) { stage = 0; phase ^= 1u; }
+      }
+    }
+  } else if (warp == 1) {
+    // ---- MMA issuer (leader CTA only) --------------------------------------------------------------
+    if (rank == 0) {
+      int stage = 0, acc_stage = 0;
+      uint32_t phase = 0, acc_phase = 0;
+      WgradTile t;
+      bool ok = true;
+      for (int tile = pair; ok && wgrad_tile(p, s_counts, tile, t); tile += npairs) {
+        if (t.rows == 0) continue;
+        ok = __all_sync(0xffffffffu, mbar_wait_cluster(tempty_bar + 8 * acc_stage, acc_phase ^ 1u, abort_flag, p.wait_limit));
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t d_tmem = tmem_base + (uint32_t)(acc_stage * 256);
+        const uint32_t id = p.idesc | ((uint32_t)(t.nt >> 3) << 17);
+        auto mma = [&](int kk, bool first) {
+          const uint32_t sa = tiles_base + stage * WG_STAGE_BYTES;
+          tc_mma_pair(d_tmem, make_smem_desc(sa + kk * 2048u, blk, 1024u),
+                      make_smem_desc(sa + 2 * TC_BOX_BYTES + kk * 2048u, blk, 1024u), id, first ? 0u : 1u);
+        };
+        auto block = [&](int steps, bool first, bool last) {      // one K block; false: a wait ran out
+          if (!__all_sync(0xffffffffu, mbar_wait_cluster(full_bar + 8 * stage, phase, abort_flag, p.wait_limit))) return false;
+          tc_fence_after();
+          if (elect_one()) {
+#pragma unroll
+            for (int kk = 0; kk < TC_BK / 16; ++kk)
+              if (steps == TC_BK / 16 || kk < steps) mma(kk, first && kk == 0);
+            tc_commit_pair(empty_bar + 8 * stage);                       // frees the stage in both CTAs
+            if (last) tc_commit_pair(tfull_bar + 8 * acc_stage);         // accumulators complete in both CTAs
+          }
+          __syncwarp();
+          if (++stage == WG_STAGES) { stage = 0; phase ^= 1u; }
+          return true;
+        };
+        // The last K block is peeled off: it runs only the 16-row steps that hold rows in use (the others would add the
+        // zeros of pad rows), and a test in the loop costs more than it saves.
+        const int nloop = (t.rows - 1) / p.krows;
+        if (p.krows == TC_BK) {
+          for (int kb = 0; ok && kb < nloop; ++kb) ok = block(TC_BK / 16, kb == 0, false);
+        } else {
+          for (int kb = 0; ok && kb < nloop; ++kb) ok = block(p.krows / 16, kb == 0, false);
+        }
+        ok = ok && block((t.rows - nloop * p.krows + 15) >> 4, nloop == 0, true);
+        if (!ok) break;
+        if (++acc_stage == 2) { acc_stage = 0; acc_phase ^= 1u; }
+      }
+    }
+  } else {
+    // ---- epilogue warps (both CTAs, own 128 rows; 128 of the tile's columns each) -------------------------
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    const uint32_t box = tiles_base + WG_STAGES * WG_STAGE_BYTES + (uint32_t)(warp - 2) * 2 * WG_BOX_BYTES;
+    int acc_stage = 0, turn = 0;
+    uint32_t acc_phase = 0;
+    WgradTile t;
+    bool ok = true;
+    for (int tile = pair; ok && wgrad_tile(p, s_counts, tile, t); tile += npairs) {
+      const CUtensorMap* mo = t.which == 0 ? &maps.W2 : t.which == 1 ? &maps.W1g : &maps.W1u;
+      const int row = t.m0 + 128 * (int)rank + 32 * q, col = t.n0 + 128 * half;
+      uint32_t r[4][32];
+      if (t.rows == 0) {                             // nothing to contract: zeros
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+          for (int i = 0; i < 32; ++i) r[c][i] = 0u;
+      } else {
+        ok = __all_sync(0xffffffffu, mbar_wait_cluster(tfull_bar + 8 * acc_stage, acc_phase, abort_flag, p.wait_limit));
+        if (!ok) break;
+        tc_fence_after();
+        // all 128 columns are read at once and the accumulators released before anything is stored
+        const uint32_t taddr = tmem_base + (uint32_t)(acc_stage * 256 + 128 * half) + ((uint32_t)(32 * q) << 16);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tc_ld32(taddr + 32 * c, r[c]);
+        tc_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(leader_tempty + 8 * acc_stage);
+        if (++acc_stage == 2) { acc_stage = 0; acc_phase ^= 1u; }
+      }
+      if (row >= t.M) continue;
+      if (p.out_f32) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          if (col + 32 * c >= t.N) break;
+          wgrad_store_box(box + turn * WG_BOX_BYTES, lane, r[c], mo, col + 32 * c, row, t.e);
+          turn ^= 1;
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          if (col + 64 * c >= t.N) break;
+          uint32_t w[32];
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            w[i] = pack_bf16(__uint_as_float(r[2 * c + (i >> 4)][2 * (i & 15)]), __uint_as_float(r[2 * c + (i >> 4)][2 * (i & 15) + 1]));
+          wgrad_store_box(box + turn * WG_BOX_BYTES, lane, w, mo, col + 64 * c, row, t.e);
+          turn ^= 1;
+        }
+      }
+    }
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");      // every box is in the output
+  }
+
+  // ---- teardown: neither CTA leaves while the other may still touch its barriers or memory -------
+  __syncwarp();
+  if (*abort_flag) {
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2000000ll) { }
+    if (tid == 0) atomicExch(&p.stats->error_word, 0x7c0c);
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+  }
+  cluster_sync_all();                 // the next kernel's blocks may start on an SM as soon as its CTA is gone
+}
+
 // ---- host side --------------------------------------------------------------------------------------
 // Row-major bf16 tensor [E, rows, cols] as a 3-D map (cols, rows, E), boxes of 64 columns x box_rows, 128-byte swizzle.
 static etr_status make_map(CUtensorMap* m, const void* base, int cols, int rows, int E, int box_rows = 64) {
@@ -1759,7 +2009,7 @@ static etr_status tc_launch_pair(const char* name, const CUtensorMap& a0, const 
                                  cudaStream_t st) {
   const int cfg = (p.a_mn ? 1 : 0) | (p.b_mn ? 2 : 0) | (p.dual_b ? 4 : 0) | (p.k1_blocks > 0 ? 8 : 0);
   constexpr int C0 = EPI == TC_EPI_SWIGLU ? 4 : EPI == TC_EPI_DSWIGLU ? 2 : 0;      // first use
-  constexpr int C1 = EPI == TC_EPI_STORE ? 3 : C0, C2 = EPI == TC_EPI_STORE ? 10 : C0;
+  constexpr int C1 = EPI == TC_EPI_STORE && GATHER == 2 ? 3 : C0, C2 = EPI == TC_EPI_STORE ? 10 : C0;
   if (cfg == C0) return tc_launch_pair_cfg<EPI, GATHER, C0>(name, a0, a1, b0, b1, p, max_tiles, st);
   if (cfg == C1) return tc_launch_pair_cfg<EPI, GATHER, C1>(name, a0, a1, b0, b1, p, max_tiles, st);
   if (cfg == C2) return tc_launch_pair_cfg<EPI, GATHER, C2>(name, a0, a1, b0, b1, p, max_tiles, st);
@@ -1871,6 +2121,69 @@ static etr_status swap_launch(const char* name, const CUtensorMap& a0, const CUt
   return ETR_OK;
 }
 
+// ---- weight gradients: host side ------------------------------------------------------------------------
+// Row-major bf16 tensor [E, rows, cols] as a 4-D map (64 columns, rows, blocks of 64 columns, E): a box of 64 columns x
+// box_rows x 2 blocks is 128 columns, each block of 64 with its 128-byte swizzle.  cols is a multiple of 64.
+static etr_status make_map_blocks(CUtensorMap* m, const void* base, int cols, int rows, int E, int box_rows) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return ETR_ERR_CUDA;
+  const cuuint64_t dims[4] = {64, (cuuint64_t)rows, (cuuint64_t)(cols / 64), (cuuint64_t)E};
+  const cuuint64_t strides[3] = {(cuuint64_t)cols * 2, 128, (cuuint64_t)cols * 2 * (cuuint64_t)rows};
+  const cuuint32_t box[4] = {64, (cuuint32_t)box_rows, 2, 1};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? ETR_OK : ETR_ERR_CUDA;
+}
+// Row-major output [E, rows, cols], bf16 or fp32, stored in boxes of 128 bytes x 32 rows.
+static etr_status make_map_out(CUtensorMap* m, void* base, int cols, int rows, int E, bool f32) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return ETR_ERR_CUDA;
+  const cuuint64_t eb = f32 ? 4 : 2;
+  const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)E};
+  const cuuint64_t strides[2] = {cols * eb, cols * eb * (cuuint64_t)rows};
+  const cuuint32_t box[3] = {f32 ? 32u : 64u, 32, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  const CUresult r = fn(m, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides,
+                        box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                        CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? ETR_OK : ETR_ERR_CUDA;
+}
+// Xp == nullptr: dW2 alone.
+static etr_status wgrad_launch(const etr_config* c, const etr_route* rt, const void* dO, const void* Xp, const void* H,
+                               const void* dG, const void* dU, void* dW1g, void* dW1u, void* dW2, etr_stats* stats,
+                               cudaStream_t st) {
+  const int d = c->d, h = c->h, Cs = c_stride_of(c), E = c->E;
+  WgradParams p = {};
+  p.d = d; p.h = h; p.E = E; p.nout = Xp ? 3 : 1;
+  p.krows = c->capacity <= 16 ? 16 : c->capacity <= 32 ? 32 : TC_BK;      // the rows behind are not even fetched
+  p.out_f32 = c->grad_fp32 != 0;
+  p.counts = rt->counts; p.stats = stats;
+  p.wait_limit = c->wait_limit_cycles > 0 ? (long long)c->wait_limit_cycles : TC_WAIT_LIMIT_CYCLES;
+  p.idesc = make_idesc(1, 1, 0, 256);
+  WgradMaps m;
+  ETR_TRY(make_map_blocks(&m.dO, dO, d, Cs, E, p.krows));
+  ETR_TRY(make_map_blocks(&m.H, H, h, Cs, E, p.krows));
+  ETR_TRY(make_map_out(&m.W2, dW2, h, d, E, p.out_f32));
+  m.dG = m.dU = m.Xp = m.dO; m.W1g = m.W1u = m.W2;
+  if (Xp) {
+    ETR_TRY(make_map_blocks(&m.dG, dG, h, Cs, E, p.krows));
+    ETR_TRY(make_map_blocks(&m.dU, dU, h, Cs, E, p.krows));
+    ETR_TRY(make_map_blocks(&m.Xp, Xp, d, Cs, E, p.krows));
+    ETR_TRY(make_map_out(&m.W1g, dW1g, d, h, E, p.out_f32));
+    ETR_TRY(make_map_out(&m.W1u, dW1u, d, h, E, p.out_f32));
+  }
+  static std::atomic<unsigned long long> attr_done{0};      // one bit per device
+  if (!ensure_dyn_smem(tc_wgrad_pair_kernel, WG_SMEM, attr_done)) return ETR_ERR_CUDA;
+  const long long tiles = (long long)E * p.nout * ceil_div(d, 256) * ceil_div(h, 256);
+  const int pairs = (int)std::min(tiles, (long long)(sm_count() / 2));
+  ETR_TIME_BEGIN("tc_gemm_dw");
+  launch_kernel(tc_wgrad_pair_kernel, 2 * pairs, TC_THREADS, WG_SMEM, st, 2, m, p);
+  ETR_LAUNCH_CHECK();
+  return ETR_OK;
+}
+
 static TcParams tc_params(const etr_config* c) {
   TcParams p = {};
   p.wait_limit = c->wait_limit_cycles > 0 ? (long long)c->wait_limit_cycles : TC_WAIT_LIMIT_CYCLES;
@@ -1977,20 +2290,23 @@ etr_status tc_ffn_backward(const etr_config* c, const etr_route* rt, const void*
     ETR_TRY((tc_run<TC_EPI_STORE>(tc_form_of(c, TC_EPI_STORE, p), "tc_gemm_dxp", mdG, mdU, mW1g, mW1u, p,
                                           E * mt * ceil_div(d, 256), st)));
   }
-  {  // dW2 = dO^T H: contraction over the expert's rows, both operands MN-major
-    TcParams p = tc_params(c);
-    p.a_mn = 1; p.b_mn = 1; p.M = d; p.N = h; p.dyn = TC_DYN_K; p.E = E; p.counts = rt->counts;
-    p.out0 = (__nv_bfloat16*)dW2; p.out_bs = (long long)d * h; p.ld_out = h; p.stats = stats;
-    p.out_f32 = c->grad_fp32 != 0;
-    ETR_TRY((tc_run<TC_EPI_STORE>(tc_form_of(c, TC_EPI_STORE, p), "tc_gemm_dw2", mdO, mdO, mH, mH, p,
-                                          E * ceil_div(d, TC_BM) * ceil_div(h, 256), st)));
+  // Weight gradients, contractions over the expert's rows.  The pair form takes all three in one launch; the forms that
+  // gemm_impl forces, and rows gathered from X (fuse_dispatch), run them one by one.
+  TcParams dw2 = tc_params(c);
+  dw2.a_mn = 1; dw2.b_mn = 1; dw2.M = d; dw2.N = h; dw2.dyn = TC_DYN_K; dw2.E = E; dw2.counts = rt->counts;
+  dw2.out0 = (__nv_bfloat16*)dW2; dw2.out_bs = (long long)d * h; dw2.ld_out = h; dw2.stats = stats;
+  dw2.out_f32 = c->grad_fp32 != 0;
+  const TcForm form = tc_form_of(c, TC_EPI_STORE, dw2);
+  if (form == TC_FORM_PAIR) {
+    ETR_TRY(wgrad_launch(c, rt, dO, Xtok ? nullptr : Xp, H, dG, dU, dW1g, dW1u, dW2, stats, st));
+    if (!Xtok) return ETR_OK;
+  } else {
+    ETR_TRY((tc_run<TC_EPI_STORE>(form, "tc_gemm_dw2", mdO, mdO, mH, mH, dw2, E * ceil_div(d, TC_BM) * ceil_div(h, 256), st)));
   }
   for (int which = 0; which < 2; ++which) {  // dW1g = dG^T Xp, dW1u = dU^T Xp
-    TcParams p = tc_params(c);
-    p.a_mn = 1; p.b_mn = 1; p.M = h; p.N = d; p.dyn = TC_DYN_K; p.E = E; p.counts = rt->counts;
+    TcParams p = dw2;
+    p.M = h; p.N = d; p.ld_out = d; p.out0 = (__nv_bfloat16*)(which ? dW1u : dW1g);
     if (Xtok) { p.gather = 2; p.gather_ld = Cs; p.gather_oob = c->T; p.gather_idx = rt->slot_token; }
-    p.out0 = (__nv_bfloat16*)(which ? dW1u : dW1g); p.out_bs = (long long)h * d; p.ld_out = d; p.stats = stats;
-    p.out_f32 = c->grad_fp32 != 0;
     const CUtensorMap& ma = which ? mdU : mdG;
     ETR_TRY((tc_run<TC_EPI_STORE>(tc_form_of(c, TC_EPI_STORE, p), "tc_gemm_dw1", ma, ma, mXp, mXp, p,
                                           E * ceil_div(h, TC_BM) * ceil_div(d, 256), st)));
