@@ -1661,13 +1661,18 @@ tc_grouped_gemm_swap_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
 // operands MN-major, CTA pairs on tiles of 256 x up to 256 (the last column tile has 128 columns where that is all that is
 // left).  What bounds it: with many rows per expert the tensor pipe and the operands' way into the SMs; with few (one to
 // four K blocks a tile) the stream of outputs to HBM.  For the latter the epilogue writes nothing itself: it packs 64
-// columns of its 32 rows into a swizzled box in shared memory and hands that to TMA, two boxes per warp in turn, so that the
-// stores of one tile drain under the next ones.  Before, each warp turned 32 x 32 blocks and stored 64-byte row pieces, 1.5
-// to 3 us a tile, and a launch per gradient left the last round of tiles of each part-filled.
+// columns of its 32 rows into a swizzled box in shared memory and hands that to TMA.  A tile's way through it is a chain
+// of latencies all the same (in cycles: 1300 to 4400 for 128 columns of tensor memory while all warps read, 240 to release them, twice
+// 700 for a box), so there are two sets of eight epilogue warps that take alternate tiles, one per accumulator stage.
+// Measured, the three gradients: one launch each, warps turning 32 x 32 blocks and storing 64-byte row pieces; one launch,
+// boxes, eight warps; this.  10 rows per expert (E 32, d 2048, h 4096) 500, 385, 292 us (5.5 TB/s of outputs); 112 rows (E 16,
+// h 2816) 195, 176, 139; 512 rows (E 16, d 1024, h 2816) 147, 120, 121; 1024 rows (E 32, d 2048, h 1408) 486, 457, 449; 722 rows
+// (E 64, d 4096, h 2048) 1880, 1815, 1767.  No gain: columns of tiles first, two or four boxes per warp; three stages: 15 % slower.
 constexpr int WG_STAGES = 5;
 constexpr uint32_t WG_STAGE_BYTES = 4 * TC_BOX_BYTES;        // per CTA: 128 columns of A, 128 of B, 64 rows each
 constexpr uint32_t WG_BOX_BYTES = 32 * 128;                  // an output box: 32 rows of 128 bytes
-constexpr size_t WG_SMEM = WG_STAGES * WG_STAGE_BYTES + 8 * 2 * WG_BOX_BYTES + 1024;
+constexpr int WG_EPI_WARPS = 16, WG_THREADS = 64 + 32 * WG_EPI_WARPS;
+constexpr size_t WG_SMEM = WG_STAGES * WG_STAGE_BYTES + WG_EPI_WARPS * WG_BOX_BYTES + 1024;
 
 struct WgradParams {
   int d, h, E;
@@ -1680,23 +1685,35 @@ struct WgradParams {
   uint32_t idesc;        // without N
 };
 struct WgradMaps { CUtensorMap dO, H, dG, dU, Xp, W2, W1g, W1u; };
-struct WgradTile { int e, which, m0, n0, nt, M, N, rows; };      // nt: columns of the tile, 128 or 256
-
-__device__ __forceinline__ bool wgrad_tile(const WgradParams& p, const int* counts_s, int tile, WgradTile& t) {
-  const int td = (p.d + 255) >> 8, th = (p.h + 255) >> 8, per = td * th;
-  t.e = tile / (p.nout * per);
-  if (t.e >= p.E) return false;
-  const int in_e = tile - t.e * p.nout * per;
-  t.which = in_e / per;
-  const int local = in_e - t.which * per, tm = t.which ? th : td;
-  t.M = t.which ? p.h : p.d;
-  t.N = t.which ? p.d : p.h;
-  t.m0 = (local % tm) * 256;
-  t.n0 = (local / tm) * 256;
-  t.nt = t.N - t.n0 > 128 ? 256 : 128;
-  t.rows = counts_s[t.e];
-  return true;
-}
+// The tiles of a pair, every npairs-th: of an expert those of dW2, then dW1g, then dW1u, row tiles first.
+struct WgradTiles {
+  int e, which, m0, n0, nt, M, N, rows;      // the current tile; nt: its columns, 128 or 256
+  int in_e, per, step_e, step_i;
+  __device__ __forceinline__ bool first(const WgradParams& p, const int* counts_s, int tile, int step) {
+    per = ((p.d + 255) >> 8) * ((p.h + 255) >> 8);
+    const int all = p.nout * per;
+    e = tile / all; in_e = tile - e * all;
+    step_e = step / all; step_i = step - step_e * all;
+    return set(p, counts_s);
+  }
+  __device__ __forceinline__ bool next(const WgradParams& p, const int* counts_s) {
+    e += step_e; in_e += step_i;
+    if (in_e >= p.nout * per) { in_e -= p.nout * per; ++e; }
+    return set(p, counts_s);
+  }
+  __device__ __forceinline__ bool set(const WgradParams& p, const int* counts_s) {
+    if (e >= p.E) return false;
+    which = (in_e >= per) + (in_e >= 2 * per);
+    M = which ? p.h : p.d;
+    N = which ? p.d : p.h;
+    const int local = in_e - which * per, tm = (M + 255) >> 8, tn = local / tm;
+    m0 = (local - tn * tm) * 256;
+    n0 = tn * 256;
+    nt = N - n0 > 128 ? 256 : 128;
+    rows = counts_s[e];
+    return true;
+  }
+};
 
 __device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar_cluster, int c0, int c1,
                                                  int c2, int c3) {
@@ -1708,7 +1725,7 @@ __device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap
 // 32 words of this lane's row (128 bytes) into the swizzled box at buf, then the whole box to (col, row, e) of the output.
 __device__ __forceinline__ void wgrad_store_box(uint32_t buf, int lane, const uint32_t* w, const CUtensorMap* map, int col,
                                                 int row, int e) {
-  if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");      // the box before last has been read
+  if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");      // the last box has been read
   __syncwarp();
 #pragma unroll
   for (int c = 0; c < 8; ++c)
@@ -1723,7 +1740,7 @@ __device__ __forceinline__ void wgrad_store_box(uint32_t buf, int lane, const ui
   }
 }
 
-__global__ void __launch_bounds__(TC_THREADS, 1)
+__global__ void __launch_bounds__(WG_THREADS, 1)
 tc_wgrad_pair_kernel(const __grid_constant__ WgradMaps maps, const WgradParams p) {
   constexpr uint32_t TMEM_COLS = 512;              // two accumulator stages
   extern __shared__ uint8_t smem_raw[];
@@ -1755,7 +1772,7 @@ tc_wgrad_pair_kernel(const __grid_constant__ WgradMaps maps, const WgradParams p
   __syncwarp();
   cluster_sync_all();                 // both CTAs' barriers exist before any remote arrive
   grid_wait();
-  for (int e = tid; e < p.E; e += TC_THREADS) s_counts[e] = p.counts[e];
+  for (int e = tid; e < p.E; e += WG_THREADS) s_counts[e] = p.counts[e];
   tc_fence_before();
   __syncthreads();
   grid_release();
@@ -1769,9 +1786,9 @@ tc_wgrad_pair_kernel(const __grid_constant__ WgradMaps maps, const WgradParams p
     // ---- TMA producer (both CTAs) ---------------------------------------------------------------
     int stage = 0;
     uint32_t phase = 0;
-    WgradTile t;
+    WgradTiles t;
     bool ok = true;
-    for (int tile = pair; ok && wgrad_tile(p, s_counts, tile, t); tile += npairs) {
+    for (bool more = t.first(p, s_counts, pair, npairs); ok && more; more = t.next(p, s_counts)) {
       const CUtensorMap* ma = t.which == 0 ? &maps.dO : t.which == 1 ? &maps.dG : &maps.dU;
       const CUtensorMap* mb = t.which == 0 ? &maps.H : &maps.Xp;
       const int ca = (t.m0 + 128 * (int)rank) >> 6, cb = (t.n0 + (t.nt >> 1) * (int)rank) >> 6;      // in blocks of 64 columns
@@ -1793,9 +1810,9 @@ tc_wgrad_pair_kernel(const __grid_constant__ WgradMaps maps, const WgradParams p
     if (rank == 0) {
       int stage = 0, acc_stage = 0;
       uint32_t phase = 0, acc_phase = 0;
-      WgradTile t;
+      WgradTiles t;
       bool ok = true;
-      for (int tile = pair; ok && wgrad_tile(p, s_counts, tile, t); tile += npairs) {
+      for (bool more = t.first(p, s_counts, pair, npairs); ok && more; more = t.next(p, s_counts)) {
         if (t.rows == 0) continue;
         ok = __all_sync(0xffffffffu, mbar_wait_cluster(tempty_bar + 8 * acc_stage, acc_phase ^ 1u, abort_flag, p.wait_limit));
         if (!ok) break;
@@ -1836,53 +1853,50 @@ tc_wgrad_pair_kernel(const __grid_constant__ WgradMaps maps, const WgradParams p
     }
   } else {
     // ---- epilogue warps (both CTAs, own 128 rows; 128 of the tile's columns each) -------------------------
-    const int q = warp & 3, half = (warp - 2) >> 2;
-    const uint32_t box = tiles_base + WG_STAGES * WG_STAGE_BYTES + (uint32_t)(warp - 2) * 2 * WG_BOX_BYTES;
-    int acc_stage = 0, turn = 0;
+    const int q = warp & 3, half = ((warp - 2) >> 2) & 1, mine = (warp - 2) >> 3;
+    const uint32_t box = tiles_base + WG_STAGES * WG_STAGE_BYTES + (uint32_t)(warp - 2) * WG_BOX_BYTES;
+    int turn = 0, empties = 0;                       // which set takes the next tile with rows, and without
     uint32_t acc_phase = 0;
-    WgradTile t;
-    bool ok = true;
-    for (int tile = pair; ok && wgrad_tile(p, s_counts, tile, t); tile += npairs) {
+    WgradTiles t;
+    for (bool more = t.first(p, s_counts, pair, npairs); more; more = t.next(p, s_counts)) {
       const CUtensorMap* mo = t.which == 0 ? &maps.W2 : t.which == 1 ? &maps.W1g : &maps.W1u;
       const int row = t.m0 + 128 * (int)rank + 32 * q, col = t.n0 + 128 * half;
-      uint32_t r[4][32];
-      if (t.rows == 0) {                             // nothing to contract: zeros
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-#pragma unroll
-          for (int i = 0; i < 32; ++i) r[c][i] = 0u;
-      } else {
-        ok = __all_sync(0xffffffffu, mbar_wait_cluster(tfull_bar + 8 * acc_stage, acc_phase, abort_flag, p.wait_limit));
-        if (!ok) break;
+      int& whose = t.rows == 0 ? empties : turn;
+      const bool own = whose == mine;
+      whose ^= 1;
+      if (!own) continue;
+      const uint32_t taddr = tmem_base + (uint32_t)(mine * 256 + 128 * half) + ((uint32_t)(32 * q) << 16);
+      if (t.rows > 0) {
+        if (!__all_sync(0xffffffffu, mbar_wait_cluster(tfull_bar + 8 * mine, acc_phase, abort_flag, p.wait_limit))) break;
+        acc_phase ^= 1u;
         tc_fence_after();
-        // all 128 columns are read at once and the accumulators released before anything is stored
-        const uint32_t taddr = tmem_base + (uint32_t)(acc_stage * 256 + 128 * half) + ((uint32_t)(32 * q) << 16);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) tc_ld32(taddr + 32 * c, r[c]);
-        tc_wait_ld();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(leader_tempty + 8 * acc_stage);
-        if (++acc_stage == 2) { acc_stage = 0; acc_phase ^= 1u; }
       }
-      if (row >= t.M) continue;
-      if (p.out_f32) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          if (col + 32 * c >= t.N) break;
-          wgrad_store_box(box + turn * WG_BOX_BYTES, lane, r[c], mo, col + 32 * c, row, t.e);
-          turn ^= 1;
+      for (int c = 0; c < 2; ++c) {                  // 64 columns at a time
+        uint32_t r[2][32];
+        if (t.rows == 0) {                           // nothing to contract: zeros
+#pragma unroll
+          for (int i = 0; i < 32; ++i) r[0][i] = r[1][i] = 0u;
+        } else {
+          tc_ld32(taddr + 64 * c, r[0]);
+          tc_ld32(taddr + 64 * c + 32, r[1]);
+          tc_wait_ld();
+          if (c == 1) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(leader_tempty + 8 * mine);
+          }
         }
-      } else {
+        if (row >= t.M || col + 64 * c >= t.N) continue;
+        if (p.out_f32) {
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          if (col + 64 * c >= t.N) break;
+          for (int u = 0; u < 2; ++u) wgrad_store_box(box, lane, r[u], mo, col + 64 * c + 32 * u, row, t.e);
+        } else {
           uint32_t w[32];
 #pragma unroll
           for (int i = 0; i < 32; ++i)
-            w[i] = pack_bf16(__uint_as_float(r[2 * c + (i >> 4)][2 * (i & 15)]), __uint_as_float(r[2 * c + (i >> 4)][2 * (i & 15) + 1]));
-          wgrad_store_box(box + turn * WG_BOX_BYTES, lane, w, mo, col + 64 * c, row, t.e);
-          turn ^= 1;
+            w[i] = pack_bf16(__uint_as_float(r[i >> 4][2 * (i & 15)]), __uint_as_float(r[i >> 4][2 * (i & 15) + 1]));
+          wgrad_store_box(box, lane, w, mo, col + 64 * c, row, t.e);
         }
       }
     }
@@ -2179,7 +2193,7 @@ static etr_status wgrad_launch(const etr_config* c, const etr_route* rt, const v
   const long long tiles = (long long)E * p.nout * ceil_div(d, 256) * ceil_div(h, 256);
   const int pairs = (int)std::min(tiles, (long long)(sm_count() / 2));
   ETR_TIME_BEGIN("tc_gemm_dw");
-  launch_kernel(tc_wgrad_pair_kernel, 2 * pairs, TC_THREADS, WG_SMEM, st, 2, m, p);
+  launch_kernel(tc_wgrad_pair_kernel, 2 * pairs, WG_THREADS, WG_SMEM, st, 2, m, p);
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }
