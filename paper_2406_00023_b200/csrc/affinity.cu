@@ -835,7 +835,12 @@ __device__ __forceinline__ void dx_chunk_cz(float* __restrict__ cz, float* __res
 
 
 
-template <class T, int NV, bool GROUP8>
+// GPV: pooled columns that 8 elements span, 1 (D = 2^d_shift >= 8) or 2 (D = 4): their R values are then gathered in the
+// streaming pass itself, beside the rows (R is a few KiB to a few hundred and stays in L1 and L2), and step (2) shrinks to
+// beta, one thread per token: a quarter of a block's life went into cz, with no byte of X or dXp in flight.  cz through
+// shared memory against this: 89 -> 71 us (T 16384, d 2048, two rows a token), 260 -> 240 (T 65536, d 4096), 17 -> 13
+// (T 4096, d 1024), 5.6 -> 4.6 (T 512, d 256, fp32).  0: any other D, through cz.
+template <class T, int NV, int GPV>
 __global__ void __launch_bounds__(256, 4)
 affinity_bwd_dx_chunk_kernel(const T* X, const float* R,
                              const float* delta, const float* xnorm,
@@ -844,7 +849,7 @@ affinity_bwd_dx_chunk_kernel(const T* X, const float* R,
                              const T* dXp, T* __restrict__ dX,
                              int Ttok, int d, int D, int E, int m, int C_stride, int tpb, int d_shift) {
   grid_sync();
-  extern __shared__ __align__(16) float cz[];      // [tpb][m]
+  extern __shared__ __align__(16) float cz[];      // [tpb][m], GPV = 0 only
   __shared__ int s_ptr[DXC_MAX_TOKENS + 1];
   __shared__ int s_row[DXC_ROWS];
   __shared__ int s_exp[DXC_ROWS];                  // expert of the entry, -1 if ||R_i|| = 0
@@ -875,9 +880,24 @@ affinity_bwd_dx_chunk_kernel(const T* X, const float* R,
     s_w[e] = dg * sqD / (a * b) / (float)D;
   }
   __syncthreads();
-  dx_chunk_cz(cz, s_beta, s_ptr, s_exp, s_w, s_dg, s_dl, s_a, R, rnorm, delta, dgate, tok_row, base,
-              DXC_ROWS, nt, m, E, C_stride, t0, sqD, D, tid);
+  if (GPV == 0) {
+    dx_chunk_cz(cz, s_beta, s_ptr, s_exp, s_w, s_dg, s_dl, s_a, R, rnorm, delta, dgate, tok_row, base,
+                DXC_ROWS, nt, m, E, C_stride, t0, sqD, D, tid);
+  } else if (tid < nt) {                           // beta of a token: its entries in list order
+    const float a = s_a[tid];
+    float beta = 0.f;
+    for (int q = s_ptr[tid] - base; q < s_ptr[tid + 1] - base; ++q) {
+      if (q < DXC_ROWS) {
+        if (s_exp[q] >= 0 && a != 0.f) beta = fmaf(s_dg[q], s_dl[q], beta);
+      } else {
+        const int r = tok_row[base + q], i = r / C_stride;
+        if (rnorm[i] != 0.f && a != 0.f) beta = fmaf(dgate[r], delta[(size_t)(t0 + tid) * E + i], beta);
+      }
+    }
+    s_beta[tid] = a != 0.f ? beta / (a * a) : 0.f;
+  }
   __syncthreads();
+  constexpr int G = GPV > 0 ? GPV : 1;
   const int vpt = d / 8 / NV;                      // threads per token
   for (int wi = tid; wi < nt * vpt; wi += 256) {
     const int tl = wi / vpt, v = wi - tl * vpt;
@@ -897,41 +917,86 @@ affinity_bwd_dx_chunk_kernel(const T* X, const float* R,
     Vec8<T> xv[NV];
 #pragma unroll
     for (int u = 0; u < NV; ++u) xv[u] = Vec8<T>::load(x + (size_t)(v + u * vpt) * 8);
+    float acc[NV][G];                              // cz of the thread's pooled columns
+#pragma unroll
+    for (int u = 0; u < NV; ++u)
+#pragma unroll
+      for (int g2 = 0; g2 < G; ++g2) acc[u][g2] = 0.f;
+    struct Entry { int r, i; float w; };           // a row of the token, its expert (-1: R does not count) and R's weight
+    auto entry = [&](int q) {
+      Entry n;
+      if (q < DXC_ROWS) {
+        n.r = s_row[q]; n.i = s_exp[q]; n.w = s_w[q];
+      } else {
+        n.r = tok_row[base + q]; n.i = n.r / C_stride;
+        const float b = rnorm[n.i];
+        n.w = dgate[n.r] * sqD / (s_a[tl] * b) / (float)D;
+        if (b == 0.f) n.i = -1;
+      }
+      if (s_a[tl] == 0.f) n.i = -1;
+      return n;
+    };
+    struct RVal { float v[NV][G]; };
+    auto load_r = [&](const Entry& n) {
+      RVal y;
+#pragma unroll
+      for (int u = 0; u < NV; ++u) {
+        const int c0 = (v + u * vpt) * 8;
+        if (GPV == 1) {
+          y.v[u][0] = n.i >= 0 ? R[(size_t)n.i * m + (c0 >> d_shift)] : 0.f;
+        } else if (GPV == 2) {
+          const float2 f = n.i >= 0 ? *reinterpret_cast<const float2*>(R + (size_t)n.i * m + (c0 >> 2)) : make_float2(0.f, 0.f);
+          y.v[u][0] = f.x; y.v[u][G - 1] = f.y;
+        }
+      }
+      return y;
+    };
+    auto add_r = [&](const Entry& n, const RVal& y) {
+      if (GPV > 0 && n.i >= 0) {
+#pragma unroll
+        for (int u = 0; u < NV; ++u)
+#pragma unroll
+          for (int g2 = 0; g2 < G; ++g2) acc[u][g2] = fmaf(n.w, y.v[u][g2], acc[u][g2]);
+      }
+    };
     int q = beg;
     for (; q + 2 <= end; q += 2) {
-      const int r0 = q < DXC_ROWS ? s_row[q] : tok_row[base + q];
-      const int r1 = q + 1 < DXC_ROWS ? s_row[q + 1] : tok_row[base + q + 1];
+      const Entry n0 = entry(q), n1 = entry(q + 1);
       Vec8<T> v0[NV], v1[NV];
 #pragma unroll
-      for (int u = 0; u < NV; ++u) v0[u] = Vec8<T>::load(dXp + (size_t)r0 * d + (size_t)(v + u * vpt) * 8);
+      for (int u = 0; u < NV; ++u) v0[u] = Vec8<T>::load(dXp + (size_t)n0.r * d + (size_t)(v + u * vpt) * 8);
 #pragma unroll
-      for (int u = 0; u < NV; ++u) v1[u] = Vec8<T>::load(dXp + (size_t)r1 * d + (size_t)(v + u * vpt) * 8);
+      for (int u = 0; u < NV; ++u) v1[u] = Vec8<T>::load(dXp + (size_t)n1.r * d + (size_t)(v + u * vpt) * 8);
+      const RVal y0 = load_r(n0), y1 = load_r(n1);
 #pragma unroll
       for (int u = 0; u < NV; ++u)
 #pragma unroll
         for (int e = 0; e < 8; ++e) bs[u][e] = (bs[u][e] + v0[u].v[e]) + v1[u].v[e];
+      add_r(n0, y0);
+      add_r(n1, y1);
     }
     if (q < end) {
-      const int r = q < DXC_ROWS ? s_row[q] : tok_row[base + q];
+      const Entry n0 = entry(q);
       Vec8<T> v0[NV];
 #pragma unroll
-      for (int u = 0; u < NV; ++u) v0[u] = Vec8<T>::load(dXp + (size_t)r * d + (size_t)(v + u * vpt) * 8);
+      for (int u = 0; u < NV; ++u) v0[u] = Vec8<T>::load(dXp + (size_t)n0.r * d + (size_t)(v + u * vpt) * 8);
+      const RVal y0 = load_r(n0);
 #pragma unroll
       for (int u = 0; u < NV; ++u)
 #pragma unroll
         for (int e = 0; e < 8; ++e) bs[u][e] += v0[u].v[e];
+      add_r(n0, y0);
     }
     const float beta = s_beta[tl];
-    const float* czt = cz + (size_t)tl * m;
 #pragma unroll
     for (int u = 0; u < NV; ++u) {
       const int c0 = (v + u * vpt) * 8;
       float out[8];
-      if (GROUP8) {                                // D = 2^d_shift >= 8: the 8 elements share one group
-        const float czv = czt[c0 >> d_shift];
+      if (GPV > 0) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) out[e] = bs[u][e] + (czv - beta * xv[u].v[e]);
+        for (int e = 0; e < 8; ++e) out[e] = bs[u][e] + (acc[u][e * G / 8] - beta * xv[u].v[e]);
       } else {
+        const float* czt = cz + (size_t)tl * m;
         int gi = c0 / D, rem = c0 - gi * D;        // group of the first element, then stepped
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
@@ -1334,18 +1399,18 @@ static etr_status launch_bwd_dx(const etr_config* c, const void* X, const float*
                                (const T*)dXp_fused, (T*)dX, c->T, c->d, c->D, c->E, m, Cs);
     return ETR_OK;
   };
-  // chunked form of the fused kernel: as many tokens per block as keep cz, beside the 10.2 KiB of its row lists,
-  // within the 48 KiB a launch gets without opting in (at most 16)
-  constexpr size_t cz_max = 37 * 1024;
-  int tpb = DXC_MAX_TOKENS;
-  while (tpb > 2 && (size_t)tpb * m * sizeof(float) > cz_max) tpb /= 2;
-  // a short batch: fewer tokens, so that every SM has two blocks (512 tokens, d 256: 16.8 -> 10.9 us)
-  while (tpb > 2 && ceil_div(c->T, tpb) < 2 * current_sm_count()) tpb /= 2;
   int d_shift = 0;
   while ((1 << d_shift) < c->D) ++d_shift;
-  const bool group8 = c->D >= 8 && (1 << d_shift) == c->D;
-  if (dXp_fused && !ddelta && (size_t)tpb * m * sizeof(float) <= cz_max) {
-    const size_t csm = (size_t)tpb * m * sizeof(float);
+  const int gpv = (1 << d_shift) != c->D ? 0 : c->D >= 8 ? 1 : c->D == 4 ? 2 : 0;
+  // chunked form of the fused kernel: at most 16 tokens per block; where cz goes through shared memory as many as keep it,
+  // beside the 10.2 KiB of the row lists, within the 48 KiB a launch gets without opting in
+  constexpr size_t cz_max = 37 * 1024;
+  int tpb = DXC_MAX_TOKENS;
+  while (gpv == 0 && tpb > 2 && (size_t)tpb * m * sizeof(float) > cz_max) tpb /= 2;
+  // a short batch: fewer tokens, so that every SM has two blocks (512 tokens, d 256: 16.8 -> 10.9 us)
+  while (tpb > 2 && ceil_div(c->T, tpb) < 2 * current_sm_count()) tpb /= 2;
+  const size_t csm = gpv == 0 ? (size_t)tpb * m * sizeof(float) : 0;
+  if (dXp_fused && !ddelta && csm <= cz_max) {
     ETR_TIME_BEGIN("affinity_bwd_dx_fused_kernel");
     auto go = [&](auto k) {
       launch_kernel(k, ceil_div(c->T, tpb), 256, csm, st, 1, (const T*)X, R, delta, xnorm, rnorm, rt->tok_ptr, rt->tok_row, dgate,
@@ -1353,11 +1418,13 @@ static etr_status launch_bwd_dx(const etr_config* c, const void* X, const float*
                                                d_shift);
     };
     if (c->d % 16 == 0) {
-      if (group8) go(affinity_bwd_dx_chunk_kernel<T, 2, true>);
-      else go(affinity_bwd_dx_chunk_kernel<T, 2, false>);
+      if (gpv == 1) go(affinity_bwd_dx_chunk_kernel<T, 2, 1>);
+      else if (gpv == 2) go(affinity_bwd_dx_chunk_kernel<T, 2, 2>);
+      else go(affinity_bwd_dx_chunk_kernel<T, 2, 0>);
     } else {
-      if (group8) go(affinity_bwd_dx_chunk_kernel<T, 1, true>);
-      else go(affinity_bwd_dx_chunk_kernel<T, 1, false>);
+      if (gpv == 1) go(affinity_bwd_dx_chunk_kernel<T, 1, 1>);
+      else if (gpv == 2) go(affinity_bwd_dx_chunk_kernel<T, 1, 2>);
+      else go(affinity_bwd_dx_chunk_kernel<T, 1, 0>);
     }
   } else if (dXp_fused) {
     if (ddelta) ETR_TRY(launch(affinity_bwd_dx_kernel<T, true, true>, "affinity_bwd_dx_fused_kernel"));
