@@ -27,6 +27,7 @@
 // mbarriers are bounded; on expiry the kernel records a code in etr_stats.error_word,
 // stops issuing work, releases its tensor memory and returns.
 #include <algorithm>
+#include <cstring>
 
 #include "common.cuh"
 #include "tcgen05_ptx.cuh"
@@ -40,7 +41,7 @@ constexpr int TC_THREADS = 320;        // TMA warp, MMA warp, 8 epilogue warps
 constexpr uint32_t TC_BOX_BYTES = 64 * 64 * 2;
 constexpr long long TC_WAIT_LIMIT_CYCLES = ETR_WAIT_LIMIT_CYCLES;
 
-enum { TC_EPI_STORE = 0, TC_EPI_SWIGLU = 1, TC_EPI_DSWIGLU = 2 };
+enum { TC_EPI_STORE = 0, TC_EPI_SWIGLU = 1, TC_EPI_DSWIGLU = 2, TC_EPI_DSWIGLU_BOX = 3 };      // the last: pair form only
 enum { TC_DYN_M = 1, TC_DYN_K = 2 };
 
 struct TcParams {
@@ -220,6 +221,22 @@ __device__ __forceinline__ void load32_warp_turn(uint8_t* scratch, int lane, con
   for (int q = 0; q < 4; ++q)
     mine[q] = *reinterpret_cast<const uint4*>(scratch + lane * TC_SCRATCH_ROW_BYTES + q * 16);
   __syncwarp();
+}
+
+// dG and dU of two adjacent elements, in the place of the bf16 pairs of G and U.
+__device__ __forceinline__ void dswiglu_pair(float dh0, float dh1, uint32_t& gw, uint32_t& uw) {
+  const float dh[2] = {dh0, dh1};
+  const float g[2] = {__uint_as_float(gw << 16), __uint_as_float(gw & 0xffff0000u)};
+  const float u[2] = {__uint_as_float(uw << 16), __uint_as_float(uw & 0xffff0000u)};
+  float dg[2], du[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float sgm = __fdividef(1.0f, 1.0f + __expf(-g[k]));
+    dg[k] = dh[k] * u[k] * sgm * (1.0f + g[k] * (1.0f - sgm));
+    du[k] = dh[k] * g[k] * sgm;
+  }
+  gw = pack_bf16(dg[0], dg[1]);
+  uw = pack_bf16(du[0], du[1]);
 }
 
 // The epilogue of one accumulator tile for one warp: `nch` chunks of 32 columns starting at
@@ -639,39 +656,89 @@ __device__ __forceinline__ bool tile_coord_pair(const TcParams& p, const int* ti
 // and run-time branches cost there even when not taken (6-8 % of a GEMM for the operand modes,
 // 10 % per gather branch).  CFG = -1 keeps the run-time forms for combinations without an
 // instantiation of their own.
+// A second epilogue of the SwiGLU derivative (TC_EPI_DSWIGLU_BOX): G and U of a chunk of 32 columns come by TMA into a box of
+// the warp's own (32 rows of 64 bytes each, 64-byte swizzle), a lane turns its row into dG and dU in place, and TMA stores the
+// boxes.  Two boxes of each per warp: a chunk's load passes under the chunk before.  The other one fetches and stores through a
+// scratch, two more passes over shared memory for each of the four tensors, and 3000 cycles a chunk.  The boxes cost a stage of the
+// ring (five instead of six), which long contractions miss more than they gain (fetching bounds them: three stages 279, four 250,
+// five 234 us against 223 with the scratch and six at d 2048, E 128, h 768).  So below d = 2048: 89 -> 68 us at d 1024 (E 16, h 2816, 512
+// rows), 60 -> 48 at d 1088, 20 -> 17 and 17 -> 14 at d 512; at d 2048 (h 1408) 177 -> 179 with 1024 rows, 170 -> 169 with 769.
+constexpr int DSW_BOX_MAX_K = 2048;
+constexpr uint32_t DSW_BOX = 32 * 64, DSW_SLOT = 2 * DSW_BOX;      // G and U of a chunk
+struct DswMaps { CUtensorMap G, U, dG, dU; };
+// Ring and epilogue space of the pair form, and behind them what would otherwise be static shared memory: without any, the
+// dynamic block starts at a multiple of 1024, and five stages, the boxes and this are all a CTA may have.
+template <int EPI> struct PairRing {
+  static constexpr int STAGES = EPI == TC_EPI_DSWIGLU_BOX ? 5 : TC2_STAGES;
+  static constexpr uint32_t TAIL = STAGES * TC2_STAGE_BYTES + (EPI == TC_EPI_DSWIGLU_BOX ? 8 * 2 * DSW_SLOT : 8 * TC_SCRATCH_BYTES);
+};
+struct PairShared {
+  uint64_t bars[30];         // 2 STAGES + 4, the boxes' 16 more
+  uint32_t tmem_base_slot;
+  int abort_flag;
+  int tile_prefix[257];
+  int counts[256];           // the experts' row counts, read from global memory once
+};
+constexpr size_t PAIR_SLACK = 768;
+__device__ __forceinline__ uint32_t dsw_addr(uint32_t box, int lane, int c) {      // 16-byte piece c of this lane's row
+  return box + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4);
+}
+__device__ __forceinline__ void dsw_load(const DswMaps& m, uint32_t slot, uint32_t bar, int col, int row, int e) {      // one lane
+  mbar_expect_tx(bar, DSW_SLOT);
+  tma_load_3d(slot, &m.G, bar, col, row, e);
+  tma_load_3d(slot + DSW_BOX, &m.U, bar, col, row, e);
+}
+__device__ __forceinline__ void dsw_store(const DswMaps& m, uint32_t slot, int col, int row, int e) {                   // one lane
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4}], [%1];"
+               ::"l"(&m.dG), "r"(slot), "r"(col), "r"(row), "r"(e) : "memory");
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4}], [%1];"
+               ::"l"(&m.dU), "r"(slot + DSW_BOX), "r"(col), "r"(row), "r"(e) : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void lds128(uint32_t a, uint32_t* w) {
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void sts128(uint32_t a, const uint32_t* w) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+}
+
 template <int EPI, int GATHER, int CFG>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
                             const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
-                            const TcParams p) {
+                            const TcParams p, const __grid_constant__ DswMaps em) {
   constexpr int BN = 256;
   constexpr int N_TILE_COLS = (EPI == TC_EPI_SWIGLU) ? BN / 2 : BN;
   constexpr uint32_t TMEM_COLS = 512;
+  constexpr int STAGES = PairRing<EPI>::STAGES;
   // operand modes as compile-time constants when CFG >= 0 (bit 0 a_mn, 1 b_mn, 2 dual_b, 3 two K ranges)
   const bool A_MN = CFG < 0 ? p.a_mn != 0 : (CFG & 1) != 0, B_MN = CFG < 0 ? p.b_mn != 0 : (CFG & 2) != 0;
   const bool DUAL_B = CFG < 0 ? p.dual_b != 0 : (CFG & 4) != 0, TWO_K = CFG < 0 ? p.k1_blocks > 0 : (CFG & 8) != 0;
 
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2 * TC2_STAGES + 4];
-  __shared__ uint32_t tmem_base_slot;
-  __shared__ int abort_flag_s;
-  __shared__ int tile_prefix[257];
-  __shared__ int s_counts[256];      // the experts' row counts, read from global memory once
+  const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  PairShared& sh = *reinterpret_cast<PairShared*>(smem_raw + (tiles_base - smem_u32(smem_raw)) + PairRing<EPI>::TAIL);
+  uint64_t* bars = sh.bars;
+  uint32_t& tmem_base_slot = sh.tmem_base_slot;
+  int& abort_flag_s = sh.abort_flag;
+  int* tile_prefix = sh.tile_prefix;
+  int* s_counts = sh.counts;
 
   volatile int* abort_flag = &abort_flag_s;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = cluster_ctarank();
   const int pair = (int)cluster_id_x(), npairs = (int)cluster_count_x();
-  const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t full_bar = smem_u32(&bars[0]);                    // [TC2_STAGES]  used in the leader
-  const uint32_t empty_bar = smem_u32(&bars[TC2_STAGES]);          // [TC2_STAGES]  in each CTA
-  const uint32_t tfull_bar = smem_u32(&bars[2 * TC2_STAGES]);      // [2]           in each CTA
-  const uint32_t tempty_bar = smem_u32(&bars[2 * TC2_STAGES + 2]); // [2]           used in the leader
+  const uint32_t full_bar = smem_u32(&bars[0]);                    // [STAGES]  used in the leader
+  const uint32_t empty_bar = smem_u32(&bars[STAGES]);          // [STAGES]  in each CTA
+  const uint32_t tfull_bar = smem_u32(&bars[2 * STAGES]);      // [2]           in each CTA
+  const uint32_t tempty_bar = smem_u32(&bars[2 * STAGES + 2]); // [2]           used in the leader
 
   if (tid == 0) {
     abort_flag_s = 0;
-    for (int s = 0; s < TC2_STAGES; ++s) { mbar_init(full_bar + 8 * s, 1); mbar_init(empty_bar + 8 * s, 1); }
+    for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar + 8 * s, 1); mbar_init(empty_bar + 8 * s, 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar + 8 * a, 1); mbar_init(tempty_bar + 8 * a, 16); }
+    if (EPI == TC_EPI_DSWIGLU_BOX)
+      for (int b = 0; b < 16; ++b) mbar_init(smem_u32(&bars[2 * STAGES + 4 + b]), 1);      // a box pair has landed, two per epilogue warp
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -745,7 +812,7 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
             }
           }
           rows_b = rows_next;
-          if (++stage == TC2_STAGES) { stage = 0; phase ^= 1u; }
+          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
     }
@@ -781,7 +848,7 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
             tc_mma_pair(d_tmem, ad, bd, p.idesc, (kb > 0 || kk > 0) ? 1u : 0u);
           }
           tc_commit_pair(empty_bar + 8 * stage);      // frees the stage in both CTAs
-          if (++stage == TC2_STAGES) { stage = 0; phase ^= 1u; }
+          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
         if (PEEL && ok) {
           if (!mbar_wait_cluster(full_bar + 8 * stage, phase, abort_flag, p.wait_limit)) { ok = false; break; }
@@ -797,7 +864,7 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
             }
           }
           tc_commit_pair(empty_bar + 8 * stage);
-          if (++stage == TC2_STAGES) { stage = 0; phase ^= 1u; }
+          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
         tc_commit_pair(tfull_bar + 8 * acc_stage);    // accumulators complete in both CTAs
@@ -807,12 +874,12 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
   } else {
     // ---- epilogue warps (both CTAs, own 128 rows) -----------------------------------------------------
     const int q = warp & 3;
-    uint8_t* scratch = smem_raw + (tiles_base - smem_u32(smem_raw)) + TC2_STAGES * TC2_STAGE_BYTES + (warp - 2) * TC_SCRATCH_BYTES;
+    uint8_t* scratch = smem_raw + (tiles_base - smem_u32(smem_raw)) + STAGES * TC2_STAGE_BYTES + (warp - 2) * TC_SCRATCH_BYTES;
     const int half = (warp - 2) >> 2;
     constexpr int NCH = N_TILE_COLS / 32 / 2;
     const int row_in_tile = 128 * (int)rank + 32 * q + lane;
     int e_cur = 0, acc_stage = 0;
-    uint32_t acc_phase = 0;
+    uint32_t acc_phase = 0, box_phase = 0;
     TileCoord tc;
     bool ok = true;
     for (int tile = pair; ok && tile_coord_pair(p, tile_prefix, s_counts, tile, e_cur, N_TILE_COLS, tc); tile += npairs) {
@@ -826,8 +893,67 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
           store_zero_block(p, obase - (long long)lane * p.ld_out + 32 * c, lane, nz);
         continue;
       }
-      uint4 pg[4], pu[4];
       const int nvalid = min(32, max(0, tc.m_lim - (grow - lane)));
+      if constexpr (EPI == TC_EPI_DSWIGLU_BOX) {
+        const int row = grow - lane, col = tc.n0 + 32 * c_beg;
+        const int nch = nvalid > 0 ? min(NCH, (p.N - col + 31) / 32) : 0;      // N is a multiple of 64
+        const uint32_t slots = tiles_base + STAGES * TC2_STAGE_BYTES + (uint32_t)(warp - 2) * 2 * DSW_SLOT;
+        const uint32_t lbar = smem_u32(&bars[2 * STAGES + 4 + 2 * (warp - 2)]);
+        if (lane == 0) {
+          asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");      // the last tile's boxes have been read
+          for (int c = 0; c < min(nch, 2); ++c) dsw_load(em, slots + c * DSW_SLOT, lbar + 8 * c, col + 32 * c, row, tc.e);
+        }
+        __syncwarp();
+        ok = __all_sync(0xffffffffu, mbar_wait_cluster(tfull_bar + 8 * acc_stage, acc_phase, abort_flag, p.wait_limit));
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t taddr = tmem_base + (uint32_t)(acc_stage * 256 + 32 * c_beg) + ((uint32_t)(32 * q) << 16);
+        for (int c = 0; c < nch; ++c) {
+          const int b = c & 1;
+          const uint32_t slot = slots + b * DSW_SLOT;
+          uint32_t r0[32], gw[16], uw[16];
+          tc_ld32(taddr + 32 * c, r0);
+          ok = __all_sync(0xffffffffu, mbar_wait(lbar + 8 * b, (box_phase >> b) & 1u, abort_flag, p.wait_limit));
+          if (!ok) break;
+          box_phase ^= 1u << b;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            lds128(dsw_addr(slot, lane, i), gw + 4 * i);
+            lds128(dsw_addr(slot + DSW_BOX, lane, i), uw + 4 * i);
+          }
+          tc_wait_ld();
+          if (c + 1 == nch) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(leader_tempty + 8 * acc_stage);
+          }
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            dswiglu_pair(__uint_as_float(r0[2 * i]), __uint_as_float(r0[2 * i + 1]), gw[i], uw[i]);
+          if (c >= 1 && c + 1 < nch && lane == 0) {      // the other slot has been stored a chunk ago
+            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            dsw_load(em, slots + (b ^ 1) * DSW_SLOT, lbar + 8 * (b ^ 1), col + 32 * (c + 1), row, tc.e);
+          }
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            sts128(dsw_addr(slot, lane, i), gw + 4 * i);
+            sts128(dsw_addr(slot + DSW_BOX, lane, i), uw + 4 * i);
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) dsw_store(em, slot, col + 32 * c, row, tc.e);
+        }
+        if (!ok) break;
+        if (nch == 0) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(leader_tempty + 8 * acc_stage);
+        }
+        if (++acc_stage == 2) { acc_stage = 0; acc_phase ^= 1u; }
+        continue;
+      }
+      uint4 pg[4], pu[4];
       if (EPI == TC_EPI_DSWIGLU && tc.n0 + 32 * c_beg < p.N) {
         const long long wb = obase - (long long)lane * p.ld_out + 32 * c_beg;
         load32_warp_issue(p.in0 + wb, p.ld_out, lane, nvalid, pg);
@@ -874,6 +1000,7 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
       }
       if (++acc_stage == 2) { acc_stage = 0; acc_phase ^= 1u; }
     }
+    if (EPI == TC_EPI_DSWIGLU_BOX && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   }
 
   // ---- teardown: neither CTA leaves while the other may still touch its barriers or memory -------
@@ -1950,6 +2077,20 @@ static etr_status make_gather_map(CUtensorMap* m, const void* base, int cols, in
   return r == CUDA_SUCCESS ? ETR_OK : ETR_ERR_CUDA;
 }
 
+// Row-major bf16 tensor [E, rows, cols] in boxes of 32 rows x 32 columns, 64-byte swizzle.
+static etr_status make_map_chunks(CUtensorMap* m, const void* base, int cols, int rows, int E) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return ETR_ERR_CUDA;
+  const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)E};
+  const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * 2 * (cuuint64_t)rows};
+  const cuuint32_t box[3] = {32, 32, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? ETR_OK : ETR_ERR_CUDA;
+}
+
 static uint32_t make_idesc(int a_mn, int b_mn, int n, int m_instr = TC_BM) {
   uint32_t d = 0;
   d |= 1u << 4;                     // accumulator fp32
@@ -1984,15 +2125,24 @@ template <int EPI, int GATHER, int CFG>
 static etr_status tc_launch_pair_cfg(const char* name, const CUtensorMap& a0, const CUtensorMap& a1,
                                  const CUtensorMap& b0, const CUtensorMap& b1, TcParams p, int max_tiles,
                                  cudaStream_t st) {
-  constexpr size_t smem = (size_t)TC2_STAGES * TC2_STAGE_BYTES + 1024 + 8 * TC_SCRATCH_BYTES;
+  constexpr size_t smem = PairRing<EPI>::TAIL + sizeof(PairShared) + PAIR_SLACK;
+  static_assert(smem <= 232448 && 2 * PairRing<EPI>::STAGES + 4 + (EPI == TC_EPI_DSWIGLU_BOX ? 16 : 0) <= 30, "shared memory of a CTA");
   auto k = tc_grouped_gemm_pair_kernel<EPI, GATHER, CFG>;
   static std::atomic<unsigned long long> attr_done{0};      // one bit per device
   if (!ensure_dyn_smem(k, smem, attr_done)) return ETR_ERR_CUDA;
   p.idesc = make_idesc(p.a_mn, p.b_mn, 256, 256);
+  DswMaps em;
+  memset(&em, 0, sizeof(em));
+  if (EPI == TC_EPI_DSWIGLU_BOX) {
+    ETR_TRY(make_map_chunks(&em.G, p.in0, p.N, p.M, p.E));
+    ETR_TRY(make_map_chunks(&em.U, p.in1, p.N, p.M, p.E));
+    ETR_TRY(make_map_chunks(&em.dG, p.out0, p.N, p.M, p.E));
+    ETR_TRY(make_map_chunks(&em.dU, p.out1, p.N, p.M, p.E));
+  }
   const int pairs_max = sm_count() / 2;
   const int pairs = max_tiles < pairs_max ? (max_tiles < 1 ? 1 : max_tiles) : pairs_max;
   ETR_TIME_BEGIN(name);
-  launch_kernel(k, 2 * pairs, TC_THREADS, smem, st, 2, a0, a1, b0, b1, p);
+  launch_kernel(k, 2 * pairs, TC_THREADS, smem, st, 2, a0, a1, b0, b1, p, em);
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }
@@ -2022,7 +2172,7 @@ static etr_status tc_launch_pair(const char* name, const CUtensorMap& a0, const 
                                  const CUtensorMap& b0, const CUtensorMap& b1, TcParams p, int max_tiles,
                                  cudaStream_t st) {
   const int cfg = (p.a_mn ? 1 : 0) | (p.b_mn ? 2 : 0) | (p.dual_b ? 4 : 0) | (p.k1_blocks > 0 ? 8 : 0);
-  constexpr int C0 = EPI == TC_EPI_SWIGLU ? 4 : EPI == TC_EPI_DSWIGLU ? 2 : 0;      // first use
+  constexpr int C0 = EPI == TC_EPI_SWIGLU ? 4 : EPI == TC_EPI_STORE ? 0 : 2;      // first use
   constexpr int C1 = EPI == TC_EPI_STORE && GATHER == 2 ? 3 : C0, C2 = EPI == TC_EPI_STORE ? 10 : C0;
   if (cfg == C0) return tc_launch_pair_cfg<EPI, GATHER, C0>(name, a0, a1, b0, b1, p, max_tiles, st);
   if (cfg == C1) return tc_launch_pair_cfg<EPI, GATHER, C1>(name, a0, a1, b0, b1, p, max_tiles, st);
@@ -2081,6 +2231,8 @@ static etr_status tc_run(TcForm form, const char* name, const CUtensorMap& a0, c
     if (EPI == TC_EPI_STORE && p.gather == 2)
       return tc_launch_pair<EPI, EPI == TC_EPI_STORE ? 2 : 0>(name, a0, a1, b0, b1, p, (max_tiles + 1) / 2, st);
     if (p.gather) return ETR_ERR_UNSUPPORTED;
+    if (EPI == TC_EPI_DSWIGLU && p.K < DSW_BOX_MAX_K)
+      return tc_launch_pair<EPI == TC_EPI_DSWIGLU ? TC_EPI_DSWIGLU_BOX : EPI, 0>(name, a0, a1, b0, b1, p, (max_tiles + 1) / 2, st);
     return tc_launch_pair<EPI, 0>(name, a0, a1, b0, b1, p, (max_tiles + 1) / 2, st);
   }
   if (p.gather) return ETR_ERR_UNSUPPORTED;
