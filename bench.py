@@ -38,7 +38,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu captures summarised
 # under profiles/ (absent: not captured for the current version of that kernel).
 NCU_TRAFFIC_BYTES = {}
-# The grouped GEMMs as AUTO launches them at the mid workload (d = 2048), all 7 launches of one step
+# The grouped GEMMs of one step at the mid workload (d = 2048)
 # (profiles/tc_grouped_gemm_mid_ncu.md): 3636.2 MB of DRAM traffic against 3799.7 MB of algorithmic bytes
 # (part of the output is still in L2 when a kernel ends).  The large workload is too big for a
 # multi-pass capture, so its traffic is this ratio times its own algorithmic bytes.
@@ -46,7 +46,7 @@ TC_GEMM_DRAM_OVER_ALGORITHMIC = 3636.2 / 3799.7
 
 
 def tc_gemm_algorithmic_bytes(w, rows_padded):
-    """Bytes the seven grouped GEMMs of one step must move (bf16): activations once per use, every
+    """Bytes the seven contractions of one step must move (bf16): activations once per use, every
     expert weight once per GEMM that reads it, every output once."""
     ad, ah, wt = rows_padded * w.d * 2, rows_padded * w.h * 2, w.E * w.d * w.h * 2
     reads = (ad + 2 * wt) + (ah + wt) + (ad + wt + 2 * ah) + (2 * ah + 2 * wt) + (ad + ah) + 2 * (ah + ad)
