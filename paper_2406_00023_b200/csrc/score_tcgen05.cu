@@ -101,6 +101,37 @@ affinity_score_tc_kernel(const __grid_constant__ CUtensorMap mapZ, const __grid_
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(SCT_TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // ||R_i|| by the epilogue warps, a warp per row, lanes over the columns, the same sums as the other score kernels (eight
+  // columns per lane and four rows requested together).  With up to 32 experts before the wait: the kernel before this one is
+  // always the pooling of the same call, which does not write R and had waited itself, so whatever did write R is complete.
+  // More rows take longer than that kernel leaves: behind the wait, while the first tile is on its way.
+  // Together with half of the epilogue left out there: 9.0 -> 7.2 us (64 tokens, E 16, m 128), 8.5 -> 5.6 (512, E 8, m 64), 12.1 -> 9.7
+  // (6113, E 32, m 256); with 64 experts before the wait instead 10.1 -> 11.7 (300 tokens).
+  auto norms = [&]() {
+    for (int i0 = warp & 3; i0 < E; i0 += 16) {
+      float sq[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int j0 = lane; j0 < m; j0 += 256) {
+        float v[4][8];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            v[r][u] = i0 + 4 * r < E && j0 + 32 * u < m ? R[(size_t)(i0 + 4 * r) * m + j0 + 32 * u] : 0.f;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int u = 0; u < 8; ++u) sq[r] += v[r][u] * v[r][u];
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float acc_q = warp_sum(sq[r]);
+        if (lane == 0) rn[i0 + 4 * r] = sqrtf(acc_q);
+      }
+    }
+  };
+  const bool early = E <= 32;
+  if (early && warp >= 6) norms();
+  __syncwarp();
   grid_wait();
   tc_fence_before();
   __syncthreads();
@@ -191,36 +222,11 @@ affinity_score_tc_kernel(const __grid_constant__ CUtensorMap mapZ, const __grid_
     // ---- epilogue warps: a lane owns a token --------------------------------------------------------------
     const int q = warp & 3;                      // tensor-memory lanes 32 q .. 32 q + 31
     float* stg = reinterpret_cast<float*>(tiles + (size_t)SCT_STAGES * SCT_STAGE_BYTES) + (warp - 6) * 32 * 33;
-    // ||R_i|| while the first tile is on its way: a warp per row, lanes over the columns, the same sums
-    // as the other score kernels (eight columns per lane requested together)
-    // (and four rows of a warp: a row at a time is a round of L2 latency each, sixteen of them at E = 64)
-    for (int i0 = q; i0 < SCT_N; i0 += 16) {
-      float sq[4] = {0.f, 0.f, 0.f, 0.f};
-      if (i0 < E) {
-        for (int j0 = lane; j0 < m; j0 += 256) {
-          float v[4][8];
-#pragma unroll
-          for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-              v[r][u] = i0 + 4 * r < E && j0 + 32 * u < m ? R[(size_t)(i0 + 4 * r) * m + j0 + 32 * u] : 0.f;
-#pragma unroll
-          for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int u = 0; u < 8; ++u) sq[r] += v[r][u] * v[r][u];
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int i = i0 + 4 * r;
-        const float acc_q = warp_sum(sq[r]);
-        if (lane == 0) {
-          rn[i] = sqrtf(acc_q);
-          if (blockIdx.x == 0 && i < E) rnorm[i] = rn[i];
-        }
-      }
+    if (!early) {
+      norms();
+      asm volatile("bar.sync 1, 128;" ::: "memory");      // the four epilogue warps: rn is complete
     }
-    asm volatile("bar.sync 1, 128;" ::: "memory");      // the four epilogue warps: rn is complete
+    if (blockIdx.x == 0 && tid - 192 < E) rnorm[tid - 192] = rn[tid - 192];      // 128 threads, E <= 64
     int acc = 0;
     uint32_t acc_phase = 0;
     float best = -INFINITY;
@@ -231,49 +237,48 @@ affinity_score_tc_kernel(const __grid_constant__ CUtensorMap mapZ, const __grid_
       if (!mbar_wait(tfull_bar + 8 * acc, acc_phase, abort_flag, wait_limit)) { ok = false; break; }
       tc_fence_after();
       const uint32_t taddr = tmem_base + (uint32_t)(acc * SCT_CHAINS * SCT_N) + ((uint32_t)(32 * q) << 16);
-      uint32_t r[SCT_N];
-      tc_ld32(taddr, r);
-      tc_ld32(taddr + 32, r + 32);
-      tc_wait_ld();
+      // Half of the expert columns at a time (the upper half only where there are that many experts): the chains' partial
+      // sums added in order, then delta = sqrt(D) s / (||x|| ||R_i||), 0 where a norm is 0.  A fast division (reciprocal and
+      // product, 2 ulp) taken unconditionally and selected afterwards: correctly rounded divisions, each behind its own zero
+      // test, overlapped with nothing and were the longest stage of the kernel; the result is compared at 1e-5, not to the
+      // last bit.
+      // Store: a lane holds a token's row, but 32 lanes writing 32 different rows would send 16 bytes per sector.  The warp
+      // turns 32 x 32 blocks through its staging tile (row stride 33 words: no bank conflicts either way) and writes 128
+      // contiguous bytes of one token per instruction.
+      const int t_warp = tile * SCT_BM + 32 * q, nrow = min(32, Ttok - t_warp);
+#pragma unroll 1
+      for (int half = 0; 32 * half < E; ++half) {
+        uint32_t r[32];
+        {
+          uint32_t p[SCT_CHAINS][32];
 #pragma unroll
-      for (int ch = 1; ch < SCT_CHAINS; ++ch) {      // the partial sums of the other accumulators, added in order
-        uint32_t p[SCT_N];
-        tc_ld32(taddr + ch * SCT_N, p);
-        tc_ld32(taddr + ch * SCT_N + 32, p + 32);
-        tc_wait_ld();
+          for (int ch = 0; ch < SCT_CHAINS; ++ch) tc_ld32(taddr + ch * SCT_N + 32 * half, p[ch]);
+          tc_wait_ld();
+          if (32 * half + 32 >= E) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(tempty_bar + 8 * acc);      // the values are in registers
+          }
 #pragma unroll
-        for (int i = 0; i < SCT_N; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) + __uint_as_float(p[i]));
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(tempty_bar + 8 * acc);      // the values are in registers
-      // scale: delta = sqrt(D) s / (||x|| ||R_i||), 0 where a norm is 0.  A fast division (reciprocal and product,
-      // 2 ulp) taken unconditionally and selected afterwards: 64 correctly rounded divisions per token, each behind
-      // its own zero test, overlapped with nothing and were the longest stage of the kernel; the result is
-      // compared at 1e-5, not to the last bit.
+          for (int i = 0; i < 32; ++i) {
+            float v = __uint_as_float(p[0][i]);
 #pragma unroll
-      for (int i = 0; i < SCT_N; ++i) {
-        const float den = xn * rn[i];
-        const float quot = __fdividef(sqD * __uint_as_float(r[i]), den);
-        const float v = den == 0.f ? 0.f : quot;
-        r[i] = __float_as_uint(v);
-        if (i < E && t < Ttok) best = fmaxf(best, v);
-      }
-      // store: a lane holds a token's row, but 32 lanes writing 32 different rows would send 16 bytes per
-      // sector.  The warp turns 32 x 32 blocks through its staging tile (row stride 33 words: no bank
-      // conflicts either way) and writes 128 contiguous bytes of one token per instruction.
-      const int t_warp = tile * SCT_BM + 32 * q;
+            for (int ch = 1; ch < SCT_CHAINS; ++ch) v += __uint_as_float(p[ch][i]);
+            const float den = xn * rn[32 * half + i];
+            const float quot = __fdividef(sqD * v, den);
+            const float dl = den == 0.f ? 0.f : quot;
+            r[i] = __float_as_uint(dl);
+            if (32 * half + i < E && t < Ttok) best = fmaxf(best, dl);
+          }
+        }
+        __syncwarp();
 #pragma unroll
-      for (int half = 0; half < SCT_N / 32; ++half) {
-        if (32 * half < E) {
-          __syncwarp();
-#pragma unroll
-          for (int j = 0; j < 32; ++j) stg[lane * 33 + j] = __uint_as_float(r[32 * half + j]);
-          __syncwarp();
-          const int i = 32 * half + lane;
-          const int nrow = min(32, Ttok - t_warp);
-          for (int rr = 0; rr < nrow; ++rr)
-            if (i < E) delta[(size_t)(t_warp + rr) * E + i] = stg[rr * 33 + lane];
+        for (int j = 0; j < 32; ++j) stg[lane * 33 + j] = __uint_as_float(r[j]);
+        __syncwarp();
+        const int i = 32 * half + lane;
+        if (i < E) {
+#pragma unroll 4
+          for (int rr = 0; rr < nrow; ++rr) delta[(size_t)(t_warp + rr) * E + i] = stg[rr * 33 + lane];
         }
       }
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
