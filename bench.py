@@ -104,8 +104,7 @@ def algorithmic_work(w, rows, kernel, unrouted=0):
         "tf32x3_gemm_down": (2 * rows * d * h, "flops"),
         "tf32x3_gemm_dswiglu": (2 * rows * d * h, "flops"),
         "tf32x3_gemm_dxp": (4 * rows * d * h, "flops"),
-        "tf32x3_gemm_dw2": (2 * rows * d * h, "flops"),
-        "tf32x3_gemm_dw1": (4 * rows * d * h, "flops"),
+        "tf32x3_gemm_dw": (6 * rows * d * h, "flops"),
         # tcgen05 grouped GEMMs: selected rows only (not the rows padding a 128-row tile)
         "tc_gemm_swiglu": (4 * rows * d * h, "flops"),
         "tc_gemm_down": (2 * rows * d * h, "flops"),

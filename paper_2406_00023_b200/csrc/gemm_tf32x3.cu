@@ -14,7 +14,7 @@
 // therefore end a chain after two MMAs: 0.6e-7 short, that layer 7.1e-7, 158 -> 161 us.  (For all of them that would be
 // 651 -> 739 us at T 1531, d 768, h 1000; four MMAs are already below the FMAs there.  Chains of eight: 2.0e-7.)
 //
-// One persistent kernel serves the six contractions.  Roles in a CTA of 640 threads:
+// One persistent kernel serves the six contractions (the three weight gradients in one launch).  Roles in a CTA of 640 threads:
 //   warp 0       TMA: a K block arrives as plain fp32 in the place of its hi tiles
 //   warp 1       issues the MMAs (kind::tf32, 128 x 2 BN and 128 x BN, 8 values of K each)
 //   warps 4-11   split a block into hi (in place) and lo, both K-major with the 128-byte swizzle, in two groups of
@@ -47,7 +47,8 @@ static_assert(128 * F3_REGS_IO + 256 * F3_REGS_CONV + 256 * F3_REGS_EPI <= F3_TH
 constexpr int F3_SHORT_WIDTH = 384, F3_SHORT_ROWS = 256;
 constexpr int F3_SCRATCH = 32 * 80;              // per epilogue warp: 32 rows of 64 bytes, 16 bytes of pad each
 
-enum { F3_STORE = 0, F3_SWIGLU = 1, F3_DSWIGLU = 2 };
+// F3_WGRAD: the three weight gradients in one launch (plain stores; M = d and N = h of the first, exchanged for the others).
+enum { F3_STORE = 0, F3_SWIGLU = 1, F3_DSWIGLU = 2, F3_WGRAD = 3 };
 
 struct F3Params {
   int two_k;               // the first half of the K blocks from (A0, B0), the rest from (A1, B1); both ranges are K long
@@ -62,7 +63,7 @@ struct F3Params {
   long long wait_limit;
 };
 
-struct F3Tile { int e, m0, n0, K, kblocks, m_lim; };
+struct F3Tile { int e, m0, n0, K, kblocks, m_lim, N, which; };      // which: the gradient, 0 where there is one output
 
 __device__ __forceinline__ void f3_mma(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
   asm volatile(
@@ -139,17 +140,41 @@ __device__ __forceinline__ void f3_add16(f32x2* sum, const uint32_t* hh, const u
 __device__ __forceinline__ int f3_mtiles(const F3Params& p, int n_e) {
   return p.dyn_m ? (min((n_e + 127) & ~127, p.M) + F3_BM - 1) / F3_BM : (p.M + F3_BM - 1) / F3_BM;
 }
+// Tiles of an expert.
+template <int EPI>
+__device__ __forceinline__ int f3_tiles(const F3Params& p, int n_e, int cols) {
+  if (EPI != F3_WGRAD) return f3_mtiles(p, n_e) * ((p.N + cols - 1) / cols);
+  return (p.M + F3_BM - 1) / F3_BM * ((p.N + cols - 1) / cols) + 2 * ((p.N + F3_BM - 1) / F3_BM) * ((p.M + cols - 1) / cols);
+}
+template <int EPI>
 __device__ __forceinline__ bool f3_tile(const F3Params& p, const int* prefix, const int* counts, int tile, int& e_cur,
                                         int cols, F3Tile& t) {
   if (tile >= prefix[p.E]) return false;
   while (tile >= prefix[e_cur + 1]) ++e_cur;
-  const int local = tile - prefix[e_cur], n_e = counts[e_cur], mt = f3_mtiles(p, n_e);
+  int local = tile - prefix[e_cur], mt;
+  const int n_e = counts[e_cur];
   t.e = e_cur;
+  t.which = 0;
+  t.N = p.N;
+  if (EPI == F3_WGRAD) {
+    const int first = (p.M + F3_BM - 1) / F3_BM * ((p.N + cols - 1) / cols);
+    const int other = (p.N + F3_BM - 1) / F3_BM * ((p.M + cols - 1) / cols);
+    if (local >= first) {
+      local -= first;
+      t.which = local < other ? 1 : 2;
+      if (local >= other) local -= other;
+      t.N = p.M;
+    }
+    t.m_lim = t.which ? p.N : p.M;
+    mt = (t.m_lim + F3_BM - 1) / F3_BM;
+  } else {
+    mt = f3_mtiles(p, n_e);
+    t.m_lim = p.dyn_m ? min((n_e + 127) & ~127, p.M) : p.M;
+  }
   t.m0 = (local % mt) * F3_BM;
   t.n0 = (local / mt) * cols;
   t.K = p.dyn_m ? p.K : n_e;
   t.kblocks = (t.K + F3_BK - 1) / F3_BK * (p.two_k ? 2 : 1);
-  t.m_lim = p.dyn_m ? min((n_e + 127) & ~127, p.M) : p.M;
   return true;
 }
 
@@ -230,7 +255,7 @@ template <int EPI, bool A_MN, bool B_MN, int BN, int CHAIN>
 __global__ void __launch_bounds__(F3_THREADS, 1)
 tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
                    const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
-                   const F3Params p, uint32_t idesc) {
+                   const __grid_constant__ CUtensorMap mapA2, const F3Params p, uint32_t idesc) {
   constexpr int F3_STAGES = F3Ring<BN>::STAGES;
   constexpr int COLS = EPI == F3_SWIGLU ? BN / 2 : BN;               // output columns of a tile
   constexpr uint32_t A_BYTES = F3_BM * 128, B_BYTES = BN * 128;      // one of hi, lo
@@ -270,8 +295,7 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
   }
   grid_wait();
   if (warp == 2) {
-    const int nt = (p.N + COLS - 1) / COLS;
-    tile_prefix_warp(tile_prefix, s_counts, p.counts, p.E, lane, [&](int n_e) { return f3_mtiles(p, n_e) * nt; });
+    tile_prefix_warp(tile_prefix, s_counts, p.counts, p.E, lane, [&](int n_e) { return f3_tiles<EPI>(p, n_e, COLS); });
   }
   tc_fence_before();
   __syncthreads();
@@ -288,7 +312,7 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
       uint32_t phase = 0;
       F3Tile t;
       bool ok = true;
-      for (int tile = blockIdx.x; ok && f3_tile(p, tile_prefix, s_counts, tile, e_cur, COLS, t); tile += gridDim.x) {
+      for (int tile = blockIdx.x; ok && f3_tile<EPI>(p, tile_prefix, s_counts, tile, e_cur, COLS, t); tile += gridDim.x) {
         const int kb1 = p.two_k ? t.kblocks / 2 : t.kblocks;
         for (int kb = 0; kb < t.kblocks; ++kb) {
           ok = __all_sync(0xffffffffu, mbar_wait(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.wait_limit));
@@ -298,8 +322,9 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
             const int k0 = (second ? kb - kb1 : kb) * F3_BK;
             const uint32_t sa = tiles_base + stage * STAGE, sb = sa + 2 * A_BYTES, bar = full_bar + 8 * stage;
             mbar_expect_tx(bar, A_BYTES + B_BYTES);
-            f3_fetch<A_MN, F3_BM>(sa, second ? &mapA1 : &mapA0, bar, t.m0, k0, t.e);
-            f3_fetch<B_MN, B_ROWS>(sb, second ? &mapB1 : &mapB0, bar, t.n0, k0, t.e);
+            const bool alt = EPI == F3_WGRAD ? t.which != 0 : second;
+            f3_fetch<A_MN, F3_BM>(sa, EPI == F3_WGRAD && t.which == 2 ? &mapA2 : alt ? &mapA1 : &mapA0, bar, t.m0, k0, t.e);
+            f3_fetch<B_MN, B_ROWS>(sb, alt ? &mapB1 : &mapB0, bar, t.n0, k0, t.e);
             if (EPI == F3_SWIGLU) f3_fetch<B_MN, B_ROWS>(sb + B_BYTES / 2, &mapB1, bar, t.n0, k0, t.e);
           }
           __syncwarp();
@@ -313,7 +338,7 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
       uint32_t phase = 0, acc_phase = 0;
       F3Tile t;
       bool ok = true;
-      for (int tile = blockIdx.x; ok && f3_tile(p, tile_prefix, s_counts, tile, e_cur, COLS, t); tile += gridDim.x) {
+      for (int tile = blockIdx.x; ok && f3_tile<EPI>(p, tile_prefix, s_counts, tile, e_cur, COLS, t); tile += gridDim.x) {
         for (int kb = 0; kb < t.kblocks; ++kb) {
           ok = __all_sync(0xffffffffu, mbar_wait(conv_bar + 8 * stage, phase, abort_flag, p.wait_limit));
           const uint32_t a_hi = tiles_base + stage * STAGE, a_lo = a_hi + A_BYTES, b_hi = a_hi + 2 * A_BYTES;
@@ -353,7 +378,7 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
     uint32_t phase = 0;
     F3Tile t;
     bool ok = true;
-    for (int tile = blockIdx.x; ok && f3_tile(p, tile_prefix, s_counts, tile, e_cur, COLS, t); tile += gridDim.x) {
+    for (int tile = blockIdx.x; ok && f3_tile<EPI>(p, tile_prefix, s_counts, tile, e_cur, COLS, t); tile += gridDim.x) {
       for (int kb = 0; kb < t.kblocks; ++kb) {
         if (turn == group) {
           ok = __all_sync(0xffffffffu, mbar_wait(full_bar + 8 * stage, phase, abort_flag, p.wait_limit));
@@ -388,7 +413,7 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
     uint32_t acc_phase = 0;
     F3Tile t;
     bool ok = true;
-    for (int tile = blockIdx.x; ok && f3_tile(p, tile_prefix, s_counts, tile, e_cur, COLS, t); tile += gridDim.x) {
+    for (int tile = blockIdx.x; ok && f3_tile<EPI>(p, tile_prefix, s_counts, tile, e_cur, COLS, t); tile += gridDim.x) {
       f32x2 run[GW];                                                 // 2 GW running sums
 #pragma unroll
       for (int i = 0; i < GW; ++i) run[i] = 0ull;
@@ -414,7 +439,9 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
       }
       if (!ok) break;
       const int row0 = t.m0 + 32 * q, nvalid = min(32, t.m_lim - row0);
-      const long long wb = (long long)t.e * p.out_bs + (long long)row0 * p.ld_out;
+      const int ld_out = EPI == F3_WGRAD ? t.N : p.ld_out;
+      float* const out = EPI == F3_WGRAD && t.which ? (t.which == 1 ? p.out1 : p.out2) : p.out0;
+      const long long wb = (long long)t.e * p.out_bs + (long long)row0 * ld_out;
       float sum[2][GW];
 #pragma unroll
       for (int i = 0; i < GW; ++i) {
@@ -443,7 +470,7 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
 #pragma unroll
           for (int c = 0; c < GW; c += 16) {
             const int n = t.n0 + (g ? g1 : g0) + c;
-            if (n >= p.N) break;
+            if (n >= t.N) break;
             if (EPI == F3_DSWIGLU) {
               float du[16];
               const float4* G = reinterpret_cast<const float4*>(p.in0 + wb + (long long)lane * p.ld_out + n);
@@ -462,7 +489,7 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
               }
               f3_store16(scratch, lane, nvalid, p.N - n, p.out1 + wb + n, p.ld_out, du);
             }
-            f3_store16(scratch, lane, nvalid, p.N - n, p.out0 + wb + n, p.ld_out, &sum[g][c]);
+            f3_store16(scratch, lane, nvalid, t.N - n, out + wb + n, ld_out, &sum[g][c]);
           }
         }
       }
@@ -520,18 +547,24 @@ static etr_status f3_launch_bn(const char* name, const F3Operand* A, const F3Ope
     ETR_TRY(f3_map(&a[i], oa.ptr, oa.cols, oa.rows, p.E, A_MN ? F3_BK : F3_BM));
     ETR_TRY(f3_map(&b[i], ob.ptr, ob.cols, ob.rows, p.E, B_MN ? F3_BK : (EPI == F3_SWIGLU ? BN / 2 : BN)));
   }
+  CUtensorMap a2 = a[0];
+  if (EPI == F3_WGRAD) ETR_TRY(f3_map(&a2, A[2].ptr, A[2].cols, A[2].rows, p.E, F3_BK));
   ETR_TIME_BEGIN(name);
-  launch_kernel(k, std::max(1, std::min(max_tiles, current_sm_count())), F3_THREADS, smem, st, 1, a[0], a[1], b[0], b[1], p, idesc);
+  launch_kernel(k, std::max(1, std::min(max_tiles, current_sm_count())), F3_THREADS, smem, st, 1, a[0], a[1], b[0], b[1], a2, p, idesc);
   ETR_LAUNCH_CHECK();
   return ETR_OK;
 }
 // k_max: the longest contraction that the launch can hold.
 template <int EPI, bool A_MN, bool B_MN>
-static etr_status f3_launch(const char* name, const F3Operand (&A)[2], const F3Operand (&B)[2], const F3Params& p,
+static etr_status f3_launch(const char* name, const F3Operand* A, const F3Operand* B, const F3Params& p,
                             int tiles_m, int k_max, cudaStream_t st) {
   // 128-column tiles unless they leave SMs without one
   constexpr int C128 = EPI == F3_SWIGLU ? 64 : 128, C64 = C128 / 2;
-  const int t128 = tiles_m * ceil_div(p.N, C128), t64 = tiles_m * ceil_div(p.N, C64);
+  int t128 = tiles_m * ceil_div(p.N, C128), t64 = tiles_m * ceil_div(p.N, C64);
+  if (EPI == F3_WGRAD) {
+    t128 += 2 * p.E * ceil_div(p.N, F3_BM) * ceil_div(p.M, C128);
+    t64 += 2 * p.E * ceil_div(p.N, F3_BM) * ceil_div(p.M, C64);
+  }
   const bool wide = t128 >= current_sm_count();
   if (k_max <= (p.dyn_m ? F3_SHORT_WIDTH : F3_SHORT_ROWS))
     return wide ? f3_launch_bn<EPI, A_MN, B_MN, 128, 2>(name, A, B, p, t128, st)
@@ -585,19 +618,13 @@ etr_status tf32x3_ffn_backward(const etr_config* c, const etr_route* rt, const v
     p.two_k = 1; p.M = Cs; p.N = d; p.K = h; p.dyn_m = 1; p.out0 = (float*)dXp; p.out_bs = ldx; p.ld_out = d;
     ETR_TRY((f3_launch<F3_STORE, false, true>("tf32x3_gemm_dxp", A, B, p, mt, 2 * h, st)));
   }
-  {  // dW2 = dO^T H over the expert's rows
-    F3Params p = f3_params(c, rt, stats);
-    const F3Operand A[2] = {{dO, d, Cs}, {}}, B[2] = {{H, h, Cs}, {}};
-    p.M = d; p.N = h; p.out0 = (float*)dW2; p.out_bs = w; p.ld_out = h;
-    ETR_TRY((f3_launch<F3_STORE, true, true>("tf32x3_gemm_dw2", A, B, p, E * ceil_div(d, F3_BM), c->capacity, st)));
-  }
-  for (int which = 0; which < 2; ++which) {  // dW1g = dG^T Xp, dW1u = dU^T Xp
-    F3Params p = f3_params(c, rt, stats);
-    const F3Operand A[2] = {{which ? dU : dG, h, Cs}, {}}, B[2] = {{Xp, d, Cs}, {}};
-    p.M = h; p.N = d; p.out0 = (float*)(which ? dW1u : dW1g); p.out_bs = w; p.ld_out = d;
-    ETR_TRY((f3_launch<F3_STORE, true, true>("tf32x3_gemm_dw1", A, B, p, E * ceil_div(h, F3_BM), c->capacity, st)));
-  }
-  return ETR_OK;
+  // dW2 = dO^T H, dW1g = dG^T Xp, dW1u = dU^T Xp over the expert's rows, one launch: a launch each left its last (at 512 tokens
+  // its only) round of tiles part-filled and paid the head and the tail of a tile's chain three times.  30 -> 21 us at T 512, d 256,
+  // h 512, E 8; 152 -> 128 at T 1531, d 768, h 1000, E 12 (tiles of 64 columns up to two rounds of 128: the same).
+  F3Params p = f3_params(c, rt, stats);
+  const F3Operand A[3] = {{dO, d, Cs}, {dG, h, Cs}, {dU, h, Cs}}, B[2] = {{H, h, Cs}, {Xp, d, Cs}};
+  p.M = d; p.N = h; p.out0 = (float*)dW2; p.out1 = (float*)dW1g; p.out2 = (float*)dW1u; p.out_bs = w;
+  return f3_launch<F3_WGRAD, true, true>("tf32x3_gemm_dw", A, B, p, E * ceil_div(d, F3_BM), c->capacity, st);
 }
 
 }  // namespace etr
