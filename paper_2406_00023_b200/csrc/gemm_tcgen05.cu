@@ -1,6 +1,6 @@
 // Grouped GEMMs of the expert FFN on the 5th-generation tensor cores (bf16 in, fp32
 // accumulate in tensor memory).  One persistent, warp-specialised design serves all six
-// contractions of the forward and backward pass, in four tile forms:
+// contractions of the forward and backward pass, in four tile forms (and one more kernel):
 //
 //   tc_grouped_gemm_kernel            one CTA per 128 x 256 tile (cta_group::1), 4-stage ring
 //   tc_grouped_gemm_pair_kernel       a cluster of two CTAs per 256 x 256 tile (cta_group::2),
@@ -9,6 +9,7 @@
 //                                     share the A operand, 4-stage ring, halves released separately
 //   tc_grouped_gemm_swap_kernel       the pair form with the operands exchanged: 256 rows of the weights are M, up
 //                                     to 256 tokens (a multiple of 16) are N (contractions over d or h)
+//   tc_wgrad_pair_kernel              the pair form's weight gradients, all three in one launch
 //
 //   warp 0      TMA producer: 64x64-element boxes (128-byte swizzle) into the ring
 //   warp 1      allocates tensor memory, issues tcgen05.mma (the pair's leader CTA only)
