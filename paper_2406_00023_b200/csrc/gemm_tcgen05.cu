@@ -897,7 +897,9 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
       const int nvalid = min(32, max(0, tc.m_lim - (grow - lane)));
       if constexpr (EPI == TC_EPI_DSWIGLU_BOX) {
         const int row = grow - lane, col = tc.n0 + 32 * c_beg;
-        const int nch = nvalid > 0 ? min(NCH, (p.N - col + 31) / 32) : 0;      // N is a multiple of 64
+        // Chunks of this warp, none where its rows or its half of the columns are past the edge (N - col is then as low as
+        // -64, at N = 64 mod 256): never negative, the accumulator is given back below for none and at the last one else.
+        const int nch = nvalid > 0 ? min(NCH, (max(0, p.N - col) + 31) / 32) : 0;
         const uint32_t slots = tiles_base + STAGES * TC2_STAGE_BYTES + (uint32_t)(warp - 2) * 2 * DSW_SLOT;
         const uint32_t lbar = smem_u32(&bars[2 * STAGES + 4 + 2 * (warp - 2)]);
         if (lane == 0) {

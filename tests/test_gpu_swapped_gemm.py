@@ -23,10 +23,10 @@ def rel(got, ref):
     return float((got.double() - ref).norm()) / n if n else float(got.double().norm())
 
 
-def run(E, d, h, cap, counts, impl, grad_fp32=False):
+def run(E, d, h, cap, counts, impl, grad_fp32=False, wait_limit_cycles=0):
     g = torch.Generator(device="cuda").manual_seed(1)
     cfg = etr.make_config(T=max(8, cap), d=d, D=1, E=E, k=1, h=h, capacity=cap, dtype=etr.BF16, mode=etr.MODE_TCR,
-                          gemm_impl=impl, grad_fp32=grad_fp32)
+                          gemm_impl=impl, grad_fp32=grad_fp32, wait_limit_cycles=wait_limit_cycles)
     assert etr.validate(cfg) == etr.OK
     b = etr.LayerBuffers(cfg)
     b.block.fill_(0xFF)                                      # NaN wherever nothing is written
