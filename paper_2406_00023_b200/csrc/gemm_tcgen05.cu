@@ -667,8 +667,9 @@ __device__ __forceinline__ bool tile_coord_pair(const TcParams& p, const int* ti
 constexpr int DSW_BOX_MAX_K = 2048;
 constexpr uint32_t DSW_BOX = 32 * 64, DSW_SLOT = 2 * DSW_BOX;      // G and U of a chunk
 struct DswMaps { CUtensorMap G, U, dG, dU; };
-// Ring and epilogue space of the pair form, and behind them what would otherwise be static shared memory: without any, the
-// dynamic block starts at a multiple of 1024, and five stages, the boxes and this are all a CTA may have.
+// Ring and epilogue space of the pair form, and behind them what would otherwise be static shared memory.  The swizzled boxes
+// want a multiple of 1024: the kernel declares its dynamic block so, instead of rounding the address up as the other forms do,
+// for which five stages, the boxes and this leave no room.
 template <int EPI> struct PairRing {
   static constexpr int STAGES = EPI == TC_EPI_DSWIGLU_BOX ? 5 : TC2_STAGES;
   static constexpr uint32_t TAIL = STAGES * TC2_STAGE_BYTES + (EPI == TC_EPI_DSWIGLU_BOX ? 8 * 2 * DSW_SLOT : 8 * TC_SCRATCH_BYTES);
@@ -680,7 +681,6 @@ struct PairShared {
   int tile_prefix[257];
   int counts[256];           // the experts' row counts, read from global memory once
 };
-constexpr size_t PAIR_SLACK = 768;
 __device__ __forceinline__ uint32_t dsw_addr(uint32_t box, int lane, int c) {      // 16-byte piece c of this lane's row
   return box + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4);
 }
@@ -716,9 +716,9 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
   const bool A_MN = CFG < 0 ? p.a_mn != 0 : (CFG & 1) != 0, B_MN = CFG < 0 ? p.b_mn != 0 : (CFG & 2) != 0;
   const bool DUAL_B = CFG < 0 ? p.dual_b != 0 : (CFG & 4) != 0, TWO_K = CFG < 0 ? p.k1_blocks > 0 : (CFG & 8) != 0;
 
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  PairShared& sh = *reinterpret_cast<PairShared*>(smem_raw + (tiles_base - smem_u32(smem_raw)) + PairRing<EPI>::TAIL);
+  extern __shared__ __align__(1024) uint8_t pair_smem[];
+  const uint32_t tiles_base = smem_u32(pair_smem);
+  PairShared& sh = *reinterpret_cast<PairShared*>(pair_smem + PairRing<EPI>::TAIL);
   uint64_t* bars = sh.bars;
   uint32_t& tmem_base_slot = sh.tmem_base_slot;
   int& abort_flag_s = sh.abort_flag;
@@ -875,7 +875,7 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
   } else {
     // ---- epilogue warps (both CTAs, own 128 rows) -----------------------------------------------------
     const int q = warp & 3;
-    uint8_t* scratch = smem_raw + (tiles_base - smem_u32(smem_raw)) + STAGES * TC2_STAGE_BYTES + (warp - 2) * TC_SCRATCH_BYTES;
+    uint8_t* scratch = pair_smem + STAGES * TC2_STAGE_BYTES + (warp - 2) * TC_SCRATCH_BYTES;
     const int half = (warp - 2) >> 2;
     constexpr int NCH = N_TILE_COLS / 32 / 2;
     const int row_in_tile = 128 * (int)rank + 32 * q + lane;
@@ -2128,7 +2128,7 @@ template <int EPI, int GATHER, int CFG>
 static etr_status tc_launch_pair_cfg(const char* name, const CUtensorMap& a0, const CUtensorMap& a1,
                                  const CUtensorMap& b0, const CUtensorMap& b1, TcParams p, int max_tiles,
                                  cudaStream_t st) {
-  constexpr size_t smem = PairRing<EPI>::TAIL + sizeof(PairShared) + PAIR_SLACK;
+  constexpr size_t smem = PairRing<EPI>::TAIL + sizeof(PairShared);
   static_assert(smem <= 232448 && 2 * PairRing<EPI>::STAGES + 4 + (EPI == TC_EPI_DSWIGLU_BOX ? 16 : 0) <= 30, "shared memory of a CTA");
   auto k = tc_grouped_gemm_pair_kernel<EPI, GATHER, CFG>;
   static std::atomic<unsigned long long> attr_done{0};      // one bit per device

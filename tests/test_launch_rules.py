@@ -46,3 +46,25 @@ def test_overlapped_launches(name):
 def test_the_kernels_are_found():
     names = [k for f in SOURCES for k, _, _ in kernels(text(f))]
     assert len(names) >= 30 and "tc_grouped_gemm_swap_kernel" in names and "combine_kernel" in names
+
+
+TILED = [f for f in SOURCES if re.search(r"extern __shared__ [^;]*uint8_t", text(f))]
+
+
+@pytest.mark.parametrize("name", TILED)
+def test_tiles_start_at_a_multiple_of_1024(name):
+    """The dynamic shared memory of a kernel with swizzled tiles is declared so aligned and its address taken as it is, or the
+    address is rounded up and the launch asks for the 1024 bytes that this may skip."""
+    src = text(name)
+    rounds = []
+    for kernel, _, body in kernels(src):
+        block = re.search(r"extern __shared__ ([^;]*)uint8_t", body)
+        if block:
+            rounds.append("1023u" in body)
+            assert rounds[-1] != ("__align__(1024)" in block.group(1)), kernel
+    sizes = re.findall(r"constexpr size_t (?:smem|\w+_SMEM) = ([^;]*);", src)
+    assert len(sizes) == len(rounds) and sum("+ 1024" in s for s in sizes) == sum(rounds)
+
+
+def test_the_tiled_kernels_are_found():
+    assert TILED == ["gemm_tcgen05.cu", "gemm_tf32x3.cu", "score_tcgen05.cu"]
