@@ -57,7 +57,7 @@ template <> struct Raw16<float> {                  // 4 elements
 // 8 independent pieces per lane before any is consumed, so one warp keeps 4 KiB in flight.
 // Out-of-range groups re-read the lane's first group and are discarded (no predicated loads).
 template <class T, int PPG>
-__device__ inline float pool_groups(const T* __restrict__ x, float* __restrict__ zrow, int m, int lane,
+__device__ inline float pool_groups(const T* x, float* __restrict__ zrow, int m, int lane,
                                     float invD) {
   constexpr int GB = PPG >= 8 ? 1 : 8 / PPG;      // groups per batch
   constexpr int D = Raw16<T>::ELEMS * PPG;
@@ -85,7 +85,7 @@ __device__ inline float pool_groups(const T* __restrict__ x, float* __restrict__
 
 // Pools one token row into zrow[0..m) (lane-strided) and returns this lane's share of ||x||^2.
 template <class T>
-__device__ inline float pool_token_partial(const T* __restrict__ x, float* __restrict__ zrow, int d,
+__device__ inline float pool_token_partial(const T* x, float* __restrict__ zrow, int d,
                                            int D, int m, int lane) {
   const float invD = 1.0f / (float)D;
   constexpr int PE = Raw16<T>::ELEMS;
@@ -128,7 +128,7 @@ __device__ inline float pool_token_partial(const T* __restrict__ x, float* __res
 }
 
 template <class T>
-__device__ inline void pool_token(const T* __restrict__ x, float* __restrict__ zrow, int d, int D,
+__device__ inline void pool_token(const T* x, float* __restrict__ zrow, int d, int D,
                                   int m, int lane, float& sumsq) {
   sumsq = warp_sum(pool_token_partial<T>(x, zrow, d, D, m, lane));
 }
@@ -768,12 +768,12 @@ constexpr int DXC_ROWS = 512;          // row entries held in shared memory; lat
 // are still added in list order (same sums, bit for bit, as a loop per token).  Entries beyond the
 // staged ones (DXC_ROWS) are read in place.
 __device__ __forceinline__ void dx_chunk_cz(float* __restrict__ cz, float* __restrict__ s_beta,
-                                            const int* __restrict__ s_ptr, const int* __restrict__ s_exp,
-                                            const float* __restrict__ s_w, const float* __restrict__ s_dg,
-                                            const float* __restrict__ s_dl, const float* __restrict__ s_a,
-                                            const float* __restrict__ R, const float* __restrict__ rnorm,
-                                            const float* __restrict__ delta, const float* __restrict__ dgate,
-                                            const int32_t* __restrict__ tok_row, int base, int staged_max,
+                                            const int* s_ptr, const int* s_exp,
+                                            const float* s_w, const float* s_dg,
+                                            const float* s_dl, const float* s_a,
+                                            const float* R, const float* rnorm,
+                                            const float* delta, const float* dgate,
+                                            const int32_t* tok_row, int base, int staged_max,
                                             int nt, int m, int E, int C_stride, int t0, float sqD, int D,
                                             int tid) {
   for (int j = tid; j < m; j += 256) {

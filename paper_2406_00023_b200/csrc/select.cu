@@ -272,7 +272,7 @@ select_threshold_limit_kernel(const uint32_t* keyT, int32_t* __restrict__ limit,
 constexpr int SEL_KPT = 4;
 constexpr int SEL_SWEEP = 1024 * SEL_KPT;
 
-__device__ __forceinline__ void load_keys(const uint32_t* __restrict__ row, int t0, int T, uint32_t* k) {
+__device__ __forceinline__ void load_keys(const uint32_t* row, int t0, int T, uint32_t* k) {
 #pragma unroll
   for (int u = 0; u < SEL_KPT; ++u) k[u] = t0 + u < T ? row[t0 + u] : 0u;
 }

@@ -29,6 +29,7 @@ def kernels(src):
 def test_overlapped_launches(name):
     src = text(name)
     assert "__ldg" not in src and "ld.global.nc" not in src
+    assert not re.search(r"const\s+\w+\s*\*\s*(const\s+)?__restrict__", src)      # functions called by kernels too
     for kernel, params, body in kernels(src):
         assert not re.search(r"const\s+\w+\s*\*\s*(const\s+)?__restrict__", params), kernel
         if re.search(kernel + r"\s*<<<", src):
