@@ -95,27 +95,40 @@ def test_group_sizes(D, dtype):
     layer_vs_oracle(w, gw.make_inputs(w), ob.MODE_TCR)
 
 
-@pytest.mark.parametrize("dtype", ["bf16", "f32"])
-def test_tokens_kept_by_every_expert_overflow_the_staged_row_lists(dtype):
-    """Expert choice with C = T and 128 experts: every token has 128 rows, so the chunks of 8
-    (combine) and 16 (fused dX) consecutive tokens hold 1024 and 2048 row entries, more than the
-    512 those kernels stage in shared memory: the entries beyond are read in place.  T = 40 also
-    leaves a ragged last chunk in both."""
-    w = gw.scaled(W["small"], T=40, d=1024, D=8, E=128, h=64, cf=64.0, dtype=dtype)
+@pytest.mark.parametrize("T,E,d,D,h,dtype", [
+    (40, 128, 1024, 8, 64, "bf16"), (40, 128, 1024, 8, 64, "f32"),
+    (2400, 72, 584, 8, 8, "f32"),                            # 576 entries a block in both kernels
+    (4747, 40, 320, 8, 64, "bf16"), (4747, 40, 328, 8, 8, "f32"), (4747, 40, 168, 4, 8, "f32"),      # R gathered beside the rows
+    (4747, 40, 200, 5, 8, "f32"),                            # any other group size: through shared memory
+])
+def test_tokens_kept_by_every_expert_overflow_the_staged_row_lists(T, E, d, D, h, dtype):
+    """Expert choice with C = T: every token has a row of every expert.  The combine kernel takes up to 8 tokens a block and the
+    fused dX kernel up to 16, as many as leave every SM two blocks, and each stages 512 row entries in shared memory: the
+    entries beyond are read in place.  2400 tokens: 8 a block in both.  4747: 16 in dX, the last block 11.  40 tokens are one
+    and two a block, whose 128 and 256 entries fit.  (The router's part of dX, which the entries beyond enter in two ways, is
+    over half of dX here.)"""
+    w = gw.scaled(W["small"], T=T, d=d, D=D, E=E, h=h, cf=E / 2, dtype=dtype)
     assert w.capacity == w.T
+    if T > 40:
+        two_a_sm = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+        assert (T // 8 >= two_a_sm and 8 * E > 512) or (T // 16 >= two_a_sm and 16 * E > 512)
     fw, got, out = layer_vs_oracle(w, gw.make_inputs(w), ob.MODE_ECR)
     assert np.all(np.diff(got.tok_ptr) == w.E)
 
 
-@pytest.mark.parametrize("d,D,dtype", [(2048, 16, "bf16"), (2048, 4, "bf16"), (2048, 8, "f32"), (4096, 32, "bf16"),
-                                       (8192, 64, "bf16")])
-def test_fused_dx_at_wide_hidden_sizes(d, D, dtype):
-    """Hidden sizes of 2048, 4096 and 8192 in the fused dX kernel (whole 4 to 16 KiB rows per token and
-    row of dXp), power-of-two and generic group sizes, a ragged last chunk of tokens (T = 215 =
-    13 * 16 + 7), and expert choice with C = T / 4, which gives tokens anything from no row (zeros,
-    X not read) to the rows of most of the 16 experts, so that one chunk's flat list of row entries
-    crosses many token boundaries."""
-    w = gw.scaled(W["small"], T=215, d=d, D=D, E=16, h=64, cf=2.0, dtype=dtype)
+@pytest.mark.parametrize("d,D,dtype,T,C", [
+    (2048, 16, "bf16", 215, 54), (2048, 4, "bf16", 215, 54), (2048, 8, "f32", 215, 54), (4096, 32, "bf16", 215, 54),
+    (8192, 64, "bf16", 215, 54),
+    # capacities whose cuts leave at least 1e-5 between the last affinity kept and the first one not
+    (512, 8, "bf16", 4747, 1042), (512, 4, "f32", 4747, 1114), (512, 2, "bf16", 4747, 1177),
+])
+def test_fused_dx_at_wide_hidden_sizes(d, D, dtype, T, C):
+    """Hidden sizes of 2048, 4096 and 8192 in the fused dX kernel (whole 4 to 16 KiB rows per token and row of dXp),
+    power-of-two and generic group sizes, and expert choice with C of about T / 4, which gives tokens anything from no row
+    (zeros, X not read) to the rows of most of the 16 experts.  215 tokens are two a block, the last one alone; 4747 are 16 a
+    block (the last 11), whose list of row entries crosses many token boundaries."""
+    w = gw.scaled(W["small"], T=T, d=d, D=D, E=16, h=64, cf=(C - 0.5) * 8 / T, dtype=dtype)
+    assert w.capacity == C
     fw, got, out = layer_vs_oracle(w, gw.make_inputs(w), ob.MODE_ECR)
     n = np.diff(got.tok_ptr)
     assert n.min() == 0 and n.max() >= 6 and n.sum() > 3 * w.T
