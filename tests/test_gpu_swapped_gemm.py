@@ -1,7 +1,8 @@
 """The bf16 grouped GEMMs with the weights as the M operand and the tokens as N, stage by stage: row counts around
 the 16-row steps and the 256-row tiles, column counts that end inside a tile, every size of token box, all four
 epilogues, against 64-bit products of the same bf16 inputs, and bit for bit against the CTA-pair form; beside them the
-weight gradients (always the pair form) in bf16 and in fp32, whose buffers start as NaN: experts without rows included.
+weight gradients (one launch of their own in both) against the same products and bit for bit against the single-CTA form, in
+bf16 and in fp32, whose buffers start as NaN: experts without rows included.
 
 Tolerance (relative 2-norm): an output is one rounding to bf16, at most 2^-8 of a value and 1.66e-3 in the root mean
 square; the fp32 sums are three orders below.  2.5e-3 leaves room for small blocks, whose rms scatters.  fp32 gradients
@@ -57,9 +58,10 @@ def run(E, d, h, cap, counts, impl, grad_fp32=False, wait_limit_cycles=0):
 ])
 def test_stages(E, d, h, cap, counts):
     b, W, Cs, dW = run(E, d, h, cap, counts, etr.GEMM_AUTO)
-    p, _, _, dWp = run(E, d, h, cap, counts, etr.GEMM_TCGEN05_2CTA)
+    p, *_ = run(E, d, h, cap, counts, etr.GEMM_TCGEN05_2CTA)
+    *_, dWs = run(E, d, h, cap, counts, etr.GEMM_TCGEN05)
     f, _, _, dWf = run(E, d, h, cap, counts, etr.GEMM_AUTO, grad_fp32=True)
-    assert all(torch.equal(u, v) for u, v in zip(dW, dWp)) and all(torch.equal(u, v.bfloat16()) for u, v in zip(dW, dWf))
+    assert all(torch.equal(u, v) for u, v in zip(dW, dWs)) and all(torch.equal(u, v.bfloat16()) for u, v in zip(dW, dWf))
     for i, n in enumerate(counts):
         pad = (n + 127) // 128 * 128
         x, G, U, H, O, dO, dG, dU, dXp = (t.view(E, Cs, -1)[i].double() for t in
