@@ -652,11 +652,10 @@ __device__ __forceinline__ bool tile_coord_pair(const TcParams& p, const int* ti
   return true;
 }
 
-// GATHER is TcParams::gather, and CFG the operand modes (a_mn, b_mn, dual_b, two K ranges), as
+// GATHER is TcParams::gather, and CFG the operand modes (bit 0 a_mn, 1 b_mn, 2 dual_b, 3 two K ranges), as
 // compile-time constants: the single-lane producer and MMA loops are on the kernel's critical path,
 // and run-time branches cost there even when not taken (6-8 % of a GEMM for the operand modes,
-// 10 % per gather branch).  CFG = -1 keeps the run-time forms for combinations without an
-// instantiation of their own.
+// 10 % per gather branch).
 // A second epilogue of the SwiGLU derivative (TC_EPI_DSWIGLU_BOX): G and U of a chunk of 32 columns come by TMA into a box of
 // the warp's own (32 rows of 64 bytes each, 64-byte swizzle), a lane turns its row into dG and dU in place, and TMA stores the
 // boxes.  Two boxes of each per warp: a chunk's load passes under the chunk before.  The other one fetches and stores through a
@@ -712,9 +711,7 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
   constexpr int N_TILE_COLS = (EPI == TC_EPI_SWIGLU) ? BN / 2 : BN;
   constexpr uint32_t TMEM_COLS = 512;
   constexpr int STAGES = PairRing<EPI>::STAGES;
-  // operand modes as compile-time constants when CFG >= 0 (bit 0 a_mn, 1 b_mn, 2 dual_b, 3 two K ranges)
-  const bool A_MN = CFG < 0 ? p.a_mn != 0 : (CFG & 1) != 0, B_MN = CFG < 0 ? p.b_mn != 0 : (CFG & 2) != 0;
-  const bool DUAL_B = CFG < 0 ? p.dual_b != 0 : (CFG & 4) != 0, TWO_K = CFG < 0 ? p.k1_blocks > 0 : (CFG & 8) != 0;
+  constexpr bool A_MN = (CFG & 1) != 0, B_MN = (CFG & 2) != 0, DUAL_B = (CFG & 4) != 0, TWO_K = (CFG & 8) != 0;
 
   extern __shared__ __align__(1024) uint8_t pair_smem[];
   const uint32_t tiles_base = smem_u32(pair_smem);
@@ -835,7 +832,7 @@ tc_grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __g
         // whose last 16-wide steps may hold pad rows only: that block is peeled off the loop and runs
         // just the steps with rows in use (the skipped ones would add zeros).  The loop itself stays
         // free of the test: anything extra in it shows in the GEMM time.
-        constexpr bool PEEL = CFG < 0 || CFG == 3;
+        constexpr bool PEEL = CFG == 3;
         const int nloop = PEEL ? tc.kblocks - 1 : tc.kblocks;
         for (int kb = 0; kb < nloop; ++kb) {
           if (!mbar_wait_cluster(full_bar + 8 * stage, phase, abort_flag, p.wait_limit)) { ok = false; break; }
@@ -1068,9 +1065,7 @@ tc_grouped_gemm_pair_wide_kernel(const __grid_constant__ CUtensorMap mapA0, cons
   constexpr int BN = 256;
   constexpr int N_TILE_COLS = (EPI == TC_EPI_SWIGLU) ? BN / 2 : BN;
   constexpr uint32_t TMEM_COLS = 512;
-  // operand modes as compile-time constants when CFG >= 0 (bit 0 a_mn, 1 b_mn, 2 dual_b, 3 two K ranges)
-  const bool A_MN = CFG < 0 ? p.a_mn != 0 : (CFG & 1) != 0, B_MN = CFG < 0 ? p.b_mn != 0 : (CFG & 2) != 0;
-  const bool DUAL_B = CFG < 0 ? p.dual_b != 0 : (CFG & 4) != 0, TWO_K = CFG < 0 ? p.k1_blocks > 0 : (CFG & 8) != 0;
+  constexpr bool A_MN = (CFG & 1) != 0, B_MN = (CFG & 2) != 0, DUAL_B = (CFG & 4) != 0, TWO_K = (CFG & 8) != 0;
 
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bars[2 * TCW_STAGES + 3];
@@ -2168,30 +2163,31 @@ static etr_status tc_launch_pair_wide_cfg(const char* name, const CUtensorMap& a
 }
 
 
-// The operand modes each epilogue is used with get their own instantiation; anything else runs the
-// generic one (CFG = -1).
+// An instantiation for each set of operand modes that an epilogue is used with: one of SwiGLU and its derivative; of plain
+// stores the down GEMM, dXp, and weight gradients (of gathered rows in the pair form, forced by gemm_impl in the wide one).
+static int tc_cfg(const TcParams& p) { return (p.a_mn ? 1 : 0) | (p.b_mn ? 2 : 0) | (p.dual_b ? 4 : 0) | (p.k1_blocks > 0 ? 8 : 0); }
 template <int EPI, int GATHER>
 static etr_status tc_launch_pair(const char* name, const CUtensorMap& a0, const CUtensorMap& a1,
-                                 const CUtensorMap& b0, const CUtensorMap& b1, TcParams p, int max_tiles,
+                                 const CUtensorMap& b0, const CUtensorMap& b1, const TcParams& p, int max_tiles,
                                  cudaStream_t st) {
-  const int cfg = (p.a_mn ? 1 : 0) | (p.b_mn ? 2 : 0) | (p.dual_b ? 4 : 0) | (p.k1_blocks > 0 ? 8 : 0);
-  constexpr int C0 = EPI == TC_EPI_SWIGLU ? 4 : EPI == TC_EPI_STORE ? 0 : 2;      // first use
-  constexpr int C1 = EPI == TC_EPI_STORE && GATHER == 2 ? 3 : C0, C2 = EPI == TC_EPI_STORE ? 10 : C0;
+  constexpr int C0 = EPI == TC_EPI_SWIGLU ? 4 : EPI != TC_EPI_STORE ? 2 : GATHER == 2 ? 3 : 0;
+  constexpr int C1 = EPI == TC_EPI_STORE && GATHER == 0 ? 10 : C0;
+  const int cfg = tc_cfg(p);
   if (cfg == C0) return tc_launch_pair_cfg<EPI, GATHER, C0>(name, a0, a1, b0, b1, p, max_tiles, st);
   if (cfg == C1) return tc_launch_pair_cfg<EPI, GATHER, C1>(name, a0, a1, b0, b1, p, max_tiles, st);
-  if (cfg == C2) return tc_launch_pair_cfg<EPI, GATHER, C2>(name, a0, a1, b0, b1, p, max_tiles, st);
-  return tc_launch_pair_cfg<EPI, GATHER, -1>(name, a0, a1, b0, b1, p, max_tiles, st);
+  return ETR_ERR_UNSUPPORTED;
 }
 template <int EPI, int GATHER>
 static etr_status tc_launch_pair_wide(const char* name, const CUtensorMap& a0, const CUtensorMap& a1,
-                                      const CUtensorMap& b0, const CUtensorMap& b1, TcParams p, int max_tiles,
+                                      const CUtensorMap& b0, const CUtensorMap& b1, const TcParams& p, int max_tiles,
                                       cudaStream_t st) {
-  const int cfg = (p.a_mn ? 1 : 0) | (p.b_mn ? 2 : 0) | (p.dual_b ? 4 : 0) | (p.k1_blocks > 0 ? 8 : 0);
-  constexpr int C0 = EPI == TC_EPI_SWIGLU ? 4 : EPI == TC_EPI_DSWIGLU ? 2 : 0;
-  constexpr int C2 = EPI == TC_EPI_STORE ? 10 : C0;
+  constexpr int C0 = EPI == TC_EPI_SWIGLU ? 4 : EPI != TC_EPI_STORE ? 2 : 0;
+  constexpr int C1 = EPI == TC_EPI_STORE ? 10 : C0, C2 = EPI == TC_EPI_STORE ? 3 : C0;
+  const int cfg = tc_cfg(p);
   if (cfg == C0) return tc_launch_pair_wide_cfg<EPI, GATHER, C0>(name, a0, a1, b0, b1, p, max_tiles, st);
+  if (cfg == C1) return tc_launch_pair_wide_cfg<EPI, GATHER, C1>(name, a0, a1, b0, b1, p, max_tiles, st);
   if (cfg == C2) return tc_launch_pair_wide_cfg<EPI, GATHER, C2>(name, a0, a1, b0, b1, p, max_tiles, st);
-  return tc_launch_pair_wide_cfg<EPI, GATHER, -1>(name, a0, a1, b0, b1, p, max_tiles, st);
+  return ETR_ERR_UNSUPPORTED;
 }
 
 // The three forms of one contraction; max_tiles is an upper bound counted in 128-row tiles of one

@@ -17,8 +17,8 @@ pytestmark = pytest.mark.gpu
     (2, 192, 320, 17, (17, 16)),                             # of 32; last column tiles of 64 and 192 columns
     (2, 320, 128, 33, (33, 32)),                             # of 64, the last one with one row
     (4, 256, 640, 200, (200, 0, 65, 129)),                   # whole tiles and a last one of 128 columns
-    (40, 576, 256, 300, tuple((53 * i) % 301 for i in range(40))),      # more tiles than pairs, three and more per pair
-    (2, 1984, 64, 260, (260, 257)),                          # the longest derivative that goes through boxes
+    (40, 576, 256, 300, tuple((53 * i) % 301 for i in range(40))),      # 360 tiles of gradients, four and five a pair
+    (2, 1984, 64, 260, (260, 257)),                          # the longest derivative that goes through boxes (4 tiles)
     (2, 2048, 64, 260, (260, 257)),                          # the shortest that does not
 ])
 def test_against_the_single_cta_form(E, d, h, cap, counts, grad_fp32):
