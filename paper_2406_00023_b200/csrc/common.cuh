@@ -36,10 +36,6 @@ void timing_end(cudaStream_t st);
 //   - A kernel waits (grid_wait) before its first access to global memory: the kernel before it is then complete and
 //     its writes are visible.  Only after that wait does it let the next kernel in (grid_release), so never more than two
 //     kernels of a stream are in flight, and a kernel sees the writes of all kernels before it.
-//   - One exception: the tensor-core score kernel reads R before it waits (the norms of up to 32 experts).  R is an input of
-//     the call, the kernel before is always the pooling of the same call (affinity_forward_split launches the two back to
-//     back), and that one writes no R and lets the score kernel in only behind its own wait: whatever wrote R is complete.
-//     Nothing may be launched between the two.
 //   - Inputs are plain `const` pointers, not `const __restrict__`, and never read by __ldg: the compiler may send such reads
 //     through the read-only path, which asks for memory that nobody writes during the kernel's lifetime, and that
 //     lifetime begins while the kernel before it still writes.  (Outputs are `__restrict__`: that orders nothing away.)

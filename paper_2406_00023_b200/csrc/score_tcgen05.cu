@@ -101,37 +101,6 @@ affinity_score_tc_kernel(const __grid_constant__ CUtensorMap mapZ, const __grid_
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(SCT_TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  // ||R_i|| by the epilogue warps, a warp per row, lanes over the columns, the same sums as the other score kernels (eight
-  // columns per lane and four rows requested together).  With up to 32 experts before the wait: the kernel before this one is
-  // always the pooling of the same call, which does not write R and had waited itself, so whatever did write R is complete.
-  // More rows take longer than that kernel leaves: behind the wait, while the first tile is on its way.
-  // Together with half of the epilogue left out there: 9.0 -> 7.2 us (64 tokens, E 16, m 128), 8.5 -> 5.6 (512, E 8, m 64), 12.1 -> 9.7
-  // (6113, E 32, m 256); with 64 experts before the wait instead 10.1 -> 11.7 (300 tokens).
-  auto norms = [&]() {
-    for (int i0 = warp & 3; i0 < E; i0 += 16) {
-      float sq[4] = {0.f, 0.f, 0.f, 0.f};
-      for (int j0 = lane; j0 < m; j0 += 256) {
-        float v[4][8];
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int u = 0; u < 8; ++u)
-            v[r][u] = i0 + 4 * r < E && j0 + 32 * u < m ? R[(size_t)(i0 + 4 * r) * m + j0 + 32 * u] : 0.f;
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int u = 0; u < 8; ++u) sq[r] += v[r][u] * v[r][u];
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const float acc_q = warp_sum(sq[r]);
-        if (lane == 0) rn[i0 + 4 * r] = sqrtf(acc_q);
-      }
-    }
-  };
-  const bool early = E <= 32;
-  if (early && warp >= 6) norms();
-  __syncwarp();
   grid_wait();
   tc_fence_before();
   __syncthreads();
@@ -222,10 +191,31 @@ affinity_score_tc_kernel(const __grid_constant__ CUtensorMap mapZ, const __grid_
     // ---- epilogue warps: a lane owns a token --------------------------------------------------------------
     const int q = warp & 3;                      // tensor-memory lanes 32 q .. 32 q + 31
     float* stg = reinterpret_cast<float*>(tiles + (size_t)SCT_STAGES * SCT_STAGE_BYTES) + (warp - 6) * 32 * 33;
-    if (!early) {
-      norms();
-      asm volatile("bar.sync 1, 128;" ::: "memory");      // the four epilogue warps: rn is complete
+    // ||R_i|| while the first tile is on its way: a warp per row, lanes over the columns, the same sums as the other score
+    // kernels (eight columns per lane and four rows requested together; a row at a time is a round of L2 latency each).
+    // Before the wait, under the pooling's last blocks, they cost more than they hid: the affinity call 7.4 -> 8.2 us (64 tokens,
+    // E 16, m 128), 6.3 -> 7.0 (512, E 8, m 64), 13.6 both (6113, E 32, m 256), 18.6 -> 19.8 (16384, the same).
+    for (int i0 = q; i0 < E; i0 += 16) {
+      float sq[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int j0 = lane; j0 < m; j0 += 256) {
+        float v[4][8];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            v[r][u] = i0 + 4 * r < E && j0 + 32 * u < m ? R[(size_t)(i0 + 4 * r) * m + j0 + 32 * u] : 0.f;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int u = 0; u < 8; ++u) sq[r] += v[r][u] * v[r][u];
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float acc_q = warp_sum(sq[r]);
+        if (lane == 0) rn[i0 + 4 * r] = sqrtf(acc_q);
+      }
     }
+    asm volatile("bar.sync 1, 128;" ::: "memory");      // the four epilogue warps: rn is complete
     if (blockIdx.x == 0 && tid - 192 < E) rnorm[tid - 192] = rn[tid - 192];      // 128 threads, E <= 64
     int acc = 0;
     uint32_t acc_phase = 0;
@@ -237,7 +227,9 @@ affinity_score_tc_kernel(const __grid_constant__ CUtensorMap mapZ, const __grid_
       if (!mbar_wait(tfull_bar + 8 * acc, acc_phase, abort_flag, wait_limit)) { ok = false; break; }
       tc_fence_after();
       const uint32_t taddr = tmem_base + (uint32_t)(acc * SCT_CHAINS * SCT_N) + ((uint32_t)(32 * q) << 16);
-      // Half of the expert columns at a time (the upper half only where there are that many experts): the chains' partial
+      // Half of the expert columns at a time, the upper half only where there are that many experts (against both at once and
+      // always, the affinity call: 10.0 -> 7.4 us at 64 tokens, E 16, m 128; 9.6 -> 6.3 at 512, E 8, m 64; 15.6 -> 13.6 at 6113,
+      // E 32, m 256; 12.8 -> 12.4 at 300, E 64, m 256; 142.1 -> 141.9 at 65536, the same): the chains' partial
       // sums added in order, then delta = sqrt(D) s / (||x|| ||R_i||), 0 where a norm is 0.  A fast division (reciprocal and
       // product, 2 ulp) taken unconditionally and selected afterwards: correctly rounded divisions, each behind its own zero
       // test, overlapped with nothing and were the longest stage of the kernel; the result is compared at 1e-5, not to the

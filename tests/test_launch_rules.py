@@ -48,7 +48,7 @@ def test_overlapped_launches(name):
             assert not re.search(r"\bp\.\w+\[|stats->|\w+\[", re.sub(r"__shared__[^;]*;", "", body[:first])), kernel
             continue
         early = global_reads(params, body[:body.index("grid_wait();")])
-        assert early == ({"R"} if kernel == "affinity_score_tc_kernel" else set()), kernel
+        assert not early, kernel
         order = [body.index(s) for s in ("tcgen05.alloc", "grid_wait();", "__syncthreads();", "grid_release();")]
         assert order == sorted(order) and "grid_sync" not in body, kernel
         if "tcgen05.dealloc.cta_group::2" in body:           # the pair leaves together
@@ -58,27 +58,6 @@ def test_overlapped_launches(name):
 def test_the_kernels_are_found():
     names = [k for f in SOURCES for k, _, _ in kernels(text(f))]
     assert len(names) >= 30 and "tc_grouped_gemm_swap_kernel" in names and "combine_kernel" in names
-
-
-def test_the_score_kernel_reads_r_early_because_pooling_comes_directly_before():
-    """R before the wait is sound as long as the kernel before is the pooling of the same call: it waits for all that came
-    before it, which is whatever wrote R, and writes no R itself."""
-    src = text("affinity.cu")
-    calls = [(f, m.start()) for f in SOURCES for m in re.finditer(r"(?<!etr_status )\baffinity_score_tc\(", text(f))]
-    assert [f for f, _ in calls] == ["affinity.cu"]
-    before = src[:calls[0][1]]
-    between = before[before.rindex("launch_pool<float>("):]
-    assert not re.search(r"launch_kernel|<<<|cuda[A-Z]\w+\(|launch_(?!pool)\w+|return", between), between
-    assert re.search(r"if \(c->dtype == ETR_BF16\) ETR_TRY\(launch_pool<__nv_bfloat16>\([^;]*;\s*else ETR_TRY\(\s*$",
-                     before[:before.rindex("launch_pool<float>(")])      # one of the two, always
-    pool = next((p, b) for k, p, b in kernels(src) if k == "grap_pool_kernel")
-    assert not re.search(r"\bR\b", pool[0]) and pool[1].lstrip().startswith("grid_sync();")
-    launch = src[src.index("static etr_status launch_pool("):]
-    launch = launch[:launch.index("\n}")]
-    assert set(re.findall(r"launch_kernel\((\w+)", launch)) == {"grap_pool_kernel"} and "<<<" not in launch
-    score = text("score_tcgen05.cu")
-    body = score[score.rindex("etr_status affinity_score_tc("):]
-    assert body.count("launch_kernel(") == 1 and not re.search(r"<<<|cudaMem|cudaStream[A-Z]", body)
 
 
 TILED = [f for f in SOURCES if re.search(r"extern __shared__ [^;]*uint8_t", text(f))]
