@@ -38,18 +38,18 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu captures summarised
 # under profiles/ (absent: not captured for the current version of that kernel).
 NCU_TRAFFIC_BYTES = {}
-# The grouped GEMMs of one step at the mid workload (d = 2048)
-# (profiles/tc_grouped_gemm_mid_ncu.md): 3636.2 MB of DRAM traffic against 3799.7 MB of algorithmic bytes
+# The five tensor-core launches of one step at the mid workload (d = 2048, 1024 rows per expert, the forms AUTO launches;
+# profiles/tc_grouped_gemm_mid_ncu.md): 3576.1 MB of DRAM traffic against 3665.8 MB of algorithmic bytes
 # (part of the output is still in L2 when a kernel ends).  The large workload is too big for a
 # multi-pass capture, so its traffic is this ratio times its own algorithmic bytes.
-TC_GEMM_DRAM_OVER_ALGORITHMIC = 3636.2 / 3799.7
+TC_GEMM_DRAM_OVER_ALGORITHMIC = 3576.1 / 3665.8
 
 
 def tc_gemm_algorithmic_bytes(w, rows_padded):
-    """Bytes the seven contractions of one step must move (bf16): activations once per use, every
-    expert weight once per GEMM that reads it, every output once."""
+    """Bytes the five launches of one step must move (bf16): every activation and every expert weight once per launch
+    that reads it (the launch of the weight gradients reads dO, H, dG, dU and Xp), every output once."""
     ad, ah, wt = rows_padded * w.d * 2, rows_padded * w.h * 2, w.E * w.d * w.h * 2
-    reads = (ad + 2 * wt) + (ah + wt) + (ad + wt + 2 * ah) + (2 * ah + 2 * wt) + (ad + ah) + 2 * (ah + ad)
+    reads = (ad + 2 * wt) + (ah + wt) + (ad + wt + 2 * ah) + (2 * ah + 2 * wt) + (2 * ad + 3 * ah)
     writes = 3 * ah + ad + 2 * ah + ad + wt + 2 * wt
     return reads + writes
 
@@ -554,12 +554,12 @@ def main():
     g = gemm_summary(w, kernels, rows)
     roofline = None
     if g and g["share_of_step"] >= 0.5:
-        # The six tcgen05 contractions run on one persistent grouped-GEMM design in several tile forms
-        # (--gemm can force one); the roofline entry covers all their launches.  The ncu traffic ratio was
+        # The tcgen05 contractions run on one persistent grouped-GEMM design in several tile forms, the weight gradients
+        # on a kernel of their own (--gemm can force a form); the roofline entry covers all their launches.  The ncu traffic ratio was
         # taken with the library's own choice at d = 2048; narrower layers take other forms.
         pair = args.gemm == "auto" and w.d >= 2048
-        kname = {"auto": "tc_grouped_gemm_*_kernel (form chosen per contraction)",
-                 "tcgen05_2cta": "tc_grouped_gemm_pair_kernel", "tcgen05_2cta_wide": "tc_grouped_gemm_pair_wide_kernel",
+        kname = {"auto": "tc_grouped_gemm_*_kernel (form chosen per contraction), tc_wgrad_pair_kernel",
+                 "tcgen05_2cta": "tc_grouped_gemm_pair_kernel, tc_wgrad_pair_kernel", "tcgen05_2cta_wide": "tc_grouped_gemm_pair_wide_kernel",
                  "tcgen05": "tc_grouped_gemm_kernel"}.get(args.gemm, "tc_grouped_gemm")
         roofline = {"kernel": kname, "launches_per_step": g["launches_per_step"], "bound": "tensor",
                     "achieved": g["tflops"], "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
