@@ -155,13 +155,13 @@ grap_pool_kernel(const T* X, float* __restrict__ Z, float* __restrict__ xnorm,
   float sq = 0.f;
   if (PPG > 0) {
     const float invD = 1.0f / (float)D;
-    const int npieces = m * PPG;
+    const int npieces = m * PPG, in_row = min(lane, npieces - 1);      // a row may have fewer pieces than the warp lanes
     for (int p0 = 0; p0 < npieces; p0 += 32 * BATCH) {
       Raw16<T> q[BATCH];
 #pragma unroll
       for (int g = 0; g < BATCH; ++g) {
         const int p = p0 + 32 * g + lane;
-        q[g].load(x + (size_t)(p < npieces ? p : lane) * PE);
+        q[g].load(x + (size_t)(p < npieces ? p : in_row) * PE);
       }
       asm volatile("" ::: "memory");      // no load moves behind the stores below
 #pragma unroll

@@ -80,3 +80,19 @@ def test_tiles_start_at_a_multiple_of_1024(name):
 
 def test_the_tiled_kernels_are_found():
     assert TILED == ["gemm_tcgen05.cu", "gemm_tf32x3.cu", "score_tcgen05.cu"]
+
+
+def test_pooling_reads_stay_inside_the_row():
+    """The pooling kernel loads without predicates: a piece beyond the row is replaced by one of the row's own.  Every lane and
+    batch of rows of 1 to 600 pieces of 16 bytes (a row of 64 bf16 values has 8, fewer than the lanes of a warp)."""
+    body = next(b for k, _, b in kernels(text("affinity.cu")) if k == "grap_pool_kernel")
+    batch = int(re.search(r"constexpr int BATCH = (\d+);", body).group(1))
+    cond, there, else_ = re.search(r"q\[g\]\.load\(x \+ \(size_t\)\((.+?) \? (.+?) : (.+?)\) \* PE\);", body).groups()
+    named = dict(re.findall(r"(\w+) = (min\(lane, npieces - 1\))", body))
+    pick = compile(f"({there}) if ({cond}) else ({named.get(else_, else_)})", "piece", "eval")
+    for npieces in range(1, 601):
+        for p0 in range(0, npieces, 32 * batch):
+            for g in range(batch):
+                for lane in range(32):
+                    at = eval(pick, {"min": min}, {"p": p0 + 32 * g + lane, "lane": lane, "npieces": npieces})
+                    assert 0 <= at < npieces, (npieces, p0, g, lane)
