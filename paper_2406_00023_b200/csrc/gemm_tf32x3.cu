@@ -381,7 +381,12 @@ tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_const
     for (int tile = blockIdx.x; ok && f3_tile<EPI>(p, tile_prefix, s_counts, tile, e_cur, COLS, t); tile += gridDim.x) {
       for (int kb = 0; kb < t.kblocks; ++kb) {
         if (turn == group) {
-          ok = __all_sync(0xffffffffu, mbar_wait(full_bar + 8 * stage, phase, abort_flag, p.wait_limit));
+          // With an odd number of stages the use of this stage before this one is the other group's, and the parity of a
+          // barrier tells its last two uses apart only: were that block still on its way (behind the one after it), the
+          // wait for this one would pass on the parity of the use before.  So that use has to be split first.
+          if (F3_STAGES % 2 != 0)
+            ok = __all_sync(0xffffffffu, mbar_wait(conv_bar + 8 * stage, phase ^ 1u, abort_flag, p.wait_limit));
+          ok = ok && __all_sync(0xffffffffu, mbar_wait(full_bar + 8 * stage, phase, abort_flag, p.wait_limit));
           if (!ok) break;
           uint8_t* st = tiles + (size_t)stage * STAGE;
           uint8_t* sb = st + 2 * A_BYTES;

@@ -96,3 +96,26 @@ def test_pooling_reads_stay_inside_the_row():
                 for lane in range(32):
                     at = eval(pick, {"min": min}, {"p": p0 + 32 * g + lane, "lane": lane, "npieces": npieces})
                     assert 0 <= at < npieces, (npieces, p0, g, lane)
+
+
+@pytest.mark.parametrize("stages", [3, 4])
+def test_the_split_of_fp32_operands_waits_for_the_block_it_takes(stages):
+    """Two groups of converter warps take alternate K blocks of a ring of 3 or 4 stages, and a wait tells the uses of a stage
+    apart by their parity: it passes when the number of completed uses is of the other one.  Over every state that a group
+    may find when it comes to use `u` of a stage (`split`: uses split so far, `landed`: uses whose copy has landed, both only
+    grow), its waits, as the source has them, may pass in turn only when use u has landed."""
+    src = text("gemm_tf32x3.cu")
+    branch = src[src.index("if (turn == group) {"):src.index("f3_split_box<A_MN>(st")]
+    waits = re.findall(r"(if \(F3_STAGES % 2 != 0\)\s+ok = |ok = (?:ok && )?)__all_sync\(0xffffffffu, "
+                       r"mbar_wait\((\w+)_bar \+ 8 \* stage, phase( \^ 1u)?", branch)
+    assert len(waits) == branch.count("mbar_wait(")
+    waits = [(bar, 1 if flip else 0) for cond, bar, flip in waits if stages % 2 or not cond.startswith("if")]
+    for u in range(2, 8):
+        # the group's own last use of the stage, u - 2 or u - 1, is split, this one is not; a stage holds one block
+        states = [(split, landed) for split in range(u - 1 if stages % 2 else u, u + 1) for landed in (split, split + 1)]
+        at = set(states)
+        for bar, flip in waits:
+            done = {"conv": 0, "full": 1}[bar]
+            later = {b for a in at for b in states if b[0] >= a[0] and b[1] >= a[1]}
+            at = {x for x in later if x[done] & 1 != (u ^ flip) & 1}
+        assert at and all(landed > u for _, landed in at), (u, at)
